@@ -24,11 +24,9 @@ cudaError_t walk_tc_prepare(const Geom& G, const Arena& A, int64_t total_rows, v
 void walk_tc_release(void* tmaps);
 bool decode_mma_supported(const Geom& G);
 int decode_mma_ctas_per_sm();
+int decode_mma_tile_tokens();
 cudaError_t decode_mma_prepare(const Geom& G, const Arena& A, int64_t total_rows, void** maps_out);
 void decode_mma_release(void* maps);
-cudaError_t launch_decode_parts_mma(const Geom& G, const Arena& A, int layer, const void* q, float* raw_acc, float* raw_ml,
-                                    float* scratch, int splits, int* status, const void* maps, int keys_only,
-                                    cudaStream_t st);
 cudaError_t launch_decode_parts_mma_slots(const Geom& G, const Arena& A, const int* slot_layers, int n_slots,
                                           unsigned keys_mask, const void* q, float* raw_acc, float* raw_ml, float* scratch,
                                           size_t z_stride_words, int splits, int* status, const void* maps,
@@ -85,7 +83,7 @@ struct balancekv_ctx {
   int decode_slots = 148;        // CTAs of the decode kernel that are resident at once
   bool use_tc = false;
   void* tmaps = nullptr;
-  void* decode_maps = nullptr;   // tensor maps of the tensor-core decode kernel (bf16, d = 128)
+  void* decode_maps = nullptr;   // tensor maps of the tensor-core decode kernel (bf16)
 
   // descriptor ring: two halves of pinned host memory mirrored on the device
   char* h_ring = nullptr;
@@ -740,7 +738,7 @@ static int pick_splits(balancekv_ctx* c, int layer) {
       for (int l = 1; l <= f.levels; ++l) rows += S.lvl_len[l];
       max_rows = std::max(max_rows, rows);
     }
-  const int tile_tokens = 16384 / (f.head_dim * c->esz);
+  const int tile_tokens = c->decode_maps ? decode_mma_tile_tokens() : 16384 / (f.head_dim * c->esz);
   const int64_t tiles = (max_rows + tile_tokens - 1) / tile_tokens + f.levels;
   int splits = (int)std::max<int64_t>(1, std::min<int64_t>(c->max_splits, (tiles + 1) / 2));
   // the fewest splits with the same number of tiles per CTA: the tile phase is as long, the combine shorter
@@ -820,7 +818,7 @@ int balancekv_decode_attn_merged(balancekv_ctx* c, const int32_t* layers_num, in
                                  int n_den, const void* q, void* out, void* stream) {
   if (!c || !q || !out || !layers_num || !layers_den || n_num < 1 || n_den < 1) return BALANCEKV_E_INVAL;
   if (!aligned16(q) || !aligned16(out)) return BALANCEKV_E_INVAL;
-  if (!c->decode_maps) return BALANCEKV_E_INVAL;          // bf16, head_dim 128, group <= 8 only
+  if (!c->decode_maps || c->cfg.head_dim != 128) return BALANCEKV_E_INVAL;   // bf16, head_dim 128, group <= 8 only
   if (timed_out(c)) return BALANCEKV_E_TIMEOUT;
   c->decode_chain = false;
   // distinct slots in order of first appearance, with the sides they enter

@@ -1,4 +1,4 @@
-// Split-K decode attention over the weighted compressed cache, bf16 / d = 128, on tensor cores.
+// Split-K decode attention over the weighted compressed cache, bf16, d = 128 or 64, on tensor cores.
 //
 //   out = sum_i w_i e^{<k_i,q>/sqrt d} v_i / sum_i w_i e^{<k_i,q>/sqrt d},   w_i = 2^level(i)
 //
@@ -9,10 +9,11 @@
 // HBM speed, this one needs ~3.
 //
 // Grid (streams of the layer, splits [+ g - 1], slots), CTAs of four warps in two groups, two per SM.  A CTA
-// walks its share of the stream's 64-token tiles through a 3-stage ring filled by TMA (tensor maps over the K
-// and V arenas, boxes of 64 dims x 64 rows, 128-byte swizzle, so ldmatrix reads are bank-conflict free); the
+// walks its share of the stream's 64-token tiles through a 96 KB ring (3 stages at d = 128, 6 at d = 64) filled by
+// TMA (tensor maps over the K and V arenas, boxes of 64 dims x 64 rows, 128-byte swizzle, so ldmatrix reads are
+// bank-conflict free); the
 // groups take tiles in turn.  Warp w of a group owns tokens 32w..32w+31 of a tile -- the tokens are the M
-// dimension of both products -- and keeps a private online softmax (running max, sum, 128 x 8 accumulator)
+// dimension of both products -- and keeps a private online softmax (running max, sum, d x 8 accumulator)
 // in registers; warps merge through shared memory, splits through a global scratch whose words are their own
 // arrival flags: with more than one split, head 0 of a stream is combined by the CTA of its last split and
 // head h > 0 by a CTA of its own (grid y = splits + h - 1), which polls the partial rows of its head.
@@ -21,6 +22,8 @@
 // CTAs score it in fp32 and add it as one more partial (weight 1), and the combiner of head 0 writes its
 // row, its position and the stream's new level-0 length once its polls have shown that every CTA of the
 // stream is past its tiles, i.e. has finished reading the old segment table.
+// d = 64 takes this kernel too: on CUDA cores a launch over 8 streams x 2900 rows, 8 query heads each, took 24.6 us
+// (issue bound, and the last CTA of a stream summed the splits one load after the other), here 9.0 us.
 // Rows of a tile beyond a segment's end are masked in the scores; their V rows are whatever the
 // arena holds there (zero-initialised at creation or finite older rows) times an exact zero.
 #include <cuda.h>
@@ -32,24 +35,32 @@ namespace bkv {
 namespace {
 
 // Shape of a CTA: kGroups warp groups that take the CTA's tiles in turn, each warp of a group owning
-// kTB blocks of 16 tokens of a 64-token tile; kStages tiles in flight; kCtasPerSm resident CTAs.
+// kTB blocks of 16 tokens of a 64-token tile; kCtasPerSm resident CTAs.
 constexpr int kGroups = 2;
 constexpr int kTB = 2;
-constexpr int kStages = 3;
 constexpr int kCtasPerSm = 2;
 constexpr int kWarpTokens = 16 * kTB;
 constexpr int kGroupWarps = 64 / kWarpTokens;
 constexpr int kGroupThreads = 32 * kGroupWarps;
 constexpr int kWarps = kGroups * kGroupWarps;
 constexpr int kThreads = 32 * kWarps;
-constexpr int kBars = kGroups * kStages;      // tile i: stage i % kStages, barrier i % kBars (a multiple of kStages and kGroups)
 constexpr int kTN = 64;                      // tokens per tile
-constexpr int kD = 128;
 constexpr uint32_t kHalf = kTN * 128;        // bytes of one [64 tokens][64 dims] bf16 box
-constexpr uint32_t kTensorBytes = 2 * kHalf; // K (or V) tile: two boxes
-constexpr uint32_t kStageBytes = 2 * kTensorBytes;
 constexpr long long kWaitCycles = 100000000LL;   // about 50 ms: a bulk copy that has not landed by then never will
-constexpr int PS = kD + 4;                   // row of the in-CTA merge buffer: acc[D], max, sum, 2 pad (bank-conflict free)
+
+// What depends on the head dimension.
+template <int D>
+struct Dim {
+  static_assert(D == 128 || D == 64, "boxes of 64 dims; the output columns belong to whole warps");
+  static constexpr uint32_t kTensorBytes = (D / 64) * kHalf;   // K (or V) tile: one box per 64 dims
+  static constexpr uint32_t kStageBytes = 2 * kTensorBytes;
+  static constexpr int kStages = 98304 / kStageBytes;          // tiles in flight: 3 or 6, so that two CTAs share an SM
+  static constexpr int kBars = 6;                              // tile i: stage i % kStages, barrier i % kBars (a multiple of kStages and kGroups)
+  static_assert(kBars % kStages == 0 && kBars % kGroups == 0, "a barrier serves tiles of one stage and one group");
+  static constexpr int PS = D + 4;                             // row of the in-CTA merge buffer: acc[D], max, sum, 2 pad (bank-conflict free)
+  static constexpr int kColWarps = D / 32;                     // warps that combine: 32 output columns each
+  static constexpr size_t kSmemBytes = 1024 + (size_t)kStages * kStageBytes + kBars * sizeof(uint64_t);
+};
 
 struct DecodeMaps {
   CUtensorMap k, v;
@@ -115,7 +126,7 @@ __device__ inline float fast_exp2(float x) {     // -inf -> 0
 constexpr uint32_t kEmptyWord = 0xffffffffu;
 constexpr int kMaxSplits = 64;
 static_assert(2 * kWarps <= 8, "the scratch holds 8 floats of (max, sum) copies per partial row (decode_scratch_bytes)");
-static_assert(kThreads == kD, "the combine maps a warp to 32 output columns");
+static_assert(Dim<128>::kColWarps <= kWarps, "the combine maps a warp to 32 output columns");
 __device__ inline bool is_empty(float x) { return __float_as_uint(x) == kEmptyWord; }
 // Plain loads as volatile asm statements: they keep their place among the polling loads, i.e. they are issued
 // before the polls and not where their values are first used.
@@ -149,9 +160,9 @@ __device__ inline uint32_t pack_bf16(float lo, float hi) {
   const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&v);
 }
-// Byte offset of (token row, 16-byte chunk of dims) inside a K or V tile: two 64-dim boxes of
+// Byte offset of (token row, 16-byte chunk of dims) inside a K or V tile: 64-dim boxes of
 // 64 rows x 128 bytes, chunk index XORed with (row % 8) by the 128-byte swizzle.
-__device__ inline uint32_t tile_off(int token, int chunk16) {   // chunk16 in [0, 16)
+__device__ inline uint32_t tile_off(int token, int chunk16) {   // chunk16 in [0, d / 8)
   return (uint32_t)(chunk16 >> 3) * kHalf + (uint32_t)token * 128u + (uint32_t)(((chunk16 & 7) ^ (token & 7)) << 4);
 }
 
@@ -228,10 +239,15 @@ __device__ inline bool group_bar_or(int group, bool pred) {
   return r != 0;
 }
 
+template <int D>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ out,
                   float* __restrict__ part_base, int* __restrict__ status,
                   const StepAppend ap, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV) {
+  constexpr int kStages = Dim<D>::kStages, kBars = Dim<D>::kBars, PS = Dim<D>::PS, kColWarps = Dim<D>::kColWarps;
+  constexpr uint32_t kTensorBytes = Dim<D>::kTensorBytes, kStageBytes = Dim<D>::kStageBytes;
+  constexpr int kRowPieces = D / 8;                // 16-byte pieces of a row
+  constexpr int kLines = D / 64;                   // 128-byte lines of a row
   float* part = part_base;
   float* raw_acc = ap.raw_acc;
   float* raw_ml = ap.raw_ml;
@@ -241,7 +257,7 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
     layer = ap.slot_layer[z];
     keys_only = (int)((ap.keys_mask >> z) & 1u);
     part += (size_t)z * ap.z_stride;
-    raw_acc += (size_t)z * G.B * G.H * G.g * kD;
+    raw_acc += (size_t)z * G.B * G.H * G.g * D;
     raw_ml += (size_t)z * G.B * G.H * G.g * 2;
   }
   extern __shared__ unsigned char smem_raw[];
@@ -282,13 +298,13 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
   // (the producer's write updates that line; nothing is taken into L1 here).
   if (ap.in_flag) {
     // operands still in flight: nothing to ask for yet
-  } else if (tid < 2 * g) {
-    const char* qrow = reinterpret_cast<const char*>(q + ((size_t)seq * (G.H * g) + (size_t)head * g + (tid >> 1)) * kD);
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(qrow + 128 * (tid & 1)));
-  } else if (ap.k_new && tid < 2 * g + 4) {
-    const int k = tid - 2 * g;
-    const char* row = reinterpret_cast<const char*>((k & 2 ? ap.v_new : ap.k_new) + (size_t)sl * kD);
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(row + 128 * (k & 1)));
+  } else if (tid < kLines * g) {                      // the stream's g query rows are contiguous
+    const char* qrow = reinterpret_cast<const char*>(q + ((size_t)seq * (G.H * g) + (size_t)head * g) * D);
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(qrow + 128 * tid));
+  } else if (ap.k_new && tid < kLines * (g + 2)) {
+    const int k = tid - kLines * g;
+    const char* row = reinterpret_cast<const char*>((k >= kLines ? ap.v_new : ap.k_new) + (size_t)sl * D);
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(row + 128 * (k % kLines)));
   }
   const bool early = ap.early && ap.n_seg;
   if (!early) {
@@ -312,11 +328,11 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
     unsigned char* st = tiles + (size_t)(i % kStages) * kStageBytes;
     uint64_t* bar = &full[i % kBars];
     mbar_expect_tx(bar, keys_only ? kTensorBytes : kStageBytes);
-    tma_load_2d(st, &tmK, 0, (int)tr.row, bar);
-    tma_load_2d(st + kHalf, &tmK, 64, (int)tr.row, bar);
+#pragma unroll
+    for (int b = 0; b < D / 64; ++b) tma_load_2d(st + b * kHalf, &tmK, 64 * b, (int)tr.row, bar);
     if (!keys_only) {
-      tma_load_2d(st + kTensorBytes, &tmV, 0, (int)tr.row, bar);
-      tma_load_2d(st + kTensorBytes + kHalf, &tmV, 64, (int)tr.row, bar);
+#pragma unroll
+      for (int b = 0; b < D / 64; ++b) tma_load_2d(st + kTensorBytes + b * kHalf, &tmV, 64 * b, (int)tr.row, bar);
     }
   };
   int issued = 0;
@@ -349,11 +365,13 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
   // joins as one more partial (level 0, weight 1, <q, k_new> in fp32), the ratio or the raw parts are
   // written, and with h == 0 the token's row goes into the cache.
   struct NewTok {
-    uint2 kn;                  // 4 dims of k_new per lane
+    uint2 kn;                  // 4 dims of k_new per lane (lanes < d / 4)
     uint2 qv[kMaxGroup];       // 4 dims of q per lane and head (one head: slot 0)
     uint2 vn;                  // lanes 0-7: the columns 32 warp + 4 lane .. + 3 of v_new
-    uint4 row_new;             // last warp: lanes 0-15 a piece of the row of K, lanes 16-31 of V
+    uint4 row_new;             // last column warp: the first d / 8 lanes a piece of the row of K, the next d / 8 of V
   };
+  const bool col_warp = warp < kColWarps;          // owns the output columns 32 warp .. 32 warp + 31
+  const bool has_dims = 4 * lane < D;
   // h < 0: the queries of all heads
   auto load_new = [&](int h) -> NewTok {
     NewTok nt;
@@ -363,18 +381,19 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
 #pragma unroll
     for (int k = 0; k < kMaxGroup; ++k) nt.qv[k] = make_uint2(0u, 0u);
     if (ap.k_new) {
-      nt.kn = ld_early_v2(ap.k_new + (size_t)sl * kD + 4 * lane);
-      if (lane < 8) nt.vn = ld_early_v2(ap.v_new + (size_t)sl * kD + 32 * warp + 4 * lane);
-      const __nv_bfloat16* qs = q + ((size_t)seq * (G.H * g) + (size_t)head * g) * kD + 4 * lane;
-      if (h >= 0) {
-        nt.qv[0] = ld_early_v2(qs + (size_t)h * kD);
+      if (has_dims) nt.kn = ld_early_v2(ap.k_new + (size_t)sl * D + 4 * lane);
+      if (col_warp && lane < 8) nt.vn = ld_early_v2(ap.v_new + (size_t)sl * D + 32 * warp + 4 * lane);
+      const __nv_bfloat16* qs = q + ((size_t)seq * (G.H * g) + (size_t)head * g) * D + 4 * lane;
+      if (!has_dims) {
+      } else if (h >= 0) {
+        nt.qv[0] = ld_early_v2(qs + (size_t)h * D);
       } else {
 #pragma unroll
         for (int k = 0; k < kMaxGroup; ++k)
-          if (k < g) nt.qv[k] = ld_early_v2(qs + (size_t)k * kD);
+          if (k < g) nt.qv[k] = ld_early_v2(qs + (size_t)k * D);
       }
-      if (h <= 0 && warp == kWarps - 1)
-        nt.row_new = ld_early_v4(reinterpret_cast<const uint4*>((lane < 16 ? ap.k_new : ap.v_new) + (size_t)sl * kD) + (lane & 15));
+      if (h <= 0 && warp == kColWarps - 1 && lane < 2 * kRowPieces)
+        nt.row_new = ld_early_v4(reinterpret_cast<const uint4*>((lane < kRowPieces ? ap.k_new : ap.v_new) + (size_t)sl * D) + lane % kRowPieces);
     }
     return nt;
   };
@@ -401,10 +420,10 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
       M = Mn;
     }
     const size_t qh = (size_t)seq * (G.H * g) + (size_t)head * g + h;
-    if (lane < 8) {
+    if (col_warp && lane < 8) {
       const int c = 32 * warp + 4 * lane;
       if (raw_acc) {
-        *reinterpret_cast<float4*>(raw_acc + qh * kD + c) = a;
+        *reinterpret_cast<float4*>(raw_acc + qh * D + c) = a;
         if (c == 0) { raw_ml[2 * qh] = M; raw_ml[2 * qh + 1] = L; }
       } else {
         const float inv = L > 0.f ? 1.0f / L : 0.f;
@@ -412,14 +431,14 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
         uint2 w;
         w.x = *reinterpret_cast<uint32_t*>(&o01);
         w.y = *reinterpret_cast<uint32_t*>(&o23);
-        *reinterpret_cast<uint2*>(out + qh * kD + c) = w;
+        *reinterpret_cast<uint2*>(out + qh * D + c) = w;
       }
     }
-    if (ap.k_new && h == 0 && warp == kWarps - 1) {
-      // append: one 256-byte row of K and of V, the position, the new length of C^0
+    if (ap.k_new && h == 0 && warp == kColWarps - 1) {
+      // append: one row of K and of V, the position, the new length of C^0
       const size_t dst_row = (size_t)stream_base + G.region_off[0] + ap.rel_row;
-      __nv_bfloat16* dstp = static_cast<__nv_bfloat16*>(lane < 16 ? A.K : A.V) + dst_row * kD;
-      reinterpret_cast<uint4*>(dstp)[lane & 15] = nt.row_new;
+      __nv_bfloat16* dstp = static_cast<__nv_bfloat16*>(lane < kRowPieces ? A.K : A.V) + dst_row * D;
+      if (lane < 2 * kRowPieces) reinterpret_cast<uint4*>(dstp)[lane % kRowPieces] = nt.row_new;
       float s2 = 0.f;                                         // ||k||^2 / ||v||^2 travel with the row
       const __nv_bfloat162* h2 = reinterpret_cast<const __nv_bfloat162*>(&nt.row_new);
 #pragma unroll
@@ -429,8 +448,8 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
         s2 = fmaf(fv.y, fv.y, s2);
       }
 #pragma unroll
-      for (int o = 8; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-      const float v2 = __shfl_sync(0xffffffffu, s2, 16);
+      for (int o = kRowPieces / 2; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+      const float v2 = __shfl_sync(0xffffffffu, s2, kRowPieces);
       if (lane == 0 && A.nrm) A.nrm[dst_row] = make_float2(s2, v2);
       if (lane == 1) {
         A.idx[dst_row] = ap.idx0;
@@ -443,10 +462,11 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
   // takes the rows rg, rg + 4, ... (vector loads and stores: a quarter of the memory instructions that a
   // lane per column would need), and the four row groups meet by two shuffle steps.
   auto combine_head = [&](int h) {
+    if (!col_warp) return;
     const int rg = lane >> 3;
-    const float* rows = part + ((size_t)sl * splits * g + h) * kD + 32 * warp + 4 * (lane & 7);        // row of split sp: + sp rstep
-    const float* mls = part + (size_t)gridDim.x * splits * g * kD + (((size_t)sl * g + h) * kWarps + warp) * splits * 2;   // this warp's copies of the head's pairs, split by split: one line or two for a polling warp
-    const size_t rstep = (size_t)g * kD, mstep = 2;
+    const float* rows = part + ((size_t)sl * splits * g + h) * D + 32 * warp + 4 * (lane & 7);        // row of split sp: + sp rstep
+    const float* mls = part + (size_t)gridDim.x * splits * g * D + (((size_t)sl * g + h) * kColWarps + warp) * splits * 2;   // this warp's copies of the head's pairs, split by split: one line or two for a polling warp
+    const size_t rstep = (size_t)g * D, mstep = 2;
     const NewTok nt = load_new(h);              // in flight during the polls
     const float* mlp[2] = {mls + (size_t)lane * mstep, mls + (size_t)(lane + 32) * mstep};
     float2 ml[2];
@@ -530,12 +550,12 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
   // in the second product the columns 0-3 carry the high parts of the probabilities and the columns 4-7 their
   // low parts, so that one MMA does what takes two with more heads; the halves are added before the merge.
   const bool packed = g <= 4;
-  uint32_t qb[8][2];
+  uint32_t qb[D / 16][2];
   {
     const int hr = packed ? hq & 3 : hq;
-    const __nv_bfloat16* qp = q + ((size_t)seq * (G.H * g) + (size_t)head * g + hr) * kD;
+    const __nv_bfloat16* qp = q + ((size_t)seq * (G.H * g) + (size_t)head * g + hr) * D;
 #pragma unroll
-    for (int ks = 0; ks < 8; ++ks) {
+    for (int ks = 0; ks < D / 16; ++ks) {
       uint32_t lo = 0, hi = 0;
       if (hr < g) {
         lo = *reinterpret_cast<const uint32_t*>(qp + ks * 16 + 2 * tq);
@@ -546,9 +566,10 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
   }
 
   // O^T of this warp's tokens: o[mb][j] = dim 16 mb + hq + 8 (j >> 1), query head 2 tq + (j & 1)
-  float o[8][4];
+  constexpr int kMB = D / 16;
+  float o[kMB][4];
 #pragma unroll
-  for (int n = 0; n < 8; ++n) { o[n][0] = o[n][1] = o[n][2] = o[n][3] = 0.f; }
+  for (int n = 0; n < kMB; ++n) { o[n][0] = o[n][1] = o[n][2] = o[n][3] = 0.f; }
   float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};   // heads 2 tq, 2 tq + 1; l over this thread's tokens
 
   // ldmatrix row addresses of this lane (see the fragment layouts of mma.m16n8k16), for the first of
@@ -584,7 +605,7 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
 #pragma unroll
         for (int c = 0; c < 4; ++c) { sa[tb][c][0] = sa[tb][c][1] = sa[tb][c][2] = sa[tb][c][3] = 0.f; }
 #pragma unroll
-      for (int kh = 0; kh < 2; ++kh) {
+      for (int kh = 0; kh < D / 64; ++kh) {
         uint32_t ka[4][kTB][4];
 #pragma unroll
         for (int k4 = 0; k4 < 4; ++k4)
@@ -596,12 +617,12 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
           for (int tb = 0; tb < kTB; ++tb) mma_bf16(sa[tb][k4], ka[k4][tb], qb[kh * 4 + k4][0], qb[kh * 4 + k4][1]);
       }
       // the value operands do not depend on the probabilities: their loads are in flight during the softmax
-      uint32_t va[kTB][8][4];
+      uint32_t va[kTB][kMB][4];
       if (!keys_only) {
 #pragma unroll
         for (int tb = 0; tb < kTB; ++tb)
 #pragma unroll
-          for (int mb = 0; mb < 8; ++mb) ldsm_x4_trans(Vt + tile_off(v_tok + 16 * tb, mb * 2 + v_chunk), va[tb][mb]);
+          for (int mb = 0; mb < kMB; ++mb) ldsm_x4_trans(Vt + tile_off(v_tok + 16 * tb, mb * 2 + v_chunk), va[tb][mb]);
       }
       // this thread: per block tb the tokens tok0 (x[tb][0], x[tb][1]) and tok0 + 8 (x[tb][2], x[tb][3]),
       // heads 2 tq (even index) and 2 tq + 1
@@ -628,7 +649,7 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
         const float a0 = fast_exp2(m_run[0] - mn0), a1 = fast_exp2(m_run[1] - mn1);   // m_run = -inf -> 0
         l_run[0] *= a0; l_run[1] *= a1;
 #pragma unroll
-        for (int n = 0; n < 8; ++n) { o[n][0] *= a0; o[n][1] *= a1; o[n][2] *= a0; o[n][3] *= a1; }
+        for (int n = 0; n < kMB; ++n) { o[n][0] *= a0; o[n][1] *= a1; o[n][2] *= a0; o[n][3] *= a1; }
         m_run[0] = mn0; m_run[1] = mn1;
       }
       // The probabilities enter the second MMA as bf16: split them into a high and a low part
@@ -652,21 +673,21 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
           bl[tb][0] = movm_trans(pl0); bl[tb][1] = movm_trans(pl1);
         }
       }
-      // ---- O^T[128 x 8] += V^T[128 x 16 kTB] P^T[16 kTB x 8]: the high parts of a block, then its low
+      // ---- O^T[d x 8] += V^T[d x 16 kTB] P^T[16 kTB x 8]: the high parts of a block, then its low
       // parts, so that no MMA follows its predecessor on the same accumulator
       if (!keys_only) {
         if (packed) {
 #pragma unroll
           for (int tb = 0; tb < kTB; ++tb)
 #pragma unroll
-            for (int mb = 0; mb < 8; ++mb) mma_bf16(o[mb], va[tb][mb], bh[tb][0], bh[tb][1]);
+            for (int mb = 0; mb < kMB; ++mb) mma_bf16(o[mb], va[tb][mb], bh[tb][0], bh[tb][1]);
         } else {
 #pragma unroll
           for (int tb = 0; tb < kTB; ++tb) {
 #pragma unroll
-            for (int mb = 0; mb < 8; ++mb) mma_bf16(o[mb], va[tb][mb], bh[tb][0], bh[tb][1]);
+            for (int mb = 0; mb < kMB; ++mb) mma_bf16(o[mb], va[tb][mb], bh[tb][0], bh[tb][1]);
 #pragma unroll
-            for (int mb = 0; mb < 8; ++mb) mma_bf16(o[mb], va[tb][mb], bl[tb][0], bl[tb][1]);
+            for (int mb = 0; mb < kMB; ++mb) mma_bf16(o[mb], va[tb][mb], bl[tb][0], bl[tb][1]);
           }
         }
       }
@@ -686,7 +707,7 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
   }
   if (packed) {                                // high + low halves: the columns 2 tq + e and 2 tq + e + 4
 #pragma unroll
-    for (int n = 0; n < 8; ++n)
+    for (int n = 0; n < kMB; ++n)
 #pragma unroll
       for (int j = 0; j < 4; ++j) o[n][j] += __shfl_xor_sync(0xffffffffu, o[n][j], 2);
   }
@@ -697,8 +718,8 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
     if (h < g) {
       float* rowp = mrg + ((size_t)warp * g + h) * PS;
 #pragma unroll
-      for (int n = 0; n < 8; ++n) { rowp[16 * n + hq] = o[n][e]; rowp[16 * n + 8 + hq] = o[n][2 + e]; }
-      if (hq == 0) { rowp[kD] = m_run[e]; rowp[kD + 1] = l_run[e]; }
+      for (int n = 0; n < kMB; ++n) { rowp[16 * n + hq] = o[n][e]; rowp[16 * n + 8 + hq] = o[n][2 + e]; }
+      if (hq == 0) { rowp[D] = m_run[e]; rowp[D + 1] = l_run[e]; }
     }
   }
   __syncthreads();
@@ -707,12 +728,12 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
   constexpr uint32_t kMrg2Off = kWarps * kMaxGroup * PS * 4;        // behind mrg: [ways][g][PS] first-level merges
   constexpr uint32_t kSingleOff = 4352 + kWarps * kMaxGroup * 32 * 16 + 4096;   // behind the merge buffers and the combine's tables
   const bool single = splits == 1;
-  // Partial results: per (stream, split, head) a row of kD column sums, and behind all rows the
-  // (max, sum) pairs.  Rows of 512 bytes keep the staging copy 128-byte aligned.
+  // Partial results: per (stream, split, head) a row of d column sums, and behind all rows the
+  // (max, sum) pairs.
   const size_t n_rows_all = (size_t)gridDim.x * splits * g;
-  float* my_acc = single ? reinterpret_cast<float*>(tiles + kSingleOff) : part + ((size_t)sl * splits + split) * g * kD;
-  float* my_ml = single ? reinterpret_cast<float*>(tiles + kSingleOff) + kMaxGroup * kD
-                        : part + n_rows_all * kD + (size_t)sl * g * kWarps * splits * 2;       // pair of (head, copy, split): + ((h kWarps + copy) splits + split) 2
+  float* my_acc = single ? reinterpret_cast<float*>(tiles + kSingleOff) : part + ((size_t)sl * splits + split) * g * D;
+  float* my_ml = single ? reinterpret_cast<float*>(tiles + kSingleOff) + kMaxGroup * D
+                        : part + n_rows_all * D + (size_t)sl * g * kColWarps * splits * 2;    // pair of (head, copy, split): + ((h kColWarps + copy) splits + split) 2
   // Work items of the merge and combine phases: (head mh, way mw), item r = mw g + mh, ways =
   // max(1, warps / g); a warp takes items r = warp, warp + kWarps, ... (lane = 4 output columns).
   // The ways of a head share its rows: way mw takes the rows mw, mw + ways, ...
@@ -726,7 +747,7 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
 #pragma unroll
       for (int k = 0; k < kWarps; ++k) {
         const int w = mw + k * ways;
-        mv[k] = w < kWarps ? mrg[((size_t)w * g + mh) * PS + kD] : -INFINITY;
+        mv[k] = w < kWarps ? mrg[((size_t)w * g + mh) * PS + D] : -INFINITY;
         M = fmaxf(M, mv[k]);
       }
       float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -737,14 +758,14 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
         if (w < kWarps && mv[k] != -INFINITY) {
           const float* rowp = mrg + ((size_t)w * g + mh) * PS;
           const float f = fast_exp2(mv[k] - M);
-          const float4 v = *reinterpret_cast<const float4*>(rowp + 4 * lane);
+          const float4 v = has_dims ? *reinterpret_cast<const float4*>(rowp + 4 * lane) : make_float4(0.f, 0.f, 0.f, 0.f);
           acc.x = fmaf(v.x, f, acc.x); acc.y = fmaf(v.y, f, acc.y); acc.z = fmaf(v.z, f, acc.z); acc.w = fmaf(v.w, f, acc.w);
-          L = fmaf(rowp[kD + 1], f, L);
+          L = fmaf(rowp[D + 1], f, L);
         }
       }
       float* dst = mrg2 + ((size_t)mw * g + mh) * PS;
-      *reinterpret_cast<float4*>(dst + 4 * lane) = acc;
-      if (lane == 0) { dst[kD] = M; dst[kD + 1] = L; }
+      if (has_dims) *reinterpret_cast<float4*>(dst + 4 * lane) = acc;
+      if (lane == 0) { dst[D] = M; dst[D + 1] = L; }
     }
     __syncthreads();
     mrg = mrg2;                                 // the second level reads `ways` rows per head
@@ -753,23 +774,23 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
     const int n_src = ways > 1 ? ways : kWarps;
     for (int h = warp; h < g; h += kWarps) {
       float M = -INFINITY;
-      for (int k = 0; k < n_src; ++k) M = fmaxf(M, mrg[((size_t)k * g + h) * PS + kD]);
+      for (int k = 0; k < n_src; ++k) M = fmaxf(M, mrg[((size_t)k * g + h) * PS + D]);
       float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
       float L = 0.f;
       for (int k = 0; k < n_src; ++k) {
         const float* rowp = mrg + ((size_t)k * g + h) * PS;
-        const float mk = rowp[kD];
+        const float mk = rowp[D];
         const float f = mk == -INFINITY ? 0.f : fast_exp2(mk - M);
-        const float4 v = *reinterpret_cast<const float4*>(rowp + 4 * lane);
+        const float4 v = has_dims ? *reinterpret_cast<const float4*>(rowp + 4 * lane) : make_float4(0.f, 0.f, 0.f, 0.f);
         acc.x = fmaf(v.x, f, acc.x); acc.y = fmaf(v.y, f, acc.y); acc.z = fmaf(v.z, f, acc.z); acc.w = fmaf(v.w, f, acc.w);
-        L = fmaf(rowp[kD + 1], f, L);
+        L = fmaf(rowp[D + 1], f, L);
       }
       if (single) {
-        *reinterpret_cast<float4*>(my_acc + h * kD + 4 * lane) = acc;
+        if (has_dims) *reinterpret_cast<float4*>(my_acc + h * D + 4 * lane) = acc;
         if (lane == 0) *reinterpret_cast<float2*>(my_ml + 2 * h) = make_float2(M, L);
       } else {                                  // published: see the combine below
-        st_scratch4(my_acc + h * kD + 4 * lane, acc);
-        if (lane < kWarps) st_scratch2(my_ml + ((size_t)(h * kWarps + lane) * splits + split) * 2, make_float2(M, L));   // a copy per combining warp
+        if (has_dims) st_scratch4(my_acc + h * D + 4 * lane, acc);
+        if (lane < kColWarps) st_scratch2(my_ml + ((size_t)(h * kColWarps + lane) * splits + split) * 2, make_float2(M, L));   // a copy per combining warp
       }
     }
   }
@@ -785,12 +806,12 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
   if (single) {
     __syncthreads();                            // the rows in shared memory are complete
     const float* acc1 = reinterpret_cast<const float*>(tiles + kSingleOff);
-    const float* ml1 = acc1 + kMaxGroup * kD;
+    const float* ml1 = acc1 + kMaxGroup * D;
     NewTok nt = load_new(-1);
 #pragma unroll
     for (int h = 0; h < kMaxGroup; ++h)
       if (h < g)
-        finish(h, *reinterpret_cast<const float4*>(acc1 + h * kD + 32 * warp + 4 * (lane & 7)), ml1[2 * h], ml1[2 * h + 1], nt,
+        finish(h, *reinterpret_cast<const float4*>(acc1 + h * D + (32 * warp) % D + 4 * (lane & 7)), ml1[2 * h], ml1[2 * h + 1], nt,
                ap.k_new ? score_new(nt, h) : 0.f);
     return;
   }
@@ -801,41 +822,79 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-constexpr size_t kSmemBytes = 1024 + (size_t)kStages * kStageBytes + kBars * sizeof(uint64_t);
+// Tensor maps over K and V viewed as [total_rows, d] bf16, boxes of 64 dims x 64 rows.
+cudaError_t encode_maps(DecodeMaps* tm, void* K, void* V, int d, int64_t total_rows) {
+  if (total_rows < 1 || total_rows >= ((int64_t)1 << 31)) return cudaErrorNotSupported;
+  struct Entry {
+    EncodeTiledFn fn = nullptr;
+    cudaError_t err = cudaSuccess;
+    Entry() {
+      void* p = nullptr;
+      cudaDriverEntryPointQueryResult qres;
+      err = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &qres);
+      if (err == cudaSuccess && (!p || qres != cudaDriverEntryPointSuccess)) err = cudaErrorNotSupported;
+      if (err == cudaSuccess) fn = reinterpret_cast<EncodeTiledFn>(p);
+    }
+  };
+  static const Entry entry;                 // the driver's encoder: looked up once
+  if (entry.err != cudaSuccess) return entry.err;
+  const cuuint64_t dims[2] = {(cuuint64_t)d, (cuuint64_t)total_rows};
+  const cuuint64_t strides[1] = {(cuuint64_t)d * 2};
+  const cuuint32_t box[2] = {64, (cuuint32_t)kTN};
+  const cuuint32_t estr[2] = {1, 1};
+  void* bases[2] = {K, V};
+  CUtensorMap* maps[2] = {&tm->k, &tm->v};
+  for (int i = 0; i < 2; ++i) {
+    CUresult r = entry.fn(maps[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, bases[i], dims, strides, box, estr,
+                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
+  }
+  return cudaSuccess;
+}
+
+cudaError_t set_smem(int d) {
+  return d == 128 ? cudaFuncSetAttribute(decode_mma_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Dim<128>::kSmemBytes)
+                  : cudaFuncSetAttribute(decode_mma_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Dim<64>::kSmemBytes);
+}
+
+// CTAs per stream of a launch with `splits` splits: the combiners of the heads 1 .. g - 1 have CTAs of their own.
+unsigned grid_y(const Geom& G, int splits) { return (unsigned)(splits > 1 ? splits + G.g - 1 : 1); }
+
+// Scratch layout of all launches: the CUDA-core kernel's ticket counters (unused here), then (stream, split,
+// head) rows of d column sums, then per row d / 32 copies of its (max, sum) pair.
+float* partial_rows(const Geom& G, float* scratch) { return scratch + (((size_t)G.B * G.H + 63) / 64) * 64; }
+
+// Launches with programmatic stream serialization: back-to-back decode launches overlap a launch with the previous
+// kernel's tail (see the kernel's prologue).
+cudaError_t launch(const Geom& G, const Arena& A, int layer, const void* q, void* out, float* part, int* status,
+                   const StepAppend& ap, const DecodeMaps& tm, int n_slots, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(G.B * G.H, grid_y(G, ap.splits), n_slots);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = G.d == 128 ? Dim<128>::kSmemBytes : Dim<64>::kSmemBytes;
+  cfg.stream = st;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, G.d == 128 ? decode_mma_kernel<128> : decode_mma_kernel<64>, G, A, layer,
+                            static_cast<const __nv_bfloat16*>(q), static_cast<__nv_bfloat16*>(out), part, status, ap, tm.k, tm.v);
+}
 
 }  // namespace
 
-bool decode_mma_supported(const Geom& G) { return G.is_bf16 && G.d == kD && G.g <= 8; }
+bool decode_mma_supported(const Geom& G) { return G.is_bf16 && (G.d == 128 || G.d == 64) && G.g <= 8; }
 int decode_mma_ctas_per_sm() { return kCtasPerSm; }
+int decode_mma_tile_tokens() { return kTN; }
 
-// CTAs per stream of a launch with `splits` splits: the combiners of the heads 1 .. g - 1 have CTAs of their own.
-int decode_mma_ctas_per_stream(int g, int splits) { return splits > 1 ? splits + g - 1 : 1; }
-static unsigned grid_y(const Geom& G, int splits) { return (unsigned)decode_mma_ctas_per_stream(G.g, splits); }
-
-// Tensor maps over the K and V arenas viewed as [total_rows, 128] bf16, boxes of 64 dims x 64 rows.
 cudaError_t decode_mma_prepare(const Geom& G, const Arena& A, int64_t total_rows, void** maps_out) {
   *maps_out = nullptr;
-  if (!decode_mma_supported(G) || total_rows >= ((int64_t)1 << 31)) return cudaErrorNotSupported;
-  void* fn = nullptr;
-  cudaDriverEntryPointQueryResult qres;
-  cudaError_t e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres);
-  if (e != cudaSuccess) return e;
-  if (!fn || qres != cudaDriverEntryPointSuccess) return cudaErrorNotSupported;
-  EncodeTiledFn encode = reinterpret_cast<EncodeTiledFn>(fn);
+  if (!decode_mma_supported(G)) return cudaErrorNotSupported;
   DecodeMaps* tm = new DecodeMaps();
-  const cuuint64_t dims[2] = {(cuuint64_t)kD, (cuuint64_t)total_rows};
-  const cuuint64_t strides[1] = {(cuuint64_t)kD * 2};
-  const cuuint32_t box[2] = {64, (cuuint32_t)kTN};
-  const cuuint32_t estr[2] = {1, 1};
-  void* bases[2] = {A.K, A.V};
-  CUtensorMap* maps[2] = {&tm->k, &tm->v};
-  for (int i = 0; i < 2; ++i) {
-    CUresult r = encode(maps[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, bases[i], dims, strides, box, estr,
-                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) { delete tm; return cudaErrorInvalidValue; }
-  }
-  e = cudaFuncSetAttribute(decode_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+  cudaError_t e = encode_maps(tm, A.K, A.V, G.d, total_rows);
+  if (e == cudaSuccess) e = set_smem(G.d);
   if (e != cudaSuccess) { delete tm; return e; }
   *maps_out = tm;
   return cudaSuccess;
@@ -843,44 +902,18 @@ cudaError_t decode_mma_prepare(const Geom& G, const Arena& A, int64_t total_rows
 
 void decode_mma_release(void* maps) { delete static_cast<DecodeMaps*>(maps); }
 
-cudaError_t launch_decode_step_mma(const Geom& G, const Arena& A, int layer, const void* q, void* out, float* scratch,
-                                   int splits, int* status, const void* maps, const void* k_new, const void* v_new,
-                                   int rel_row, int idx0, int new_len, const Seg* seg_hint, int early, const int* in_flag,
-                                   int in_expect, cudaStream_t st);
-
-// Scratch layout of all launches: the CUDA-core kernel's ticket counters (unused here), then (stream, split,
-// head) rows of kD column sums, then per row kWarps copies of its (max, sum) pair.
-// Un-normalised parts (see StepAppend::raw_acc) of the layer's streams, for decode merged over slots.
-cudaError_t launch_decode_parts_mma(const Geom& G, const Arena& A, int layer, const void* q, float* raw_acc, float* raw_ml,
-                                    float* scratch, int splits, int* status, const void* maps, int keys_only,
-                                    cudaStream_t st) {
-  if (!maps || !raw_acc || !raw_ml) return cudaErrorInvalidValue;
-  const DecodeMaps* tm = static_cast<const DecodeMaps*>(maps);
-  const int n_sl = G.B * G.H;
-  float* part = scratch + ((n_sl + 63) / 64) * 64;
-  dim3 grid(n_sl, grid_y(G, splits));
-  const StepAppend ap{nullptr, nullptr, 0, 0, 0, raw_acc, raw_ml, keys_only, 0, {}, 0, {}, 0u, 0u, 0, nullptr, 0, splits};
-  decode_mma_kernel<<<grid, kThreads, kSmemBytes, st>>>(G, A, layer, static_cast<const __nv_bfloat16*>(q), nullptr, part,
-                                                        status, ap, tm->k, tm->v);
-  return cudaGetLastError();
-}
-
-// The same for n_slots layer slots in one launch (grid z = slot): raw_acc / raw_ml hold one block per
-// slot, scratch one block of z_stride_words 4-byte words per slot (laid out as for a single slot).
+// Un-normalised parts (see StepAppend::raw_acc) of n_slots layer slots in one launch (grid z = slot), for decode
+// merged over slots: raw_acc / raw_ml hold one block per slot, scratch one block of z_stride_words 4-byte words per
+// slot (laid out as for a single slot).
 cudaError_t launch_decode_parts_mma_slots(const Geom& G, const Arena& A, const int* slot_layers, int n_slots,
                                           unsigned keys_mask, const void* q, float* raw_acc, float* raw_ml, float* scratch,
                                           size_t z_stride_words, int splits, int* status, const void* maps,
                                           cudaStream_t st) {
   if (!maps || !raw_acc || !raw_ml || n_slots < 1 || n_slots > 8 || z_stride_words > 0xffffffffull) return cudaErrorInvalidValue;
-  const DecodeMaps* tm = static_cast<const DecodeMaps*>(maps);
-  const int n_sl = G.B * G.H;
-  float* part = scratch + ((n_sl + 63) / 64) * 64;
-  dim3 grid(n_sl, grid_y(G, splits), n_slots);
   StepAppend ap{nullptr, nullptr, 0, 0, 0, raw_acc, raw_ml, 0, 0, {}, n_slots, {}, keys_mask, (unsigned)z_stride_words, 0, nullptr, 0, splits};
   for (int i = 0; i < n_slots; ++i) ap.slot_layer[i] = slot_layers[i];
-  decode_mma_kernel<<<grid, kThreads, kSmemBytes, st>>>(G, A, slot_layers[0], static_cast<const __nv_bfloat16*>(q), nullptr,
-                                                        part, status, ap, tm->k, tm->v);
-  return cudaGetLastError();
+  return launch(G, A, slot_layers[0], q, nullptr, partial_rows(G, scratch), status, ap, *static_cast<const DecodeMaps*>(maps),
+                n_slots, st);
 }
 
 // Ratio of merged parts: the value sums of the numerator slots over the weight sums of the
@@ -924,10 +957,6 @@ cudaError_t launch_decode_step_mma(const Geom& G, const Arena& A, int layer, con
                                    int rel_row, int idx0, int new_len, const Seg* seg_hint, int early, const int* in_flag,
                                    int in_expect, cudaStream_t st) {
   if (!maps) return cudaErrorInvalidValue;
-  const DecodeMaps* tm = static_cast<const DecodeMaps*>(maps);
-  const int n_sl = G.B * G.H;
-  float* part = scratch + ((n_sl + 63) / 64) * 64;
-  dim3 grid(n_sl, grid_y(G, splits));
   StepAppend ap{static_cast<const __nv_bfloat16*>(k_new), static_cast<const __nv_bfloat16*>(v_new), rel_row, idx0,
                 new_len, nullptr, nullptr, 0, 0, {}, 0, {}, 0u, 0u, 0, nullptr, 0, splits};
   if (seg_hint) {
@@ -937,20 +966,7 @@ cudaError_t launch_decode_step_mma(const Geom& G, const Arena& A, int layer, con
   }
   ap.in_flag = in_flag;
   ap.in_expect = in_expect;
-  // programmatic stream serialization: back-to-back decode steps overlap a launch with the
-  // previous kernel's tail (see the kernel's prologue)
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = kSmemBytes;
-  cfg.stream = st;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, decode_mma_kernel, G, A, layer, static_cast<const __nv_bfloat16*>(q),
-                            static_cast<__nv_bfloat16*>(out), part, status, ap, tm->k, tm->v);
+  return launch(G, A, layer, q, out, partial_rows(G, scratch), status, ap, *static_cast<const DecodeMaps*>(maps), 1, st);
 }
 
 }  // namespace bkv

@@ -164,25 +164,24 @@ int balancekv_decode_attn_host(balancekv_ctx* ctx, int layer, const void* q_host
  * sum_i w_i e^{<k_i,q>/sqrt d} v_i / sum_i w_i e^{<k_i,q>/sqrt d}, the same arithmetic as
  * balancekv_decode_attn.
  *
- * The split-K scratch is a fixed 8 MiB array inside the library image (held by every GPU
- * that loads the library, until the process exits); the call performs no cudaMalloc, cudaFree
- * or other allocating call.  A problem whose scratch (256 bytes, a segment table of
- * n_streams * (level+1) * 8 bytes, n_streams ticket words rounded up to 64, and n_streams *
- * splits * group * (head_dim+8) * 4 bytes of partial rows, splits <= 64 chosen from the SM
- * count) exceeds the array is rejected with BALANCEKV_E_NOMEM and a message on stderr.  The
+ * The split-K scratch is a fixed array inside the library image (13.5 MiB: 8 MiB of fp32 scratch and four
+ * blocks of rows for bf16; held by every GPU that loads the library, until the process exits); the call
+ * performs no cudaMalloc, cudaFree or other allocating call.  A problem whose fp32 scratch would need more
+ * (256 bytes, a segment table of n_streams * (level+1) * 8 bytes, n_streams ticket words rounded up to 64,
+ * and n_streams * splits * group * (head_dim+8) * 4 bytes of partial rows, splits <= 64 chosen from the SM
+ * count) is rejected with BALANCEKV_E_NOMEM and a message on stderr, whatever its type.  The
  * first call on a device -- of this function or of balancekv_decode_attn_static_status,
- * whichever host thread gets there first -- looks up the array's device address
- * (cudaGetSymbolAddress) and clears its status word with a synchronous memset; make that first
- * call outside any stream capture.  All calls share the array: the part a call uses is
- * re-initialised by the call itself, but two calls that overlap on the GPU (different CUDA
- * streams) race on it -- issue them on one stream. */
+ * whichever host thread gets there first -- looks up the arrays' device addresses
+ * (cudaGetSymbolAddress) and initialises them synchronously; make that first
+ * call outside any stream capture.  Issue the calls on one stream: fp32 calls that overlap on the GPU
+ * (different CUDA streams) race on the scratch array, and so do bf16 calls of which more than four overlap. */
 int balancekv_decode_attn_static(const void* K, const void* V, int n_streams, int cache_len, int n_heavy,
                                  int level, const void* q, void* out, int group, int head_dim, int dtype,
                                  void* stream);
 /* The entry point above returns before its kernel has run, so a bounded device-side wait that
  * gives up cannot show in its return value; it sets a status word in the built-in array
  * instead, which this call copies to *status_host (0 = fine, 1 = a wait gave up since the last
- * read; the outputs of that launch are then not valid) and clears.  Allocates nothing;
+ * read; the outputs of that launch and of later ones are then not valid) and clears, the scratch with it.  Allocates nothing;
  * synchronises `stream`.  The paper has no counterpart. */
 int balancekv_decode_attn_static_status(int* status_host, void* stream);
 

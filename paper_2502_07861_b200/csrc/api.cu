@@ -25,7 +25,7 @@ void walk_tc_release(void* tmaps);
 bool decode_mma_supported(const Geom& G);
 int decode_mma_ctas_per_sm();
 int decode_mma_tile_tokens();
-cudaError_t decode_mma_prepare(const Geom& G, const Arena& A, int64_t total_rows, void** maps_out);
+cudaError_t decode_mma_prepare(const Geom& G, const Arena& A, void** maps_out);
 void decode_mma_release(void* maps);
 cudaError_t launch_decode_parts_mma_slots(const Geom& G, const Arena& A, const int* slot_layers, int n_slots,
                                           unsigned keys_mask, const void* q, float* raw_acc, float* raw_ml, float* scratch,
@@ -388,7 +388,7 @@ int balancekv_create(const balancekv_config* cfg, balancekv_ctx** out) {
   // prepared is an error, never a quiet change of kernels.
   const bool rows_ok = c->total_rows < ((int64_t)1 << 31);
   if (f.gram_path != 1 && decode_mma_supported(G) && rows_ok) {
-    if (decode_mma_prepare(G, c->A, c->total_rows, &c->decode_maps) != cudaSuccess) return fail(BALANCEKV_E_CUDA);
+    if (decode_mma_prepare(G, c->A, &c->decode_maps) != cudaSuccess) return fail(BALANCEKV_E_CUDA);
   }
   const bool tc_ok = walk_tc_supported(G) && rows_ok;
   if (f.gram_path == 2 && !tc_ok) return fail(BALANCEKV_E_INVAL);
@@ -719,7 +719,6 @@ static bool layer_seg_hint(balancekv_ctx* c, int layer, Seg* out) {
   return true;
 }
 
-// Split-K factor of a decode launch over the layer's current caches.
 // The tensor-core decode kernel adds g - 1 combining CTAs per stream to a launch with more than one split:
 // the largest split factor <= splits whose grid over n_streams streams still fits one wave.
 static int one_wave_splits(balancekv_ctx* c, int splits, int n_streams) {
@@ -728,6 +727,7 @@ static int one_wave_splits(balancekv_ctx* c, int splits, int n_streams) {
   return std::max(1, std::min(splits, room));
 }
 
+// Split-K factor of a decode launch over the layer's current caches.
 static int pick_splits(balancekv_ctx* c, int layer) {
   const balancekv_config& f = c->cfg;
   int64_t max_rows = 0;
@@ -740,11 +740,8 @@ static int pick_splits(balancekv_ctx* c, int layer) {
     }
   const int tile_tokens = c->decode_maps ? decode_mma_tile_tokens() : 16384 / (f.head_dim * c->esz);
   const int64_t tiles = (max_rows + tile_tokens - 1) / tile_tokens + f.levels;
-  int splits = (int)std::max<int64_t>(1, std::min<int64_t>(c->max_splits, (tiles + 1) / 2));
-  // the fewest splits with the same number of tiles per CTA: the tile phase is as long, the combine shorter
-  const int64_t tiles_per = std::max<int64_t>(1, (tiles + splits - 1) / splits);
-  splits = (int)std::max<int64_t>(1, (tiles + tiles_per - 1) / tiles_per);
-  if (c->decode_maps) splits = one_wave_splits(c, splits, c->cfg.n_seqs * c->cfg.n_kv_heads);
+  int splits = pick_decode_splits(tiles, c->max_splits, c->decode_slots, f.n_seqs * f.n_kv_heads,
+                                  f.n_q_heads / f.n_kv_heads, c->decode_maps != nullptr);
   if (f.decode_splits > 0) splits = std::min(f.decode_splits, c->max_splits);
   return splits;
 }

@@ -9,9 +9,10 @@
 // scratch (per-split partial sums, the ticket counters, the small segment table and a status
 // word) lives in a fixed array that is part of the library image.
 //
-// The array is a file-scope __device__ array, so every GPU that loads the library holds its
-// kStaticBytes until the process exits.  In host code the array's name is only a handle; the
+// The arrays are file-scope __device__ arrays, so every GPU that loads the library holds them
+// until the process exits.  In host code an array's name is only a handle; the
 // device address is obtained once per device with cudaGetSymbolAddress.
+#include <atomic>
 #include <cstdio>
 #include <mutex>
 
@@ -20,13 +21,29 @@
 
 namespace bkv {
 
+int decode_mma_ctas_per_sm();
+int decode_mma_tile_tokens();
+size_t decode_mma_static_bytes(const Geom& G, int splits);
+cudaError_t decode_mma_static_setup();
+cudaError_t launch_decode_static_mma(const Geom& G, void* K, void* V, const Seg* seg, const void* q, void* out, float* rows,
+                                     int splits, int* status, cudaStream_t st);
+
 namespace {
 
 constexpr size_t kStaticBytes = (size_t)8 << 20;   // 8 MiB per GPU
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticBytes];
+// Split-K rows of the tensor-core kernel (bf16), whose words are their own arrival flags: all of them hold the empty
+// pattern between launches, and every launch puts it back.  Four blocks, used in turn, so that calls on different
+// CUDA streams do not meet in one unless more than four of them overlap.  A block holds the rows of one wave of CTAs
+// (splits > 1 only where streams x (splits + group - 1) CTAs fit 2 x 148: at most 289 rows of 8 heads).
+constexpr size_t kRowBlockBytes = (size_t)11 << 17;
+constexpr int kRowBlocks = 4;
+static __device__ __align__(256) unsigned char g_static_rows[kRowBlocks * kRowBlockBytes];
 
 constexpr int kMaxDevices = 64;
 unsigned char* g_scratch_addr[kMaxDevices] = {};    // device address of the array, per device
+unsigned char* g_rows_addr[kMaxDevices] = {};
+std::atomic<unsigned> g_next_rows[kMaxDevices];
 int g_sm_count[kMaxDevices] = {};
 std::once_flag g_setup_once[kMaxDevices];           // the per-device set-up runs once, whichever host thread comes first
 cudaError_t g_setup_err[kMaxDevices] = {};
@@ -46,9 +63,9 @@ __global__ void static_setup_kernel(unsigned char* base, int n_streams, int T, i
   }
 }
 
-// Once per device, with that device current: resolve the array's device address (in host code the
-// array's name is only a handle) and clear the status word.  The array is not otherwise initialised:
-// every call sets up the part it uses.
+// Once per device, with that device current: resolve the arrays' device addresses (in host code the
+// names are only handles), clear the status word and empty the tensor-core kernel's rows.  The scratch array is not
+// otherwise initialised: every call that uses it sets up its part.
 void static_setup_device(int dev) {
   void* p = nullptr;
   cudaError_t e = cudaGetSymbolAddress(&p, g_static_scratch);
@@ -57,8 +74,14 @@ void static_setup_device(int dev) {
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess && sms < 1) e = cudaErrorInvalidValue;
   if (e == cudaSuccess) e = cudaMemset(p, 0, 256);
+  void* rows = nullptr;
+  if (e == cudaSuccess) e = cudaGetSymbolAddress(&rows, g_static_rows);
+  if (e == cudaSuccess) e = cudaMemset(rows, 0xff, sizeof(g_static_rows));
+  if (e == cudaSuccess) e = decode_mma_static_setup();
+  if (e == cudaSuccess) e = cudaDeviceSynchronize();
   g_setup_err[dev] = e;
   if (e != cudaSuccess) return;
+  g_rows_addr[dev] = static_cast<unsigned char*>(rows);
   g_sm_count[dev] = sms;
   g_scratch_addr[dev] = static_cast<unsigned char*>(p);
 }
@@ -125,6 +148,28 @@ extern "C" int balancekv_decode_attn_static(const void* K, const void* V, int n_
     return BALANCEKV_E_NOMEM;
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  if (dtype == 1) {
+    // bf16: the tensor-core kernel, one launch (the CUDA-core kernel took 34 us + 2 us of set-up launch for 16 streams x
+    // 4500 rows x 4 heads of 128 dims; this one with
+    // the host's share of the call 15.6 us)
+    Seg seg[kMaxLevels + 1] = {};
+    seg[T] = Seg{0, n_heavy};
+    seg[0] = T > 0 ? Seg{0, n_tail} : Seg{0, cache_len};
+    const int slots = decode_mma_ctas_per_sm() * g_sm_count[dev];
+    const int64_t mma_tiles = (n_heavy + decode_mma_tile_tokens() - 1) / decode_mma_tile_tokens() +
+                              (n_tail + decode_mma_tile_tokens() - 1) / decode_mma_tile_tokens();
+    int sp = pick_decode_splits(mma_tiles, 64, slots, n_streams, group, true);
+    while (decode_mma_static_bytes(G, sp) > kRowBlockBytes) --sp;
+    const unsigned block = g_next_rows[dev].fetch_add(1, std::memory_order_relaxed) % kRowBlocks;
+    const cudaError_t e = launch_decode_static_mma(G, const_cast<void*>(K), const_cast<void*>(V), seg, q, out,
+                                                   reinterpret_cast<float*>(g_rows_addr[dev] + block * kRowBlockBytes), sp,
+                                                   reinterpret_cast<int*>(base), st);
+    if (e != cudaSuccess) {
+      std::fprintf(stderr, "balancekv_decode_attn_static: launch failed: %s\n", cudaGetErrorString(e));
+      return BALANCEKV_E_CUDA;
+    }
+    return BALANCEKV_OK;
+  }
   static_setup_kernel<<<(n_streams + 255) / 256, 256, 0, st>>>(base, n_streams, T, n_heavy, n_tail, seg_off, scratch_off);
   if (cudaGetLastError() != cudaSuccess) return BALANCEKV_E_CUDA;
   Arena A{};
@@ -151,6 +196,10 @@ extern "C" int balancekv_decode_attn_static_status(int* status_host, void* strea
   if (cudaMemcpyAsync(&v, g_scratch_addr[dev], sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess) return BALANCEKV_E_CUDA;
   if (cudaMemsetAsync(g_scratch_addr[dev], 0, sizeof(int), st) != cudaSuccess) return BALANCEKV_E_CUDA;
   if (cudaStreamSynchronize(st) != cudaSuccess) return BALANCEKV_E_CUDA;
+  // a launch that gave up may have left partial rows behind
+  if (v != 0 && (cudaMemsetAsync(g_rows_addr[dev], 0xff, kRowBlocks * kRowBlockBytes, st) != cudaSuccess ||
+                 cudaStreamSynchronize(st) != cudaSuccess))
+    return BALANCEKV_E_CUDA;
   *status_host = v;
   return BALANCEKV_OK;
 }

@@ -24,8 +24,9 @@
 // stream is past its tiles, i.e. has finished reading the old segment table.
 // d = 64 takes this kernel too: on CUDA cores a launch over 8 streams x 2900 rows, 8 query heads each, took 24.6 us
 // (issue bound, and the last CTA of a stream summed the splits one load after the other), here 9.0 us.
-// Rows of a tile beyond a segment's end are masked in the scores; their V rows are whatever the
-// arena holds there (zero-initialised at creation or finite older rows) times an exact zero.
+// Rows of a tile beyond a segment's end are masked in the scores; their V rows are whatever the stream's own region
+// holds there (zero-initialised at creation or finite older rows; zeros beyond the stream's last row: the tensor maps
+// have the stream as a dimension of their own) times an exact zero.
 #include <cuda.h>
 
 #include "common.cuh"
@@ -90,10 +91,10 @@ __device__ inline bool mbar_wait(uint64_t* bar, uint32_t parity) {
   }
   return true;
 }
-__device__ inline void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
+__device__ inline void tma_load_3d(void* dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar) {
   asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-      ::"r"(smem_u32(dst)), "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(y) : "memory");
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
+      ::"r"(smem_u32(dst)), "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(z) : "memory");
 }
 __device__ inline void ldsm_x4(uint32_t addr, uint32_t (&r)[4]) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
@@ -207,17 +208,16 @@ struct StepAppend {
 };
 
 struct TileRef {
-  int64_t row;
+  int row;           // first row, counted inside the stream
   int rows, level;
 };
-__device__ inline TileRef locate_tile(int tile, const int* lvl_tiles, const Seg* seg, int T, int64_t stream_base,
-                                      const int32_t* region_off) {
+__device__ inline TileRef locate_tile(int tile, const int* lvl_tiles, const Seg* seg, int T, const int32_t* region_off) {
   TileRef r{0, 0, 0};
   for (int l = T; l >= 0; --l) {
     const int nt = lvl_tiles[l];
     if (tile < nt) {
       r.level = l;
-      r.row = stream_base + region_off[l] + seg[l].start + (int64_t)tile * kTN;
+      r.row = region_off[l] + seg[l].start + tile * kTN;
       r.rows = min(kTN, seg[l].len - tile * kTN);
       return r;
     }
@@ -324,15 +324,15 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
   const int my_tiles = split < splits ? t_end - t_begin : 0;
 
   auto issue = [&](int i) {   // one thread
-    const TileRef tr = locate_tile(t_begin + i, lvl_tiles, seg_s, G.T, stream_base, G.region_off);
+    const TileRef tr = locate_tile(t_begin + i, lvl_tiles, seg_s, G.T, G.region_off);
     unsigned char* st = tiles + (size_t)(i % kStages) * kStageBytes;
     uint64_t* bar = &full[i % kBars];
     mbar_expect_tx(bar, keys_only ? kTensorBytes : kStageBytes);
 #pragma unroll
-    for (int b = 0; b < D / 64; ++b) tma_load_2d(st + b * kHalf, &tmK, 64 * b, (int)tr.row, bar);
+    for (int b = 0; b < D / 64; ++b) tma_load_3d(st + b * kHalf, &tmK, 64 * b, tr.row, stream, bar);
     if (!keys_only) {
 #pragma unroll
-      for (int b = 0; b < D / 64; ++b) tma_load_2d(st + kTensorBytes + b * kHalf, &tmV, 64 * b, (int)tr.row, bar);
+      for (int b = 0; b < D / 64; ++b) tma_load_3d(st + kTensorBytes + b * kHalf, &tmV, 64 * b, tr.row, stream, bar);
     }
   };
   int issued = 0;
@@ -593,7 +593,7 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
     if (lane == 0) arrived = mbar_wait(&full[i % kBars], (uint32_t)((i / kBars) & 1));
     arrived = __shfl_sync(0xffffffffu, arrived, 0);
     __syncwarp();                  // the polling lane's view of the landed tile, for the whole warp
-    const TileRef tr = locate_tile(t_begin + i, lvl_tiles, seg_s, G.T, stream_base, G.region_off);
+    const TileRef tr = locate_tile(t_begin + i, lvl_tiles, seg_s, G.T, G.region_off);
     const uint32_t Kt = smem_u32(tiles + (size_t)s * kStageBytes), Vt = Kt + kTensorBytes;
     if (arrived && wq * kWarpTokens < tr.rows) {
       // ---- scores of the warp's tokens against the group's heads: S^T[16 x 8] = K Q^T per block.
@@ -822,9 +822,9 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// Tensor maps over K and V viewed as [total_rows, d] bf16, boxes of 64 dims x 64 rows.
-cudaError_t encode_maps(DecodeMaps* tm, void* K, void* V, int d, int64_t total_rows) {
-  if (total_rows < 1 || total_rows >= ((int64_t)1 << 31)) return cudaErrorNotSupported;
+// Tensor maps over K and V viewed as [n_streams, rows, d] bf16, boxes of 64 dims x 64 rows of one stream.
+cudaError_t encode_maps(DecodeMaps* tm, void* K, void* V, int d, int64_t rows, int n_streams) {
+  if (rows < 1 || rows >= ((int64_t)1 << 31)) return cudaErrorNotSupported;
   struct Entry {
     EncodeTiledFn fn = nullptr;
     cudaError_t err = cudaSuccess;
@@ -838,14 +838,14 @@ cudaError_t encode_maps(DecodeMaps* tm, void* K, void* V, int d, int64_t total_r
   };
   static const Entry entry;                 // the driver's encoder: looked up once
   if (entry.err != cudaSuccess) return entry.err;
-  const cuuint64_t dims[2] = {(cuuint64_t)d, (cuuint64_t)total_rows};
-  const cuuint64_t strides[1] = {(cuuint64_t)d * 2};
-  const cuuint32_t box[2] = {64, (cuuint32_t)kTN};
-  const cuuint32_t estr[2] = {1, 1};
+  const cuuint64_t dims[3] = {(cuuint64_t)d, (cuuint64_t)rows, (cuuint64_t)n_streams};
+  const cuuint64_t strides[2] = {(cuuint64_t)d * 2, (cuuint64_t)d * 2 * rows};
+  const cuuint32_t box[3] = {64, (cuuint32_t)kTN, 1};
+  const cuuint32_t estr[3] = {1, 1, 1};
   void* bases[2] = {K, V};
   CUtensorMap* maps[2] = {&tm->k, &tm->v};
   for (int i = 0; i < 2; ++i) {
-    CUresult r = entry.fn(maps[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, bases[i], dims, strides, box, estr,
+    CUresult r = entry.fn(maps[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, bases[i], dims, strides, box, estr,
                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
@@ -889,11 +889,11 @@ bool decode_mma_supported(const Geom& G) { return G.is_bf16 && (G.d == 128 || G.
 int decode_mma_ctas_per_sm() { return kCtasPerSm; }
 int decode_mma_tile_tokens() { return kTN; }
 
-cudaError_t decode_mma_prepare(const Geom& G, const Arena& A, int64_t total_rows, void** maps_out) {
+cudaError_t decode_mma_prepare(const Geom& G, const Arena& A, void** maps_out) {
   *maps_out = nullptr;
   if (!decode_mma_supported(G)) return cudaErrorNotSupported;
   DecodeMaps* tm = new DecodeMaps();
-  cudaError_t e = encode_maps(tm, A.K, A.V, G.d, total_rows);
+  cudaError_t e = encode_maps(tm, A.K, A.V, G.d, G.rows_per_stream, G.B * G.L * G.H);
   if (e == cudaSuccess) e = set_smem(G.d);
   if (e != cudaSuccess) { delete tm; return e; }
   *maps_out = tm;
@@ -914,6 +914,27 @@ cudaError_t launch_decode_parts_mma_slots(const Geom& G, const Arena& A, const i
   for (int i = 0; i < n_slots; ++i) ap.slot_layer[i] = slot_layers[i];
   return launch(G, A, slot_layers[0], q, nullptr, partial_rows(G, scratch), status, ap, *static_cast<const DecodeMaps*>(maps),
                 n_slots, st);
+}
+
+// balancekv_decode_attn_static: caches owned by the caller, [B streams][rows_per_stream][d] with the segments `seg`
+// (level l of every stream: rows seg[l] behind region_off[l]).  The tensor maps are encoded on the host for each call
+// (plain arithmetic, no allocation) and travel as kernel parameters.  rows: scratch of decode_mma_static_bytes().
+size_t decode_mma_static_bytes(const Geom& G, int splits) {
+  return splits > 1 ? sizeof(float) * (size_t)G.B * G.H * splits * G.g * (G.d + 8) : 0;
+}
+cudaError_t decode_mma_static_setup() {
+  const cudaError_t e = set_smem(128);
+  return e != cudaSuccess ? e : set_smem(64);
+}
+cudaError_t launch_decode_static_mma(const Geom& G, void* K, void* V, const Seg* seg, const void* q, void* out, float* rows,
+                                     int splits, int* status, cudaStream_t st) {
+  DecodeMaps tm;
+  const cudaError_t e = encode_maps(&tm, K, V, G.d, G.rows_per_stream > 0 ? G.rows_per_stream : 1, G.B * G.H);
+  if (e != cudaSuccess) return e;
+  StepAppend ap{nullptr, nullptr, 0, 0, 0, nullptr, nullptr, 0, G.T + 1, {}, 0, {}, 0u, 0u, 0, nullptr, 0, splits};
+  for (int l = 0; l <= G.T; ++l) ap.seg[l] = seg[l];
+  const Arena A{K, V, nullptr, nullptr, nullptr};
+  return launch(G, A, 0, q, out, rows, status, ap, tm, 1, st);
 }
 
 // Ratio of merged parts: the value sums of the numerator slots over the weight sums of the

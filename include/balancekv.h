@@ -164,17 +164,17 @@ int balancekv_decode_attn_host(balancekv_ctx* ctx, int layer, const void* q_host
  * sum_i w_i e^{<k_i,q>/sqrt d} v_i / sum_i w_i e^{<k_i,q>/sqrt d}, the same arithmetic as
  * balancekv_decode_attn.
  *
- * The split-K scratch is a fixed array inside the library image (13.5 MiB: 8 MiB of fp32 scratch and four
- * blocks of rows for bf16; held by every GPU that loads the library, until the process exits); the call
- * performs no cudaMalloc, cudaFree or other allocating call.  A problem whose fp32 scratch would need more
- * (256 bytes, a segment table of n_streams * (level+1) * 8 bytes, n_streams ticket words rounded up to 64,
- * and n_streams * splits * group * (head_dim+8) * 4 bytes of partial rows, splits <= 64 chosen from the SM
- * count) is rejected with BALANCEKV_E_NOMEM and a message on stderr, whatever its type.  The
+ * The split-K scratch is a fixed array inside the library image (5.5 MiB in four blocks; held by every GPU
+ * that loads the library, until the process exits); the call
+ * performs no cudaMalloc, cudaFree or other allocating call.  A problem is rejected with BALANCEKV_E_NOMEM and
+ * a message on stderr if 256 bytes, a segment table of n_streams * (level+1) * 8 bytes, n_streams words rounded
+ * up to 64, and n_streams * splits * group * (head_dim+8) * 4 bytes of partial rows (splits <= 64: two waves
+ * of CTAs, two 16 KB tiles each) exceed 8 MiB.  The
  * first call on a device -- of this function or of balancekv_decode_attn_static_status,
  * whichever host thread gets there first -- looks up the arrays' device addresses
  * (cudaGetSymbolAddress) and initialises them synchronously; make that first
- * call outside any stream capture.  Issue the calls on one stream: fp32 calls that overlap on the GPU
- * (different CUDA streams) race on the scratch array, and so do bf16 calls of which more than four overlap. */
+ * call outside any stream capture.  Calls take the blocks in turn: of calls that overlap on the GPU (different
+ * CUDA streams) more than four race on them -- issue the calls on one stream. */
 int balancekv_decode_attn_static(const void* K, const void* V, int n_streams, int cache_len, int n_heavy,
                                  int level, const void* q, void* out, int group, int head_dim, int dtype,
                                  void* stream);
@@ -319,9 +319,8 @@ int balancekv_debug_set_status(balancekv_ctx* ctx, int value);
 
 /* Testing aid: the number of 4-byte words of the split-K decode scratch that do not hold the
  * "empty" pattern (Algorithm 1's output ratio is summed over splits through that scratch; the
- * tensor-core decode kernel uses each word as its own arrival flag and must leave every word
- * empty behind every launch).  0 for contexts on the CUDA-core decode kernel.  Synchronises the
- * device.  words: host pointer. */
+ * decode kernels use each word as its own arrival flag and must leave every word empty behind
+ * every launch).  Synchronises the device.  words: host pointer. */
 int balancekv_debug_scratch_used(balancekv_ctx* ctx, int64_t* words);
 
 /* Synchronises the device.  Returns BALANCEKV_E_TIMEOUT (record filled) if a device-side wait gave up. */

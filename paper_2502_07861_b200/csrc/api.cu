@@ -13,7 +13,7 @@
 #include <cuda.h>
 
 #include "../../include/balancekv.h"
-#include "common.cuh"
+#include "decode_common.cuh"
 #include "sched.h"
 
 using namespace bkv;
@@ -23,7 +23,6 @@ bool walk_tc_supported(const Geom& G);
 cudaError_t walk_tc_prepare(const Geom& G, const Arena& A, int64_t total_rows, void** tmaps_out);
 void walk_tc_release(void* tmaps);
 bool decode_mma_supported(const Geom& G);
-int decode_mma_ctas_per_sm();
 int decode_mma_tile_tokens();
 cudaError_t decode_mma_prepare(const Geom& G, const Arena& A, void** maps_out);
 void decode_mma_release(void* maps);
@@ -34,9 +33,7 @@ cudaError_t launch_decode_parts_mma_slots(const Geom& G, const Arena& A, const i
 cudaError_t launch_merged_ratio(const float* acc, const float* ml, int n_parts, unsigned num_mask, unsigned den_mask,
                                 void* out, int n_heads, int d, cudaStream_t st);
 cudaError_t launch_decode_step_mma(const Geom& G, const Arena& A, int layer, const void* q, void* out, float* scratch,
-                                   int splits, int* status, const void* maps, const void* k_new, const void* v_new,
-                                   int rel_row, int idx0, int new_len, const Seg* seg_hint, int early, const int* in_flag,
-                                   int in_expect, cudaStream_t st);
+                                   const StepAppend& ap, int* status, const void* maps, cudaStream_t st);
 }  // namespace bkv
 
 #define BKV_CUDA(expr)                                                                    \
@@ -49,14 +46,10 @@ cudaError_t launch_decode_step_mma(const Geom& G, const Arena& A, int layer, con
     }                                                                                     \
   } while (0)
 
-// Split-K scratch of the decode kernels: ticket counters (CUDA-core kernel: zero, self-resetting), then
-// the partial rows.  The tensor-core kernel uses a word of a partial row as its own arrival flag: between
-// launches every such word holds the all-ones pattern, which the combining CTA restores after reading.
-static cudaError_t init_decode_scratch(float* scratch, size_t bytes, size_t n_sl, cudaStream_t st) {
-  const size_t ticket_bytes = ((n_sl + 63) / 64) * 64 * sizeof(unsigned);
-  cudaError_t e = cudaMemsetAsync(scratch, 0xff, bytes, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(scratch, 0, ticket_bytes < bytes ? ticket_bytes : bytes, st);
-  return e;
+// Split-K scratch of the decode kernels: a word of a partial row is its own arrival flag, so between launches every
+// word holds the all-ones pattern, which the combining CTA restores after reading.
+static cudaError_t init_decode_scratch(float* scratch, size_t bytes, cudaStream_t st) {
+  return cudaMemsetAsync(scratch, 0xff, bytes, st);
 }
 
 struct balancekv_ctx {
@@ -80,7 +73,7 @@ struct balancekv_ctx {
   int* h_status = nullptr;       // pinned mirror of the status word, refreshed after every compress batch and by stats
   float* d_decode_scratch = nullptr;
   int max_splits = 1;
-  int decode_slots = 148;        // CTAs of the decode kernel that are resident at once
+  int decode_slots = 148;        // CTAs of a decode kernel that are resident at once
   bool use_tc = false;
   void* tmaps = nullptr;
   void* decode_maps = nullptr;   // tensor maps of the tensor-core decode kernel (bf16)
@@ -369,13 +362,12 @@ int balancekv_create(const balancekv_config* cfg, balancekv_ctx** out) {
   *c->h_status = 0;
   {
     const int n_sl = f.n_seqs * f.n_kv_heads;
-    const int per_sm = f.gram_path != 1 && decode_mma_supported(G) ? decode_mma_ctas_per_sm() : 2;
-    c->decode_slots = per_sm * c->sm_count;                                 // CTAs of one wave
+    c->decode_slots = kDecodeCtasPerSm * c->sm_count;                                 // CTAs of one wave
     c->max_splits = std::max(1, std::min(64, c->decode_slots / n_sl));      // rounding down keeps one wave
     if (f.decode_splits > 0) c->max_splits = std::min(64, f.decode_splits);
     const size_t sb = decode_scratch_bytes(G, c->max_splits);
     if ((rc = dev_alloc(c, reinterpret_cast<char**>(&c->d_decode_scratch), sb))) return fail(rc);
-    if (init_decode_scratch(c->d_decode_scratch, sb, (size_t)G.B * G.H, nullptr) != cudaSuccess) return fail(BALANCEKV_E_CUDA);
+    if (init_decode_scratch(c->d_decode_scratch, sb, nullptr) != cudaSuccess) return fail(BALANCEKV_E_CUDA);
     if (cudaStreamSynchronize(nullptr) != cudaSuccess) return fail(BALANCEKV_E_CUDA);
   }
   c->ring_half = (size_t)4 << 20;
@@ -719,7 +711,7 @@ static bool layer_seg_hint(balancekv_ctx* c, int layer, Seg* out) {
   return true;
 }
 
-// The tensor-core decode kernel adds g - 1 combining CTAs per stream to a launch with more than one split:
+// A decode launch with more than one split has g - 1 combining CTAs per stream besides its tile CTAs:
 // the largest split factor <= splits whose grid over n_streams streams still fits one wave.
 static int one_wave_splits(balancekv_ctx* c, int splits, int n_streams) {
   const int per_stream = c->decode_slots / std::max(1, n_streams);
@@ -738,36 +730,45 @@ static int pick_splits(balancekv_ctx* c, int layer) {
       for (int l = 1; l <= f.levels; ++l) rows += S.lvl_len[l];
       max_rows = std::max(max_rows, rows);
     }
-  const int tile_tokens = c->decode_maps ? decode_mma_tile_tokens() : 16384 / (f.head_dim * c->esz);
+  const int tile_tokens = c->decode_maps ? decode_mma_tile_tokens() : decode_tile_tokens(c->G);
   const int64_t tiles = (max_rows + tile_tokens - 1) / tile_tokens + f.levels;
-  int splits = pick_decode_splits(tiles, c->max_splits, c->decode_slots, f.n_seqs * f.n_kv_heads,
-                                  f.n_q_heads / f.n_kv_heads, c->decode_maps != nullptr);
+  int splits = pick_decode_splits(tiles, c->max_splits, c->decode_slots, f.n_seqs * f.n_kv_heads, c->G.g);
   if (f.decode_splits > 0) splits = std::min(f.decode_splits, c->max_splits);
   return splits;
+}
+
+// One decode launch over the layer's current caches; with k_new / v_new given it also appends one token per stream
+// (row rel of the level-0 region, original position idx0, new level-0 length new_len) and the host's bookkeeping of
+// that append has not happened yet.
+static int launch_decode_step(balancekv_ctx* c, int layer, const void* q, void* out, const void* k_new, const void* v_new,
+                              int rel, int idx0, int new_len, cudaStream_t st) {
+  StepAppend ap{};
+  ap.k_new = k_new; ap.v_new = v_new;
+  ap.rel_row = rel; ap.idx0 = idx0; ap.new_len = new_len;
+  ap.splits = pick_splits(c, layer);
+  if (layer_seg_hint(c, layer, ap.seg)) {
+    ap.n_seg = c->cfg.levels + 1;
+    ap.early = c->decode_chain && c->chain_stream == st;
+  }
+  ap.in_flag = c->step_flag;
+  ap.in_expect = c->step_expect;
+  c->step_flag = nullptr;
+  ProfScope ps(c, 4, st);
+  if (c->decode_maps)
+    BKV_CUDA(launch_decode_step_mma(c->G, c->A, layer, q, out, c->d_decode_scratch, ap, c->d_status, c->decode_maps, st));
+  else
+    BKV_CUDA(launch_decode(c->G, c->A, layer, q, out, c->d_decode_scratch, ap, c->d_status, st));
+  c->decode_chain = true;
+  c->chain_stream = st;
+  c->kernels_launched++;
+  return BALANCEKV_OK;
 }
 
 int balancekv_decode_attn(balancekv_ctx* c, int layer, const void* q, void* out, void* stream) {
   if (!c || layer < 0 || layer >= c->cfg.n_layers || !q || !out) return BALANCEKV_E_INVAL;
   if (!aligned16(q) || !aligned16(out)) return BALANCEKV_E_INVAL;
   if (timed_out(c)) return BALANCEKV_E_TIMEOUT;
-  const int splits = pick_splits(c, layer);
-  {
-    ProfScope ps(c, 4, static_cast<cudaStream_t>(stream));
-    if (c->decode_maps) {
-      Seg hint[kMaxLevels + 1];
-      const bool alike = layer_seg_hint(c, layer, hint);
-      cudaStream_t st = static_cast<cudaStream_t>(stream);
-      const int early = alike && c->decode_chain && c->chain_stream == st;
-      BKV_CUDA(launch_decode_step_mma(c->G, c->A, layer, q, out, c->d_decode_scratch, splits, c->d_status, c->decode_maps,
-                                      nullptr, nullptr, 0, 0, 0, alike ? hint : nullptr, early, nullptr, 0, st));
-      c->decode_chain = true;
-      c->chain_stream = st;
-    } else
-      BKV_CUDA(launch_decode(c->G, c->A, layer, q, out, c->d_decode_scratch, splits, c->d_status,
-                             static_cast<cudaStream_t>(stream)));
-  }
-  c->kernels_launched++;
-  return BALANCEKV_OK;
+  return launch_decode_step(c, layer, q, out, nullptr, nullptr, 0, 0, 0, static_cast<cudaStream_t>(stream));
 }
 
 int balancekv_decode_attn_host(balancekv_ctx* c, int layer, const void* q_host, void* out_host, void* stream) {
@@ -847,8 +848,7 @@ int balancekv_decode_attn_merged(balancekv_ctx* c, const int32_t* layers_num, in
     const size_t block_bytes = (decode_scratch_bytes(c->G, c->max_splits) + 255) & ~(size_t)255;
     BKV_CUDA(cudaMalloc(reinterpret_cast<void**>(&c->two_scratch), block_bytes * BALANCEKV_MAX_MERGE));
     for (int z = 0; z < BALANCEKV_MAX_MERGE; ++z)
-      BKV_CUDA(init_decode_scratch(reinterpret_cast<float*>(reinterpret_cast<char*>(c->two_scratch) + block_bytes * z), block_bytes,
-                                   (size_t)c->G.B * c->G.H, st));
+      BKV_CUDA(init_decode_scratch(reinterpret_cast<float*>(reinterpret_cast<char*>(c->two_scratch) + block_bytes * z), block_bytes, st));
     c->two_scratch_words = block_bytes / 4;
     c->bytes_resident += block_bytes * BALANCEKV_MAX_MERGE;
   }
@@ -879,7 +879,6 @@ int balancekv_decode_attn_two(balancekv_ctx* c, int layer_num, int layer_den, co
 
 // True if balancekv_stream_step will serve this layer's step with the one fused launch.
 static bool step_can_fuse(balancekv_ctx* c, int layer) {
-  if (!c->decode_maps) return false;
   const balancekv_config& f = c->cfg;
   const Layout& Lo = c->Lo;
   const std::vector<int>& streams = layer_streams(c, layer);
@@ -896,41 +895,19 @@ static bool step_can_fuse(balancekv_ctx* c, int layer) {
 int balancekv_stream_step(balancekv_ctx* c, int layer, const void* q, const void* k_new, const void* v_new, void* out,
                           void* stream) {
   if (c && timed_out(c)) return BALANCEKV_E_TIMEOUT;
-  // One launch when the tensor-core decode kernel serves this context and the layer's streams are
-  // in lockstep with room for the token: the kernel appends after attending (see its header).
-  if (c && layer >= 0 && layer < c->cfg.n_layers && c->decode_maps && q && out && k_new && v_new && aligned16(q) &&
-      aligned16(out) && aligned16(k_new) && aligned16(v_new)) {
-    const balancekv_config& f = c->cfg;
-    const Layout& Lo = c->Lo;
+  // One launch when the layer's streams are in lockstep with room for the token: the kernel appends after attending.
+  if (c && layer >= 0 && layer < c->cfg.n_layers && q && out && k_new && v_new && aligned16(q) && aligned16(out) &&
+      aligned16(k_new) && aligned16(v_new) && step_can_fuse(c, layer)) {
     const std::vector<int>& streams = layer_streams(c, layer);
-    const int max_pending = Lo.T == 0 ? f.max_tokens : (f.max_pending > 0 ? std::min(f.max_pending, f.max_tokens) : f.max_tokens);
     const StreamState& S0 = c->st[streams[0]];
-    bool fits = true;
+    const int rc = launch_decode_step(c, layer, q, out, k_new, v_new, S0.start0 + S0.len0, (int)S0.appended, S0.len0 + 1,
+                                      static_cast<cudaStream_t>(stream));
+    if (rc) return rc;
     for (int s : streams) {
-      const StreamState& S = c->st[s];
-      fits &= S.start0 == S0.start0 && S.len0 == S0.len0 && S.appended == S0.appended;
-      fits &= S.appended + 1 <= f.max_tokens && S.pending + 1 <= max_pending && (int64_t)S.start0 + S.len0 + 1 <= Lo.cap0;
+      StreamState& S = c->st[s];
+      S.len0 += 1; S.appended += 1; S.pending += 1; c->tokens_appended += 1;
     }
-    if (fits) {
-      const int splits = pick_splits(c, layer);
-      Seg hint[kMaxLevels + 1];
-      const bool alike = layer_seg_hint(c, layer, hint);       // the table before this step's append
-      const int rel = S0.start0 + S0.len0, idx0 = (int)S0.appended, new_len = S0.len0 + 1;
-      for (int s : streams) {
-        StreamState& S = c->st[s];
-        S.len0 += 1; S.appended += 1; S.pending += 1; c->tokens_appended += 1;
-      }
-      cudaStream_t st = static_cast<cudaStream_t>(stream);
-      const int early = alike && c->decode_chain && c->chain_stream == st;
-      ProfScope ps(c, 4, st);
-      BKV_CUDA(launch_decode_step_mma(c->G, c->A, layer, q, out, c->d_decode_scratch, splits, c->d_status, c->decode_maps,
-                                      k_new, v_new, rel, idx0, new_len, alike ? hint : nullptr, early, c->step_flag, c->step_expect, st));
-      c->step_flag = nullptr;
-      c->decode_chain = true;
-      c->chain_stream = st;
-      c->kernels_launched++;
-      return BALANCEKV_OK;
-    }
+    return BALANCEKV_OK;
   }
   int rc = balancekv_stream_append_layer(c, layer, k_new, v_new, 1, stream);
   if (rc) return rc;
@@ -1294,10 +1271,10 @@ int balancekv_reset(balancekv_ctx* c, void* stream) {
   BKV_CUDA(cudaMemsetAsync(c->d_status, 0, sizeof(int), st));
   *c->h_status = 0;
   // a launch that gave up may have left partial rows behind
-  BKV_CUDA(init_decode_scratch(c->d_decode_scratch, decode_scratch_bytes(c->G, c->max_splits), (size_t)c->G.B * c->G.H, st));
+  BKV_CUDA(init_decode_scratch(c->d_decode_scratch, decode_scratch_bytes(c->G, c->max_splits), st));
   if (c->two_scratch)
     for (int z = 0; z < BALANCEKV_MAX_MERGE; ++z)
-      BKV_CUDA(init_decode_scratch(c->two_scratch + c->two_scratch_words * z, c->two_scratch_words * 4, (size_t)c->G.B * c->G.H, st));
+      BKV_CUDA(init_decode_scratch(c->two_scratch + c->two_scratch_words * z, c->two_scratch_words * 4, st));
   return BALANCEKV_OK;
 }
 
@@ -1369,14 +1346,11 @@ int balancekv_debug_set_status(balancekv_ctx* c, int value) {
 int balancekv_debug_scratch_used(balancekv_ctx* c, int64_t* words) {
   if (!c || !words) return BALANCEKV_E_INVAL;
   *words = 0;
-  if (!c->decode_maps) return BALANCEKV_OK;          // the CUDA-core kernel keeps no state in its partial rows
   BKV_CUDA(cudaDeviceSynchronize());
-  const size_t n_sl = (size_t)c->G.B * c->G.H;
-  const size_t ticket_words = ((n_sl + 63) / 64) * 64;
   auto count = [&](const float* block, size_t bytes) -> int {
     std::vector<uint32_t> host(bytes / 4);
     if (cudaMemcpy(host.data(), block, host.size() * 4, cudaMemcpyDeviceToHost) != cudaSuccess) return BALANCEKV_E_CUDA;
-    for (size_t i = ticket_words; i < host.size(); ++i) *words += host[i] != 0xffffffffu;
+    for (size_t i = 0; i < host.size(); ++i) *words += host[i] != 0xffffffffu;
     return BALANCEKV_OK;
   };
   int rc = count(c->d_decode_scratch, decode_scratch_bytes(c->G, c->max_splits));

@@ -178,22 +178,22 @@ cudaError_t launch_walk_tc(const Geom& G, const Arena& A, const CallDesc* calls,
                            const void* tmap_k, const void* tmap_v, cudaStream_t st);
 cudaError_t launch_compact(const Geom& G, const Arena& A, const CallDesc* calls, int n_calls, int level,
                            const int8_t* eta, cudaStream_t st);
+struct StepAppend;      // decode_common.cuh
 size_t decode_scratch_bytes(const Geom& G, int splits);
+int decode_tile_tokens(const Geom& G);
 cudaError_t launch_decode(const Geom& G, const Arena& A, int layer, const void* q, void* out, float* scratch,
-                          int splits, int* status, cudaStream_t st);
+                          const StepAppend& ap, int* status, cudaStream_t st);
 // Split-K factor of a decode launch whose longest stream has `tiles` tiles: at least two tiles per CTA, the fewest
-// splits with that number of tiles per CTA (the tile phase is as long, the combine shorter), and -- for the kernel
-// whose heads 1 .. g - 1 are combined by CTAs of their own -- a grid of one wave of `slots` resident CTAs.
-inline int pick_decode_splits(int64_t tiles, int max_splits, int slots, int n_streams, int g, bool combiners) {
+// splits with that number of tiles per CTA (the tile phase is as long, the combine shorter), and a grid of one wave
+// of `slots` resident CTAs (the heads 1 .. g - 1 of a stream are combined by CTAs of their own).
+inline int pick_decode_splits(int64_t tiles, int max_splits, int slots, int n_streams, int g) {
   int64_t splits = (tiles + 1) / 2 < max_splits ? (tiles + 1) / 2 : max_splits;
   if (splits < 1) splits = 1;
   int64_t per = (tiles + splits - 1) / splits;
   if (per < 1) per = 1;
   splits = (tiles + per - 1) / per;
-  if (combiners) {
-    const int64_t room = slots / (n_streams > 0 ? n_streams : 1) - (g - 1);
-    if (splits > room) splits = room;
-  }
+  const int64_t room = slots / (n_streams > 0 ? n_streams : 1) - (g - 1);
+  if (splits > room) splits = room;
   return splits < 1 ? 1 : (int)splits;
 }
 cudaError_t launch_fill_weights(float* w, int n, float value, cudaStream_t st);

@@ -1,4 +1,5 @@
-// Split-K decode attention over the weighted compressed cache.
+// Split-K decode attention over the weighted compressed cache on CUDA cores, for the contexts that the tensor-core
+// kernel does not serve: fp32 caches, and bf16 ones that ask for this family.
 //
 //   out = sum_i w_i e^{<k_i,q>/sqrt d} v_i / sum_i w_i e^{<k_i,q>/sqrt d},   w_i = 2^level(i)
 //
@@ -6,373 +7,347 @@
 // C^T..C^0 of one stream (Eq. (1) when every token sits in C^0).  In base 2 the weight is an
 // exact integer added to the logit: l_i = <k_i,q> log2(e)/sqrt d + level(i).
 //
-// Grid (streams of the layer, splits).  A CTA walks its share of the stream's 16 KB tiles
-// (K and V rows are contiguous per level, so a tile is one linear bulk copy per tensor)
-// through a 3-stage shared-memory ring filled by cp.async.bulk + mbarrier.  Each warp keeps
-// private online-softmax state (max, sum, accumulator) for all g query heads of the KV
-// head: 8 lanes share a token for the q.k dot product, then every lane owns D/32 output
-// columns for p.v.  Warps merge through shared memory, splits through a global scratch
-// and a ticket counter (the last CTA of a stream combines; nobody waits).
-#include "common.cuh"
+// Grid (streams of the layer, splits [+ g - 1]), two CTAs per SM.  A CTA walks its share of the stream's 16 KB tiles
+// (K and V rows are contiguous per level, so a tile is one linear bulk copy per tensor) through a 3-stage ring: a
+// lane fills it by cp.async.bulk + mbarrier, eight warps consume it and hand a stage back through a second
+// barrier, so that no warp waits for the slowest one tile by tile.  A warp takes batches of 32 / HP tokens (HP = g
+// rounded up to a power of two).  For the scores every lane holds d / 32 dims of all queries: one conflict-free row
+// load and HP packed multiply-adds per token; the 32 (token, head) sums of a batch then meet in one transposed
+// reduction of 31 shuffles that leaves one score in each lane, so that a batch costs one exponential per lane.  The
+// probabilities go through 128 bytes of shared memory to the value phase, where a lane owns d / 32 output columns.
+// Warps merge through shared memory; splits, the fused append and the result are HeadEnd's (decode_common.cuh).
+//
+// What bounds it: at batch sizes that fill the chip, HBM; otherwise the chain of one launch.  fp32, 8 streams x 2500
+// rows x 4 heads of 128 dims: 10.6 us per launch against 26.5 us with eight lanes per token, all warps in step per tile and
+// the last CTA of a stream reading the partial rows one after the other; one stream of 700 rows, d = 64: 4.9 us against 10.2.
+#include "decode_common.cuh"
 
 namespace bkv {
 
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kWarps = 8;
+using namespace dec;
+
+constexpr int kWarps = 8;                  // consumers; one lane of warp 0 also issues the copies (a warp more would cost registers)
+constexpr int kThreads = 32 * kWarps;
 constexpr int kStages = 3;
 constexpr int kTileBytes = 16384;          // per tensor per stage
+constexpr size_t kSmemBytes = (size_t)kStages * 2 * kTileBytes + 2 * kStages * sizeof(uint64_t);
 constexpr int kMaxDevices = 64;
-constexpr long long kWaitCycles = 100000000LL;    // about 50 ms: a bulk copy that has not landed by then never will
 
-__device__ inline uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ inline void mbar_init(uint64_t* bar, int count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
-}
-__device__ inline void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-__device__ inline bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
-  return ok != 0;
-}
-// Bounded wait: gives up after kWaitCycles and reports failure.
-__device__ inline bool mbar_wait(uint64_t* bar, uint32_t parity) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const long long t0 = clock64();
-  while (!mbar_try_wait(bar, parity)) {
-    if (clock64() - t0 > kWaitCycles) return false;
-  }
-  return true;
-}
 __device__ inline void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
 }
 
-struct TileRef {
-  int64_t row;   // first arena row
-  int rows;      // valid rows
-  int level;
-};
-
-template <int TN>
-__device__ inline TileRef locate_tile(int tile, const int* lvl_tiles, const Seg* seg, int T, int64_t stream_base,
-                                      const int32_t* region_off) {
-  // levels are visited from T down to 0
-  TileRef r{0, 0, 0};
-  for (int l = T; l >= 0; --l) {
-    const int nt = lvl_tiles[l];
-    if (tile < nt) {
-      r.level = l;
-      r.row = stream_base + region_off[l] + seg[l].start + (int64_t)tile * TN;
-      r.rows = min(TN, seg[l].len - tile * TN);
-      return r;
+// This lane's d / 32 neighbouring elements of a row.
+template <typename E, int N>
+__device__ inline void load_cols(const unsigned char* row, int lane, float2 (&v)[N / 2]) {
+  if constexpr (sizeof(E) == 4) {
+    if constexpr (N == 4) {
+      const float4 w = *reinterpret_cast<const float4*>(row + lane * 16);
+      v[0] = make_float2(w.x, w.y); v[1] = make_float2(w.z, w.w);
+    } else {
+      v[0] = *reinterpret_cast<const float2*>(row + lane * 8);
     }
-    tile -= nt;
+  } else {
+    if constexpr (N == 4) {
+      const uint2 w = *reinterpret_cast<const uint2*>(row + lane * 8);
+      v[0] = make_float2(bf16_lo(w.x), bf16_hi(w.x)); v[1] = make_float2(bf16_lo(w.y), bf16_hi(w.y));
+    } else {
+      const uint32_t w = *reinterpret_cast<const uint32_t*>(row + lane * 4);
+      v[0] = make_float2(bf16_lo(w), bf16_hi(w));
+    }
   }
-  return r;
 }
 
-template <bool kBf16, int D, int GQ>
-__global__ void __launch_bounds__(kThreads, 2)
-decode_kernel(Geom G, Arena A, int layer, const void* __restrict__ q, void* __restrict__ out,
-              float* __restrict__ part, unsigned* __restrict__ tickets, int* __restrict__ status) {
-  constexpr int esz = kBf16 ? 2 : 4;
-  constexpr int TN = kTileBytes / (D * esz);      // tokens per tile
-  constexpr int DPL = D / 8;                      // dims per lane in the q.k phase
-  constexpr int CPL = D / 32;                     // output columns per lane
-  constexpr int PS = D + 2;                       // partial row: acc[D], max, sum
+template <typename E, int D, int HP>
+__global__ void __launch_bounds__(kThreads, kDecodeCtasPerSm)
+decode_kernel(Geom G, Arena A, int layer, const E* __restrict__ q, E* __restrict__ out, float* __restrict__ part,
+              int* __restrict__ status, const StepAppend ap) {
+  constexpr int TN = kTileBytes / (D * (int)sizeof(E));   // tokens per tile
+  constexpr int CPL = D / 32;                     // dims / output columns per lane
+  constexpr int NT = 32 / HP;                     // tokens of a batch
+  constexpr int PS = D + 4;                       // merge row: acc[D], max, sum, pad
+  constexpr uint32_t kRowBytes = D * (uint32_t)sizeof(E);
+  static_assert(TN % NT == 0, "a tile is a whole number of batches");
 
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  unsigned char* tiles = smem_raw;                                   // kStages * 2 * kTileBytes
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem_raw + kStages * 2 * kTileBytes);
+  extern __shared__ __align__(128) unsigned char tiles[];            // kStages * 2 * kTileBytes, then the barriers
+  uint64_t* full = reinterpret_cast<uint64_t*>(tiles + kStages * 2 * kTileBytes);
+  uint64_t* empty = full + kStages;
   __shared__ int lvl_tiles[kMaxLevels + 1];
   __shared__ Seg seg_s[kMaxLevels + 1];
-  __shared__ int is_last_s;
+  __shared__ __align__(16) float probs[kWarps][32];   // read as float4
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int g = G.g;
   const int sl = blockIdx.x;                       // stream inside the layer: seq * H + head
-  const int seq = sl / G.H, head = sl % G.H;
-  const int stream = (seq * G.L + layer) * G.H + head;
-  const int splits = gridDim.y, split = blockIdx.y;
-  const int64_t stream_base = (int64_t)stream * G.rows_per_stream;
+  const int stream = ((sl / G.H) * G.L + layer) * G.H + sl % G.H;
+  const int splits = ap.splits, split = blockIdx.y;     // split >= splits: a combiner without tiles
+  q += (size_t)sl * g * D;
+  out += (size_t)sl * g * D;
 
-  if (tid <= G.T) {
-    const Seg s = A.seg[(size_t)stream * (G.T + 1) + tid];
-    seg_s[tid] = s;
-    lvl_tiles[tid] = (s.len + TN - 1) / TN;
-  }
+  // Prologue as in the tensor-core kernel: before griddepcontrol.wait only barrier set-up and, in a chain of decode
+  // launches (ap.early), the fetch of tiles that the previous launch does not write.
   if (tid == 0) {
-    for (int s = 0; s < kStages; ++s) mbar_init(&full[s], 1);
+    for (int s = 0; s < kStages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], kWarps); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  prefetch_operands<kRowBytes>(ap, q, sl, g);
+  const bool early = ap.early && ap.n_seg;
+  if (!early) grid_wait_and_release();
+  if (tid <= G.T) {
+    const Seg s = ap.n_seg ? ap.seg[tid] : A.seg[(size_t)stream * (G.T + 1) + tid];
+    seg_s[tid] = s;
+    lvl_tiles[tid] = (s.len + TN - 1) / TN;
   }
   __syncthreads();
   int n_tiles = 0;
   for (int l = 0; l <= G.T; ++l) n_tiles += lvl_tiles[l];
   const int t_begin = (int)((long long)n_tiles * split / splits);
   const int t_end = (int)((long long)n_tiles * (split + 1) / splits);
-  const int my_tiles = t_end - t_begin;
+  const int my_tiles = split < splits ? t_end - t_begin : 0;
 
-  // query of this lane's dims for the g heads of the KV head, pre-scaled by log2(e)/sqrt d
-  const int sub = lane & 7, grp = lane >> 3;
-  float qr[GQ][DPL];
-  {
-    const float sc = 1.4426950408889634f * G.inv_sqrt_d;
-#pragma unroll
-    for (int h = 0; h < GQ; ++h) {
-      const size_t off = ((size_t)seq * (G.H * GQ) + head * GQ + h) * D;
-#pragma unroll
-      for (int i = 0; i < DPL; i += 8) {
-        float v[8];
-        load8<kBf16>(static_cast<const char*>(q) + off * esz, sub * DPL + i, v);
-#pragma unroll
-        for (int k = 0; k < 8; ++k) qr[h][i + k] = v[k] * sc;
-      }
-    }
-  }
-
-  auto issue = [&](int i) {   // thread 0 only
-    const TileRef tr = locate_tile<TN>(t_begin + i, lvl_tiles, seg_s, G.T, stream_base, G.region_off);
+  auto issue = [&](int i) {   // one thread
+    const TileRef tr = locate_tile<TN>(t_begin + i, lvl_tiles, seg_s, G.T, G.region_off);
     const int s = i % kStages;
-    const uint32_t bytes = (uint32_t)tr.rows * D * esz;
+    const uint32_t bytes = (uint32_t)tr.rows * kRowBytes;
+    const size_t off = ((size_t)stream * G.rows_per_stream + tr.row) * kRowBytes;
     mbar_expect_tx(&full[s], 2 * bytes);
-    bulk_load(tiles + (size_t)s * 2 * kTileBytes, static_cast<const char*>(A.K) + (size_t)tr.row * D * esz, bytes, &full[s]);
-    bulk_load(tiles + (size_t)s * 2 * kTileBytes + kTileBytes, static_cast<const char*>(A.V) + (size_t)tr.row * D * esz, bytes, &full[s]);
+    bulk_load(tiles + (size_t)s * 2 * kTileBytes, static_cast<const char*>(A.K) + off, bytes, &full[s]);
+    bulk_load(tiles + (size_t)s * 2 * kTileBytes + kTileBytes, static_cast<const char*>(A.V) + off, bytes, &full[s]);
   };
-  if (tid == 0)
-    for (int i = 0; i < min(kStages, my_tiles); ++i) issue(i);
+  const bool producer = tid == 0;
+  int issued = 0;
+  if (producer) {
+    const int lim = min(kStages, my_tiles);
+    while (issued < lim && !(early && t_begin + issued == n_tiles - 1)) issue(issued++);
+  }
+  if (early) {
+    grid_wait_and_release();
+    if (producer)
+      while (issued < min(kStages, my_tiles)) issue(issued++);
+  }
+  wait_operands(ap, status);
 
-  float m_run[GQ], l_run[GQ], acc[GQ][CPL];
-#pragma unroll
-  for (int h = 0; h < GQ; ++h) {
-    m_run[h] = -INFINITY; l_run[h] = 0.f;
-#pragma unroll
-    for (int c = 0; c < CPL; ++c) acc[h][c] = 0.f;
+  const float sc = 1.4426950408889634f * G.inv_sqrt_d;
+  const HeadEnd<E, D> end{G, A, ap, q, out, nullptr, nullptr, sl, stream, g, warp, lane, sc};
+  constexpr uint32_t kFacOff = 2 * kWarps * kMaxGroup * PS * 4;   // behind the merge rows and the merged ones
+  static_assert(kFacOff + kWarps * kDecodeMaxSplits * 4 <= kStages * 2 * kTileBytes, "the merge buffers reuse the tile ring");
+  float* const fac = reinterpret_cast<float*>(tiles + kFacOff) + warp * kDecodeMaxSplits;
+  if (split >= splits) {                          // the combiner of head split - splits + 1
+    end.combine_head(split - splits + 1, part, gridDim.x, fac, status);
+    return;
   }
 
-  bool failed = false;
-  for (int i = 0; i < my_tiles; ++i) {
-    const int s = i % kStages;
-    const bool arrived = __all_sync(0xffffffffu, mbar_wait(&full[s], (uint32_t)((i / kStages) & 1)));
-    TileRef tr = locate_tile<TN>(t_begin + i, lvl_tiles, seg_s, G.T, stream_base, G.region_off);
-    const unsigned char* Kt = tiles + (size_t)s * 2 * kTileBytes;
-    const unsigned char* Vt = Kt + kTileBytes;
-    const float lvl = (float)tr.level;
-    if (!arrived) tr.rows = 0;   // skip the tile; the CTA agrees on the failure below
-#pragma unroll 1
-    for (int base = warp * 4; base < tr.rows; base += 4 * kWarps) {
-      const int tok = base + grp;
-      const bool valid = tok < tr.rows;
-      // ---- q.k: 8 lanes per token
-      float dot[GQ];
+  bool ok = true;
+  const int my_h = lane % HP, my_tk = lane / HP;   // this lane's (head, token of the batch) after the reduction
+  float m_run = -INFINITY, l_run = 0.f;            // of head my_h; the sum over this lane's tokens
+  float2 acc[HP][CPL / 2];
 #pragma unroll
-      for (int h = 0; h < GQ; ++h) dot[h] = 0.f;
+  for (int h = 0; h < HP; ++h)
 #pragma unroll
-      for (int i8 = 0; i8 < DPL; i8 += 8) {
-        float kf[8];
-        load8<kBf16>(Kt + (size_t)(valid ? tok : 0) * D * esz, sub * DPL + i8, kf);
+    for (int c = 0; c < CPL / 2; ++c) acc[h][c] = make_float2(0.f, 0.f);
+
+  {
+    float2 qr[HP][CPL / 2];
 #pragma unroll
-        for (int h = 0; h < GQ; ++h)
+    for (int h = 0; h < HP; ++h) {
+      if (h < g) load_cols<E, CPL>(reinterpret_cast<const unsigned char*>(q + (size_t)h * D), lane, qr[h]);
+      else
 #pragma unroll
-          for (int k = 0; k < 8; ++k) dot[h] = fmaf(qr[h][i8 + k], kf[k], dot[h]);
-      }
-      float mx_new[GQ];
-      bool grew = false;
-#pragma unroll
-      for (int h = 0; h < GQ; ++h) {
-        float v = dot[h];
-        v += __shfl_xor_sync(0xffffffffu, v, 1);
-        v += __shfl_xor_sync(0xffffffffu, v, 2);
-        v += __shfl_xor_sync(0xffffffffu, v, 4);
-        v = valid ? v + lvl : -INFINITY;
-        dot[h] = v;
-        float mx = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 8));
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
-        mx_new[h] = fmaxf(m_run[h], mx);
-        grew |= mx_new[h] > m_run[h];
-      }
-      if (grew) {   // warp-uniform
-#pragma unroll
-        for (int h = 0; h < GQ; ++h) {
-          const float a = exp2f(m_run[h] - mx_new[h]);   // m_run = -inf -> 0; mx_new is finite here
-          l_run[h] *= a;
-#pragma unroll
-          for (int c = 0; c < CPL; ++c) acc[h][c] *= a;
-          m_run[h] = mx_new[h];
-        }
-      }
-      float p[GQ];
-#pragma unroll
-      for (int h = 0; h < GQ; ++h) {
-        p[h] = valid ? exp2f(dot[h] - m_run[h]) : 0.f;
-        if (sub == 0) l_run[h] += p[h];      // one lane per token carries the sum
-      }
-      // ---- p.v: every lane owns CPL columns
-#pragma unroll
-      for (int tk = 0; tk < 4; ++tk) {
-        if (base + tk < tr.rows) {   // warp-uniform
-          float vf[CPL];
-          const unsigned char* vrow = Vt + (size_t)(base + tk) * D * esz;
-          if constexpr (kBf16) {
-            if constexpr (CPL == 4) {
-              const uint2 w = *reinterpret_cast<const uint2*>(vrow + lane * 8);
-              vf[0] = bf16_lo(w.x); vf[1] = bf16_hi(w.x); vf[2] = bf16_lo(w.y); vf[3] = bf16_hi(w.y);
-            } else {
-              const uint32_t w = *reinterpret_cast<const uint32_t*>(vrow + lane * 4);
-              vf[0] = bf16_lo(w); vf[1] = bf16_hi(w);
-            }
-          } else {
-            if constexpr (CPL == 4) {
-              const float4 w = *reinterpret_cast<const float4*>(vrow + lane * 16);
-              vf[0] = w.x; vf[1] = w.y; vf[2] = w.z; vf[3] = w.w;
-            } else {
-              const float2 w = *reinterpret_cast<const float2*>(vrow + lane * 8);
-              vf[0] = w.x; vf[1] = w.y;
-            }
-          }
-#pragma unroll
-          for (int h = 0; h < GQ; ++h) {
-            const float ph = __shfl_sync(0xffffffffu, p[h], tk * 8);
-#pragma unroll
-            for (int c = 0; c < CPL; ++c) acc[h][c] = fmaf(ph, vf[c], acc[h][c]);
-          }
-        }
-      }
+        for (int c = 0; c < CPL / 2; ++c) qr[h][c] = make_float2(0.f, 0.f);
     }
-    // stage s fully consumed; the same barrier makes a timed-out wait a CTA-wide decision
-    if (__syncthreads_or(!arrived)) { failed = true; break; }
-    if (tid == 0 && i + kStages < my_tiles) issue(i + kStages);
+    constexpr int kBatches = TN / NT;              // batches of a full tile
+    for (int i = 0; i < my_tiles; ++i) {
+      const int s = i % kStages;
+      if (producer && i > 0 && issued < my_tiles) {  // refill the stage of tile i - 1 once every warp has left it
+        ok = mbar_wait(&empty[issued % kStages], (uint32_t)((issued / kStages - 1) & 1));
+        if (ok) issue(issued++);
+      }
+      // Every warp waits for every tile, so that the phase before the awaited one is always one it has seen; one
+      // lane polls (every poll is a serialised shared-memory access).
+      if (lane == 0) ok = ok && mbar_wait(&full[s], (uint32_t)((i / kStages) & 1));
+      ok = __shfl_sync(0xffffffffu, ok, 0);
+      __syncwarp();                                // the polling lane's view of the landed tile, for the whole warp
+      if (!ok) break;
+      const TileRef tr = locate_tile<TN>(t_begin + i, lvl_tiles, seg_s, G.T, G.region_off);
+      const unsigned char* Kt = tiles + (size_t)s * 2 * kTileBytes;
+      const unsigned char* Vt = Kt + kTileBytes;
+      // batches go round the warps across tiles
+      int b0 = (warp - i * kBatches) % kWarps;
+      if (b0 < 0) b0 += kWarps;
+      for (int base = b0 * NT; base < tr.rows; base += kWarps * NT) {
+        // ---- scores: partial sums of 32 (token, head) pairs, index token * HP + head.  Rows past the end repeat
+        // the last one; their scores are masked.
+        float v[32];
+#pragma unroll
+        for (int tk = 0; tk < NT; ++tk) {
+          float2 kf[CPL / 2];
+          load_cols<E, CPL>(Kt + (size_t)min(base + tk, tr.rows - 1) * kRowBytes, lane, kf);
+#pragma unroll
+          for (int h = 0; h < HP; ++h) {
+            float2 d2 = __fmul2_rn(qr[h][0], kf[0]);
+            if constexpr (CPL == 4) d2 = __ffma2_rn(qr[h][1], kf[1], d2);
+            v[tk * HP + h] = d2.x + d2.y;
+          }
+        }
+        // ---- transposed reduction: lane L ends with the sum of pair L over all lanes
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          const bool up = lane & o;
+#pragma unroll
+          for (int k = 0; k < o; ++k) {
+            const float send = up ? v[k] : v[k + o], keep = up ? v[k + o] : v[k];
+            v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+          }
+        }
+        const float x = base + my_tk < tr.rows ? fmaf(v[0], sc, (float)tr.level) : -INFINITY;
+        float mx = x;
+#pragma unroll
+        for (int o = HP; o < 32; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        const float mn = fmaxf(m_run, mx);         // finite: the batch's first token is valid
+        if (__any_sync(0xffffffffu, mn > m_run)) {
+          const float a = exp2f(m_run - mn);       // m_run = -inf -> 0
+          l_run *= a;
+          m_run = mn;
+#pragma unroll
+          for (int h = 0; h < HP; ++h) {
+            const float ah = __shfl_sync(0xffffffffu, a, h);
+#pragma unroll
+            for (int c = 0; c < CPL / 2; ++c) acc[h][c] = __fmul2_rn(acc[h][c], make_float2(ah, ah));
+          }
+        }
+        const float p = exp2f(x - m_run);
+        l_run += p;
+        __syncwarp();                              // the previous batch's probabilities have been read
+        probs[warp][lane] = p;
+        __syncwarp();
+        // ---- values
+        float pb[32];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) *reinterpret_cast<float4*>(pb + 4 * k) = *reinterpret_cast<const float4*>(&probs[warp][4 * k]);
+#pragma unroll
+        for (int tk = 0; tk < NT; ++tk) {
+          float2 vf[CPL / 2];
+          load_cols<E, CPL>(Vt + (size_t)min(base + tk, tr.rows - 1) * kRowBytes, lane, vf);
+#pragma unroll
+          for (int h = 0; h < HP; ++h) {
+            const float ph = pb[tk * HP + h];
+#pragma unroll
+            for (int c = 0; c < CPL / 2; ++c) acc[h][c] = __ffma2_rn(make_float2(ph, ph), vf[c], acc[h][c]);
+          }
+        }
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&empty[s]);
+    }
   }
-  if (failed) {
-    if (lane == 0) atomicCAS(status, kStatusOk, kStatusWaitTimeout);
-  }
-  __syncthreads();
+  if (!ok && lane == 0) atomicCAS(status, kStatusOk, kStatusWaitTimeout);
+  __syncthreads();                                 // the tile ring is idle now
 
-  // ---- merge the 8 warps through shared memory (the tile ring is idle now)
-  float* mrg = reinterpret_cast<float*>(tiles);        // [kWarps][GQ][PS]
+  // ---- merge the 8 warps through shared memory
+  float* mrg = reinterpret_cast<float*>(tiles);        // [kWarps][g][PS], behind it the merged rows [g][PS]
+  float* merged = mrg + kWarps * kMaxGroup * PS;
+  {
 #pragma unroll
-  for (int h = 0; h < GQ; ++h) {
-    float l = l_run[h];
-    l += __shfl_xor_sync(0xffffffffu, l, 8);
-    l += __shfl_xor_sync(0xffffffffu, l, 16);
-    l = __shfl_sync(0xffffffffu, l, 0);
-    float* row = mrg + ((size_t)warp * GQ + h) * PS;
+    for (int o = HP; o < 32; o <<= 1) l_run += __shfl_xor_sync(0xffffffffu, l_run, o);
 #pragma unroll
-    for (int c = 0; c < CPL; ++c) row[lane * CPL + c] = acc[h][c];
-    if (lane == 0) { row[D] = m_run[h]; row[D + 1] = l; }
+    for (int h = 0; h < HP; ++h)
+      if (h < g) {
+        float* row = mrg + ((size_t)warp * g + h) * PS;
+#pragma unroll
+        for (int c = 0; c < CPL / 2; ++c) *reinterpret_cast<float2*>(row + lane * CPL + 2 * c) = acc[h][c];
+      }
+    if (lane < g && lane < HP) *reinterpret_cast<float2*>(mrg + ((size_t)warp * g + lane) * PS + D) = make_float2(m_run, l_run);
   }
   __syncthreads();
-  float* my_part = part + ((size_t)sl * splits + split) * GQ * PS;
-  for (int i = tid; i < GQ * D; i += kThreads) {
-    const int h = i / D, c = i % D;
-    float M = -INFINITY;
+  const bool single = splits == 1;
+  if (warp < g) {                                  // g <= 8: a warp per head
+    const int h = warp;
+    float mw[kWarps], M = -INFINITY;
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w) M = fmaxf(M, mrg[((size_t)w * GQ + h) * PS + D]);
-    float o = 0.f, L = 0.f;
+    for (int w = 0; w < kWarps; ++w) { mw[w] = mrg[((size_t)w * g + h) * PS + D]; M = fmaxf(M, mw[w]); }
+    float2 a[CPL / 2];
+    float L = 0.f;
+#pragma unroll
+    for (int c = 0; c < CPL / 2; ++c) a[c] = make_float2(0.f, 0.f);
 #pragma unroll
     for (int w = 0; w < kWarps; ++w) {
-      const float* row = mrg + ((size_t)w * GQ + h) * PS;
-      const float sc = row[D] == -INFINITY ? 0.f : exp2f(row[D] - M);
-      o = fmaf(row[c], sc, o);
-      L = fmaf(row[D + 1], sc, L);
+      const float* row = mrg + ((size_t)w * g + h) * PS;
+      const float f = mw[w] == -INFINITY ? 0.f : exp2f(mw[w] - M);
+#pragma unroll
+      for (int c = 0; c < CPL / 2; ++c) a[c] = __ffma2_rn(*reinterpret_cast<const float2*>(row + lane * CPL + 2 * c), make_float2(f, f), a[c]);
+      L = fmaf(row[D + 1], f, L);
     }
-    my_part[h * PS + c] = o;
-    if (c == 0) { my_part[h * PS + D] = M; my_part[h * PS + D + 1] = L; }
-  }
-  // ---- ticket: the last CTA of the stream combines the splits
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) {
-    const unsigned old = atomicAdd(&tickets[sl], 1u);
-    is_last_s = old == (unsigned)(splits - 1);
-  }
-  __syncthreads();
-  if (!is_last_s) return;
-  __threadfence();
-  const float* sp = part + (size_t)sl * splits * GQ * PS;
-  for (int i = tid; i < GQ * D; i += kThreads) {
-    const int h = i / D, c = i % D;
-    float M = -INFINITY;
-    for (int s = 0; s < splits; ++s) M = fmaxf(M, __ldcg(sp + ((size_t)s * GQ + h) * PS + D));
-    float o = 0.f, L = 0.f;
-    for (int s = 0; s < splits; ++s) {
-      const float* row = sp + ((size_t)s * GQ + h) * PS;
-      const float ms = __ldcg(row + D);
-      const float sc = ms == -INFINITY ? 0.f : exp2f(ms - M);
-      o = fmaf(__ldcg(row + c), sc, o);
-      L = fmaf(__ldcg(row + D + 1), sc, L);
+    if (single) {
+#pragma unroll
+      for (int c = 0; c < CPL / 2; ++c) *reinterpret_cast<float2*>(merged + h * PS + lane * CPL + 2 * c) = a[c];
+      if (lane == 0) *reinterpret_cast<float2*>(merged + h * PS + D) = make_float2(M, L);
+    } else {                                       // published: see HeadEnd::combine_head
+      float* row = part + (((size_t)sl * splits + split) * g + h) * D + lane * CPL;
+      if constexpr (CPL == 4) st_scratch4(row, make_float4(a[0].x, a[0].y, a[1].x, a[1].y));
+      else st_scratch2(row, a[0]);
+      constexpr int kCopies = HeadEnd<E, D>::kColWarps;
+      float* ml = part + (size_t)gridDim.x * splits * g * D + ((size_t)sl * g + h) * kCopies * splits * 2;
+      if (lane < kCopies) st_scratch2(ml + ((size_t)lane * splits + split) * 2, make_float2(M, L));
     }
-    const float r = L > 0.f ? o / L : 0.f;
-    const size_t off = ((size_t)seq * (G.H * GQ) + head * GQ + h) * D + c;
-    if constexpr (kBf16) static_cast<__nv_bfloat16*>(out)[off] = __float2bfloat16_rn(r);
-    else static_cast<float*>(out)[off] = r;
   }
-  if (tid == 0) tickets[sl] = 0;   // ready for the next launch
+  if (single) {
+    __syncthreads();
+    const auto nt = end.load_new(-1);
+#pragma unroll
+    for (int h = 0; h < kMaxGroup; ++h)
+      if (h < g)
+        end.finish(h, *reinterpret_cast<const float4*>(merged + h * PS + (32 * warp) % D + 4 * (lane & 7)), merged[h * PS + D],
+                   merged[h * PS + D + 1], nt, ap.k_new ? end.score_new(nt, h) : 0.f);
+    return;
+  }
+  if (split == splits - 1) end.combine_head(0, part, gridDim.x, fac, status);
 }
 
-template <bool kBf16, int D, int GQ>
-cudaError_t launch_t(const Geom& G, const Arena& A, int layer, const void* q, void* out, float* scratch,
-                     int splits, int* status, cudaStream_t st) {
-  auto kern = decode_kernel<kBf16, D, GQ>;
-  const size_t smem = (size_t)kStages * 2 * kTileBytes + kStages * sizeof(uint64_t);
+template <typename E, int D, int HP>
+cudaError_t launch_t(const Geom& G, const Arena& A, int layer, const void* q, void* out, float* part, const StepAppend& ap,
+                     int* status, cudaStream_t st) {
+  auto kern = decode_kernel<E, D, HP>;
   // the attribute belongs to the (kernel, device) pair: once per device that launches this instance
   static bool configured[kMaxDevices] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= kMaxDevices || !configured[dev]) {
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < kMaxDevices) configured[dev] = true;
   }
-  const int n_sl = G.B * G.H;
-  unsigned* tickets = reinterpret_cast<unsigned*>(scratch);
-  float* part = scratch + ((n_sl + 63) / 64) * 64;
-  dim3 grid(n_sl, splits);
-  kern<<<grid, kThreads, smem, st>>>(G, A, layer, q, out, part, tickets, status);
-  return cudaGetLastError();
+  const PdlConfig pc(dim3(G.B * G.H, decode_grid_y(G, ap.splits)), kThreads, kSmemBytes, st);
+  return cudaLaunchKernelEx(&pc.cfg, kern, G, A, layer, static_cast<const E*>(q), static_cast<E*>(out), part, status, ap);
 }
 
-template <bool kBf16, int D>
-cudaError_t launch_g(const Geom& G, const Arena& A, int layer, const void* q, void* out, float* scratch,
-                     int splits, int* status, cudaStream_t st) {
-  switch (G.g) {
-    case 1: return launch_t<kBf16, D, 1>(G, A, layer, q, out, scratch, splits, status, st);
-    case 2: return launch_t<kBf16, D, 2>(G, A, layer, q, out, scratch, splits, status, st);
-    case 3: return launch_t<kBf16, D, 3>(G, A, layer, q, out, scratch, splits, status, st);
-    case 4: return launch_t<kBf16, D, 4>(G, A, layer, q, out, scratch, splits, status, st);
-    case 5: return launch_t<kBf16, D, 5>(G, A, layer, q, out, scratch, splits, status, st);
-    case 6: return launch_t<kBf16, D, 6>(G, A, layer, q, out, scratch, splits, status, st);
-    case 7: return launch_t<kBf16, D, 7>(G, A, layer, q, out, scratch, splits, status, st);
-    case 8: return launch_t<kBf16, D, 8>(G, A, layer, q, out, scratch, splits, status, st);
-  }
+template <typename E, int D>
+cudaError_t launch_g(const Geom& G, const Arena& A, int layer, const void* q, void* out, float* part, const StepAppend& ap,
+                     int* status, cudaStream_t st) {
+  if (G.g == 1) return launch_t<E, D, 1>(G, A, layer, q, out, part, ap, status, st);
+  if (G.g == 2) return launch_t<E, D, 2>(G, A, layer, q, out, part, ap, status, st);
+  if (G.g <= 4) return launch_t<E, D, 4>(G, A, layer, q, out, part, ap, status, st);
+  if (G.g <= 8) return launch_t<E, D, 8>(G, A, layer, q, out, part, ap, status, st);
   return cudaErrorInvalidValue;
 }
 
 }  // namespace
 
-// Scratch layout: ticket counters (zero-initialised once by the owner; self-resetting),
-// then per (stream, split, head) partial rows of D+2 floats.
-size_t decode_scratch_bytes(const Geom& G, int splits) {
-  const size_t n_sl = (size_t)G.B * G.H;
-  return sizeof(float) * (((n_sl + 63) / 64) * 64 + n_sl * splits * G.g * (G.d + 8));   // rows of d + 8 floats cover both decode kernels' layouts
-}
+// Scratch of both decode kernels (see HeadEnd::combine_head): per (stream, split, head) d column sums and at most 8
+// floats of (max, sum) copies.  Every word holds the empty pattern (all ones) between launches.
+size_t decode_scratch_bytes(const Geom& G, int splits) { return sizeof(float) * (size_t)G.B * G.H * splits * G.g * (G.d + 8); }
+int decode_tile_tokens(const Geom& G) { return kTileBytes / (G.d * (G.is_bf16 ? 2 : 4)); }
 
 cudaError_t launch_decode(const Geom& G, const Arena& A, int layer, const void* q, void* out, float* scratch,
-                          int splits, int* status, cudaStream_t st) {
-  if (G.d == 128) return G.is_bf16 ? launch_g<true, 128>(G, A, layer, q, out, scratch, splits, status, st)
-                                   : launch_g<false, 128>(G, A, layer, q, out, scratch, splits, status, st);
-  if (G.d == 64) return G.is_bf16 ? launch_g<true, 64>(G, A, layer, q, out, scratch, splits, status, st)
-                                  : launch_g<false, 64>(G, A, layer, q, out, scratch, splits, status, st);
+                          const StepAppend& ap, int* status, cudaStream_t st) {
+  if (G.d == 128) return G.is_bf16 ? launch_g<__nv_bfloat16, 128>(G, A, layer, q, out, scratch, ap, status, st)
+                                   : launch_g<float, 128>(G, A, layer, q, out, scratch, ap, status, st);
+  if (G.d == 64) return G.is_bf16 ? launch_g<__nv_bfloat16, 64>(G, A, layer, q, out, scratch, ap, status, st)
+                                  : launch_g<float, 64>(G, A, layer, q, out, scratch, ap, status, st);
   return cudaErrorInvalidValue;
 }
 

@@ -29,17 +29,19 @@
 // have the stream as a dimension of their own) times an exact zero.
 #include <cuda.h>
 
-#include "common.cuh"
+#include "decode_common.cuh"
 
 namespace bkv {
 
 namespace {
 
+using namespace dec;
+
 // Shape of a CTA: kGroups warp groups that take the CTA's tiles in turn, each warp of a group owning
-// kTB blocks of 16 tokens of a 64-token tile; kCtasPerSm resident CTAs.
+// kTB blocks of 16 tokens of a 64-token tile; two CTAs per SM.
 constexpr int kGroups = 2;
 constexpr int kTB = 2;
-constexpr int kCtasPerSm = 2;
+constexpr int kCtasPerSm = kDecodeCtasPerSm;
 constexpr int kWarpTokens = 16 * kTB;
 constexpr int kGroupWarps = 64 / kWarpTokens;
 constexpr int kGroupThreads = 32 * kGroupWarps;
@@ -47,7 +49,6 @@ constexpr int kWarps = kGroups * kGroupWarps;
 constexpr int kThreads = 32 * kWarps;
 constexpr int kTN = 64;                      // tokens per tile
 constexpr uint32_t kHalf = kTN * 128;        // bytes of one [64 tokens][64 dims] bf16 box
-constexpr long long kWaitCycles = 100000000LL;   // about 50 ms: a bulk copy that has not landed by then never will
 
 // What depends on the head dimension.
 template <int D>
@@ -67,30 +68,6 @@ struct DecodeMaps {
   CUtensorMap k, v;
 };
 
-__device__ inline uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ inline void mbar_init(uint64_t* bar, int count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
-}
-__device__ inline void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-__device__ inline bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
-  return ok != 0;
-}
-__device__ inline bool mbar_wait(uint64_t* bar, uint32_t parity) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const long long t0 = clock64();
-  while (!mbar_try_wait(bar, parity)) {
-    if (clock64() - t0 > kWaitCycles) return false;
-  }
-  return true;
-}
 __device__ inline void tma_load_3d(void* dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar) {
   asm volatile(
       "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
@@ -117,46 +94,8 @@ __device__ inline uint32_t movm_trans(uint32_t a) {
   asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(d) : "r"(a));
   return d;
 }
-__device__ inline float fast_exp2(float x) {     // -inf -> 0
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-// Accesses to the split-K scratch (see the combine).  Publishing stores and polling loads are relaxed operations at
-// GPU scope -- never served by L1, and not a data race although nothing else orders them: each word validates itself.
-constexpr uint32_t kEmptyWord = 0xffffffffu;
-constexpr int kMaxSplits = 64;
-static_assert(2 * kWarps <= 8, "the scratch holds 8 floats of (max, sum) copies per partial row (decode_scratch_bytes)");
-static_assert(Dim<128>::kColWarps <= kWarps, "the combine maps a warp to 32 output columns");
-__device__ inline bool is_empty(float x) { return __float_as_uint(x) == kEmptyWord; }
-// Plain loads as volatile asm statements: they keep their place among the polling loads, i.e. they are issued
-// before the polls and not where their values are first used.
-__device__ inline uint2 ld_early_v2(const void* p) {
-  uint2 v;
-  asm volatile("ld.global.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");
-  return v;
-}
-__device__ inline uint4 ld_early_v4(const void* p) {
-  uint4 v;
-  asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
-  return v;
-}
-__device__ inline float4 ld_poll4(const float* p) {
-  float4 v;
-  asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p) : "memory");
-  return v;
-}
-__device__ inline float2 ld_poll2(const float* p) {
-  float2 v;
-  asm volatile("ld.relaxed.gpu.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p) : "memory");
-  return v;
-}
-__device__ inline void st_scratch4(float* p, float4 v) {
-  asm volatile("st.relaxed.gpu.global.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
-}
-__device__ inline void st_scratch2(float* p, float2 v) {
-  asm volatile("st.relaxed.gpu.global.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(v.x), "f"(v.y) : "memory");
-}
+static_assert(Dim<128>::kColWarps <= kWarps && 2 * Dim<128>::kColWarps <= 8,
+              "a warp per 32 output columns; the scratch holds 8 floats of (max, sum) copies per partial row");
 __device__ inline uint32_t pack_bf16(float lo, float hi) {
   const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&v);
@@ -165,65 +104,6 @@ __device__ inline uint32_t pack_bf16(float lo, float hi) {
 // 64 rows x 128 bytes, chunk index XORed with (row % 8) by the 128-byte swizzle.
 __device__ inline uint32_t tile_off(int token, int chunk16) {   // chunk16 in [0, d / 8)
   return (uint32_t)(chunk16 >> 3) * kHalf + (uint32_t)token * 128u + (uint32_t)(((chunk16 & 7) ^ (token & 7)) << 4);
-}
-
-// One appended token per stream of the layer (lockstep fill): source rows [B*H, d] and where they go.
-struct StepAppend {
-  const __nv_bfloat16* k_new;   // nullptr: plain decode
-  const __nv_bfloat16* v_new;
-  int rel_row, idx0, new_len;   // row inside the level-0 region, original position, new level-0 length
-  // Un-normalised result instead of the ratio (both nullptr: ratio in `out`): per query head
-  // sum_i w_i e^{l_i - M} v_i as fp32 [B, H g, d] and (M, sum_i w_i e^{l_i - M}) as fp32 [B, H g, 2],
-  // M the largest base-2 logit incl. log2 w_i.  Algorithm 1 divides the numerator of one
-  // MergeAndReduce instance by the denominator of another; this is one such part.
-  float* raw_acc;
-  float* raw_ml;
-  int keys_only;                // 1: only (M, sum) are wanted (a denominator instance): V is neither loaded nor multiplied
-  // Segment table of the layer's streams when they are all alike (the host mirrors it): saves the
-  // dependent global read at the start of a latency-bound launch.  n_seg = 0: read the table.
-  int n_seg;
-  Seg seg[kMaxLevels + 1];
-  // One launch over several layer slots (decode merged over slots): blockIdx.z selects the slot.
-  // n_slots = 0: a launch over the one slot `layer`.  z_stride: 4-byte words between the scratch
-  // blocks (partial rows and their pairs) of consecutive slots; raw_acc / raw_ml advance by one
-  // [B, H g, d] / [B, H g, 2] block per slot; bit z of keys_mask = keys_only of slot z.
-  int n_slots;
-  int slot_layer[8];
-  unsigned keys_mask;
-  unsigned z_stride;
-  // 1: the library's previous launch on this CUDA stream was a decode launch of this context, so
-  // the only arena rows that can still be in flight are the one row per stream that launch
-  // appended.  Every other tile may then be fetched before the grid dependency is resolved (see
-  // the kernel's prologue).  Needs the segment table as a parameter (n_seg > 0).
-  int early;
-  // The step's operands (q, k_new, v_new) arrive by a copy on another CUDA stream that no event ties to
-  // this launch: the copy is followed by a copy of the word `in_expect` to *in_flag, and the kernel
-  // waits (bounded) for that word before it reads them.  nullptr: the operands are ordered before the
-  // launch in the usual way.
-  const int* in_flag;
-  int in_expect;
-  // Splits of a stream's tiles.  With more than one the grid has g - 1 more CTAs per stream, which combine
-  // the heads 1 .. g - 1 (see the kernel's combine).
-  int splits;
-};
-
-struct TileRef {
-  int row;           // first row, counted inside the stream
-  int rows, level;
-};
-__device__ inline TileRef locate_tile(int tile, const int* lvl_tiles, const Seg* seg, int T, const int32_t* region_off) {
-  TileRef r{0, 0, 0};
-  for (int l = T; l >= 0; --l) {
-    const int nt = lvl_tiles[l];
-    if (tile < nt) {
-      r.level = l;
-      r.row = region_off[l] + seg[l].start + tile * kTN;
-      r.rows = min(kTN, seg[l].len - tile * kTN);
-      return r;
-    }
-    tile -= nt;
-  }
-  return r;
 }
 
 // Named barrier of one warp group (ids 1, 2; id 0 is __syncthreads) that also votes: true if any
@@ -273,7 +153,6 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
   const int seq = sl / G.H, head = sl % G.H;
   const int stream = (seq * G.L + layer) * G.H + head;
   const int splits = ap.splits, split = blockIdx.y;     // split >= splits: a combiner without tiles (see the combine)
-  const int64_t stream_base = (int64_t)stream * G.rows_per_stream;
   // Merge and combine phases: the first work item of this warp, (head mh, way mw) with warp = mw g + mh.
   int mh = warp, mw = 0;
   if (g < kWarps)
@@ -293,24 +172,9 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
-  // The step's operands are wanted right after the dependency resolves: ask for them in L2 now.  A
-  // line fetched before its producer has written it is harmless, L2 being the point of coherence
-  // (the producer's write updates that line; nothing is taken into L1 here).
-  if (ap.in_flag) {
-    // operands still in flight: nothing to ask for yet
-  } else if (tid < kLines * g) {                      // the stream's g query rows are contiguous
-    const char* qrow = reinterpret_cast<const char*>(q + ((size_t)seq * (G.H * g) + (size_t)head * g) * D);
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(qrow + 128 * tid));
-  } else if (ap.k_new && tid < kLines * (g + 2)) {
-    const int k = tid - kLines * g;
-    const char* row = reinterpret_cast<const char*>((k >= kLines ? ap.v_new : ap.k_new) + (size_t)sl * D);
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(row + 128 * (k % kLines)));
-  }
+  prefetch_operands<2 * D>(ap, q + (size_t)sl * g * D, sl, g);
   const bool early = ap.early && ap.n_seg;
-  if (!early) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  }
+  if (!early) grid_wait_and_release();
   if (tid <= G.T) {
     const Seg s = ap.n_seg ? ap.seg[tid] : A.seg[(size_t)stream * (G.T + 1) + tid];
     seg_s[tid] = s;
@@ -324,7 +188,7 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
   const int my_tiles = split < splits ? t_end - t_begin : 0;
 
   auto issue = [&](int i) {   // one thread
-    const TileRef tr = locate_tile(t_begin + i, lvl_tiles, seg_s, G.T, G.region_off);
+    const TileRef tr = locate_tile<kTN>(t_begin + i, lvl_tiles, seg_s, G.T, G.region_off);
     unsigned char* st = tiles + (size_t)(i % kStages) * kStageBytes;
     uint64_t* bar = &full[i % kBars];
     mbar_expect_tx(bar, keys_only ? kTensorBytes : kStageBytes);
@@ -341,203 +205,19 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
     while (issued < lim && !(early && t_begin + issued == n_tiles - 1)) issue(issued++);
   }
   if (early) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    grid_wait_and_release();
     if (tid == 0)
       while (issued < min(kStages, my_tiles)) issue(issued++);
   }
-  if (ap.in_flag) {
-    // the copy engine writes the operands, then the flag word (two copies in stream order)
-    if (tid == 0) {
-      const long long t0 = clock64();
-      while (*reinterpret_cast<const volatile int*>(ap.in_flag) != ap.in_expect) {
-        if (clock64() - t0 > kWaitCycles) { atomicCAS(status, kStatusOk, kStatusWaitTimeout); break; }
-      }
-      __threadfence();
-    }
-    __syncthreads();
-  }
+  wait_operands(ap, status);
 
   const float sc = 1.4426950408889634f * G.inv_sqrt_d;
   constexpr uint32_t kFacOff = 4352 + kWarps * kMaxGroup * 32 * 16 + 4096;   // = the single-split rows' place (never both)
 
-  // ---- the end of a head's path, by all threads of a CTA (thread = output column): the appended token
-  // joins as one more partial (level 0, weight 1, <q, k_new> in fp32), the ratio or the raw parts are
-  // written, and with h == 0 the token's row goes into the cache.
-  struct NewTok {
-    uint2 kn;                  // 4 dims of k_new per lane (lanes < d / 4)
-    uint2 qv[kMaxGroup];       // 4 dims of q per lane and head (one head: slot 0)
-    uint2 vn;                  // lanes 0-7: the columns 32 warp + 4 lane .. + 3 of v_new
-    uint4 row_new;             // last column warp: the first d / 8 lanes a piece of the row of K, the next d / 8 of V
-  };
-  const bool col_warp = warp < kColWarps;          // owns the output columns 32 warp .. 32 warp + 31
-  const bool has_dims = 4 * lane < D;
-  // h < 0: the queries of all heads
-  auto load_new = [&](int h) -> NewTok {
-    NewTok nt;
-    nt.kn = make_uint2(0u, 0u);
-    nt.vn = make_uint2(0u, 0u);
-    nt.row_new = make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-    for (int k = 0; k < kMaxGroup; ++k) nt.qv[k] = make_uint2(0u, 0u);
-    if (ap.k_new) {
-      if (has_dims) nt.kn = ld_early_v2(ap.k_new + (size_t)sl * D + 4 * lane);
-      if (col_warp && lane < 8) nt.vn = ld_early_v2(ap.v_new + (size_t)sl * D + 32 * warp + 4 * lane);
-      const __nv_bfloat16* qs = q + ((size_t)seq * (G.H * g) + (size_t)head * g) * D + 4 * lane;
-      if (!has_dims) {
-      } else if (h >= 0) {
-        nt.qv[0] = ld_early_v2(qs + (size_t)h * D);
-      } else {
-#pragma unroll
-        for (int k = 0; k < kMaxGroup; ++k)
-          if (k < g) nt.qv[k] = ld_early_v2(qs + (size_t)k * D);
-      }
-      if (h <= 0 && warp == kColWarps - 1 && lane < 2 * kRowPieces)
-        nt.row_new = ld_early_v4(reinterpret_cast<const uint4*>((lane < kRowPieces ? ap.k_new : ap.v_new) + (size_t)sl * D) + lane % kRowPieces);
-    }
-    return nt;
-  };
-  // base-2 logit of the appended token for the head whose query sits in slot qslot (by a whole warp)
-  auto score_new = [&](const NewTok& nt, int qslot) -> float {
-    const uint2 qv = nt.qv[qslot];
-    const __nv_bfloat162 k01 = *reinterpret_cast<const __nv_bfloat162*>(&nt.kn.x), k23 = *reinterpret_cast<const __nv_bfloat162*>(&nt.kn.y);
-    const __nv_bfloat162 q01 = *reinterpret_cast<const __nv_bfloat162*>(&qv.x), q23 = *reinterpret_cast<const __nv_bfloat162*>(&qv.y);
-    float dot = __bfloat162float(q01.x) * __bfloat162float(k01.x);
-    dot = fmaf(__bfloat162float(q01.y), __bfloat162float(k01.y), dot);
-    dot = fmaf(__bfloat162float(q23.x), __bfloat162float(k23.x), dot);
-    dot = fmaf(__bfloat162float(q23.y), __bfloat162float(k23.y), dot);
-    return warp_sum(dot) * sc;
-  };
-  // a: lanes 0-7 of every warp hold the sums of the output columns 32 warp + 4 lane .. + 3
-  auto finish = [&](int h, float4 a, float M, float L, const NewTok& nt, float x) {
-    if (ap.k_new) {
-      const float Mn = fmaxf(M, x);
-      const float f = M == -INFINITY ? 0.f : fast_exp2(M - Mn), fN = fast_exp2(x - Mn);
-      const __nv_bfloat162 v01 = *reinterpret_cast<const __nv_bfloat162*>(&nt.vn.x), v23 = *reinterpret_cast<const __nv_bfloat162*>(&nt.vn.y);
-      a.x = fmaf(__bfloat162float(v01.x), fN, a.x * f); a.y = fmaf(__bfloat162float(v01.y), fN, a.y * f);
-      a.z = fmaf(__bfloat162float(v23.x), fN, a.z * f); a.w = fmaf(__bfloat162float(v23.y), fN, a.w * f);
-      L = fmaf(L, f, fN);
-      M = Mn;
-    }
-    const size_t qh = (size_t)seq * (G.H * g) + (size_t)head * g + h;
-    if (col_warp && lane < 8) {
-      const int c = 32 * warp + 4 * lane;
-      if (raw_acc) {
-        *reinterpret_cast<float4*>(raw_acc + qh * D + c) = a;
-        if (c == 0) { raw_ml[2 * qh] = M; raw_ml[2 * qh + 1] = L; }
-      } else {
-        const float inv = L > 0.f ? 1.0f / L : 0.f;
-        __nv_bfloat162 o01 = __floats2bfloat162_rn(a.x * inv, a.y * inv), o23 = __floats2bfloat162_rn(a.z * inv, a.w * inv);
-        uint2 w;
-        w.x = *reinterpret_cast<uint32_t*>(&o01);
-        w.y = *reinterpret_cast<uint32_t*>(&o23);
-        *reinterpret_cast<uint2*>(out + qh * D + c) = w;
-      }
-    }
-    if (ap.k_new && h == 0 && warp == kColWarps - 1) {
-      // append: one row of K and of V, the position, the new length of C^0
-      const size_t dst_row = (size_t)stream_base + G.region_off[0] + ap.rel_row;
-      __nv_bfloat16* dstp = static_cast<__nv_bfloat16*>(lane < kRowPieces ? A.K : A.V) + dst_row * D;
-      if (lane < 2 * kRowPieces) reinterpret_cast<uint4*>(dstp)[lane % kRowPieces] = nt.row_new;
-      float s2 = 0.f;                                         // ||k||^2 / ||v||^2 travel with the row
-      const __nv_bfloat162* h2 = reinterpret_cast<const __nv_bfloat162*>(&nt.row_new);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float2 fv = __bfloat1622float2(h2[i]);
-        s2 = fmaf(fv.x, fv.x, s2);
-        s2 = fmaf(fv.y, fv.y, s2);
-      }
-#pragma unroll
-      for (int o = kRowPieces / 2; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-      const float v2 = __shfl_sync(0xffffffffu, s2, kRowPieces);
-      if (lane == 0 && A.nrm) A.nrm[dst_row] = make_float2(s2, v2);
-      if (lane == 1) {
-        A.idx[dst_row] = ap.idx0;
-        A.seg[(size_t)stream * (G.T + 1)].len = ap.new_len;
-      }
-    }
-  };
-  // Combine head h of this CTA's stream (see the combine below).  Warp w sums the columns 32 w .. 32 w + 31,
-  // a 128-byte line of every partial row: lane = (row group rg = lane / 8, 16-byte piece lane % 8), the lane
-  // takes the rows rg, rg + 4, ... (vector loads and stores: a quarter of the memory instructions that a
-  // lane per column would need), and the four row groups meet by two shuffle steps.
-  auto combine_head = [&](int h) {
-    if (!col_warp) return;
-    const int rg = lane >> 3;
-    const float* rows = part + ((size_t)sl * splits * g + h) * D + 32 * warp + 4 * (lane & 7);        // row of split sp: + sp rstep
-    const float* mls = part + (size_t)gridDim.x * splits * g * D + (((size_t)sl * g + h) * kColWarps + warp) * splits * 2;   // this warp's copies of the head's pairs, split by split: one line or two for a polling warp
-    const size_t rstep = (size_t)g * D, mstep = 2;
-    const NewTok nt = load_new(h);              // in flight during the polls
-    const float* mlp[2] = {mls + (size_t)lane * mstep, mls + (size_t)(lane + 32) * mstep};
-    float2 ml[2];
-#pragma unroll
-    for (int e = 0; e < 2; ++e) ml[e] = lane + 32 * e < splits ? ld_poll2(mlp[e]) : make_float2(-INFINITY, 0.f);
-    constexpr int kPer = kMaxSplits / 4;
-    float4 v[kPer];
-#pragma unroll
-    for (int i = 0; i < kPer; ++i)
-      if (rg + 4 * i < splits) v[i] = ld_poll4(rows + (size_t)(rg + 4 * i) * rstep);
-    const float x_new = ap.k_new ? score_new(nt, 0) : 0.f;      // while the polls are in flight
-    // A round re-reads everything that was still empty, all loads in flight together (words checked one
-    // after the other would cost a round trip each).
-    const long long t0 = clock64();
-    bool ok = true;
-    for (;;) {
-      bool pending = false;
-#pragma unroll
-      for (int e = 0; e < 2; ++e)
-        if (lane + 32 * e < splits && (is_empty(ml[e].x) || is_empty(ml[e].y))) {
-          ml[e] = ld_poll2(mlp[e]);
-          pending = true;
-        }
-#pragma unroll
-      for (int i = 0; i < kPer; ++i)
-        if (rg + 4 * i < splits && (is_empty(v[i].x) || is_empty(v[i].y) || is_empty(v[i].z) || is_empty(v[i].w))) {
-          v[i] = ld_poll4(rows + (size_t)(rg + 4 * i) * rstep);
-          pending = true;
-        }
-      if (!pending) break;
-      if (clock64() - t0 > kWaitCycles) { ok = false; break; }
-    }
-    __syncwarp();
-    const float M = warp_max(fmaxf(ml[0].x, ml[1].x));
-    const float f0 = ml[0].x == -INFINITY ? 0.f : fast_exp2(ml[0].x - M);
-    const float f1 = ml[1].x == -INFINITY ? 0.f : fast_exp2(ml[1].x - M);
-    const float L = warp_sum(fmaf(ml[0].y, f0, ml[1].y * f1));
-    // the factors of all splits through shared memory (behind the merge buffers, which other warps of the
-    // last split's CTA may still be reading)
-    float* fac = reinterpret_cast<float*>(tiles + kFacOff) + warp * kMaxSplits;
-    fac[lane] = f0;
-    fac[lane + 32] = f1;
-    __syncwarp();
-    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-    for (int i = 0; i < kPer; ++i)
-      if (rg + 4 * i < splits) {
-        const float f = fac[rg + 4 * i];
-        a.x = fmaf(v[i].x, f, a.x); a.y = fmaf(v[i].y, f, a.y); a.z = fmaf(v[i].z, f, a.z); a.w = fmaf(v[i].w, f, a.w);
-      }
-#pragma unroll
-    for (int o = 8; o < 32; o <<= 1) {
-      a.x += __shfl_xor_sync(0xffffffffu, a.x, o); a.y += __shfl_xor_sync(0xffffffffu, a.y, o);
-      a.z += __shfl_xor_sync(0xffffffffu, a.z, o); a.w += __shfl_xor_sync(0xffffffffu, a.w, o);
-    }
-    finish(h, a, M, L, nt, x_new);
-    // the empty pattern again, for the next launch (every warp has its own copy of the pairs, so nobody else
-    // still wants these words)
-    {
-      const float e = __uint_as_float(kEmptyWord);
-#pragma unroll
-      for (int i = 0; i < kPer; ++i)
-        if (rg + 4 * i < splits) st_scratch4(const_cast<float*>(rows + (size_t)(rg + 4 * i) * rstep), make_float4(e, e, e, e));
-#pragma unroll
-      for (int k = 0; k < 2; ++k)
-        if (lane + 32 * k < splits) st_scratch2(const_cast<float*>(mlp[k]), make_float2(e, e));
-    }
-    if (!ok && lane == 0) atomicCAS(status, kStatusOk, kStatusWaitTimeout);
-  };
+  const HeadEnd<__nv_bfloat16, D> end{G, A, ap, q + (size_t)sl * g * D, out + (size_t)sl * g * D, raw_acc, raw_ml, sl, stream, g, warp, lane, sc};
+  float* const fac = reinterpret_cast<float*>(tiles + kFacOff) + warp * kDecodeMaxSplits;   // behind the merge buffers, which other warps may still be reading
   if (split >= splits) {                        // a CTA without tiles: the combiner of head split - splits + 1
-    combine_head(split - splits + 1);
+    end.combine_head(split - splits + 1, part, gridDim.x, fac, status);
     return;
   }
 
@@ -593,7 +273,7 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
     if (lane == 0) arrived = mbar_wait(&full[i % kBars], (uint32_t)((i / kBars) & 1));
     arrived = __shfl_sync(0xffffffffu, arrived, 0);
     __syncwarp();                  // the polling lane's view of the landed tile, for the whole warp
-    const TileRef tr = locate_tile(t_begin + i, lvl_tiles, seg_s, G.T, G.region_off);
+    const TileRef tr = locate_tile<kTN>(t_begin + i, lvl_tiles, seg_s, G.T, G.region_off);
     const uint32_t Kt = smem_u32(tiles + (size_t)s * kStageBytes), Vt = Kt + kTensorBytes;
     if (arrived && wq * kWarpTokens < tr.rows) {
       // ---- scores of the warp's tokens against the group's heads: S^T[16 x 8] = K Q^T per block.
@@ -758,13 +438,13 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
         if (w < kWarps && mv[k] != -INFINITY) {
           const float* rowp = mrg + ((size_t)w * g + mh) * PS;
           const float f = fast_exp2(mv[k] - M);
-          const float4 v = has_dims ? *reinterpret_cast<const float4*>(rowp + 4 * lane) : make_float4(0.f, 0.f, 0.f, 0.f);
+          const float4 v = end.has_dims() ? *reinterpret_cast<const float4*>(rowp + 4 * lane) : make_float4(0.f, 0.f, 0.f, 0.f);
           acc.x = fmaf(v.x, f, acc.x); acc.y = fmaf(v.y, f, acc.y); acc.z = fmaf(v.z, f, acc.z); acc.w = fmaf(v.w, f, acc.w);
           L = fmaf(rowp[D + 1], f, L);
         }
       }
       float* dst = mrg2 + ((size_t)mw * g + mh) * PS;
-      if (has_dims) *reinterpret_cast<float4*>(dst + 4 * lane) = acc;
+      if (end.has_dims()) *reinterpret_cast<float4*>(dst + 4 * lane) = acc;
       if (lane == 0) { dst[D] = M; dst[D + 1] = L; }
     }
     __syncthreads();
@@ -781,41 +461,32 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
         const float* rowp = mrg + ((size_t)k * g + h) * PS;
         const float mk = rowp[D];
         const float f = mk == -INFINITY ? 0.f : fast_exp2(mk - M);
-        const float4 v = has_dims ? *reinterpret_cast<const float4*>(rowp + 4 * lane) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 v = end.has_dims() ? *reinterpret_cast<const float4*>(rowp + 4 * lane) : make_float4(0.f, 0.f, 0.f, 0.f);
         acc.x = fmaf(v.x, f, acc.x); acc.y = fmaf(v.y, f, acc.y); acc.z = fmaf(v.z, f, acc.z); acc.w = fmaf(v.w, f, acc.w);
         L = fmaf(rowp[D + 1], f, L);
       }
       if (single) {
-        if (has_dims) *reinterpret_cast<float4*>(my_acc + h * D + 4 * lane) = acc;
+        if (end.has_dims()) *reinterpret_cast<float4*>(my_acc + h * D + 4 * lane) = acc;
         if (lane == 0) *reinterpret_cast<float2*>(my_ml + 2 * h) = make_float2(M, L);
       } else {                                  // published: see the combine below
-        if (has_dims) st_scratch4(my_acc + h * D + 4 * lane, acc);
+        if (end.has_dims()) st_scratch4(my_acc + h * D + 4 * lane, acc);
         if (lane < kColWarps) st_scratch2(my_ml + ((size_t)(h * kColWarps + lane) * splits + split) * 2, make_float2(M, L));   // a copy per combining warp
       }
     }
   }
-  // ---- combine.  No ticket, no fence and no staging copy: a word of the scratch is its own arrival flag.
-  // Between launches every word of the partial rows holds kEmptyWord, a NaN pattern that arithmetic never
-  // produces (results are canonical NaNs, and -inf is a legal maximum).  A CTA publishes its rows with relaxed
-  // stores.  Head 0 of a stream is combined by the stream's CTA of the last split, head h > 0 by the CTA
-  // (stream, splits + h - 1), which has no tiles: the g combiners of a stream run side by side on different
-  // SMs, each polls the words of its head until none is empty, sums, and puts the empty pattern back for the
-  // next launch.  CTAs are dispatched in index order, so everything a combiner waits for was dispatched
-  // before it and never waits itself: the wait ends (and is bounded anyway).  The chain behind the last tile
-  // is then one store and about one load through L2 instead of fence, ticket, fence and copy.
   if (single) {
     __syncthreads();                            // the rows in shared memory are complete
     const float* acc1 = reinterpret_cast<const float*>(tiles + kSingleOff);
     const float* ml1 = acc1 + kMaxGroup * D;
-    NewTok nt = load_new(-1);
+    const auto nt = end.load_new(-1);
 #pragma unroll
     for (int h = 0; h < kMaxGroup; ++h)
       if (h < g)
-        finish(h, *reinterpret_cast<const float4*>(acc1 + h * D + (32 * warp) % D + 4 * (lane & 7)), ml1[2 * h], ml1[2 * h + 1], nt,
-               ap.k_new ? score_new(nt, h) : 0.f);
+        end.finish(h, *reinterpret_cast<const float4*>(acc1 + h * D + (32 * warp) % D + 4 * (lane & 7)), ml1[2 * h], ml1[2 * h + 1], nt,
+               ap.k_new ? end.score_new(nt, h) : 0.f);
     return;
   }
-  if (split == splits - 1) combine_head(0);
+  if (split == splits - 1) end.combine_head(0, part, gridDim.x, fac, status);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -858,35 +529,17 @@ cudaError_t set_smem(int d) {
                   : cudaFuncSetAttribute(decode_mma_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Dim<64>::kSmemBytes);
 }
 
-// CTAs per stream of a launch with `splits` splits: the combiners of the heads 1 .. g - 1 have CTAs of their own.
-unsigned grid_y(const Geom& G, int splits) { return (unsigned)(splits > 1 ? splits + G.g - 1 : 1); }
-
-// Scratch layout of all launches: the CUDA-core kernel's ticket counters (unused here), then (stream, split,
-// head) rows of d column sums, then per row d / 32 copies of its (max, sum) pair.
-float* partial_rows(const Geom& G, float* scratch) { return scratch + (((size_t)G.B * G.H + 63) / 64) * 64; }
-
-// Launches with programmatic stream serialization: back-to-back decode launches overlap a launch with the previous
-// kernel's tail (see the kernel's prologue).
 cudaError_t launch(const Geom& G, const Arena& A, int layer, const void* q, void* out, float* part, int* status,
                    const StepAppend& ap, const DecodeMaps& tm, int n_slots, cudaStream_t st) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(G.B * G.H, grid_y(G, ap.splits), n_slots);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = G.d == 128 ? Dim<128>::kSmemBytes : Dim<64>::kSmemBytes;
-  cfg.stream = st;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, G.d == 128 ? decode_mma_kernel<128> : decode_mma_kernel<64>, G, A, layer,
+  const PdlConfig pc(dim3(G.B * G.H, decode_grid_y(G, ap.splits), n_slots), kThreads,
+                     G.d == 128 ? Dim<128>::kSmemBytes : Dim<64>::kSmemBytes, st);
+  return cudaLaunchKernelEx(&pc.cfg, G.d == 128 ? decode_mma_kernel<128> : decode_mma_kernel<64>, G, A, layer,
                             static_cast<const __nv_bfloat16*>(q), static_cast<__nv_bfloat16*>(out), part, status, ap, tm.k, tm.v);
 }
 
 }  // namespace
 
 bool decode_mma_supported(const Geom& G) { return G.is_bf16 && (G.d == 128 || G.d == 64) && G.g <= 8; }
-int decode_mma_ctas_per_sm() { return kCtasPerSm; }
 int decode_mma_tile_tokens() { return kTN; }
 
 cudaError_t decode_mma_prepare(const Geom& G, const Arena& A, void** maps_out) {
@@ -912,29 +565,21 @@ cudaError_t launch_decode_parts_mma_slots(const Geom& G, const Arena& A, const i
   if (!maps || !raw_acc || !raw_ml || n_slots < 1 || n_slots > 8 || z_stride_words > 0xffffffffull) return cudaErrorInvalidValue;
   StepAppend ap{nullptr, nullptr, 0, 0, 0, raw_acc, raw_ml, 0, 0, {}, n_slots, {}, keys_mask, (unsigned)z_stride_words, 0, nullptr, 0, splits};
   for (int i = 0; i < n_slots; ++i) ap.slot_layer[i] = slot_layers[i];
-  return launch(G, A, slot_layers[0], q, nullptr, partial_rows(G, scratch), status, ap, *static_cast<const DecodeMaps*>(maps),
+  return launch(G, A, slot_layers[0], q, nullptr, scratch, status, ap, *static_cast<const DecodeMaps*>(maps),
                 n_slots, st);
 }
 
-// balancekv_decode_attn_static: caches owned by the caller, [B streams][rows_per_stream][d] with the segments `seg`
-// (level l of every stream: rows seg[l] behind region_off[l]).  The tensor maps are encoded on the host for each call
-// (plain arithmetic, no allocation) and travel as kernel parameters.  rows: scratch of decode_mma_static_bytes().
-size_t decode_mma_static_bytes(const Geom& G, int splits) {
-  return splits > 1 ? sizeof(float) * (size_t)G.B * G.H * splits * G.g * (G.d + 8) : 0;
-}
+// balancekv_decode_attn_static: caches owned by the caller, [B streams][rows_per_stream][d] with the segments ap.seg.
+// The tensor maps are encoded on the host for each call (plain arithmetic, no allocation) and travel as kernel parameters.
 cudaError_t decode_mma_static_setup() {
   const cudaError_t e = set_smem(128);
   return e != cudaSuccess ? e : set_smem(64);
 }
-cudaError_t launch_decode_static_mma(const Geom& G, void* K, void* V, const Seg* seg, const void* q, void* out, float* rows,
-                                     int splits, int* status, cudaStream_t st) {
+cudaError_t launch_decode_static_mma(const Geom& G, const Arena& A, const StepAppend& ap, const void* q, void* out, float* rows,
+                                     int* status, cudaStream_t st) {
   DecodeMaps tm;
-  const cudaError_t e = encode_maps(&tm, K, V, G.d, G.rows_per_stream > 0 ? G.rows_per_stream : 1, G.B * G.H);
-  if (e != cudaSuccess) return e;
-  StepAppend ap{nullptr, nullptr, 0, 0, 0, nullptr, nullptr, 0, G.T + 1, {}, 0, {}, 0u, 0u, 0, nullptr, 0, splits};
-  for (int l = 0; l <= G.T; ++l) ap.seg[l] = seg[l];
-  const Arena A{K, V, nullptr, nullptr, nullptr};
-  return launch(G, A, 0, q, out, rows, status, ap, tm, 1, st);
+  const cudaError_t e = encode_maps(&tm, A.K, A.V, G.d, G.rows_per_stream > 0 ? G.rows_per_stream : 1, G.B * G.H);
+  return e != cudaSuccess ? e : launch(G, A, 0, q, out, rows, status, ap, tm, 1, st);
 }
 
 // Ratio of merged parts: the value sums of the numerator slots over the weight sums of the
@@ -974,20 +619,9 @@ cudaError_t launch_merged_ratio(const float* acc, const float* ml, int n_parts, 
 // Decode attention fused with the append of one token per stream of the layer (k_new, v_new:
 // [B*H, d] bf16; all streams of the layer have the same level-0 fill).  k_new == nullptr: plain decode.
 cudaError_t launch_decode_step_mma(const Geom& G, const Arena& A, int layer, const void* q, void* out, float* scratch,
-                                   int splits, int* status, const void* maps, const void* k_new, const void* v_new,
-                                   int rel_row, int idx0, int new_len, const Seg* seg_hint, int early, const int* in_flag,
-                                   int in_expect, cudaStream_t st) {
+                                   const StepAppend& ap, int* status, const void* maps, cudaStream_t st) {
   if (!maps) return cudaErrorInvalidValue;
-  StepAppend ap{static_cast<const __nv_bfloat16*>(k_new), static_cast<const __nv_bfloat16*>(v_new), rel_row, idx0,
-                new_len, nullptr, nullptr, 0, 0, {}, 0, {}, 0u, 0u, 0, nullptr, 0, splits};
-  if (seg_hint) {
-    ap.n_seg = G.T + 1;
-    for (int l = 0; l <= G.T; ++l) ap.seg[l] = seg_hint[l];
-    ap.early = early ? 1 : 0;
-  }
-  ap.in_flag = in_flag;
-  ap.in_expect = in_expect;
-  return launch(G, A, layer, q, out, partial_rows(G, scratch), status, ap, *static_cast<const DecodeMaps*>(maps), 1, st);
+  return launch(G, A, layer, q, out, scratch, status, ap, *static_cast<const DecodeMaps*>(maps), 1, st);
 }
 
 }  // namespace bkv

@@ -73,3 +73,38 @@ def test_static_decode_on_tensor_cores(cuda_lib, S, g, d, T, n_heavy, n_tail):
         for s in range(0, S, max(1, S // 5)):
             _check(out[s], oracle.weighted_attention(K[s], V[s], w, q[s]), "bf16", (call, s))
     assert cuda_lib.decode_attn_static_status() == 0
+
+
+@pytest.mark.parametrize("dtype,d,g,splits,n_heavy,n_tail",
+                         [("fp32", 128, 1, 1, 33, 0), ("fp32", 128, 3, 0, 1000, 31), ("fp32", 128, 8, 5, 900, 33), ("fp32", 64, 2, 64, 70, 1),
+                          ("fp32", 64, 5, 0, 2100, 64), ("bf16", 128, 4, 3, 600, 65), ("bf16", 64, 7, 0, 1300, 1)])
+def test_cuda_core_decode(cuda_lib, dtype, d, g, splits, n_heavy, n_tail):
+    """The CUDA-core kernel: every rounded group size, batches that end inside a tile, one split to more splits than
+    tiles, the fused append, and the same rows through the allocation-free entry (fp32)."""
+    B, H, T = 1, 3, 2
+    ctx = cuda_lib.Context(n_seqs=B, n_layers=1, n_kv_heads=H, n_q_heads=H * g, head_dim=d, dtype=dtype, block=64, levels=T,
+                           max_tokens=(n_heavy << T) + n_tail + 8, decode_splits=splits, gram_path=1)
+    n = n_heavy + n_tail
+    K, V = synth.layer_kv("llama", 37, 0, B, H, n + 2, d, dtype)
+    ctx.cache_load_level(0, T, to_device(K[:, :, :n_heavy], dtype), to_device(V[:, :, :n_heavy], dtype))
+    if n_tail:
+        ctx.stream_append_layer(0, to_device(K[:, :, n_heavy:n], dtype), to_device(V[:, :, n_heavy:n], dtype))
+    w = np.concatenate([np.full(n_heavy, 4.0), np.ones(n_tail + 2)])
+    for step in range(3):
+        q = synth.queries(37, 0, step, B, H * g, d, dtype)
+        qt = to_device(q, dtype)
+        if step == 0:
+            out, m = ctx.decode_attn(0, qt), n
+        else:
+            m = n + step
+            out = ctx.stream_step(0, qt, to_device(K[:, :, m - 1], dtype), to_device(V[:, :, m - 1], dtype), qt.clone())
+        assert ctx.debug_scratch_used() == 0
+        _check_heads(out.float().cpu().numpy(), K[:, :, :m], V[:, :, :m], w[:m], q, g, dtype, (g, splits, step))
+    st = ctx.stats()
+    assert st["device_status"] == 0 and st["decode_kernel"] == 1
+    if dtype == "fp32":
+        out = cuda_lib.decode_attn_static(to_device(K[0, :, :n], dtype), to_device(V[0, :, :n], dtype), n_heavy, T,
+                                          to_device(q[0].reshape(H, g, d), dtype)).cpu().numpy()
+        _check_heads(out.reshape(1, H * g, d), K[:, :, :n], V[:, :, :n], w[:n], q, g, dtype, "static")
+        assert cuda_lib.decode_attn_static_status() == 0
+    ctx.close()

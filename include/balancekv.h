@@ -164,7 +164,7 @@ int balancekv_decode_attn_host(balancekv_ctx* ctx, int layer, const void* q_host
  * sum_i w_i e^{<k_i,q>/sqrt d} v_i / sum_i w_i e^{<k_i,q>/sqrt d}, the same arithmetic as
  * balancekv_decode_attn.
  *
- * The split-K scratch is a fixed array inside the library image (5.5 MiB in four blocks; held by every GPU
+ * The split-K scratch is a fixed array inside the library image (11 MiB in four blocks; held by every GPU
  * that loads the library, until the process exits); the call
  * performs no cudaMalloc, cudaFree or other allocating call.  A problem is rejected with BALANCEKV_E_NOMEM and
  * a message on stderr if 256 bytes, a segment table of n_streams * (level+1) * 8 bytes, n_streams words rounded

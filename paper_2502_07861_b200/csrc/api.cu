@@ -24,11 +24,12 @@ cudaError_t walk_tc_prepare(const Geom& G, const Arena& A, int64_t total_rows, v
 void walk_tc_release(void* tmaps);
 bool decode_mma_supported(const Geom& G);
 int decode_mma_tile_tokens();
+int decode_mma_warps();
 cudaError_t decode_mma_prepare(const Geom& G, const Arena& A, void** maps_out);
 void decode_mma_release(void* maps);
 cudaError_t launch_decode_parts_mma_slots(const Geom& G, const Arena& A, const int* slot_layers, int n_slots,
                                           unsigned keys_mask, const void* q, float* raw_acc, float* raw_ml, float* scratch,
-                                          size_t z_stride_words, int splits, int* status, const void* maps,
+                                          size_t z_stride_words, SplitPlan plan, int* status, const void* maps,
                                           cudaStream_t st);
 cudaError_t launch_merged_ratio(const float* acc, const float* ml, int n_parts, unsigned num_mask, unsigned den_mask,
                                 void* out, int n_heads, int d, cudaStream_t st);
@@ -363,7 +364,7 @@ int balancekv_create(const balancekv_config* cfg, balancekv_ctx** out) {
   {
     const int n_sl = f.n_seqs * f.n_kv_heads;
     c->decode_slots = kDecodeCtasPerSm * c->sm_count;                                 // CTAs of one wave
-    c->max_splits = std::max(1, std::min(64, c->decode_slots / n_sl));      // rounding down keeps one wave
+    c->max_splits = max_decode_splits(c->decode_slots, n_sl);
     if (f.decode_splits > 0) c->max_splits = std::min(64, f.decode_splits);
     const size_t sb = decode_scratch_bytes(G, c->max_splits);
     if ((rc = dev_alloc(c, reinterpret_cast<char**>(&c->d_decode_scratch), sb))) return fail(rc);
@@ -711,30 +712,32 @@ static bool layer_seg_hint(balancekv_ctx* c, int layer, Seg* out) {
   return true;
 }
 
-// A decode launch with more than one split has g - 1 combining CTAs per stream besides its tile CTAs:
-// the largest split factor <= splits whose grid over n_streams streams still fits one wave.
-static int one_wave_splits(balancekv_ctx* c, int splits, int n_streams) {
-  const int per_stream = c->decode_slots / std::max(1, n_streams);
-  const int room = per_stream - (c->cfg.n_q_heads / c->cfg.n_kv_heads - 1);
-  return std::max(1, std::min(splits, room));
+// Tiles of the layer's longest stream for the decode kernels; hint: the segments of all its streams, if they are alike.
+static int64_t decode_tiles(balancekv_ctx* c, int layer, const Seg* hint) {
+  const int tn = c->decode_maps ? decode_mma_tile_tokens() : decode_tile_tokens(c->G);
+  const int T = c->cfg.levels;
+  int64_t most = 0;
+  if (hint) {
+    for (int l = 0; l <= T; ++l) most += (hint[l].len + tn - 1) / tn;
+    return most;
+  }
+  for (int s : layer_streams(c, layer)) {
+    const StreamState& S = c->st[s];
+    int64_t tiles = (S.len0 + tn - 1) / tn;
+    for (int l = 1; l <= T; ++l) tiles += (S.lvl_len[l] + tn - 1) / tn;
+    most = std::max(most, tiles);
+  }
+  return most;
 }
 
-// Split-K factor of a decode launch over the layer's current caches.
-static int pick_splits(balancekv_ctx* c, int layer) {
-  const balancekv_config& f = c->cfg;
-  int64_t max_rows = 0;
-  for (int s = 0; s < f.n_seqs; ++s)
-    for (int h = 0; h < f.n_kv_heads; ++h) {
-      const StreamState& S = c->st[stream_id(c, s, layer, h)];
-      int64_t rows = S.len0;
-      for (int l = 1; l <= f.levels; ++l) rows += S.lvl_len[l];
-      max_rows = std::max(max_rows, rows);
-    }
-  const int tile_tokens = c->decode_maps ? decode_mma_tile_tokens() : decode_tile_tokens(c->G);
-  const int64_t tiles = (max_rows + tile_tokens - 1) / tile_tokens + f.levels;
-  int splits = pick_decode_splits(tiles, c->max_splits, c->decode_slots, f.n_seqs * f.n_kv_heads, c->G.g);
-  if (f.decode_splits > 0) splits = std::min(f.decode_splits, c->max_splits);
-  return splits;
+// Split-K factor of a decode launch over n streams (see pick_decode_splits).
+static SplitPlan pick_splits(const balancekv_ctx* c, int64_t tiles, int n) {
+  const int warps = c->decode_maps ? decode_mma_warps() : decode_warps();
+  if (c->cfg.decode_splits > 0) {
+    const int s = std::min(c->cfg.decode_splits, c->max_splits);
+    return SplitPlan{s, s <= inline_limit(c->G.g, warps, tiles)};
+  }
+  return pick_decode_splits(tiles, c->max_splits, c->decode_slots, n, c->G.g, warps);
 }
 
 // One decode launch over the layer's current caches; with k_new / v_new given it also appends one token per stream
@@ -745,11 +748,14 @@ static int launch_decode_step(balancekv_ctx* c, int layer, const void* q, void* 
   StepAppend ap{};
   ap.k_new = k_new; ap.v_new = v_new;
   ap.rel_row = rel; ap.idx0 = idx0; ap.new_len = new_len;
-  ap.splits = pick_splits(c, layer);
-  if (layer_seg_hint(c, layer, ap.seg)) {
+  const bool alike = layer_seg_hint(c, layer, ap.seg);
+  if (alike) {
     ap.n_seg = c->cfg.levels + 1;
     ap.early = c->decode_chain && c->chain_stream == st;
   }
+  const SplitPlan plan = pick_splits(c, decode_tiles(c, layer, alike ? ap.seg : nullptr), c->cfg.n_seqs * c->cfg.n_kv_heads);
+  ap.splits = plan.splits;
+  ap.inline_combine = plan.inline_combine;
   ap.in_flag = c->step_flag;
   ap.in_expect = c->step_expect;
   c->step_flag = nullptr;
@@ -852,20 +858,20 @@ int balancekv_decode_attn_merged(balancekv_ctx* c, const int32_t* layers_num, in
     c->two_scratch_words = block_bytes / 4;
     c->bytes_resident += block_bytes * BALANCEKV_MAX_MERGE;
   }
-  // One launch over all slots (grid z = slot).  The split factor is the largest any slot asks for,
-  // bounded so that the whole grid stays within one wave where it can.
-  int splits = 1;
+  // One launch over all slots (grid z = slot), split for the longest of them.
+  int64_t tiles = 1;
   unsigned keys_mask = 0;
   for (int p = 0; p < n_parts; ++p) {
-    splits = std::max(splits, pick_splits(c, slots[p]));
+    Seg hint[kMaxLevels + 1];
+    const bool alike = layer_seg_hint(c, slots[p], hint);
+    tiles = std::max(tiles, decode_tiles(c, slots[p], alike ? hint : nullptr));
     if (!((num_mask >> p) & 1u)) keys_mask |= 1u << p;     // a slot that only enters the denominator: values are not read
   }
-  const int n_sl = c->cfg.n_seqs * c->cfg.n_kv_heads;
-  splits = one_wave_splits(c, splits, n_sl * n_parts);
+  const SplitPlan plan = pick_splits(c, tiles, c->cfg.n_seqs * c->cfg.n_kv_heads * n_parts);
   {
     ProfScope ps(c, 4, st);
     BKV_CUDA(launch_decode_parts_mma_slots(c->G, c->A, slots, n_parts, keys_mask, q, c->two_acc, c->two_ml, c->two_scratch,
-                                           c->two_scratch_words, splits, c->d_status, c->decode_maps, st));
+                                           c->two_scratch_words, plan, c->d_status, c->decode_maps, st));
   }
   BKV_CUDA(launch_merged_ratio(c->two_acc, c->two_ml, n_parts, num_mask, den_mask, out, n_heads, d, st));
   c->kernels_launched += 2;

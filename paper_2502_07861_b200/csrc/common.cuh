@@ -181,21 +181,9 @@ cudaError_t launch_compact(const Geom& G, const Arena& A, const CallDesc* calls,
 struct StepAppend;      // decode_common.cuh
 size_t decode_scratch_bytes(const Geom& G, int splits);
 int decode_tile_tokens(const Geom& G);
+int decode_warps();
 cudaError_t launch_decode(const Geom& G, const Arena& A, int layer, const void* q, void* out, float* scratch,
                           const StepAppend& ap, int* status, cudaStream_t st);
-// Split-K factor of a decode launch whose longest stream has `tiles` tiles: at least two tiles per CTA, the fewest
-// splits with that number of tiles per CTA (the tile phase is as long, the combine shorter), and a grid of one wave
-// of `slots` resident CTAs (the heads 1 .. g - 1 of a stream are combined by CTAs of their own).
-inline int pick_decode_splits(int64_t tiles, int max_splits, int slots, int n_streams, int g) {
-  int64_t splits = (tiles + 1) / 2 < max_splits ? (tiles + 1) / 2 : max_splits;
-  if (splits < 1) splits = 1;
-  int64_t per = (tiles + splits - 1) / splits;
-  if (per < 1) per = 1;
-  splits = (tiles + per - 1) / per;
-  const int64_t room = slots / (n_streams > 0 ? n_streams : 1) - (g - 1);
-  if (splits > room) splits = room;
-  return splits < 1 ? 1 : (int)splits;
-}
 cudaError_t launch_fill_weights(float* w, int n, float value, cudaStream_t st);
 cudaError_t launch_seg_update(const Arena& A, const SegUpdate* ups, int n, cudaStream_t st);
 int bucket_scan_chunks(int n);

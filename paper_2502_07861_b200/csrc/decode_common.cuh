@@ -3,11 +3,14 @@
 // (the combine over the splits, the appended token, the result).
 #pragma once
 
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace bkv {
 
 constexpr int kDecodeMaxSplits = 64;
+constexpr int kInlineSplits = 16;            // most splits that the last split's CTA combines alone
 constexpr int kDecodeCtasPerSm = 2;          // both kernels: about 99 KB of shared memory per CTA
 constexpr long long kDecodeWaitCycles = 100000000LL;   // about 50 ms: a copy that has not landed by then never will
 
@@ -46,13 +49,73 @@ struct StepAppend {
   // launch in the usual way.
   const int* in_flag;
   int in_expect;
-  // Splits of a stream's tiles.  With more than one the grid has g - 1 more CTAs per stream, which combine
-  // the heads 1 .. g - 1 (see combine_head).
+  // Splits of a stream's tiles.  With more than one, either the grid has g - 1 more CTAs per stream, which combine
+  // the heads 1 .. g - 1 (see HeadEnd::combine_head), or, inline_combine (at most kInlineSplits splits), the CTA of the
+  // last split combines all heads (HeadEnd::combine_inline).
   int splits;
+  int inline_combine;
 };
 
-// CTAs per stream of a launch with `splits` splits.
-inline unsigned decode_grid_y(const Geom& G, int splits) { return (unsigned)(splits > 1 ? splits + G.g - 1 : 1); }
+// CTAs per stream of a launch.
+inline unsigned decode_grid_y(const Geom& G, const StepAppend& ap) {
+  return (unsigned)(ap.splits > 1 && !ap.inline_combine ? ap.splits + G.g - 1 : ap.splits);
+}
+
+// Split-K factor of a decode launch and how its splits are combined.
+struct SplitPlan {
+  int splits;
+  bool inline_combine;
+};
+// Most splits that the last split's CTA should combine alone: its warps take a head each, or two, whose rows cost a
+// second trip.  That pays from 4096 rows on (16 streams, g = 8, 8 / 16 splits: 2048 rows 9.9 / 10.6 us, 4096 rows
+// 14.2 / 13.7).  A single head needs no combiners of its own anyway, and combine_head spreads it over the warps (fp32,
+// one stream of 700 rows: 4.9 us against 6.3).
+inline int inline_limit(int g, int warps, int64_t tiles) {
+  return g == 1 ? 1 : g > warps && tiles < 64 ? kInlineSplits / 2 : kInlineSplits;
+}
+
+// n streams whose longest has `tiles` tiles, `slots` CTAs resident at once, `warps` warps per CTA.
+//
+// Up to slots / 2 streams: one wave, at least two tiles per CTA (a CTA less is then as fast), and the fewest splits with
+// that number of tiles per CTA.  Few splits need no CTAs besides theirs; more leave room for the g - 1 combiners of each
+// stream.  Measured (d = 128, splits with / without combiners of their own): 8 streams x 8192 rows, g = 4: 34 splits
+// 10.2 us / 16 splits 13.3; 8 x 2048, g = 8: 28 splits 7.4 / 8 splits 9.1; but 24 x 1024, g = 4: 8 splits 9.3 / 6.7, and
+// 64 x 4096, g = 5, where the combiners left room for one split: 49.8 / 4 splits 28.1 (they take slots, and their polls
+// delay the tiles).
+//
+// More streams: the share of the slots that the launch's waves fill, less 0.08 per further split for what a split costs
+// (16384 rows: 160 streams, 1 / 3 splits 217 / 199 us; 200 streams, 1 / 4: 244 / 244; 256 streams, 1 / 2:
+// 302 / 307; 304 streams, 1 / 3: 491 / 394), at least 16 tiles per CTA (304 streams x 1024 rows: 42.2 / 45.1).
+inline SplitPlan pick_decode_splits(int64_t tiles, int max_splits, int slots, int n, int g, int warps) {
+  if (n < 1) n = 1;
+  const int limit = inline_limit(g, warps, tiles);
+  int64_t s = 1;
+  if (2 * n <= slots) {
+    s = std::max<int64_t>(1, std::min<int64_t>({(tiles + 1) / 2, slots / n, max_splits}));
+    if (s > limit) {
+      const int64_t room = slots / n - (g - 1);
+      if (g == 1 || room > (g > warps ? 11 : limit)) {        // combiners of their own
+        const int64_t per = (tiles + s - 1) / s;
+        return SplitPlan{(int)std::min((tiles + per - 1) / per, room), false};
+      }
+      s = limit;
+    }
+    const int64_t per = std::max<int64_t>(1, (tiles + s - 1) / s);
+    return SplitPlan{(int)std::max<int64_t>(1, (tiles + per - 1) / per), true};
+  }
+  double best = -1.0;
+  for (int64_t k = 1; k <= 4 && k <= max_splits && (k == 1 || 16 * k <= tiles); ++k) {
+    const int64_t waves = (n * k + slots - 1) / slots;
+    const double share = (double)(n * k) / (double)(waves * slots) - 0.08 * (double)(k - 1);
+    if (share > best) { best = share; s = k; }
+  }
+  return SplitPlan{(int)s, s <= limit};
+}
+// Largest value of the above for any number of tiles.
+inline int max_decode_splits(int slots, int n) {
+  if (2 * n > slots) return n < 4 * slots ? 4 : 1;
+  return slots / n < kDecodeMaxSplits ? slots / n : kDecodeMaxSplits;
+}
 
 // Launches with programmatic stream serialization: back-to-back decode launches overlap a launch with the previous
 // kernel's tail (see the kernels' prologue).
@@ -254,14 +317,23 @@ struct HeadEnd {
   struct NewTok {
     Four<E> kn;                // 4 dims of k_new per lane (lanes < d / 4)
     Four<E> qv[kMaxGroup];     // 4 dims of q per lane and head (one head: slot 0)
-    Four<E> vn;                // lanes 0-7: the columns 32 warp + 4 lane .. + 3 of v_new
-    uint4 row[kRowLoads];      // last column warp: pieces of the K row, then of the V row
+    Four<E> vn;                // this lane's four output columns of v_new
+    uint4 row[kRowLoads];      // the appending warp: pieces of the K row, then of the V row
   };
+  // Which output columns a lane finishes: c .. c + 3 if cols; row: this warp also appends the token's row.
+  struct Part {
+    int c;
+    bool cols, row;
+  };
+  // a warp owns the output columns 32 warp .. 32 warp + 31 of every head
+  __device__ Part by_columns(int h) const { return Part{32 * warp + 4 * (lane & 7), col_warp() && lane < 8, h <= 0 && warp == kColWarps - 1}; }
+  // a warp owns a head
+  __device__ Part by_head(int h) const { return Part{4 * lane, has_dims(), h == 0}; }
   __device__ bool col_warp() const { return warp < kColWarps; }   // owns the output columns 32 warp .. 32 warp + 31
   __device__ bool has_dims() const { return 4 * lane < D; }
 
   // h < 0: the queries of all heads
-  __device__ __forceinline__ NewTok load_new(int h) const {
+  __device__ __forceinline__ NewTok load_new(int h, Part pt) const {
     NewTok nt;
     nt.kn = nt.vn = Four<E>::zero();
 #pragma unroll
@@ -272,7 +344,7 @@ struct HeadEnd {
       const E* kr = static_cast<const E*>(ap.k_new) + (size_t)sl * D;
       const E* vr = static_cast<const E*>(ap.v_new) + (size_t)sl * D;
       if (has_dims()) nt.kn = Four<E>::load(kr + 4 * lane);
-      if (col_warp() && lane < 8) nt.vn = Four<E>::load(vr + 32 * warp + 4 * lane);
+      if (pt.cols) nt.vn = Four<E>::load(vr + pt.c);
       const E* qs = q + 4 * lane;
       if (!has_dims()) {
       } else if (h >= 0) {
@@ -282,7 +354,7 @@ struct HeadEnd {
         for (int k = 0; k < kMaxGroup; ++k)
           if (k < g) nt.qv[k] = Four<E>::load(qs + (size_t)k * D);
       }
-      if (h <= 0 && warp == kColWarps - 1) {
+      if (pt.row) {
         if constexpr (kRowLoads == 2) {
           nt.row[0] = ld_early_v4(reinterpret_cast<const uint4*>(kr) + lane);
           nt.row[1] = ld_early_v4(reinterpret_cast<const uint4*>(vr) + lane);
@@ -302,10 +374,9 @@ struct HeadEnd {
     dot = fmaf(x.w, k.w, dot);
     return warp_sum(dot) * sc;
   }
-  // a: lanes 0-7 of every column warp hold the sums of the output columns 32 warp + 4 lane .. + 3.  The appended token
-  // joins as one more partial (level 0, weight 1, score x in fp32), the ratio or the raw parts are written, and with
-  // h == 0 the token's row goes into the cache.
-  __device__ __forceinline__ void finish(int h, float4 a, float M, float L, const NewTok& nt, float x) const {
+  // a: the sums of the lane's output columns.  The appended token joins as one more partial (level 0, weight 1, score x
+  // in fp32), the ratio or the raw parts are written, and with h == 0 the token's row goes into the cache.
+  __device__ __forceinline__ void finish(int h, Part pt, float4 a, float M, float L, const NewTok& nt, float x) const {
     if (ap.k_new) {
       const float Mn = fmaxf(M, x);
       const float f = M == -INFINITY ? 0.f : fast_exp2(M - Mn), fN = fast_exp2(x - Mn);
@@ -315,8 +386,8 @@ struct HeadEnd {
       L = fmaf(L, f, fN);
       M = Mn;
     }
-    if (col_warp() && lane < 8) {
-      const int c = 32 * warp + 4 * lane;
+    if (pt.cols) {
+      const int c = pt.c;
       if (raw_acc) {
         const size_t qh = (size_t)sl * g + h;
         *reinterpret_cast<float4*>(raw_acc + qh * D + c) = a;
@@ -326,7 +397,7 @@ struct HeadEnd {
         Four<E>::store(out + (size_t)h * D + c, make_float4(a.x * inv, a.y * inv, a.z * inv, a.w * inv));
       }
     }
-    if (ap.k_new && h == 0 && warp == kColWarps - 1) {
+    if (ap.k_new && h == 0 && pt.row) {
       // append: one row of K and of V, the position, the new length of C^0; ||k||^2 / ||v||^2 travel with the row
       const size_t dst_row = (size_t)stream * G.rows_per_stream + G.region_off[0] + ap.rel_row;
       uint4* dk = reinterpret_cast<uint4*>(static_cast<E*>(A.K) + dst_row * D);
@@ -378,7 +449,8 @@ struct HeadEnd {
     const float* rows = part + ((size_t)sl * splits * g + h) * D + 32 * warp + 4 * (lane & 7);        // row of split sp: + sp rstep
     const float* mls = part + (size_t)n_streams * splits * g * D + (((size_t)sl * g + h) * kColWarps + warp) * splits * 2;   // this warp's copies of the head's pairs: one line or two for a polling warp
     const size_t rstep = (size_t)g * D, mstep = 2;
-    const NewTok nt = load_new(h);              // in flight during the polls
+    const Part pt = by_columns(h);
+    const NewTok nt = load_new(h, pt);          // in flight during the polls
     const float* mlp[2] = {mls + (size_t)lane * mstep, mls + (size_t)(lane + 32) * mstep};
     float2 ml[2];
 #pragma unroll
@@ -431,7 +503,7 @@ struct HeadEnd {
       a.x += __shfl_xor_sync(0xffffffffu, a.x, o); a.y += __shfl_xor_sync(0xffffffffu, a.y, o);
       a.z += __shfl_xor_sync(0xffffffffu, a.z, o); a.w += __shfl_xor_sync(0xffffffffu, a.w, o);
     }
-    finish(h, a, M, L, nt, x_new);
+    finish(h, pt, a, M, L, nt, x_new);
     // the empty pattern again, for the next launch (every warp has its own copy of the pairs, so nobody else
     // still wants these words)
     const float e = __uint_as_float(kEmptyWord);
@@ -442,6 +514,95 @@ struct HeadEnd {
     for (int k = 0; k < 2; ++k)
       if (lane + 32 * k < splits) st_scratch2(const_cast<float*>(mlp[k]), make_float2(e, e));
     if (!ok && lane == 0) atomicCAS(status, kStatusOk, kStatusWaitTimeout);
+  }
+
+  // The same by the CTA of the last split alone, for few splits: warp w takes the heads w, w + n_warps, .., NH of them at
+  // a time, lane = four output columns, all rows of its heads in flight together.  (Of the copies of a pair only the
+  // first is in use.)  fac: NH * 32 floats.
+  template <int N, int NH>
+  __device__ __forceinline__ void combine_all(float* part, int n_streams, int n_warps, float* fac, int* status) const {
+    const int splits = ap.splits;
+    const size_t rstep = (size_t)g * D;
+    for (int h0 = warp; h0 < g; h0 += NH * n_warps) {
+      float* rows[NH];
+      float* mlp[NH];
+      bool cols[NH], pair[NH];
+      NewTok nt[NH];
+      float2 ml[NH];
+      float4 v[NH][N];
+      float x_new[NH];
+#pragma unroll
+      for (int e = 0; e < NH; ++e) {
+        const int h = h0 + e * n_warps;
+        cols[e] = h < g && has_dims();
+        pair[e] = h < g && lane < splits;
+        rows[e] = part + ((size_t)sl * splits * g + h) * D + 4 * lane;
+        mlp[e] = part + (size_t)n_streams * splits * g * D + ((size_t)sl * g + h) * kColWarps * splits * 2 + 2 * lane;
+        if (h < g) nt[e] = load_new(h, by_head(h));
+        ml[e] = pair[e] ? ld_poll2(mlp[e]) : make_float2(-INFINITY, 0.f);
+#pragma unroll
+        for (int s = 0; s < N; ++s)
+          if (cols[e] && s < splits) v[e][s] = ld_poll4(rows[e] + s * rstep);
+      }
+#pragma unroll
+      for (int e = 0; e < NH; ++e) x_new[e] = ap.k_new && h0 + e * n_warps < g ? score_new(nt[e], 0) : 0.f;
+      const long long t0 = clock64();
+      bool ok = true;
+      for (;;) {
+        bool pending = false;
+#pragma unroll
+        for (int e = 0; e < NH; ++e) {
+          if (pair[e] && (is_empty(ml[e].x) || is_empty(ml[e].y))) {
+            ml[e] = ld_poll2(mlp[e]);
+            pending = true;
+          }
+#pragma unroll
+          for (int s = 0; s < N; ++s)
+            if (cols[e] && s < splits && (is_empty(v[e][s].x) || is_empty(v[e][s].y) || is_empty(v[e][s].z) || is_empty(v[e][s].w))) {
+              v[e][s] = ld_poll4(rows[e] + s * rstep);
+              pending = true;
+            }
+        }
+        if (!__any_sync(0xffffffffu, pending)) break;
+        if (__any_sync(0xffffffffu, clock64() - t0 > kDecodeWaitCycles)) { ok = false; break; }   // warp-uniform
+      }
+      const float empty = __uint_as_float(kEmptyWord);
+#pragma unroll
+      for (int e = 0; e < NH; ++e) {
+        const int h = h0 + e * n_warps;
+        if (h >= g) break;                          // warp-uniform
+        const float M = warp_max(ml[e].x);
+        const float f = ml[e].x == -INFINITY ? 0.f : fast_exp2(ml[e].x - M);
+        const float L = warp_sum(ml[e].y * f);
+        fac[32 * e + lane] = f;
+        __syncwarp();
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int s = 0; s < N; ++s)
+          if (cols[e] && s < splits) {
+            const float w = fac[32 * e + s];
+            a.x = fmaf(v[e][s].x, w, a.x); a.y = fmaf(v[e][s].y, w, a.y); a.z = fmaf(v[e][s].z, w, a.z); a.w = fmaf(v[e][s].w, w, a.w);
+          }
+        __syncwarp();
+        finish(h, by_head(h), a, M, L, nt[e], x_new[e]);
+#pragma unroll
+        for (int s = 0; s < N; ++s)
+          if (cols[e] && s < splits) st_scratch4(rows[e] + s * rstep, make_float4(empty, empty, empty, empty));
+        if (pair[e]) st_scratch2(mlp[e], make_float2(empty, empty));
+      }
+      if (!ok && lane == 0) atomicCAS(status, kStatusOk, kStatusWaitTimeout);
+    }
+  }
+  template <int kWarps>
+  __device__ __forceinline__ void combine_inline(float* part, int n_streams, float* fac, int* status) const {
+    if constexpr (kWarps < kMaxGroup) {
+      if (g > kWarps) {
+        if (ap.splits <= kInlineSplits / 2) combine_all<kInlineSplits / 2, 2>(part, n_streams, kWarps, fac, status);
+        else combine_all<kInlineSplits, 2>(part, n_streams, kWarps, fac, status);
+        return;
+      }
+    }
+    combine_all<kInlineSplits, 1>(part, n_streams, kWarps, fac, status);
   }
 };
 

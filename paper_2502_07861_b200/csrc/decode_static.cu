@@ -22,6 +22,7 @@
 namespace bkv {
 
 int decode_mma_tile_tokens();
+int decode_mma_warps();
 cudaError_t decode_mma_static_setup();
 cudaError_t launch_decode_static_mma(const Geom& G, const Arena& A, const StepAppend& ap, const void* q, void* out, float* rows,
                                      int* status, cudaStream_t st);
@@ -33,9 +34,9 @@ namespace {
 constexpr size_t kStaticBytes = (size_t)8 << 20;
 // Split-K rows, whose words are their own arrival flags: all of them hold the empty pattern between launches, and
 // every launch puts it back.  Four blocks, used in turn, so that calls on different
-// CUDA streams do not meet in one unless more than four of them overlap.  A block holds the rows of one wave of CTAs
-// (splits > 1 only where streams x (splits + group - 1) CTAs fit 2 x 148: at most 289 rows of 8 heads).
-constexpr size_t kRowBlockBytes = (size_t)11 << 17;
+// CUDA streams do not meet in one unless more than four of them overlap.  A block holds the rows of 2 x 148 CTAs with
+// tiles (1.3 MB at 8 heads) and of most launches that split more streams than that; the split factor follows the room.
+constexpr size_t kRowBlockBytes = (size_t)22 << 17;
 constexpr int kRowBlocks = 4;
 static __device__ __align__(256) unsigned char g_static_rows[kRowBlocks * kRowBlockBytes];
 static __device__ int g_static_status;
@@ -137,8 +138,11 @@ extern "C" int balancekv_decode_attn_static(const void* K, const void* V, int n_
   ap.seg[T] = Seg{0, n_heavy};
   ap.seg[0] = T > 0 ? Seg{0, n_tail} : Seg{0, cache_len};
   const int tn = dtype == 1 ? decode_mma_tile_tokens() : decode_tile_tokens(G);
-  ap.splits = pick_decode_splits((n_heavy + tn - 1) / tn + (n_tail + tn - 1) / tn, kDecodeMaxSplits,
-                                 kDecodeCtasPerSm * g_sm_count[dev], n_streams, group);
+  const SplitPlan plan = pick_decode_splits((n_heavy + tn - 1) / tn + (n_tail + tn - 1) / tn, kDecodeMaxSplits,
+                                            kDecodeCtasPerSm * g_sm_count[dev], n_streams, group,
+                                            dtype == 1 ? decode_mma_warps() : decode_warps());
+  ap.splits = plan.splits;
+  ap.inline_combine = plan.inline_combine;
   while (ap.splits > 1 && decode_scratch_bytes(G, ap.splits) > kRowBlockBytes) --ap.splits;
   const unsigned block = g_next_rows[dev].fetch_add(1, std::memory_order_relaxed) % kRowBlocks;
   float* rows = reinterpret_cast<float*>(g_rows_addr[dev] + block * kRowBlockBytes);

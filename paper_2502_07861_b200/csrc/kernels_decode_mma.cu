@@ -73,6 +73,9 @@ __device__ inline void tma_load_3d(void* dst, const CUtensorMap* map, int x, int
       "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
       ::"r"(smem_u32(dst)), "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(z) : "memory");
 }
+__device__ inline void tma_prefetch_3d(const CUtensorMap* map, int x, int y, int z) {
+  asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(map), "r"(x), "r"(y), "r"(z) : "memory");
+}
 __device__ inline void ldsm_x4(uint32_t addr, uint32_t (&r)[4]) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
@@ -119,7 +122,9 @@ __device__ inline bool group_bar_or(int group, bool pred) {
   return r != 0;
 }
 
-template <int D>
+// kInline: how the splits are combined (StepAppend::inline_combine).  Two kernels, because the code of the way not taken
+// costs a launch 0.8 us of instruction fetches (8 streams x 8272 rows: 12.2 against 13.0 us).
+template <int D, bool kInline>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ out,
                   float* __restrict__ part_base, int* __restrict__ status,
@@ -174,7 +179,8 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
   }
   prefetch_operands<2 * D>(ap, q + (size_t)sl * g * D, sl, g);
   const bool early = ap.early && ap.n_seg;
-  if (!early) grid_wait_and_release();
+  const bool late = !ap.n_seg;                     // the segment table has to be read first
+  if (late) grid_wait_and_release();
   if (tid <= G.T) {
     const Seg s = ap.n_seg ? ap.seg[tid] : A.seg[(size_t)stream * (G.T + 1) + tid];
     seg_s[tid] = s;
@@ -200,15 +206,23 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
     }
   };
   int issued = 0;
-  if (tid == 0) {
+  if (tid == 0 && early) {
     const int lim = min(kStages, my_tiles);
-    while (issued < lim && !(early && t_begin + issued == n_tiles - 1)) issue(issued++);
+    while (issued < lim && t_begin + issued != n_tiles - 1) issue(issued++);
   }
-  if (early) {
-    grid_wait_and_release();
-    if (tid == 0)
-      while (issued < min(kStages, my_tiles)) issue(issued++);
+  // Where the first tiles cannot be fetched yet they are asked for in L2 (harmless for the reason given at
+  // prefetch_operands).
+  if (!late && !early && warp == 1 && lane < min(my_tiles, kStages)) {
+    const TileRef tr = locate_tile<kTN>(t_begin + lane, lvl_tiles, seg_s, G.T, G.region_off);
+#pragma unroll
+    for (int b = 0; b < D / 64; ++b) {
+      tma_prefetch_3d(&tmK, 64 * b, tr.row, stream);
+      tma_prefetch_3d(&tmV, 64 * b, tr.row, stream);
+    }
   }
+  if (!late) grid_wait_and_release();
+  if (tid == 0)
+    while (issued < min(kStages, my_tiles)) issue(issued++);
   wait_operands(ap, status);
 
   const float sc = 1.4426950408889634f * G.inv_sqrt_d;
@@ -216,7 +230,7 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
 
   const HeadEnd<__nv_bfloat16, D> end{G, A, ap, q + (size_t)sl * g * D, out + (size_t)sl * g * D, raw_acc, raw_ml, sl, stream, g, warp, lane, sc};
   float* const fac = reinterpret_cast<float*>(tiles + kFacOff) + warp * kDecodeMaxSplits;   // behind the merge buffers, which other warps may still be reading
-  if (split >= splits) {                        // a CTA without tiles: the combiner of head split - splits + 1
+  if (!kInline && split >= splits) {            // a CTA without tiles: the combiner of head split - splits + 1
     end.combine_head(split - splits + 1, part, gridDim.x, fac, status);
     return;
   }
@@ -470,7 +484,7 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
         if (lane == 0) *reinterpret_cast<float2*>(my_ml + 2 * h) = make_float2(M, L);
       } else {                                  // published: see the combine below
         if (end.has_dims()) st_scratch4(my_acc + h * D + 4 * lane, acc);
-        if (lane < kColWarps) st_scratch2(my_ml + ((size_t)(h * kColWarps + lane) * splits + split) * 2, make_float2(M, L));   // a copy per combining warp
+        if (lane < (kInline ? 1 : kColWarps)) st_scratch2(my_ml + ((size_t)(h * kColWarps + lane) * splits + split) * 2, make_float2(M, L));   // a copy per combining warp
       }
     }
   }
@@ -478,15 +492,18 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
     __syncthreads();                            // the rows in shared memory are complete
     const float* acc1 = reinterpret_cast<const float*>(tiles + kSingleOff);
     const float* ml1 = acc1 + kMaxGroup * D;
-    const auto nt = end.load_new(-1);
+    const auto nt = end.load_new(-1, end.by_columns(-1));
 #pragma unroll
     for (int h = 0; h < kMaxGroup; ++h)
       if (h < g)
-        end.finish(h, *reinterpret_cast<const float4*>(acc1 + h * D + (32 * warp) % D + 4 * (lane & 7)), ml1[2 * h], ml1[2 * h + 1], nt,
+        end.finish(h, end.by_columns(h), *reinterpret_cast<const float4*>(acc1 + h * D + (32 * warp) % D + 4 * (lane & 7)), ml1[2 * h], ml1[2 * h + 1], nt,
                ap.k_new ? end.score_new(nt, h) : 0.f);
     return;
   }
-  if (split == splits - 1) end.combine_head(0, part, gridDim.x, fac, status);
+  if (split == splits - 1) {
+    if constexpr (kInline) end.template combine_inline<kWarps>(part, gridDim.x, fac, status);
+    else end.combine_head(0, part, gridDim.x, fac, status);
+  }
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -524,16 +541,22 @@ cudaError_t encode_maps(DecodeMaps* tm, void* K, void* V, int d, int64_t rows, i
   return cudaSuccess;
 }
 
+auto kernel_for(int d, bool inline_combine) {
+  return d == 128 ? (inline_combine ? decode_mma_kernel<128, true> : decode_mma_kernel<128, false>)
+                  : (inline_combine ? decode_mma_kernel<64, true> : decode_mma_kernel<64, false>);
+}
+size_t smem_bytes(int d) { return d == 128 ? Dim<128>::kSmemBytes : Dim<64>::kSmemBytes; }
 cudaError_t set_smem(int d) {
-  return d == 128 ? cudaFuncSetAttribute(decode_mma_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Dim<128>::kSmemBytes)
-                  : cudaFuncSetAttribute(decode_mma_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Dim<64>::kSmemBytes);
+  cudaError_t e = cudaSuccess;
+  for (int i = 0; i < 2 && e == cudaSuccess; ++i)
+    e = cudaFuncSetAttribute(kernel_for(d, i != 0), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes(d));
+  return e;
 }
 
 cudaError_t launch(const Geom& G, const Arena& A, int layer, const void* q, void* out, float* part, int* status,
                    const StepAppend& ap, const DecodeMaps& tm, int n_slots, cudaStream_t st) {
-  const PdlConfig pc(dim3(G.B * G.H, decode_grid_y(G, ap.splits), n_slots), kThreads,
-                     G.d == 128 ? Dim<128>::kSmemBytes : Dim<64>::kSmemBytes, st);
-  return cudaLaunchKernelEx(&pc.cfg, G.d == 128 ? decode_mma_kernel<128> : decode_mma_kernel<64>, G, A, layer,
+  const PdlConfig pc(dim3(G.B * G.H, decode_grid_y(G, ap), n_slots), kThreads, smem_bytes(G.d), st);
+  return cudaLaunchKernelEx(&pc.cfg, kernel_for(G.d, ap.inline_combine), G, A, layer,
                             static_cast<const __nv_bfloat16*>(q), static_cast<__nv_bfloat16*>(out), part, status, ap, tm.k, tm.v);
 }
 
@@ -541,6 +564,7 @@ cudaError_t launch(const Geom& G, const Arena& A, int layer, const void* q, void
 
 bool decode_mma_supported(const Geom& G) { return G.is_bf16 && (G.d == 128 || G.d == 64) && G.g <= 8; }
 int decode_mma_tile_tokens() { return kTN; }
+int decode_mma_warps() { return kWarps; }
 
 cudaError_t decode_mma_prepare(const Geom& G, const Arena& A, void** maps_out) {
   *maps_out = nullptr;
@@ -560,10 +584,14 @@ void decode_mma_release(void* maps) { delete static_cast<DecodeMaps*>(maps); }
 // slot (laid out as for a single slot).
 cudaError_t launch_decode_parts_mma_slots(const Geom& G, const Arena& A, const int* slot_layers, int n_slots,
                                           unsigned keys_mask, const void* q, float* raw_acc, float* raw_ml, float* scratch,
-                                          size_t z_stride_words, int splits, int* status, const void* maps,
+                                          size_t z_stride_words, SplitPlan plan, int* status, const void* maps,
                                           cudaStream_t st) {
   if (!maps || !raw_acc || !raw_ml || n_slots < 1 || n_slots > 8 || z_stride_words > 0xffffffffull) return cudaErrorInvalidValue;
-  StepAppend ap{nullptr, nullptr, 0, 0, 0, raw_acc, raw_ml, 0, 0, {}, n_slots, {}, keys_mask, (unsigned)z_stride_words, 0, nullptr, 0, splits};
+  StepAppend ap{};
+  ap.raw_acc = raw_acc; ap.raw_ml = raw_ml;
+  ap.n_slots = n_slots; ap.keys_mask = keys_mask; ap.z_stride = (unsigned)z_stride_words;
+  ap.splits = plan.splits;
+  ap.inline_combine = plan.inline_combine;
   for (int i = 0; i < n_slots; ++i) ap.slot_layer[i] = slot_layers[i];
   return launch(G, A, slot_layers[0], q, nullptr, scratch, status, ap, *static_cast<const DecodeMaps*>(maps),
                 n_slots, st);

@@ -71,6 +71,7 @@ struct balancekv_ctx {
   int8_t* d_eta = nullptr;
   unsigned long long* d_fail = nullptr;
   int* d_status = nullptr;
+  int* h_status_dev = nullptr;   // device address of h_status
   int* h_status = nullptr;       // pinned mirror of the status word, refreshed after every compress batch and by stats
   float* d_decode_scratch = nullptr;
   int max_splits = 1;
@@ -357,9 +358,10 @@ int balancekv_create(const balancekv_config* cfg, balancekv_ctx** out) {
     if (G.center_keys && (rc = dev_alloc(c, &c->d_tokshift, (size_t)c->max_calls * (t + f.head_dim)))) return fail(rc);
   }
   if ((rc = dev_alloc(c, &c->d_fail, 1))) return fail(rc);
-  if ((rc = dev_alloc(c, &c->d_status, 1))) return fail(rc);
+  if ((rc = dev_alloc(c, &c->d_status, 2))) return fail(rc);       // the word, and the counter of launch_reset
   if (cudaMemset(c->d_fail, 0, 256) != cudaSuccess || cudaMemset(c->d_status, 0, 256) != cudaSuccess) return fail(BALANCEKV_E_CUDA);
   if (cudaMallocHost(reinterpret_cast<void**>(&c->h_status), 64) != cudaSuccess) return fail(BALANCEKV_E_NOMEM);
+  if (cudaHostGetDevicePointer(reinterpret_cast<void**>(&c->h_status_dev), c->h_status, 0) != cudaSuccess) return fail(BALANCEKV_E_CUDA);
   *c->h_status = 0;
   {
     const int n_sl = f.n_seqs * f.n_kv_heads;
@@ -553,6 +555,59 @@ int balancekv_cache_load_level(balancekv_ctx* c, int layer, int level, const voi
   return append_impl(c, layer_streams(c, layer), level, K, V, orig_idx, n_tokens, static_cast<cudaStream_t>(stream), layer);
 }
 
+// One level of a batch: radii -> walk -> selection/compaction for n calls.
+static int run_calls(balancekv_ctx* c, const CallSet& calls, int n, int l, cudaStream_t st) {
+  const Geom& G = c->G;
+  // the tensor-core walk kernel takes the radii from the stored row norms itself
+  const bool need_radii = (G.center_keys || G.fixed_rk2 <= 0.f || G.fixed_rv2 <= 0.f) && !(c->use_tc && !G.center_keys);
+  if (need_radii) {
+    ProfScope ps(c, 1, st);
+    BKV_CUDA(launch_radii(G, c->A, calls, n, c->d_stats, c->d_tokshift, st));
+    c->kernels_launched += 1 + (G.center_keys ? 1 : 0);
+  }
+  if (c->use_tc) {
+    ProfScope ps(c, 2, st);
+    BKV_CUDA(launch_walk_tc(G, c->A, calls, n, l, c->d_stats, c->d_tokshift, c->d_eta, c->dbg_eta, c->dbg_S,
+                            c->dbg_p, c->d_fail, c->d_status, c->tmaps, c, st));   // selection + compaction fused at the tail
+  } else {
+    ProfScope ps(c, 2, st);
+    BKV_CUDA(launch_walk_simt(G, c->A, calls, n, l, c->d_stats, c->d_tokshift, c->d_eta, c->dbg_eta, c->dbg_S,
+                              c->dbg_p, c->d_fail, st));
+  }
+  if (!c->use_tc) {
+    ProfScope ps(c, 3, st);
+    BKV_CUDA(launch_compact(G, c->A, calls, n, l, c->d_eta, st));
+    c->kernels_launched++;
+  }
+  c->kernels_launched++;
+  c->calls_run += n;
+  return BALANCEKV_OK;
+}
+
+// A batch over streams first .. first + n - 1 (positions of the layer, or of the context for layer < 0) that are all in the
+// state of st[id of first]: no descriptors travel to the device, and one kernel ends the batch.  (The descriptor transfer,
+// the separate move and segment kernels and the transfer of the status word were 15 to 20 us of a compress.)
+static int run_lockstep(balancekv_ctx* c, int layer, int first, int n, int nb, cudaStream_t st) {
+  c->decode_chain = false;
+  StreamState S = c->st[lockstep_stream(c->G, layer, first)];
+  std::vector<CallSet> sets;
+  std::vector<int> calls;
+  BatchEnd E;
+  Seg seg[kMaxLevels + 1];
+  plan_lockstep(c->Lo, S, nb, layer, first, sets, calls, E, seg);
+  for (int l = 0; l < c->G.T; ++l) {
+    if (calls[l] == 0) break;
+    if (const int rc = run_calls(c, sets[l], n * calls[l], l, st)) return rc;
+  }
+  {
+    ProfScope ps(c, 5, st);
+    BKV_CUDA(launch_batch_end(c->G, c->A, E, n, seg, c->d_status, c->h_status_dev, st));
+    c->kernels_launched++;
+  }
+  for (int i = 0; i < n; ++i) c->st[lockstep_stream(c->G, layer, first + i)] = S;
+  return BALANCEKV_OK;
+}
+
 // Runs one planned batch: per level radii -> walk -> selection/compaction, then the
 // level-0 remainder moves and the segment-table update.
 static int run_plan(balancekv_ctx* c, Plan& P, cudaStream_t st) {
@@ -601,31 +656,9 @@ static int run_plan(balancekv_ctx* c, Plan& P, cudaStream_t st) {
         int rc = ring_push(c, calls.data() + first, (size_t)n * sizeof(CallDesc), st, &d_calls);
         if (rc) return rc;
       }
-      const CallDesc* dc = static_cast<const CallDesc*>(d_calls);
-      // the tensor-core walk kernel takes the radii from the stored row norms itself
-      const bool need_radii = (G.center_keys || G.fixed_rk2 <= 0.f || G.fixed_rv2 <= 0.f) &&
-                              !(c->use_tc && !G.center_keys && c->A.nrm);
-      if (need_radii) {
-        ProfScope ps(c, 1, st);
-        BKV_CUDA(launch_radii(G, c->A, dc, n, c->d_stats, c->d_tokshift, st));
-        c->kernels_launched += 1 + (G.center_keys ? 1 : 0);
-      }
-      if (c->use_tc) {
-        ProfScope ps(c, 2, st);
-        BKV_CUDA(launch_walk_tc(G, c->A, dc, n, l, c->d_stats, c->d_tokshift, c->d_eta, c->dbg_eta, c->dbg_S,
-                                c->dbg_p, c->d_fail, c->d_status, c->tmaps, c, st));   // selection + compaction fused at the tail
-      } else {
-        ProfScope ps(c, 2, st);
-        BKV_CUDA(launch_walk_simt(G, c->A, dc, n, l, c->d_stats, c->d_tokshift, c->d_eta, c->dbg_eta, c->dbg_S,
-                                  c->dbg_p, c->d_fail, st));
-      }
-      if (!c->use_tc) {
-        ProfScope ps(c, 3, st);
-        BKV_CUDA(launch_compact(G, c->A, dc, n, l, c->d_eta, st));
-        c->kernels_launched++;
-      }
-      c->kernels_launched++;
-      c->calls_run += n;
+      CallSet set{};
+      set.list = static_cast<const CallDesc*>(d_calls);
+      if (const int rc = run_calls(c, set, n, l, st)) return rc;
     }
   }
   if (!P.moves.empty()) {
@@ -653,11 +686,26 @@ static int run_plan(balancekv_ctx* c, Plan& P, cudaStream_t st) {
   return BALANCEKV_OK;
 }
 
-static int compress_streams(balancekv_ctx* c, const std::vector<int>& streams, int T, cudaStream_t st) {
+// layer: the layer whose streams these are, or -1 for all streams of the context.
+static int compress_streams(balancekv_ctx* c, const std::vector<int>& streams, int layer, int T, cudaStream_t st) {
   if (T != c->cfg.levels) return BALANCEKV_E_INVAL;
   if (timed_out(c)) return BALANCEKV_E_TIMEOUT;
   for (int s : streams) c->st[s].pending = 0;
   if (T == 0) return BALANCEKV_OK;
+  const int n = (int)streams.size();
+  const StreamState& S0 = c->st[streams[0]];
+  bool alike = !c->debug;                             // a context that records its calls needs their offsets
+  for (int s : streams) alike = alike && c->st[s].same_as(S0);
+  if (alike) {
+    const int64_t nb = ready_blocks(c->Lo, S0);
+    if (nb <= 0) return BALANCEKV_OK;
+    if (nb <= c->max_calls) {
+      const int batch = lockstep_batch(n, (int)nb, c->cfg.levels, (int)(c->max_calls / nb), c->sm_count);
+      for (int first = 0; first < n; first += batch)
+        if (const int rc = run_lockstep(c, layer, first, std::min(batch, n - first), (int)nb, st)) return rc;
+      return BALANCEKV_OK;
+    }
+  }
   // greedy batches of at most max_calls level-0 calls
   std::vector<int64_t> left(streams.size());
   bool any = false;
@@ -686,12 +734,12 @@ int balancekv_compress(balancekv_ctx* c, int T, void* stream) {
   if (!c) return BALANCEKV_E_INVAL;
   std::vector<int> all(c->n_streams);
   for (int i = 0; i < c->n_streams; ++i) all[i] = i;
-  return compress_streams(c, all, T, static_cast<cudaStream_t>(stream));
+  return compress_streams(c, all, -1, T, static_cast<cudaStream_t>(stream));
 }
 
 int balancekv_compress_layer(balancekv_ctx* c, int layer, int T, void* stream) {
   if (!c || layer < 0 || layer >= c->cfg.n_layers) return BALANCEKV_E_INVAL;
-  return compress_streams(c, layer_streams(c, layer), T, static_cast<cudaStream_t>(stream));
+  return compress_streams(c, layer_streams(c, layer), layer, T, static_cast<cudaStream_t>(stream));
 }
 
 // The layer's segment table as the host mirrors it, if all its streams hold the same segments
@@ -1272,15 +1320,13 @@ int balancekv_reset(balancekv_ctx* c, void* stream) {
   for (StreamState& S : c->st) S = StreamState();
   c->bucket_vmax2.clear();
   c->bucket_erase_max.clear();
-  BKV_CUDA(cudaMemsetAsync(c->A.seg, 0, sizeof(Seg) * (size_t)c->n_streams * (c->cfg.levels + 1), st));
-  // a context that gave up on a device-side wait becomes usable again
-  BKV_CUDA(cudaMemsetAsync(c->d_status, 0, sizeof(int), st));
+  // one kernel: the segment table, and -- where a device-side wait has given up -- the split-K scratch and the status word,
+  // so that the context becomes usable again
   *c->h_status = 0;
-  // a launch that gave up may have left partial rows behind
-  BKV_CUDA(init_decode_scratch(c->d_decode_scratch, decode_scratch_bytes(c->G, c->max_splits), st));
-  if (c->two_scratch)
-    for (int z = 0; z < BALANCEKV_MAX_MERGE; ++z)
-      BKV_CUDA(init_decode_scratch(c->two_scratch + c->two_scratch_words * z, c->two_scratch_words * 4, st));
+  BKV_CUDA(launch_reset(c->A.seg, (size_t)c->n_streams * (c->cfg.levels + 1), c->d_decode_scratch,
+                        decode_scratch_bytes(c->G, c->max_splits) / 4, c->two_scratch,
+                        c->two_scratch ? c->two_scratch_words * BALANCEKV_MAX_MERGE : 0, c->d_status, c->h_status_dev, st));
+  c->kernels_launched++;
   return BALANCEKV_OK;
 }
 

@@ -19,6 +19,34 @@ struct CallDesc {
   int32_t ordinal;        // call ordinal inside its level (Philox coordinate)
 };
 
+// The calls of one level of a batch: an explicit list, or (list == nullptr) the same calls for every one of a range of
+// lockstep streams, derived from the call's index so that no descriptor has to travel to the device.
+struct CallSet {
+  const CallDesc* list;
+  int32_t layer, first;      // streams: the positions first, first + 1, .. of the layer (layer >= 0) or of the context
+  int32_t per_stream;        // calls per stream; call index = stream index * per_stream + k
+  int32_t ordinal0;          // call ordinal of k = 0
+  int32_t src_rel;           // row inside the stream: calls of level 0 read src_rel + k t; above, a held pair (src_held)
+  int32_t src_held;          //   sits there and is read by k = 0
+  int64_t src_pool;          // first pool row of the other inputs (< 0: level 0)
+  int32_t src_pairs;         // pool slots (of t rows) per stream
+  int32_t top;               // 1: survivors go to level T, row dst_rel + k t/2 of the stream
+  int32_t dst_rel;
+  int32_t dst_held;          // a half is already held: the first survivors join it at row dst_held_rel of the stream
+  int32_t dst_held_rel;
+  int32_t dst_left_rel;      // row of the half that stays behind when the halves are odd in number
+  int32_t dst_pairs_all;     // pairs of halves of a stream, incl. the one that the held half completes
+  int32_t dst_pairs;         // of them in the pool
+  int64_t dst_pool;
+};
+
+// What ends a batch over lockstep streams: the level-0 remainder moves to the front of its region, the segment table
+// takes the new state, and a device-side failure is shown to the host.
+struct BatchEnd {
+  int32_t layer, first;      // streams as in CallSet
+  int32_t move_src, move_rows;   // rows of the level-0 region (move_rows == 0: none)
+};
+
 // One append (or level load) of a batched launch.
 struct AppendDesc {
   int64_t dst_row;    // first destination row in the arena
@@ -84,6 +112,51 @@ struct Geom {
   uint64_t seed;
   int32_t center_keys;
 };
+
+__host__ __device__ inline int lockstep_stream(const Geom& G, int layer, int pos) {
+  return layer >= 0 ? ((pos / G.H) * G.L + layer) * G.H + pos % G.H : pos;
+}
+// Call `call` of the set (dbg_off: lists only; a context that records its calls uses lists).
+__host__ __device__ inline CallDesc call_of(const CallSet& S, const Geom& G, int call) {
+  if (S.list) return S.list[call];
+  const int i = call / S.per_stream, k = call - i * S.per_stream;
+  CallDesc d;
+  d.stream = lockstep_stream(G, S.layer, S.first + i);
+  d.ordinal = S.ordinal0 + k;
+  d.dbg_off = -1;
+  const int64_t sb = (int64_t)d.stream * G.rows_per_stream;
+  if (S.src_pool < 0) d.src_row = sb + S.src_rel + (int64_t)k * G.t;
+  else if (S.src_held && k == 0) d.src_row = sb + S.src_rel;
+  else d.src_row = S.src_pool + ((int64_t)i * S.src_pairs + k - S.src_held) * G.t;
+  const int half = G.t / 2, j = S.dst_held + k, pr = j / 2;
+  if (S.top) d.dst_row = sb + S.dst_rel + (int64_t)k * half;
+  else if (pr >= S.dst_pairs_all) d.dst_row = sb + S.dst_left_rel;
+  else if (S.dst_held && pr == 0) d.dst_row = sb + S.dst_held_rel;
+  else d.dst_row = S.dst_pool + ((int64_t)i * S.dst_pairs + pr - S.dst_held) * G.t + (int64_t)(j & 1) * half;
+  return d;
+}
+
+// Launches with programmatic stream serialization: the kernel may become resident while its predecessor on the stream is
+// finishing.  Every such kernel calls grid_wait() before it touches anything that an earlier kernel writes or reads; it
+// then releases its own dependents, which wait for its end in the same way.
+struct PdlConfig {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr;
+  PdlConfig(dim3 grid, int threads, size_t smem, cudaStream_t st) {
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+  }
+};
+__device__ inline void grid_wait_and_release() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 
 enum DeviceStatus : int { kStatusOk = 0, kStatusWaitTimeout = 1, kStatusBadIndex = 2 };
 
@@ -167,16 +240,22 @@ cudaError_t launch_append_uniform(const Geom& G, const Arena& A, int layer, int 
                                   cudaStream_t st);
 cudaError_t launch_move(const Geom& G, const Arena& A, const MoveDesc* descs, int n_desc, int max_rows,
                         cudaStream_t st);
-cudaError_t launch_radii(const Geom& G, const Arena& A, const CallDesc* calls, int n_calls, CallStat* stats,
+cudaError_t launch_batch_end(const Geom& G, const Arena& A, const BatchEnd& E, int n_streams, const Seg* seg,
+                             const int* status, int* status_host, cudaStream_t st);
+// Forget every stream (segment table) and, if a device-side wait has given up, restore the split-K scratch: n words of
+// `scratch` and n2 of `scratch2` (may be null).  status: the status word, behind it a zero word of scratch.
+cudaError_t launch_reset(Seg* seg, size_t n_seg, float* scratch, size_t n, float* scratch2, size_t n2, int* status,
+                         int* status_host, cudaStream_t st);
+cudaError_t launch_radii(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, CallStat* stats,
                          float* tok_shift, cudaStream_t st);
-cudaError_t launch_walk_simt(const Geom& G, const Arena& A, const CallDesc* calls, int n_calls, int level,
+cudaError_t launch_walk_simt(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, int level,
                              const CallStat* stats, const float* tok_shift, int8_t* eta, int8_t* dbg_eta,
                              float* dbg_S, float* dbg_p, unsigned long long* fail_count, cudaStream_t st);
-cudaError_t launch_walk_tc(const Geom& G, const Arena& A, const CallDesc* calls, int n_calls, int level,
+cudaError_t launch_walk_tc(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, int level,
                            const CallStat* stats, const float* tok_shift, int8_t* eta, int8_t* dbg_eta,
                            float* dbg_S, float* dbg_p, unsigned long long* fail_count, int* status,
                            const void* tmap_k, const void* tmap_v, cudaStream_t st);
-cudaError_t launch_compact(const Geom& G, const Arena& A, const CallDesc* calls, int n_calls, int level,
+cudaError_t launch_compact(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, int level,
                            const int8_t* eta, cudaStream_t st);
 struct StepAppend;      // decode_common.cuh
 size_t decode_scratch_bytes(const Geom& G, int splits);

@@ -117,23 +117,6 @@ inline int max_decode_splits(int slots, int n) {
   return slots / n < kDecodeMaxSplits ? slots / n : kDecodeMaxSplits;
 }
 
-// Launches with programmatic stream serialization: back-to-back decode launches overlap a launch with the previous
-// kernel's tail (see the kernels' prologue).
-struct PdlConfig {
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr;
-  PdlConfig(dim3 grid, int threads, size_t smem, cudaStream_t st) {
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-  }
-};
-
 namespace dec {
 
 __device__ inline uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -168,10 +151,6 @@ __device__ inline float fast_exp2(float x) {     // -inf -> 0
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
-}
-__device__ inline void grid_wait_and_release() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // Accesses to the split-K scratch (see combine_head).  Publishing stores and polling loads are relaxed operations at

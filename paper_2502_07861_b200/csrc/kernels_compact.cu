@@ -40,10 +40,11 @@ __device__ inline int block_exclusive_scan(int v, int* warp_sums, int& total) {
 }
 
 __global__ void __launch_bounds__(kThreads)
-compact_kernel(Geom G, Arena A, const CallDesc* __restrict__ calls, const int8_t* __restrict__ eta) {
+compact_kernel(Geom G, Arena A, const CallSet calls, const int8_t* __restrict__ eta) {
   extern __shared__ int kept_pos[];  // [t/2]
   __shared__ int warp_sums[kThreads / 32];
-  const CallDesc C = calls[blockIdx.x];
+  grid_wait_and_release();
+  const CallDesc C = call_of(calls, G, blockIdx.x);
   const int t = G.t, half = t / 2;
   const int ipt = (t + kThreads - 1) / kThreads;   // consecutive items per thread
   const int j0 = threadIdx.x * ipt;
@@ -96,14 +97,14 @@ compact_kernel(Geom G, Arena A, const CallDesc* __restrict__ calls, const int8_t
 
 }  // namespace
 
-cudaError_t launch_compact(const Geom& G, const Arena& A, const CallDesc* calls, int n_calls, int level,
+cudaError_t launch_compact(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, int level,
                            const int8_t* eta, cudaStream_t st) {
   if (n_calls <= 0) return cudaSuccess;
   const int half = G.t / 2;
   dim3 grid(n_calls, (half + kRowsPerCta - 1) / kRowsPerCta);
   (void)level;
-  compact_kernel<<<grid, kThreads, sizeof(int) * half, st>>>(G, A, calls, eta);
-  return cudaGetLastError();
+  const PdlConfig pc(grid, kThreads, sizeof(int) * half, st);
+  return cudaLaunchKernelEx(&pc.cfg, compact_kernel, G, A, calls, eta);
 }
 
 }  // namespace bkv

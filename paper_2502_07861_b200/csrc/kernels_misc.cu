@@ -2,6 +2,8 @@
 //   append / level load   (Algorithm 3: C^0 <- C^0 + {k_j, v_j})
 //   level-0 remainder move
 //   per-call radii r_key^2, r_value^2 (inputs of Algorithm 2) and the optional key shift
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace bkv {
@@ -110,6 +112,7 @@ append_kernel(Geom G, Arena A, const AppendDesc* __restrict__ descs, const void*
 __global__ void __launch_bounds__(256)
 append_uniform_kernel(Geom G, Arena A, int layer, int level, int rel_row, int idx0, int n, int new_len,
                       const void* __restrict__ Ksrc, const void* __restrict__ Vsrc, const int32_t* __restrict__ idx_src) {
+  grid_wait_and_release();
   const int sl = blockIdx.x;                                 // seq * H + head
   const int stream = ((sl / G.H) * G.L + layer) * G.H + (sl % G.H);
   const int64_t dst_row = (int64_t)stream * G.rows_per_stream + G.region_off[level] + rel_row;
@@ -126,10 +129,8 @@ append_uniform_kernel(Geom G, Arena A, int layer, int level, int rel_row, int id
   if (blockIdx.y == 0 && threadIdx.x == 0) A.seg[(size_t)stream * (G.T + 1) + level].len = new_len;
 }
 
-__global__ void __launch_bounds__(256)
-move_kernel(Geom G, Arena A, const MoveDesc* __restrict__ descs) {
-  const MoveDesc D = descs[blockIdx.x];
-  const int row0 = blockIdx.y * kCopyRows;
+// Rows row0 .. of one move.
+__device__ inline void move_rows(const Geom& G, const Arena& A, const MoveDesc& D, int row0) {
   if (row0 < D.n) {
     const int rows = min(kCopyRows, D.n - row0);
     const int esz = G.is_bf16 ? 2 : 4;
@@ -147,6 +148,49 @@ move_kernel(Geom G, Arena A, const MoveDesc* __restrict__ descs) {
   }
 }
 
+__global__ void __launch_bounds__(256)
+move_kernel(Geom G, Arena A, const MoveDesc* __restrict__ descs) {
+  move_rows(G, A, descs[blockIdx.x], blockIdx.y * kCopyRows);
+}
+
+struct SegRow {            // the segments of a lockstep stream after a batch
+  Seg seg[kMaxLevels + 1];
+};
+// grid (streams, row groups of the move)
+__global__ void __launch_bounds__(256)
+batch_end_kernel(Geom G, Arena A, BatchEnd E, SegRow row, const int* __restrict__ status, int* __restrict__ status_host) {
+  grid_wait_and_release();
+  const int stream = lockstep_stream(G, E.layer, E.first + blockIdx.x);
+  const int64_t r0 = (int64_t)stream * G.rows_per_stream + G.region_off[0];
+  move_rows(G, A, MoveDesc{r0 + E.move_src, r0, stream, E.move_rows}, blockIdx.y * kCopyRows);
+  if (blockIdx.y == 0) {
+    if (threadIdx.x <= G.T) A.seg[(size_t)stream * (G.T + 1) + threadIdx.x] = row.seg[threadIdx.x];
+    if (blockIdx.x == 0 && threadIdx.x == 0 && *status != kStatusOk) *static_cast<volatile int*>(status_host) = *status;
+  }
+}
+
+__global__ void __launch_bounds__(256)
+reset_kernel(Seg* __restrict__ seg, size_t n_seg, float* __restrict__ scratch, size_t n, float* __restrict__ scratch2, size_t n2,
+             int* __restrict__ status, int* __restrict__ status_host) {
+  grid_wait_and_release();
+  const size_t i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x, step = (size_t)gridDim.x * blockDim.x;
+  for (size_t i = i0; i < n_seg; i += step) seg[i] = Seg{0, 0};
+  if (*static_cast<volatile int*>(status) != kStatusOk) {      // a launch that gave up may have left partial rows behind
+    const float empty = __uint_as_float(0xffffffffu);
+    for (size_t i = i0; i < n; i += step) scratch[i] = empty;
+    for (size_t i = i0; i < n2; i += step) scratch2[i] = empty;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(status + 1, 1) == (int)gridDim.x - 1) {      // every CTA has read the status word
+      status[0] = kStatusOk;
+      status[1] = 0;
+      *static_cast<volatile int*>(status_host) = kStatusOk;
+    }
+  }
+}
+
 __global__ void seg_update_kernel(Arena A, const SegUpdate* __restrict__ ups, int n) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) A.seg[ups[i].index] = Seg{ups[i].start, ups[i].len};
@@ -155,8 +199,10 @@ __global__ void seg_update_kernel(Arena A, const SegUpdate* __restrict__ ups, in
 // Column means of the call's keys, one CTA per call, thread e owns column e
 // (fixed summation order, so the result is reproducible).
 template <bool kBf16>
-__global__ void mean_kernel(Geom G, Arena A, const CallDesc* __restrict__ calls, float* __restrict__ mean) {
-  const CallDesc C = calls[blockIdx.x];
+__global__ void mean_kernel(Geom G, Arena A, const CallSet calls, float* __restrict__ mean, CallStat* __restrict__ stats) {
+  grid_wait_and_release();
+  if (threadIdx.x == 0) stats[blockIdx.x] = CallStat{0.f, 0.f};     // radii_kernel takes maxima into it
+  const CallDesc C = call_of(calls, G, blockIdx.x);
   const int e = threadIdx.x;
   if (e >= G.d) return;
   float s = 0.f;
@@ -172,9 +218,10 @@ __global__ void mean_kernel(Geom G, Arena A, const CallDesc* __restrict__ calls,
 // <k_i - mean, k_j - mean> = <k_i, k_j> - a_i - a_j.
 template <bool kBf16>
 __global__ void __launch_bounds__(256)
-radii_kernel(Geom G, Arena A, const CallDesc* __restrict__ calls, CallStat* __restrict__ stats,
+radii_kernel(Geom G, Arena A, const CallSet calls, CallStat* __restrict__ stats,
              const float* __restrict__ mean, float* __restrict__ tok_shift) {
-  const CallDesc C = calls[blockIdx.x];
+  grid_wait_and_release();
+  const CallDesc C = call_of(calls, G, blockIdx.x);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int esz = kBf16 ? 2 : 4;
   float mk = 0.f, mv = 0.f;
@@ -231,8 +278,9 @@ radii_kernel(Geom G, Arena A, const CallDesc* __restrict__ calls, CallStat* __re
 
 // r_key^2, r_value^2 of a call from the stored row norms: one CTA per call.
 __global__ void __launch_bounds__(256)
-radii_norms_kernel(Geom G, Arena A, const CallDesc* __restrict__ calls, CallStat* __restrict__ stats) {
-  const CallDesc C = calls[blockIdx.x];
+radii_norms_kernel(Geom G, Arena A, const CallSet calls, CallStat* __restrict__ stats) {
+  grid_wait_and_release();
+  const CallDesc C = call_of(calls, G, blockIdx.x);
   float mk = 0.f, mv = 0.f;
   for (int j = threadIdx.x; j < G.t; j += 256) {
     const float2 n = A.nrm[C.src_row + j];
@@ -272,8 +320,8 @@ cudaError_t launch_append_uniform(const Geom& G, const Arena& A, int layer, int 
                                   int new_len, const void* Ksrc, const void* Vsrc, const int32_t* idx_src,
                                   cudaStream_t st) {
   dim3 grid(G.B * G.H, (n + kCopyRows - 1) / kCopyRows);
-  append_uniform_kernel<<<grid, n >= 16 ? 256 : 64, 0, st>>>(G, A, layer, level, rel_row, idx0, n, new_len, Ksrc, Vsrc, idx_src);
-  return cudaGetLastError();
+  const PdlConfig pc(grid, n >= 16 ? 256 : 64, 0, st);
+  return cudaLaunchKernelEx(&pc.cfg, append_uniform_kernel, G, A, layer, level, rel_row, idx0, n, new_len, Ksrc, Vsrc, idx_src);
 }
 
 cudaError_t launch_move(const Geom& G, const Arena& A, const MoveDesc* descs, int n_desc, int max_rows,
@@ -285,27 +333,35 @@ cudaError_t launch_move(const Geom& G, const Arena& A, const MoveDesc* descs, in
   return cudaGetLastError();
 }
 
+cudaError_t launch_batch_end(const Geom& G, const Arena& A, const BatchEnd& E, int n_streams, const Seg* seg,
+                             const int* status, int* status_host, cudaStream_t st) {
+  SegRow row;
+  for (int l = 0; l <= kMaxLevels; ++l) row.seg[l] = l <= G.T ? seg[l] : Seg{0, 0};
+  const PdlConfig pc(dim3(n_streams, std::max(1, (E.move_rows + kCopyRows - 1) / kCopyRows)), 256, 0, st);
+  return cudaLaunchKernelEx(&pc.cfg, batch_end_kernel, G, A, E, row, status, status_host);
+}
+
+cudaError_t launch_reset(Seg* seg, size_t n_seg, float* scratch, size_t n, float* scratch2, size_t n2, int* status,
+                         int* status_host, cudaStream_t st) {
+  const PdlConfig pc(dim3((unsigned)std::min<size_t>(148, (n_seg + 255) / 256 + 1)), 256, 0, st);
+  return cudaLaunchKernelEx(&pc.cfg, reset_kernel, seg, n_seg, scratch, n, scratch2, n2, status, status_host);
+}
+
 // stats must hold n_calls entries; tok_shift n_calls * t floats (+ n_calls * d floats of
 // mean scratch behind it) when key centering is on, else it may be null.
-cudaError_t launch_radii(const Geom& G, const Arena& A, const CallDesc* calls, int n_calls, CallStat* stats,
+cudaError_t launch_radii(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, CallStat* stats,
                          float* tok_shift, cudaStream_t st) {
   if (n_calls <= 0) return cudaSuccess;
-  if (!G.center_keys && A.nrm) {     // the norms were recorded when the rows were written
-    radii_norms_kernel<<<n_calls, 256, 0, st>>>(G, A, calls, stats);
-    return cudaGetLastError();
+  if (!G.center_keys) {              // the norms were recorded when the rows were written
+    const PdlConfig pc(dim3(n_calls), 256, 0, st);
+    return cudaLaunchKernelEx(&pc.cfg, radii_norms_kernel, G, A, calls, stats);
   }
-  cudaError_t e = cudaMemsetAsync(stats, 0, sizeof(CallStat) * (size_t)n_calls, st);
+  float* mean = tok_shift + (size_t)n_calls * G.t;
+  const PdlConfig pm(dim3(n_calls), 128, 0, st);
+  const cudaError_t e = cudaLaunchKernelEx(&pm.cfg, G.is_bf16 ? mean_kernel<true> : mean_kernel<false>, G, A, calls, mean, stats);
   if (e != cudaSuccess) return e;
-  float* mean = nullptr;
-  if (G.center_keys) {
-    mean = tok_shift + (size_t)n_calls * G.t;
-    if (G.is_bf16) mean_kernel<true><<<n_calls, 128, 0, st>>>(G, A, calls, mean);
-    else mean_kernel<false><<<n_calls, 128, 0, st>>>(G, A, calls, mean);
-  }
-  dim3 grid(n_calls, (G.t + 63) / 64);
-  if (G.is_bf16) radii_kernel<true><<<grid, 256, 0, st>>>(G, A, calls, stats, mean, tok_shift);
-  else radii_kernel<false><<<grid, 256, 0, st>>>(G, A, calls, stats, mean, tok_shift);
-  return cudaGetLastError();
+  const PdlConfig pr(dim3(n_calls, (G.t + 63) / 64), 256, 0, st);
+  return cudaLaunchKernelEx(&pr.cfg, G.is_bf16 ? radii_kernel<true> : radii_kernel<false>, G, A, calls, stats, mean, tok_shift);
 }
 
 cudaError_t launch_seg_update(const Arena& A, const SegUpdate* ups, int n, cudaStream_t st) {

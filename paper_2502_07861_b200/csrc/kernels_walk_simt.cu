@@ -47,7 +47,7 @@ __device__ inline void load_panel(float* __restrict__ dst, const void* __restric
 
 template <bool kBf16, int D>
 __global__ void __launch_bounds__(kThreads, 1)
-walk_simt_kernel(Geom G, Arena A, const CallDesc* __restrict__ calls, int level,
+walk_simt_kernel(Geom G, Arena A, const CallSet calls, int level,
                  const CallStat* __restrict__ stats, const float* __restrict__ tok_shift,
                  int8_t* __restrict__ eta_out, int8_t* __restrict__ dbg_eta, float* __restrict__ dbg_S,
                  float* __restrict__ dbg_p, unsigned long long* __restrict__ fail_count) {
@@ -63,8 +63,9 @@ walk_simt_kernel(Geom G, Arena A, const CallDesc* __restrict__ calls, int level,
   float* thr_s = eta_s + G.t;                      // [t]
   float* shift_s = thr_s + G.t;                    // [t]
 
+  grid_wait_and_release();
   const int call = blockIdx.x;
-  const CallDesc C = calls[call];
+  const CallDesc C = call_of(calls, G, call);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int t = G.t;
   const int head = C.stream % G.H;
@@ -193,15 +194,15 @@ walk_simt_kernel(Geom G, Arena A, const CallDesc* __restrict__ calls, int level,
 }
 
 template <bool kBf16, int D>
-cudaError_t launch_one(const Geom& G, const Arena& A, const CallDesc* calls, int n_calls, int level,
+cudaError_t launch_one(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, int level,
                        const CallStat* stats, const float* tok_shift, int8_t* eta, int8_t* dbg_eta, float* dbg_S,
                        float* dbg_p, unsigned long long* fail_count, cudaStream_t st) {
   const size_t smem = SimtSmem<D>::bytes(G.t);
   auto kern = walk_simt_kernel<kBf16, D>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  kern<<<n_calls, kThreads, smem, st>>>(G, A, calls, level, stats, tok_shift, eta, dbg_eta, dbg_S, dbg_p, fail_count);
-  return cudaGetLastError();
+  const PdlConfig pc(dim3(n_calls), kThreads, smem, st);
+  return cudaLaunchKernelEx(&pc.cfg, kern, G, A, calls, level, stats, tok_shift, eta, dbg_eta, dbg_S, dbg_p, fail_count);
 }
 
 }  // namespace
@@ -210,7 +211,7 @@ int walk_simt_supported(int d) { return d == 64 || d == 128; }
 
 size_t walk_simt_smem_bytes(int d, int t) { return d == 64 ? SimtSmem<64>::bytes(t) : SimtSmem<128>::bytes(t); }
 
-cudaError_t launch_walk_simt(const Geom& G, const Arena& A, const CallDesc* calls, int n_calls, int level,
+cudaError_t launch_walk_simt(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, int level,
                              const CallStat* stats, const float* tok_shift, int8_t* eta, int8_t* dbg_eta,
                              float* dbg_S, float* dbg_p, unsigned long long* fail_count, cudaStream_t st) {
   if (n_calls <= 0) return cudaSuccess;

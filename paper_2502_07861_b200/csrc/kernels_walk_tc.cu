@@ -314,7 +314,7 @@ __device__ inline void select_and_compact(const Geom& G, const Arena& A, const C
 
 template <bool kCenter>
 __global__ void __launch_bounds__(kThreads, 1)
-walk_tc_kernel(Geom G, const CallDesc* __restrict__ calls, int level, const CallStat* __restrict__ stats,
+walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restrict__ stats,
                const float* __restrict__ tok_shift, int8_t* __restrict__ eta_out, int8_t* __restrict__ dbg_eta,
                float* __restrict__ dbg_S, float* __restrict__ dbg_p, unsigned long long* __restrict__ fail_count,
                int* __restrict__ status, const float2* __restrict__ row_norms, const Arena A,
@@ -339,7 +339,7 @@ walk_tc_kernel(Geom G, const CallDesc* __restrict__ calls, int level, const Call
   int* abort_flag = reinterpret_cast<int*>(tmem_ptr_s + 1);
 
   const int call = blockIdx.x;
-  const CallDesc C = calls[call];
+  const CallDesc C = call_of(calls, G, call);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
   if (tid == 0) {
@@ -355,6 +355,14 @@ walk_tc_kernel(Geom G, const CallDesc* __restrict__ calls, int level, const Call
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_ptr_s)), "r"(kTmemCols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  // Everything above touches only this CTA's own state, and so do the coins: all of it overlaps the end of the previous
+  // launch (programmatic serialization; the wait comes before the first row or norm is read).
+  {
+    const int head = C.stream % G.H, layer = (C.stream / G.H) % G.L, seq = C.stream / (G.H * G.L);
+    for (int i = tid; i < t; i += kThreads)
+      thr_s[i] = G.c * (1.0f - 2.0f * walk_uniform(G.seed + (uint64_t)seq, layer, head, C.ordinal, level, i));
+  }
+  grid_wait_and_release();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -492,10 +500,6 @@ walk_tc_kernel(Geom G, const CallDesc* __restrict__ calls, int level, const Call
 
     constexpr int kEpiThreads = 32 * kEpiWarps;
     {
-      // all coins of the call up front (the first tile is still on its way), off the walk's critical path
-      const int head = C.stream % G.H, layer = (C.stream / G.H) % G.L, seq = C.stream / (G.H * G.L);
-      for (int i = tid; i < t; i += kEpiThreads)
-        thr_s[i] = cw * (1.0f - 2.0f * walk_uniform(G.seed + (uint64_t)seq, layer, head, C.ordinal, level, i));
       // r_key^2, r_value^2 of the call (inputs of Algorithm 2) = maxima of the stored row norms,
       // unless a separate kernel has put them (key centering changes them) or they are fixed
       if (row_norms) {
@@ -708,7 +712,7 @@ cudaError_t walk_tc_prepare(const Geom& G, const Arena& A, int64_t total_rows, v
 
 void walk_tc_release(void* tmaps) { delete static_cast<TensorMaps*>(tmaps); }
 
-cudaError_t launch_walk_tc(const Geom& G, const Arena& A, const CallDesc* calls, int n_calls, int level,
+cudaError_t launch_walk_tc(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, int level,
                            const CallStat* stats, const float* tok_shift, int8_t* eta, int8_t* dbg_eta,
                            float* dbg_S, float* dbg_p, unsigned long long* fail_count, int* status,
                            const void* tmaps, const void* fuse_compaction, cudaStream_t st) {
@@ -718,13 +722,9 @@ cudaError_t launch_walk_tc(const Geom& G, const Arena& A, const CallDesc* calls,
   const size_t smem = tc_smem_bytes(G.t);
   Arena Af = A;                       // K == nullptr: leave selection and compaction to the separate kernel
   if (!fuse_compaction) Af.K = nullptr;
-  if (G.center_keys)
-    walk_tc_kernel<true><<<n_calls, kThreads, smem, st>>>(G, calls, level, stats, tok_shift, eta, dbg_eta, dbg_S, dbg_p,
-                                                          fail_count, status, G.center_keys ? nullptr : A.nrm, Af, tm->k, tm->v);
-  else
-    walk_tc_kernel<false><<<n_calls, kThreads, smem, st>>>(G, calls, level, stats, tok_shift, eta, dbg_eta, dbg_S, dbg_p,
-                                                           fail_count, status, G.center_keys ? nullptr : A.nrm, Af, tm->k, tm->v);
-  return cudaGetLastError();
+  const PdlConfig pc(dim3(n_calls), kThreads, smem, st);
+  return cudaLaunchKernelEx(&pc.cfg, G.center_keys ? walk_tc_kernel<true> : walk_tc_kernel<false>, G, calls, level, stats, tok_shift,
+                            eta, dbg_eta, dbg_S, dbg_p, fail_count, status, G.center_keys ? nullptr : A.nrm, Af, tm->k, tm->v);
 }
 
 }  // namespace bkv

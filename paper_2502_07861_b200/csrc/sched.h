@@ -12,6 +12,8 @@
 #pragma once
 
 #include <algorithm>
+#include <climits>
+#include <cstdint>
 #include <utility>
 #include <vector>
 
@@ -26,6 +28,12 @@ struct StreamState {
   int32_t lvl_len[kMaxLevels + 1] = {};  // rows held at levels 1..T
   int32_t lvl_base[kMaxLevels + 1] = {}; // base (0 or t) of the half held at levels 1..T-1
   int64_t calls_done[kMaxLevels + 1] = {};  // calls run per level (= next call ordinal)
+  bool same_as(const StreamState& o) const {
+    bool eq = appended == o.appended && pending == o.pending && start0 == o.start0 && len0 == o.len0;
+    for (int l = 0; l <= kMaxLevels; ++l)
+      eq = eq && lvl_len[l] == o.lvl_len[l] && lvl_base[l] == o.lvl_base[l] && calls_done[l] == o.calls_done[l];
+    return eq;
+  }
 };
 
 struct Layout {
@@ -138,6 +146,76 @@ inline bool plan_batch(const Layout& Lo, StreamState* st, const std::vector<std:
     P.segs.push_back(SegUpdate{sbase + T, 0, S.lvl_len[T], 0});
   }
   return true;
+}
+
+// The same for lockstep streams -- all of them in state S, each running its nb ready blocks: one CallSet per level in
+// place of lists, the state after the batch (S is updated), the move of the remainder (E) and the segments of a stream.
+// The caller keeps n_streams * nb within the level-0 calls that the pools are sized for.
+inline void plan_lockstep(const Layout& Lo, StreamState& S, int nb, int layer, int first, std::vector<CallSet>& sets,
+                          std::vector<int>& n_calls, BatchEnd& E, Seg* seg) {
+  const int t = Lo.t, T = Lo.T, half = t / 2;
+  sets.assign(T, CallSet{});
+  n_calls.assign(T, 0);
+  int n = nb, src_rel = Lo.region_off[0] + S.start0, src_held = 0, src_pairs = 0;
+  int64_t src_pool = -1;
+  S.start0 += nb * t;
+  S.len0 -= nb * t;
+  for (int l = 0; l < T && n > 0; ++l) {
+    CallSet& C = sets[l];
+    n_calls[l] = n;
+    C.layer = layer; C.first = first; C.per_stream = n; C.ordinal0 = (int32_t)S.calls_done[l];
+    C.src_rel = src_rel; C.src_held = src_held; C.src_pool = src_pool; C.src_pairs = src_pairs;
+    S.calls_done[l] += n;
+    if (l + 1 == T) {
+      C.top = 1;
+      C.dst_rel = Lo.region_off[T] + S.lvl_len[T];
+      S.lvl_len[T] += n * half;
+      break;
+    }
+    const int h = S.lvl_len[l + 1] ? 1 : 0;       // a half is already waiting in C^{l+1}
+    const int slots = h + n, pairs = slots / 2, left = slots % 2;
+    const int pers = Lo.region_off[l + 1], old_base = S.lvl_base[l + 1];
+    const int new_base = h ? (old_base ? 0 : t) : 0;
+    C.dst_held = h;
+    C.dst_held_rel = pers + old_base + half;
+    C.dst_left_rel = pers + new_base;
+    C.dst_pairs_all = pairs;
+    C.dst_pairs = pairs - (h && pairs > 0 ? 1 : 0);
+    C.dst_pool = Lo.pool_row[l & 1];
+    src_rel = pers + old_base; src_held = h; src_pool = C.dst_pool; src_pairs = C.dst_pairs;
+    n = pairs;
+    S.lvl_len[l + 1] = left ? half : 0;
+    S.lvl_base[l + 1] = left ? new_base : 0;
+  }
+  E = BatchEnd{layer, first, 0, 0};
+  if (S.len0 == 0) {
+    S.start0 = 0;
+  } else if (S.start0 >= S.len0) {
+    E.move_src = S.start0;
+    E.move_rows = S.len0;
+    S.start0 = 0;
+  }
+  seg[0] = Seg{S.start0, S.len0};
+  for (int l = 1; l < T; ++l) seg[l] = Seg{S.lvl_base[l], S.lvl_len[l]};
+  seg[T] = Seg{0, S.lvl_len[T]};
+}
+
+// Streams per batch of n lockstep streams with nb blocks each, at most `most` (>= 1) per batch: the split with the fewest
+// waves of `slots` CTAs over all launches (a launch of 6.9 waves takes as long as one of 7).
+inline int lockstep_batch(int n, int nb, int T, int most, int slots) {
+  auto waves = [&](int streams) {
+    int64_t w = 0, calls = (int64_t)streams * nb;
+    for (int l = 0; l < T && calls > 0; ++l, calls = (int64_t)streams * (nb >> l)) w += (calls + slots - 1) / slots;
+    return w;
+  };
+  if (n <= most) return n;
+  int best = most;
+  int64_t best_w = INT64_MAX;
+  for (int b = most; b >= std::max(1, most / 2); --b) {
+    const int64_t w = (int64_t)(n / b) * waves(b) + (n % b ? waves(n % b) : 0);
+    if (w < best_w) { best_w = w; best = b; }
+  }
+  return best;
 }
 
 }  // namespace bkv

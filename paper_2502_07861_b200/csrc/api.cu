@@ -386,7 +386,7 @@ int balancekv_create(const balancekv_config* cfg, balancekv_ctx** out) {
     if (decode_mma_prepare(G, c->A, &c->decode_maps) != cudaSuccess) return fail(BALANCEKV_E_CUDA);
   }
   const bool tc_ok = walk_tc_supported(G) && rows_ok;
-  if (f.gram_path == 2 && !tc_ok) return fail(BALANCEKV_E_INVAL);
+  if (f.gram_path == 2 && !(tc_ok && f.head_dim == 128 && t % 128 == 0)) return fail(BALANCEKV_E_INVAL);   // as documented
   c->use_tc = T > 0 && tc_ok && f.gram_path != 1;
   if (c->use_tc && walk_tc_prepare(G, c->A, c->total_rows, &c->tmaps) != cudaSuccess) return fail(BALANCEKV_E_CUDA);
   if (T > 0 && !c->use_tc) {
@@ -563,7 +563,7 @@ static int run_calls(balancekv_ctx* c, const CallSet& calls, int n, int l, cudaS
   if (need_radii) {
     ProfScope ps(c, 1, st);
     BKV_CUDA(launch_radii(G, c->A, calls, n, c->d_stats, c->d_tokshift, st));
-    c->kernels_launched += 1 + (G.center_keys ? 1 : 0);
+    c->kernels_launched++;
   }
   if (c->use_tc) {
     ProfScope ps(c, 2, st);

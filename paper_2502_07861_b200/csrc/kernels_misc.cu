@@ -196,83 +196,85 @@ __global__ void seg_update_kernel(Arena A, const SegUpdate* __restrict__ ups, in
   if (i < n) A.seg[ups[i].index] = Seg{ups[i].start, ups[i].len};
 }
 
-// Column means of the call's keys, one CTA per call, thread e owns column e
-// (fixed summation order, so the result is reproducible).
+// Key centering: one CTA per call.  The mean of the call's keys (fixed summation order, so the result is reproducible),
+// the per-token shift a_j = <k_j, mean> - ||mean||^2/2, with which
+//   <k_i - mean, k_j - mean> = <k_i, k_j> - a_i - a_j   and   ||k_j - mean||^2 = ||k_j||^2 - 2 a_j,
+// and the radii: r_key^2 = max_j ||k_j - mean||^2, r_value^2 = max_j ||v_j||^2 from the stored norms.  The keys are read
+// twice, the second time from L2 or L1; the values not at all.  A column per thread over all t rows, then a second kernel
+// over K and V, took 8.4 + 7.1 us for 160 calls of 192 x 64.
+constexpr int kCenterThreads = 512;
 template <bool kBf16>
-__global__ void mean_kernel(Geom G, Arena A, const CallSet calls, float* __restrict__ mean, CallStat* __restrict__ stats) {
-  grid_wait_and_release();
-  if (threadIdx.x == 0) stats[blockIdx.x] = CallStat{0.f, 0.f};     // radii_kernel takes maxima into it
-  const CallDesc C = call_of(calls, G, blockIdx.x);
-  const int e = threadIdx.x;
-  if (e >= G.d) return;
-  float s = 0.f;
-  for (int j = 0; j < G.t; ++j) {
-    const size_t off = (size_t)(C.src_row + j) * G.d + e;
-    s += kBf16 ? __bfloat162float(static_cast<const __nv_bfloat16*>(A.K)[off]) : static_cast<const float*>(A.K)[off];
-  }
-  mean[(size_t)blockIdx.x * G.d + e] = s / (float)G.t;
-}
-
-// r_key^2 = max_j ||k_j - mean||^2, r_value^2 = max_j ||v_j||^2 over the call's tokens,
-// and the per-token shift a_j = <k_j, mean> - ||mean||^2/2, with which
-// <k_i - mean, k_j - mean> = <k_i, k_j> - a_i - a_j.
-template <bool kBf16>
-__global__ void __launch_bounds__(256)
-radii_kernel(Geom G, Arena A, const CallSet calls, CallStat* __restrict__ stats,
-             const float* __restrict__ mean, float* __restrict__ tok_shift) {
+__global__ void __launch_bounds__(kCenterThreads)
+center_kernel(Geom G, Arena A, const CallSet calls, CallStat* __restrict__ stats, float* __restrict__ tok_shift) {
+  constexpr int kEl = kBf16 ? 8 : 4;                 // elements of a 16-byte piece
+  __shared__ float part[kCenterThreads / 32][32][kEl + 1];   // per warp: sums of its lanes' columns
+  __shared__ float mean_s[256];
+  __shared__ float red[2][kCenterThreads / 32];
   grid_wait_and_release();
   const CallDesc C = call_of(calls, G, blockIdx.x);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int esz = kBf16 ? 2 : 4;
-  float mk = 0.f, mv = 0.f;
-  const float* mu = mean ? mean + (size_t)blockIdx.x * G.d : nullptr;
-  float mu2 = 0.f;
-  if (mu) {
-    for (int e = lane; e < G.d; e += 32) mu2 += mu[e] * mu[e];
-    mu2 = warp_sum(mu2);
-  }
-  // d / 8 lanes share a row (8 elements each): with d = 128 a warp works on two rows at a time
-  const int lpr = G.d / 8 < 32 ? G.d / 8 : 32;     // lanes per row
-  const int rpw = 32 / lpr;                        // rows per warp step
-  const int sub = lane / lpr, l0 = lane % lpr;
-  const int row_end = min(G.t, (int)(blockIdx.y + 1) * 64);
-  for (int r = blockIdx.y * 64 + warp * rpw + sub; r - sub < row_end; r += 8 * rpw) {
-    const bool live = r < row_end;
-    const char* krow = static_cast<const char*>(A.K) + (size_t)(C.src_row + (live ? r : 0)) * G.d * esz;
-    const char* vrow = static_cast<const char*>(A.V) + (size_t)(C.src_row + (live ? r : 0)) * G.d * esz;
-    float sk = 0.f, sv = 0.f, sm = 0.f;
-    for (int e = l0 * 8; e < G.d; e += lpr * 8) {
-      float a[8], b[8];
-      load8<kBf16>(krow, e, a);
-      load8<kBf16>(vrow, e, b);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int pieces = G.d / kEl;                      // 8, 16 or 32 lanes share a row
+  const int pc = tid % pieces, rg = tid / pieces, groups = kCenterThreads / pieces;
+  const uint4* K = reinterpret_cast<const uint4*>(A.K) + (size_t)C.src_row * pieces + pc;
+  auto piece = [&](int row, float (&x)[kEl]) {
+    const uint4 w = K[(size_t)row * pieces];
+    if constexpr (kBf16) {
+      x[0] = bf16_lo(w.x); x[1] = bf16_hi(w.x); x[2] = bf16_lo(w.y); x[3] = bf16_hi(w.y);
+      x[4] = bf16_lo(w.z); x[5] = bf16_hi(w.z); x[6] = bf16_lo(w.w); x[7] = bf16_hi(w.w);
+    } else {
+      x[0] = __uint_as_float(w.x); x[1] = __uint_as_float(w.y); x[2] = __uint_as_float(w.z); x[3] = __uint_as_float(w.w);
+    }
+  };
+  float sum[kEl];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        sk = fmaf(a[i], a[i], sk);
-        sv = fmaf(b[i], b[i], sv);
-        if (mu) sm = fmaf(a[i], mu[e + i], sm);
-      }
+  for (int e = 0; e < kEl; ++e) sum[e] = 0.f;
+#pragma unroll 4
+  for (int r = rg; r < G.t; r += groups) {
+    float x[kEl];
+    piece(r, x);
+#pragma unroll
+    for (int e = 0; e < kEl; ++e) sum[e] += x[e];
+  }
+#pragma unroll
+  for (int e = 0; e < kEl; ++e) part[warp][lane][e] = sum[e];
+  __syncthreads();
+  if (tid < G.d) {
+    const int p = tid / kEl, e = tid % kEl;
+    float s = 0.f;
+    for (int w = 0; w < kCenterThreads / 32; ++w)
+      for (int l = p; l < 32; l += pieces) s += part[w][l][e];
+    mean_s[tid] = s / (float)G.t;
+  }
+  __syncthreads();
+  float mu[kEl], mu2 = 0.f;
+#pragma unroll
+  for (int e = 0; e < kEl; ++e) { mu[e] = mean_s[pc * kEl + e]; mu2 = fmaf(mu[e], mu[e], mu2); }
+  for (int o = pieces / 2; o > 0; o >>= 1) mu2 += __shfl_xor_sync(0xffffffffu, mu2, o);
+  float mk = 0.f, mv = 0.f;
+  for (int r0 = 0; r0 < G.t; r0 += groups) {          // whole warps take part in the shuffles
+    const int r = r0 + rg;
+    float dot = 0.f;
+    if (r < G.t) {
+      float x[kEl];
+      piece(r, x);
+#pragma unroll
+      for (int e = 0; e < kEl; ++e) dot = fmaf(x[e], mu[e], dot);
     }
-    for (int o = lpr / 2; o > 0; o >>= 1) {
-      sk += __shfl_xor_sync(0xffffffffu, sk, o);
-      sv += __shfl_xor_sync(0xffffffffu, sv, o);
-      if (mu) sm += __shfl_xor_sync(0xffffffffu, sm, o);
+    for (int o = pieces / 2; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+    if (r < G.t && pc == 0) {
+      const float shift = dot - 0.5f * mu2;
+      const float2 n = A.nrm[C.src_row + r];
+      tok_shift[(size_t)blockIdx.x * G.t + r] = shift;
+      mk = fmaxf(mk, fmaxf(n.x - 2.f * shift, 0.f));
+      mv = fmaxf(mv, n.y);
     }
-    if (mu) {
-      const float shift = sm - 0.5f * mu2;
-      sk = fmaxf(sk - 2.f * shift, 0.f);
-      if (live && l0 == 0) tok_shift[(size_t)blockIdx.x * G.t + r] = shift;
-    }
-    if (live) { mk = fmaxf(mk, sk); mv = fmaxf(mv, sv); }
   }
   mk = warp_max(mk); mv = warp_max(mv);
-  __shared__ float smk[8], smv[8];
-  if (lane == 0) { smk[warp] = mk; smv[warp] = mv; }
+  if (lane == 0) { red[0][warp] = mk; red[1][warp] = mv; }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < 8; ++w) { mk = fmaxf(mk, smk[w]); mv = fmaxf(mv, smv[w]); }
-    // non-negative floats order like their bit patterns
-    atomicMax(reinterpret_cast<int*>(&stats[blockIdx.x].rk2), __float_as_int(mk));
-    atomicMax(reinterpret_cast<int*>(&stats[blockIdx.x].rv2), __float_as_int(mv));
+  if (tid == 0) {
+    for (int w = 1; w < kCenterThreads / 32; ++w) { mk = fmaxf(mk, red[0][w]); mv = fmaxf(mv, red[1][w]); }
+    stats[blockIdx.x] = CallStat{mk, mv};
   }
 }
 
@@ -347,8 +349,7 @@ cudaError_t launch_reset(Seg* seg, size_t n_seg, float* scratch, size_t n, float
   return cudaLaunchKernelEx(&pc.cfg, reset_kernel, seg, n_seg, scratch, n, scratch2, n2, status, status_host);
 }
 
-// stats must hold n_calls entries; tok_shift n_calls * t floats (+ n_calls * d floats of
-// mean scratch behind it) when key centering is on, else it may be null.
+// stats must hold n_calls entries; tok_shift n_calls * t floats when key centering is on, else it may be null.
 cudaError_t launch_radii(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, CallStat* stats,
                          float* tok_shift, cudaStream_t st) {
   if (n_calls <= 0) return cudaSuccess;
@@ -356,12 +357,8 @@ cudaError_t launch_radii(const Geom& G, const Arena& A, const CallSet& calls, in
     const PdlConfig pc(dim3(n_calls), 256, 0, st);
     return cudaLaunchKernelEx(&pc.cfg, radii_norms_kernel, G, A, calls, stats);
   }
-  float* mean = tok_shift + (size_t)n_calls * G.t;
-  const PdlConfig pm(dim3(n_calls), 128, 0, st);
-  const cudaError_t e = cudaLaunchKernelEx(&pm.cfg, G.is_bf16 ? mean_kernel<true> : mean_kernel<false>, G, A, calls, mean, stats);
-  if (e != cudaSuccess) return e;
-  const PdlConfig pr(dim3(n_calls, (G.t + 63) / 64), 256, 0, st);
-  return cudaLaunchKernelEx(&pr.cfg, G.is_bf16 ? radii_kernel<true> : radii_kernel<false>, G, A, calls, stats, mean, tok_shift);
+  const PdlConfig pc(dim3(n_calls), kCenterThreads, 0, st);
+  return cudaLaunchKernelEx(&pc.cfg, G.is_bf16 ? center_kernel<true> : center_kernel<false>, G, A, calls, stats, tok_shift);
 }
 
 cudaError_t launch_seg_update(const Arena& A, const SegUpdate* ups, int n, cudaStream_t st) {

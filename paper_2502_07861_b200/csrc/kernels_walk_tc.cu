@@ -1,6 +1,6 @@
 // SoftmaxBalance (Algorithm 2) with the Gram tiles on the 5th-generation tensor cores.
 //
-// One CTA per call.  The call's t x t kernel matrix
+// One CTA per call; d = 128 or 64, t >= 128 a multiple of 64.  The call's t x t kernel matrix
 //   Ghat_ij = exp((<k_i,k_j> - r_key^2)/sqrt d) <v_i,v_j> / r_value^2      (proof of Theorem 3.2)
 // is visited in 128 x 128 tiles of its lower triangle, row panel by row panel.  For a tile,
 // TMA brings the bf16 rows of K and V into 128B-swizzled shared memory, tcgen05.mma
@@ -19,7 +19,7 @@
 // TMEM is double buffered (2 x 256 columns); an epilogue hands its buffer back as soon as the
 // accumulator values are in registers.  Each of the two products of a tile has its own issuing
 // thread and its own barriers, so that one product's waits and commits overlap the other's
-// MMAs.  Operands live in three 64 KB slots (K tile + V tile) that rotate roles: panel r keeps
+// MMAs.  Operands live in three slots (K tile + V tile; 64 KB at d = 128) that rotate roles: panel r keeps
 // its rows in slot r % 3 and streams its column tiles through the other two, and the rows of
 // panel r + 1 are fetched into the slot that panel r's column tiles leave first, so the next
 // panel's first products are already in TMEM when the walk of the diagonal tile ends.
@@ -43,7 +43,8 @@ constexpr int kEpiWarps = 4 * kEpiGroups;
 constexpr int kTmaWarp = kEpiWarps, kMmaWarp = kEpiWarps + 1, kMmaWarpV = kEpiWarps + 2;   // TMA, MMA (K K^T), MMA (V V^T)
 constexpr int kThreads = 32 * (kEpiWarps + 3);
 constexpr uint32_t kHalfBytes = 16384;     // [128 rows][64 bf16] = one swizzle-atom column of a tile
-constexpr uint32_t kTileBytes = 32768;     // [128 rows][128 bf16]
+template <int D>
+constexpr uint32_t kTileBytesOf = (D / 64) * kHalfBytes;   // a K or V tile: [128 rows][d bf16]
 constexpr uint32_t kTmemCols = 512;
 constexpr long long kWaitCycles = 100000000LL;   // about 50 ms; every wait here is on this CTA's own copies and MMAs
 
@@ -207,9 +208,10 @@ __device__ inline float2 poly_exp2x2(float2 x) {
 // polynomial path, the others the special-function unit.
 constexpr int kPolyOf8 = 1;
 
+template <int D>
 struct Smem {
   // three operand slots first (1024-byte aligned for the 128B swizzle); a slot holds a K tile then a V tile
-  static constexpr uint32_t kSlotBytes = 2 * kTileBytes;
+  static constexpr uint32_t kSlotBytes = 2 * kTileBytesOf<D>;
   static constexpr uint32_t kTilesEnd = 3 * kSlotBytes;
 };
 constexpr int kMaxSweeps = kTile + 2;
@@ -220,6 +222,7 @@ constexpr int kMaxSweeps = kTile + 2;
 // call's destination rows with their positions and norms.  Runs at the tail of the call's CTA, whose
 // operand slots are idle by then: `scratch` holds the kept positions.  The rows were read by this
 // CTA microseconds ago and come from L2.  All kThreads threads take part.
+template <int D>
 __device__ inline void select_and_compact(const Geom& G, const Arena& A, const CallDesc& C, const int8_t* eta8, int* scratch) {
   const int t = G.t, half = t / 2;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -279,30 +282,31 @@ __device__ inline void select_and_compact(const Geom& G, const Arena& A, const C
     for (int i = 0; i < ipt; ++i)
       if (mask & (1u << i)) kept_pos[pos++] = j0 + i;
   __syncthreads();
-  // copy: a survivor row of K and of V is 2 x 16 chunks of 16 bytes; eight loads in flight per thread.
+  constexpr int kCh = D / 8;
+  // copy: a survivor row of K and of V is 2 x d / 8 chunks of 16 bytes; eight loads in flight per thread.
   // (All CTAs of a wave reach this point together, so the copy runs at the chip's memory bandwidth
   // whichever engine moves the bytes; the bulk-copy engine was measured and is no faster.)
-  const uint4* Ks = reinterpret_cast<const uint4*>(A.K) + (size_t)C.src_row * 16;
-  const uint4* Vs = reinterpret_cast<const uint4*>(A.V) + (size_t)C.src_row * 16;
-  uint4* Kd = reinterpret_cast<uint4*>(A.K) + (size_t)C.dst_row * 16;
-  uint4* Vd = reinterpret_cast<uint4*>(A.V) + (size_t)C.dst_row * 16;
-  const int items = half * 32;
+  const uint4* Ks = reinterpret_cast<const uint4*>(A.K) + (size_t)C.src_row * kCh;
+  const uint4* Vs = reinterpret_cast<const uint4*>(A.V) + (size_t)C.src_row * kCh;
+  uint4* Kd = reinterpret_cast<uint4*>(A.K) + (size_t)C.dst_row * kCh;
+  uint4* Vd = reinterpret_cast<uint4*>(A.V) + (size_t)C.dst_row * kCh;
+  const int items = half * 2 * kCh;
   for (int i0 = tid; i0 < items; i0 += 8 * kThreads) {
     uint4 v[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
       const int i = i0 + u * kThreads;
       if (i < items) {
-        const int o = i >> 5, c = i & 31;
-        v[u] = (c < 16 ? Ks : Vs)[(size_t)kept_pos[o] * 16 + (c & 15)];
+        const int o = i / (2 * kCh), c = i % (2 * kCh);
+        v[u] = (c < kCh ? Ks : Vs)[(size_t)kept_pos[o] * kCh + c % kCh];
       }
     }
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
       const int i = i0 + u * kThreads;
       if (i < items) {
-        const int o = i >> 5, c = i & 31;
-        (c < 16 ? Kd : Vd)[(size_t)o * 16 + (c & 15)] = v[u];
+        const int o = i / (2 * kCh), c = i % (2 * kCh);
+        (c < kCh ? Kd : Vd)[(size_t)o * kCh + c % kCh] = v[u];
       }
     }
   }
@@ -312,7 +316,7 @@ __device__ inline void select_and_compact(const Geom& G, const Arena& A, const C
   }
 }
 
-template <bool kCenter>
+template <int D, bool kCenter>
 __global__ void __launch_bounds__(kThreads, 1)
 walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restrict__ stats,
                const float* __restrict__ tok_shift, int8_t* __restrict__ eta_out, int8_t* __restrict__ dbg_eta,
@@ -321,13 +325,17 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
                const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  const int t = G.t, P = t / kTile;
-  float* etas = reinterpret_cast<float*>(sm + Smem::kTilesEnd);          // [t] signs scaled by 1/r_value^2 (0 = undecided)
-  float* xs = etas + t;                                                   // [3][128] partial correlations of column quarters 1..3
+  constexpr uint32_t kTileBytes = kTileBytesOf<D>, kSlotBytes = Smem<D>::kSlotBytes;
+  constexpr int kBoxes = D / 64;                                          // boxes of 64 dims per tile
+  // t is a multiple of 64: the last panel may hold 64 tokens only.  Its tile then covers 64 rows that are not the
+  // call's; what is computed for them goes nowhere.
+  const int t = G.t, P = (t + kTile - 1) / kTile, tp = P * kTile;
+  float* etas = reinterpret_cast<float*>(sm + Smem<D>::kTilesEnd);       // [tp] signs scaled by 1/r_value^2 (0 = undecided)
+  float* xs = etas + tp;                                                   // [3][128] partial correlations of column quarters 1..3
   float* xb = xs + (kEpiGroups - 1) * kTile;                              // [3][128] ... and of their sums of |Ghat|
-  float* thr_s = xb + (kEpiGroups - 1) * kTile;                           // [t] decision thresholds c (1 - 2 u_j)
-  int8_t* eta8 = reinterpret_cast<int8_t*>(thr_s + t);                    // [t] signs
-  uint64_t* bars = reinterpret_cast<uint64_t*>(eta8 + t);                 // t is a multiple of 128
+  float* thr_s = xb + (kEpiGroups - 1) * kTile;                           // [tp] decision thresholds c (1 - 2 u_j)
+  int8_t* eta8 = reinterpret_cast<int8_t*>(thr_s + tp);                   // [tp] signs
+  uint64_t* bars = reinterpret_cast<uint64_t*>(eta8 + tp);
   // x = 0: the K K^T product, x = 1: the V V^T product
   // An operand tile travels as two boxes of 64 dims (h = 0, 1); a box is refilled as soon as the
   // four MMAs that read it are done, which lengthens the prefetch distance of the column ring.
@@ -350,7 +358,7 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
-  for (int i = tid; i < t; i += kThreads) etas[i] = 0.f;
+  for (int i = tid; i < tp; i += kThreads) etas[i] = 0.f;
   if (warp == kMmaWarp) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_ptr_s)), "r"(kTmemCols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -385,10 +393,10 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
         const uint32_t ph = (par >> slot) & 1u;
         used |= 1u << slot;
         if (again) par ^= 1u << slot;
-        unsigned char* st = sm + (uint32_t)slot * Smem::kSlotBytes;
+        unsigned char* st = sm + (uint32_t)slot * kSlotBytes;
         const int y = (int)(C.src_row + (int64_t)tile_row * kTile);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
+        for (int h = 0; h < kBoxes; ++h) {
           uint64_t* fk = full + 2 * slot + h;
           uint64_t* fv = full + 6 + 2 * slot + h;
           if (again && !wait_bar(empty + 2 * slot + h, ph, abort_flag)) return false;
@@ -415,11 +423,11 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
       uint32_t par = 0;                  // per slot: parity of the next wait on its full barrier
       bool ok = true;
       const uint32_t slot0 = umma_desc_lo(smem_u32(sm + (x ? kTileBytes : 0u)));
-      constexpr uint32_t kSlotDesc = Smem::kSlotBytes >> 4;
+      constexpr uint32_t kSlotDesc = kSlotBytes >> 4;
       for (int r = 0; r < P && ok; ++r) {
         const int rs = r % 3;
         if (!(ok = wait_bar(full + 6 * x + 2 * rs, (par >> rs) & 1u, abort_flag))) break;
-        if (!(ok = wait_bar(full + 6 * x + 2 * rs + 1, (par >> rs) & 1u, abort_flag))) break;
+        if (kBoxes == 2 && !(ok = wait_bar(full + 6 * x + 2 * rs + 1, (par >> rs) & 1u, abort_flag))) break;
         par ^= 1u << rs;
         const uint32_t arow = slot0 + (uint32_t)rs * kSlotDesc;
         for (int c = 0; c <= r; ++c, ++i) {
@@ -436,9 +444,11 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
           tc_fence_after();
           umma_tile_lo(d_tmem, arow, b);
           umma_commit(empty + 6 * x + 2 * slot);       // a column slot's box after its tile, the row slot's after the diagonal tile
-          if (c < r && !(ok = wait_bar(full + 6 * x + 2 * slot + 1, ph, abort_flag))) break;
-          umma_tile_hi(d_tmem, arow, b);
-          umma_commit(empty + 6 * x + 2 * slot + 1);
+          if constexpr (kBoxes == 2) {
+            if (c < r && !(ok = wait_bar(full + 6 * x + 2 * slot + 1, ph, abort_flag))) break;
+            umma_tile_hi(d_tmem, arow, b);
+            umma_commit(empty + 6 * x + 2 * slot + 1);
+          }
           umma_commit(xdone + buf);
         }
       }
@@ -532,6 +542,7 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
     // come after the vote and contain no waits, so no thread can be left waiting at them.
     for (int r = 0; r < P; ++r) {
       const int j = r * kTile + row;                      // this thread's token in the panel
+      const bool mine = j < t;
       float nb = -rk2 * scale;                            // exponent offset of this row
       if constexpr (kCenter) nb -= shift[j] * scale;
       float acc = 0.f;
@@ -623,7 +634,9 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
           bar_sync(1, kEpiThreads);                       // all partial sums of this sweep are written
           S = (part + xs[row]) + (xs[kTile + row] + xs[2 * kTile + row]);
           const bool now = S < thr;
-          if (sweep == 0) {
+          if (!mine) {
+            changed = false;
+          } else if (sweep == 0) {
             const float bound = ((absum + xb[row]) + (xb[kTile + row] + xb[2 * kTile + row])) * inv_rv2;
             const float slack = 1e-5f * (fabsf(S) + bound) + 1e-30f;
             changed = C.dbg_off >= 0 || !(fabsf(S - thr) > bound + slack) || !(fabsf(S) + bound + slack < cw);
@@ -631,11 +644,11 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
             changed = now != plus;
           }
           plus = now;
-          etas[j] = plus ? inv_rv2 : -inv_rv2;
+          etas[j] = mine ? plus ? inv_rv2 : -inv_rv2 : 0.f;
         }
         if (!bar_red_or(2, kEpiThreads, changed)) break;  // all signs of this sweep are written; any change?
       }
-      if (wg == 0) {
+      if (wg == 0 && mine) {
         eta8[j] = plus ? 1 : -1;
         if (fabsf(S) > cw) ++fails;                          // FAIL of Algorithm 2: counted; the decision is the clamped one
         if (C.dbg_off >= 0) {
@@ -659,14 +672,21 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
       eta_out[(size_t)call * t + i] = e;
       if (C.dbg_off >= 0) dbg_eta[C.dbg_off + i] = e;
     }
-    if (A.K) select_and_compact(G, A, C, eta8, reinterpret_cast<int*>(sm));
+    if (A.K) select_and_compact<D>(G, A, C, eta8, reinterpret_cast<int*>(sm));
   }
   if (warp == kMmaWarp) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
   }
 }
 
-size_t tc_smem_bytes(int t) { return 1024 + Smem::kTilesEnd + (size_t)t * 9 + 2 * (kEpiGroups - 1) * kTile * 4 + 512; }
+size_t tc_smem_bytes(int d, int t) {
+  const size_t tp = (t + kTile - 1) / kTile * kTile;
+  return 1024 + (d == 128 ? Smem<128>::kTilesEnd : Smem<64>::kTilesEnd) + tp * 9 + 2 * (kEpiGroups - 1) * kTile * 4 + 512;
+}
+auto kernel_for(int d, bool center) {
+  return d == 128 ? (center ? walk_tc_kernel<128, true> : walk_tc_kernel<128, false>)
+                  : (center ? walk_tc_kernel<64, true> : walk_tc_kernel<64, false>);
+}
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
@@ -674,11 +694,13 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
 
 }  // namespace
 
+// Calls of a single half panel (t = 64) stay on CUDA cores: the tensor cores would work on 64 rows of 128.
 bool walk_tc_supported(const Geom& G) {
-  return G.is_bf16 && G.d == 128 && G.t % kTile == 0 && tc_smem_bytes(G.t) <= (size_t)227 * 1024;
+  return G.is_bf16 && (G.d == 128 || G.d == 64) && G.t % 64 == 0 && G.t >= kTile &&
+         tc_smem_bytes(G.d, G.t) <= (size_t)227 * 1024;
 }
 
-// Encodes the two tensor maps (K and V arenas viewed as [total_rows, 128] bf16, boxes of
+// Encodes the two tensor maps (K and V arenas viewed as [total_rows, d] bf16, boxes of
 // 64 columns x 128 rows, 128-byte swizzle).
 cudaError_t walk_tc_prepare(const Geom& G, const Arena& A, int64_t total_rows, void** tmaps_out) {
   *tmaps_out = nullptr;
@@ -702,9 +724,8 @@ cudaError_t walk_tc_prepare(const Geom& G, const Arena& A, int64_t total_rows, v
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) { delete tm; return cudaErrorInvalidValue; }
   }
-  e = cudaFuncSetAttribute(walk_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem_bytes(G.t));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(walk_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem_bytes(G.t));
+  for (int i = 0; i < 2 && e == cudaSuccess; ++i)
+    e = cudaFuncSetAttribute(kernel_for(G.d, i != 0), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem_bytes(G.d, G.t));
   if (e != cudaSuccess) { delete tm; return e; }
   *tmaps_out = tm;
   return cudaSuccess;
@@ -719,11 +740,11 @@ cudaError_t launch_walk_tc(const Geom& G, const Arena& A, const CallSet& calls, 
   if (n_calls <= 0) return cudaSuccess;
   if (!tmaps) return cudaErrorInvalidValue;
   const TensorMaps* tm = static_cast<const TensorMaps*>(tmaps);
-  const size_t smem = tc_smem_bytes(G.t);
+  const size_t smem = tc_smem_bytes(G.d, G.t);
   Arena Af = A;                       // K == nullptr: leave selection and compaction to the separate kernel
   if (!fuse_compaction) Af.K = nullptr;
   const PdlConfig pc(dim3(n_calls), kThreads, smem, st);
-  return cudaLaunchKernelEx(&pc.cfg, G.center_keys ? walk_tc_kernel<true> : walk_tc_kernel<false>, G, calls, level, stats, tok_shift,
+  return cudaLaunchKernelEx(&pc.cfg, kernel_for(G.d, G.center_keys != 0), G, calls, level, stats, tok_shift,
                             eta, dbg_eta, dbg_S, dbg_p, fail_count, status, G.center_keys ? nullptr : A.nrm, Af, tm->k, tm->v);
 }
 

@@ -1,0 +1,34 @@
+"""SoftmaxBalance kernels at the block sizes where their tiling ends raggedly, against the oracle by the teacher-forced
+procedure of parity_util (signs, margins, kept sets, stored rows, running correlations).  Tolerances of S: those of the other
+parity tests (2e-4 on tensor cores, 5e-4 with key centering, 2e-5 on CUDA cores)."""
+import numpy as np
+import pytest
+
+from paper_2502_07861_b200 import synth
+from parity_util import Harness
+
+pytestmark = pytest.mark.gpu
+
+
+def _run(cuda_lib, d, dtype, t, T, center, tol, walk_kernel, **kw):
+    B, H, n = 1, 2, 5 * t + 17
+    K, V = synth.layer_kv("llama", 61, 0, B, H, n, d, dtype)
+    K = synth.round_to(0.06 * K + (1.5 if center else 0.0), dtype)
+    hz = Harness(cuda_lib, B=B, L=1, H=H, g=1, d=d, dtype=dtype, t=t, T=T, N=n, seed=6, c_override=0.75, center_keys=center, **kw)
+    cut = 3 * t - 5
+    hz.append_layer(0, K[:, :, :cut], V[:, :, :cut])
+    hz.compress()
+    hz.append_layer(0, K[:, :, cut:], V[:, :, cut:])
+    hz.compress()
+    tot, _ = hz.check_all(tol)
+    assert tot == B * H * t * sum(5 >> l for l in range(T))
+    st = hz.ctx.stats()
+    assert st["device_status"] == 0 and st["walk_kernel"] == walk_kernel
+    hz.ctx.close()
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("t,T,center", [(128, 1, 0), (192, 2, 0), (192, 1, 1), (320, 1, 0), (1088, 1, 0), (2048, 1, 0)])
+def test_tensor_core_walk_with_ragged_panels(cuda_lib, d, t, T, center):
+    """Whole panels and a last panel of 64 tokens; d = 64 operands are a single 64-dim box."""
+    _run(cuda_lib, d, "bf16", t, T, center, 5e-4 if center else 2e-4, 2)

@@ -69,6 +69,8 @@ struct balancekv_ctx {
   CallStat* d_stats = nullptr;
   float* d_tokshift = nullptr;
   int8_t* d_eta = nullptr;
+  float* d_ghat = nullptr;       // workspace of the CUDA-core walk: ghat_calls calls
+  int ghat_calls = 0;
   unsigned long long* d_fail = nullptr;
   int* d_status = nullptr;
   int* h_status_dev = nullptr;   // device address of h_status
@@ -355,7 +357,7 @@ int balancekv_create(const balancekv_config* cfg, balancekv_ctx** out) {
   if (T > 0) {
     if ((rc = dev_alloc(c, &c->d_stats, (size_t)c->max_calls))) return fail(rc);
     if ((rc = dev_alloc(c, &c->d_eta, (size_t)c->max_calls * t))) return fail(rc);
-    if (G.center_keys && (rc = dev_alloc(c, &c->d_tokshift, (size_t)c->max_calls * (t + f.head_dim)))) return fail(rc);
+    if (G.center_keys && (rc = dev_alloc(c, &c->d_tokshift, (size_t)c->max_calls * t + 64))) return fail(rc);
   }
   if ((rc = dev_alloc(c, &c->d_fail, 1))) return fail(rc);
   if ((rc = dev_alloc(c, &c->d_status, 2))) return fail(rc);       // the word, and the counter of launch_reset
@@ -391,7 +393,9 @@ int balancekv_create(const balancekv_config* cfg, balancekv_ctx** out) {
   if (c->use_tc && walk_tc_prepare(G, c->A, c->total_rows, &c->tmaps) != cudaSuccess) return fail(BALANCEKV_E_CUDA);
   if (T > 0 && !c->use_tc) {
     if (!walk_simt_supported(G.d)) return fail(BALANCEKV_E_INVAL);
-    if (walk_simt_smem_bytes(G.d, t) > (size_t)227 * 1024) return fail(BALANCEKV_E_INVAL);
+    // workspace of the CUDA-core walk: the kernel matrices of up to 512 MB of calls at a time
+    c->ghat_calls = (int)std::max<int64_t>(1, std::min<int64_t>(c->max_calls, ((int64_t)512 << 20) / (int64_t)walk_simt_bytes(t)));
+    if ((rc = dev_alloc(c, reinterpret_cast<char**>(&c->d_ghat), walk_simt_bytes(t) * c->ghat_calls))) return fail(rc);
   }
   *out = c;
   return BALANCEKV_OK;
@@ -402,7 +406,7 @@ int balancekv_destroy(balancekv_ctx* c) {
   cudaDeviceSynchronize();
   walk_tc_release(c->tmaps);
   decode_mma_release(c->decode_maps);
-  void* ptrs[] = {c->A.K, c->A.V, c->A.idx, c->A.seg, c->A.nrm, c->d_stats, c->d_tokshift, c->d_eta, c->d_fail, c->d_status,
+  void* ptrs[] = {c->A.K, c->A.V, c->A.idx, c->A.seg, c->A.nrm, c->d_stats, c->d_tokshift, c->d_eta, c->d_ghat, c->d_fail, c->d_status,
                   c->d_decode_scratch, c->d_ring, c->dbg_eta, c->dbg_S, c->dbg_p, c->view_K, c->view_V, c->view_w,
                   c->view_idx, c->bounce_K, c->bounce_V, c->bounce_q, c->bounce_out, c->step_dev_in, c->step_dev_out, c->two_acc, c->two_ml, c->two_scratch, c->unit_V};
   for (void* p : ptrs)
@@ -558,11 +562,9 @@ int balancekv_cache_load_level(balancekv_ctx* c, int layer, int level, const voi
 // One level of a batch: radii -> walk -> selection/compaction for n calls.
 static int run_calls(balancekv_ctx* c, const CallSet& calls, int n, int l, cudaStream_t st) {
   const Geom& G = c->G;
-  // the tensor-core walk kernel takes the radii from the stored row norms itself
-  const bool need_radii = (G.center_keys || G.fixed_rk2 <= 0.f || G.fixed_rv2 <= 0.f) && !(c->use_tc && !G.center_keys);
-  if (need_radii) {
+  if (G.center_keys) {          // else the walk takes the radii from the stored row norms itself
     ProfScope ps(c, 1, st);
-    BKV_CUDA(launch_radii(G, c->A, calls, n, c->d_stats, c->d_tokshift, st));
+    BKV_CUDA(launch_center(G, c->A, calls, n, c->d_stats, c->d_tokshift, st));
     c->kernels_launched++;
   }
   if (c->use_tc) {
@@ -572,7 +574,8 @@ static int run_calls(balancekv_ctx* c, const CallSet& calls, int n, int l, cudaS
   } else {
     ProfScope ps(c, 2, st);
     BKV_CUDA(launch_walk_simt(G, c->A, calls, n, l, c->d_stats, c->d_tokshift, c->d_eta, c->dbg_eta, c->dbg_S,
-                              c->dbg_p, c->d_fail, st));
+                              c->dbg_p, c->d_fail, c->d_status, c->d_ghat, c->ghat_calls, st));
+    c->kernels_launched += 2 * ((n + c->ghat_calls - 1) / c->ghat_calls) - 1;
   }
   if (!c->use_tc) {
     ProfScope ps(c, 3, st);

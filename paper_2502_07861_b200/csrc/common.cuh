@@ -246,11 +246,12 @@ cudaError_t launch_batch_end(const Geom& G, const Arena& A, const BatchEnd& E, i
 // `scratch` and n2 of `scratch2` (may be null).  status: the status word, behind it a zero word of scratch.
 cudaError_t launch_reset(Seg* seg, size_t n_seg, float* scratch, size_t n, float* scratch2, size_t n2, int* status,
                          int* status_host, cudaStream_t st);
-cudaError_t launch_radii(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, CallStat* stats,
-                         float* tok_shift, cudaStream_t st);
+cudaError_t launch_center(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, CallStat* stats,
+                          float* tok_shift, cudaStream_t st);
 cudaError_t launch_walk_simt(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, int level,
                              const CallStat* stats, const float* tok_shift, int8_t* eta, int8_t* dbg_eta,
-                             float* dbg_S, float* dbg_p, unsigned long long* fail_count, cudaStream_t st);
+                             float* dbg_S, float* dbg_p, unsigned long long* fail_count, int* status, float* ws, int ws_calls,
+                             cudaStream_t st);
 cudaError_t launch_walk_tc(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, int level,
                            const CallStat* stats, const float* tok_shift, int8_t* eta, int8_t* dbg_eta,
                            float* dbg_S, float* dbg_p, unsigned long long* fail_count, int* status,
@@ -277,6 +278,6 @@ cudaError_t launch_bucket_scatter(const Geom& G, const Arena& A, const void* K, 
                                   int n_buckets, const int8_t* slot, const int32_t* rank, const int32_t* chunk_base,
                                   const float* ns, const BucketDst* dst, cudaStream_t st);
 int walk_simt_supported(int d);
-size_t walk_simt_smem_bytes(int d, int t);
+size_t walk_simt_bytes(int t);
 
 }  // namespace bkv

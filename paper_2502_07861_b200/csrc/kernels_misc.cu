@@ -1,7 +1,7 @@
 // Data-movement and reduction helpers of the BalanceKV library:
 //   append / level load   (Algorithm 3: C^0 <- C^0 + {k_j, v_j})
 //   level-0 remainder move
-//   per-call radii r_key^2, r_value^2 (inputs of Algorithm 2) and the optional key shift
+//   the optional key shift of a call and its radii r_key^2, r_value^2 (inputs of Algorithm 2)
 #include <algorithm>
 
 #include "common.cuh"
@@ -278,30 +278,6 @@ center_kernel(Geom G, Arena A, const CallSet calls, CallStat* __restrict__ stats
   }
 }
 
-// r_key^2, r_value^2 of a call from the stored row norms: one CTA per call.
-__global__ void __launch_bounds__(256)
-radii_norms_kernel(Geom G, Arena A, const CallSet calls, CallStat* __restrict__ stats) {
-  grid_wait_and_release();
-  const CallDesc C = call_of(calls, G, blockIdx.x);
-  float mk = 0.f, mv = 0.f;
-  for (int j = threadIdx.x; j < G.t; j += 256) {
-    const float2 n = A.nrm[C.src_row + j];
-    mk = fmaxf(mk, n.x);
-    mv = fmaxf(mv, n.y);
-  }
-  mk = warp_max(mk); mv = warp_max(mv);
-  __shared__ float smk[8], smv[8];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0) { smk[warp] = mk; smv[warp] = mv; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < 8; ++w) { mk = fmaxf(mk, smk[w]); mv = fmaxf(mv, smv[w]); }
-    CallStat S{};
-    S.rk2 = mk; S.rv2 = mv;
-    stats[blockIdx.x] = S;
-  }
-}
-
 __global__ void fill_weights_kernel(float* w, int n, float value) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) w[i] = value;
@@ -349,14 +325,9 @@ cudaError_t launch_reset(Seg* seg, size_t n_seg, float* scratch, size_t n, float
   return cudaLaunchKernelEx(&pc.cfg, reset_kernel, seg, n_seg, scratch, n, scratch2, n2, status, status_host);
 }
 
-// stats must hold n_calls entries; tok_shift n_calls * t floats when key centering is on, else it may be null.
-cudaError_t launch_radii(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, CallStat* stats,
-                         float* tok_shift, cudaStream_t st) {
-  if (n_calls <= 0) return cudaSuccess;
-  if (!G.center_keys) {              // the norms were recorded when the rows were written
-    const PdlConfig pc(dim3(n_calls), 256, 0, st);
-    return cudaLaunchKernelEx(&pc.cfg, radii_norms_kernel, G, A, calls, stats);
-  }
+// stats must hold n_calls entries, tok_shift n_calls * t floats.
+cudaError_t launch_center(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, CallStat* stats,
+                          float* tok_shift, cudaStream_t st) {
   const PdlConfig pc(dim3(n_calls), kCenterThreads, 0, st);
   return cudaLaunchKernelEx(&pc.cfg, G.is_bf16 ? center_kernel<true> : center_kernel<false>, G, A, calls, stats, tok_shift);
 }

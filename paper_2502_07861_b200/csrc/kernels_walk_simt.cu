@@ -1,4 +1,5 @@
-// SoftmaxBalance (Algorithm 2) on CUDA cores: one CTA per call.
+// SoftmaxBalance (Algorithm 2) on CUDA cores, for the contexts that the tensor-core kernel does not serve: fp32 inputs,
+// blocks of 64 tokens, and bf16 contexts that ask for this family.
 //
 // For every token j of the call, in stream order,
 //   S_j   = sum_{i<j} eta_i * Ghat_ij,   Ghat_ij = exp((<k_i,k_j> - r_key^2)/sqrt d) <v_i,v_j> / r_value^2
@@ -6,224 +7,404 @@
 //   eta_j = +1 iff u_j < 1/2 - S_j/(2c)   <=>   S_j < c (1 - 2 u_j),
 // with u_j the Philox uniform of (seed, layer, head, call ordinal, level, j).
 //
-// The kernel never materialises Ghat in global memory: 64-row panels of K and V are staged
-// in shared memory as fp32, 64x64 tiles of Ghat are formed with FFMA, off-diagonal tiles are
-// folded into the panel's partial correlations with the (already final) signs of earlier
-// panels, and the diagonal tile is consumed by a one-warp sequential walk in which lane l
-// owns token l of a 32-token group and the signs travel by warp shuffle.
+// Two kernels.  Ghat does not depend on the signs, so ghat_kernel forms its lower triangle with FFMA over the whole chip
+// (grid: tiles of all calls) into a workspace of 64 x 64 tiles; walk_kernel (a CTA per call) streams the tiles back by
+// bulk copies, folds the tiles left of the diagonal with the signs that are final, and walks the diagonal tile.
+// What bounds it: the FFMA pipe in the first kernel, the chain of panels and the L2 reads (2 t^2 bytes per call) in the
+// second.  One CTA per call doing both left most of the chip idle and ran at a third of an SM's FFMA rate: @FIGURES@
 // All accumulation is fp32 in a fixed order, so two runs give identical bits.
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace bkv {
 
 namespace {
 
-constexpr int kPanel = 64;
-constexpr int kThreads = 256;
+constexpr int kTile = 64;                               // rows and columns of a workspace tile
+constexpr int kTileFloats = kTile * kTile;
+constexpr uint32_t kTileBytes = kTileFloats * 4;
+constexpr int kChunk = 32;                              // dims per pipeline stage of ghat_kernel
+constexpr long long kWaitCycles = 100000000LL;          // about 50 ms: a bulk copy that has not landed by then never will
 
-template <int D>
-struct SimtSmem {
-  static constexpr int kStride = D + 4;
-  static constexpr size_t panel_floats = (size_t)kPanel * kStride;
-  static size_t bytes(int t) {
-    return sizeof(float) * (4 * panel_floats + (size_t)kPanel * (kPanel + 1) + kPanel + 3 * (size_t)t);
-  }
-};
+// Float index of (row, column) inside a workspace tile: 16-byte pieces, odd rows with the halves of every 128 bytes
+// swapped, so that four lanes per row read two rows without bank conflicts.
+__device__ inline int tile_at(int row, int col) { return row * kTile + (col ^ ((row & 1) << 4)); }
 
-template <bool kBf16, int D>
-__device__ inline void load_panel(float* __restrict__ dst, const void* __restrict__ base, int64_t row0) {
-  constexpr int kStride = D + 4;
-  constexpr int chunks = D / 8;
-  const int esz = kBf16 ? 2 : 4;
-  for (int i = threadIdx.x; i < kPanel * chunks; i += kThreads) {
-    const int r = i / chunks, c = i % chunks;
-    float v[8];
-    load8<kBf16>(static_cast<const char*>(base) + (size_t)(row0 + r) * D * esz, c * 8, v);
-    float4* o = reinterpret_cast<float4*>(dst + r * kStride + c * 8);
-    o[0] = make_float4(v[0], v[1], v[2], v[3]);
-    o[1] = make_float4(v[4], v[5], v[6], v[7]);
+__device__ inline uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ inline void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+
+// Four neighbouring elements in shared memory.
+template <typename E>
+__device__ inline float4 lds4(const unsigned char* p) {
+  if constexpr (sizeof(E) == 4) {
+    return *reinterpret_cast<const float4*>(p);
+  } else {
+    const uint2 w = *reinterpret_cast<const uint2*>(p);
+    return make_float4(bf16_lo(w.x), bf16_hi(w.x), bf16_lo(w.y), bf16_hi(w.y));
   }
 }
 
-template <bool kBf16, int D>
-__global__ void __launch_bounds__(kThreads, 1)
-walk_simt_kernel(Geom G, Arena A, const CallSet calls, int level,
-                 const CallStat* __restrict__ stats, const float* __restrict__ tok_shift,
-                 int8_t* __restrict__ eta_out, int8_t* __restrict__ dbg_eta, float* __restrict__ dbg_S,
-                 float* __restrict__ dbg_p, unsigned long long* __restrict__ fail_count) {
-  constexpr int kStride = D + 4;
-  extern __shared__ __align__(16) float smem[];
-  float* Kr = smem;
-  float* Vr = Kr + kPanel * kStride;
-  float* Kc = Vr + kPanel * kStride;
-  float* Vc = Kc + kPanel * kStride;
-  float* Gs = Vc + kPanel * kStride;               // [64][65]
-  float* s_row = Gs + kPanel * (kPanel + 1);       // [64]
-  float* eta_s = s_row + kPanel;                   // [t]
-  float* thr_s = eta_s + G.t;                      // [t]
-  float* shift_s = thr_s + G.t;                    // [t]
+// A block of 64 rows x 16 CM columns of one call's Ghat: 16 columns of threads, thread (ty, tx) owns the rows
+// ty + (64 / RM) a and the columns tx + 16 b.  Operands pass through two stages of 32 dims (cp.async, rows padded by 16
+// bytes: the column operand's 16 rows of a warp's load fall on all banks), first those of K, then of V.
+template <int RM>
+constexpr int kGhatThreads = kTile / RM * 16;
+template <typename E, int CM>
+constexpr size_t ghat_smem() { return 2 * (size_t)(kTile + 16 * CM) * (kChunk * sizeof(E) + 16); }
 
+template <typename E, int D, int RM, int CM>
+__global__ void __launch_bounds__(kGhatThreads<RM>, 2)
+ghat_kernel(Geom G, Arena A, const CallSet calls, int call0, const CallStat* __restrict__ stats,
+            const float* __restrict__ tok_shift, float* __restrict__ ghat, int tiles_per_call) {
+  constexpr int kThreads = kGhatThreads<RM>, kCols = 16 * CM, kRowStep = kTile / RM;
+  constexpr int kStride = kChunk * (int)sizeof(E) + 16, kPieces = kChunk * (int)sizeof(E) / 16;
+  constexpr int kStageBytes = (kTile + kCols) * kStride;
+  constexpr int kHalf = D / kChunk, kSteps = 2 * kHalf;
+  extern __shared__ __align__(128) unsigned char sm[];
+  __shared__ float red[2][kThreads / 32];
   grid_wait_and_release();
-  const int call = blockIdx.x;
+  const int call = call0 + blockIdx.y;
   const CallDesc C = call_of(calls, G, call);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int t = G.t;
-  const int head = C.stream % G.H;
-  const int layer = (C.stream / G.H) % G.L;
-  const int seq = C.stream / (G.H * G.L);
-  const float rk2 = G.fixed_rk2 > 0.f ? G.fixed_rk2 : stats[call].rk2;
-  const float rv2 = G.fixed_rv2 > 0.f ? G.fixed_rv2 : stats[call].rv2;
+  // block index -> (row tile r, column block cb): row tile r has r / (kCols / 64) + 1 column blocks
+  int r = 0, cb = blockIdx.x;
+  for (int n; cb >= (n = r * kTile / kCols + 1); ++r) cb -= n;
+  const int row0 = r * kTile, col0 = cb * kCols;
+
+  const unsigned char* src[2] = {static_cast<const unsigned char*>(A.K) + (size_t)C.src_row * D * sizeof(E),
+                                 static_cast<const unsigned char*>(A.V) + (size_t)C.src_row * D * sizeof(E)};
+  auto issue = [&](int step) {
+    unsigned char* st = sm + (step & 1) * kStageBytes;
+    const unsigned char* base = src[step / kHalf] + (size_t)(step % kHalf) * kChunk * sizeof(E);
+    for (int i = tid; i < (kTile + kCols) * kPieces; i += kThreads) {
+      const int row = i / kPieces, p = i % kPieces;
+      const int token = row < kTile ? row0 + row : min(col0 + row - kTile, t - 1);   // columns past the call are not stored
+      cp_async16(st + row * kStride + p * 16, base + (size_t)token * D * sizeof(E) + p * 16);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  issue(0);
+  issue(1);
+
+  // r_key^2, r_value^2 (inputs of Algorithm 2): maxima of the stored row norms, unless center_kernel has put them or they
+  // are fixed
+  float rk2 = G.fixed_rk2, rv2 = G.fixed_rv2;
+  if (tok_shift) {
+    if (rk2 <= 0.f) rk2 = stats[call].rk2;
+    if (rv2 <= 0.f) rv2 = stats[call].rv2;
+  } else {
+    float mk = 0.f, mv = 0.f;
+    for (int j = tid; j < t; j += kThreads) {
+      const float2 n = A.nrm[C.src_row + j];
+      mk = fmaxf(mk, n.x);
+      mv = fmaxf(mv, n.y);
+    }
+    mk = warp_max(mk); mv = warp_max(mv);
+    if (lane == 0) { red[0][warp] = mk; red[1][warp] = mv; }
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < kThreads / 32; ++w) { mk = fmaxf(mk, red[0][w]); mv = fmaxf(mv, red[1][w]); }
+    if (rk2 <= 0.f) rk2 = mk;
+    if (rv2 <= 0.f) rv2 = mv;
+  }
   const float inv_rv2 = rv2 > 0.f ? 1.0f / rv2 : 0.f;
   const float scale = 1.4426950408889634f * G.inv_sqrt_d;
-  const float c = G.c;
 
-  for (int j = tid; j < t; j += kThreads) {
-    const float u = walk_uniform(G.seed + (uint64_t)seq, layer, head, C.ordinal, level, j);
-    thr_s[j] = c * (1.0f - 2.0f * u);
-    shift_s[j] = tok_shift ? tok_shift[(size_t)call * t + j] : 0.f;
-  }
-
-  const int ty = tid >> 4, tx = tid & 15;
-  int fails = 0;
-  for (int r = 0; r < t / kPanel; ++r) {
-    __syncthreads();  // previous panel fully consumed
-    load_panel<kBf16, D>(Kr, A.K, C.src_row + (int64_t)r * kPanel);
-    load_panel<kBf16, D>(Vr, A.V, C.src_row + (int64_t)r * kPanel);
-    if (tid < kPanel) s_row[tid] = 0.f;
-    for (int cp = 0; cp <= r; ++cp) {
-      if (cp < r) {
-        load_panel<kBf16, D>(Kc, A.K, C.src_row + (int64_t)cp * kPanel);
-        load_panel<kBf16, D>(Vc, A.V, C.src_row + (int64_t)cp * kPanel);
-      }
+  const int ty = tid / 16, tx = tid % 16;
+  float acc[RM][CM], ex[RM][CM];
+#pragma unroll
+  for (int a = 0; a < RM; ++a)
+#pragma unroll
+    for (int b = 0; b < CM; ++b) acc[a][b] = 0.f;
+#pragma unroll 1
+  for (int half = 0; half < 2; ++half) {
+#pragma unroll 1
+    for (int s = 0; s < kHalf; ++s) {
+      const int step = half * kHalf + s;
+      if (step + 1 < kSteps) asm volatile("cp.async.wait_group 1;" ::: "memory");
+      else asm volatile("cp.async.wait_group 0;" ::: "memory");
       __syncthreads();
-      const float* Kcol = cp < r ? Kc : Kr;
-      const float* Vcol = cp < r ? Vc : Vr;
-      // ---- 64x64 tile: thread (ty,tx) owns rows ty+16a, cols tx+16b
-      float kk[4][4], vv[4][4];
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) { kk[a][b] = 0.f; vv[a][b] = 0.f; }
+      const unsigned char* rows = sm + (step & 1) * kStageBytes;
+      const unsigned char* cols = rows + kTile * kStride;
 #pragma unroll 2
-      for (int e = 0; e < D; e += 4) {
-        float4 kr[4], kc[4], vr[4], vc[4];
+      for (int e = 0; e < kChunk; e += 4) {
+        float4 x[RM];
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
-          kr[a] = *reinterpret_cast<const float4*>(Kr + (ty + 16 * a) * kStride + e);
-          vr[a] = *reinterpret_cast<const float4*>(Vr + (ty + 16 * a) * kStride + e);
-          kc[a] = *reinterpret_cast<const float4*>(Kcol + (tx + 16 * a) * kStride + e);
-          vc[a] = *reinterpret_cast<const float4*>(Vcol + (tx + 16 * a) * kStride + e);
-        }
+        for (int a = 0; a < RM; ++a) x[a] = lds4<E>(rows + (ty + kRowStep * a) * kStride + e * sizeof(E));
 #pragma unroll
-        for (int a = 0; a < 4; ++a)
+        for (int b = 0; b < CM; ++b) {
+          const float4 y = lds4<E>(cols + (tx + 16 * b) * kStride + e * sizeof(E));
 #pragma unroll
-          for (int b = 0; b < 4; ++b) {
-            kk[a][b] = fmaf(kr[a].x, kc[b].x, kk[a][b]);
-            kk[a][b] = fmaf(kr[a].y, kc[b].y, kk[a][b]);
-            kk[a][b] = fmaf(kr[a].z, kc[b].z, kk[a][b]);
-            kk[a][b] = fmaf(kr[a].w, kc[b].w, kk[a][b]);
-            vv[a][b] = fmaf(vr[a].x, vc[b].x, vv[a][b]);
-            vv[a][b] = fmaf(vr[a].y, vc[b].y, vv[a][b]);
-            vv[a][b] = fmaf(vr[a].z, vc[b].z, vv[a][b]);
-            vv[a][b] = fmaf(vr[a].w, vc[b].w, vv[a][b]);
+          for (int a = 0; a < RM; ++a) {
+            acc[a][b] = fmaf(x[a].x, y.x, acc[a][b]);
+            acc[a][b] = fmaf(x[a].y, y.y, acc[a][b]);
+            acc[a][b] = fmaf(x[a].z, y.z, acc[a][b]);
+            acc[a][b] = fmaf(x[a].w, y.w, acc[a][b]);
           }
+        }
       }
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          const int row = ty + 16 * a, col = tx + 16 * b;
-          const float ex = (kk[a][b] - shift_s[r * kPanel + row] - shift_s[cp * kPanel + col] - rk2) * scale;
-          Gs[row * (kPanel + 1) + col] = exp2f(ex) * (vv[a][b] * inv_rv2);
-        }
       __syncthreads();
-      if (cp < r) {
-        // fold the tile into the panel's partial correlations: 4 threads per row
-        const int row = tid >> 2, part = tid & 3;
-        float acc = 0.f;
+      if (step + 2 < kSteps) issue(step + 2);
+    }
+    if (half == 0) {
+      const float* shift = tok_shift ? tok_shift + (size_t)call * t : nullptr;
 #pragma unroll
-        for (int q = 0; q < 16; ++q) {
-          const int col = part * 16 + q;
-          acc = fmaf(Gs[row * (kPanel + 1) + col], eta_s[cp * kPanel + col], acc);
-        }
-        acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-        acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-        if (part == 0) s_row[row] += acc;
-      } else if (warp == 0) {
-        // the sequential walk over the panel's 64 tokens, 32 at a time
-        for (int grp = 0; grp < 2; ++grp) {
-          const int row = grp * 32 + lane;
-          const int jg = r * kPanel + row;
-          float S = s_row[row];
-          if (grp == 1) {
+      for (int a = 0; a < RM; ++a) {
+        const int j = row0 + ty + kRowStep * a;
+        const float off = (shift ? shift[j] : 0.f) + rk2;
 #pragma unroll
-            for (int col = 0; col < 32; ++col) S = fmaf(Gs[row * (kPanel + 1) + col], eta_s[r * kPanel + col], S);
-          }
-          float g[32];
-#pragma unroll
-          for (int j = 0; j < 32; ++j) g[j] = j < lane ? Gs[row * (kPanel + 1) + grp * 32 + j] : 0.f;
-          const float thr = thr_s[jg];
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            const float dec = S < thr ? 1.0f : -1.0f;
-            const float ej = __shfl_sync(0xffffffffu, dec, j);
-            S = fmaf(ej, g[j], S);   // g[j] = 0 once this lane's token is decided
-          }
-          const float my_eta = S < thr ? 1.0f : -1.0f;
-          eta_s[jg] = my_eta;
-          if (fabsf(S) > c) ++fails;   // FAIL of Algorithm 2: counted, decision already clamped
-          if (C.dbg_off >= 0) {
-            dbg_S[C.dbg_off + jg] = S;
-            dbg_p[C.dbg_off + jg] = 0.5f - fminf(fmaxf(S, -c), c) / (2.0f * c);
-          }
-          __syncwarp();
+        for (int b = 0; b < CM; ++b) {
+          const int i = col0 + tx + 16 * b;
+          ex[a][b] = i < j ? exp2f((acc[a][b] - (shift ? shift[i] : 0.f) - off) * scale) : 0.f;   // only earlier tokens count
+          acc[a][b] = 0.f;
         }
       }
     }
   }
-  __syncthreads();
-  for (int j = tid; j < t; j += kThreads) {
-    const int8_t e = eta_s[j] > 0.f ? 1 : -1;
-    eta_out[(size_t)call * t + j] = e;
-    if (C.dbg_off >= 0) dbg_eta[C.dbg_off + j] = e;
+  float* out = ghat + ((size_t)blockIdx.y * tiles_per_call + (size_t)r * (r + 1) / 2 + col0 / kTile) * kTileFloats;
+#pragma unroll
+  for (int b = 0; b < CM; ++b) {
+    const int ct = 16 * b / kTile, col = tx + 16 * b - ct * kTile;       // column tile of the block, column inside it
+    if (col0 / kTile + ct <= r) {
+#pragma unroll
+      for (int a = 0; a < RM; ++a) {
+        const int row = ty + kRowStep * a;
+        out[(size_t)ct * kTileFloats + tile_at(row, col)] = ex[a][b] != 0.f ? ex[a][b] * (acc[a][b] * inv_rv2) : 0.f;
+      }
+    }
   }
-  if (warp == 0) {
+}
+
+constexpr int kWalkWarps = 8, kWalkThreads = 32 * kWalkWarps + 32;       // eight warps walk, one lane of the ninth fetches
+constexpr int kWalkStages = 6;
+constexpr int kMaxSweeps = kTile + 2;
+__device__ inline bool walkers_or(bool pred) {           // barrier of the walking warps with a vote
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 q, %2, 0;\n\t"
+      "bar.red.or.pred p, 1, %1, q;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(r) : "r"(32 * kWalkWarps), "r"((uint32_t)pred) : "memory");
+  return r != 0;
+}
+__device__ inline bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+  return ok != 0;
+}
+__device__ inline bool mbar_wait(uint64_t* bar, uint32_t parity) {       // bounded
+  if (mbar_try_wait(bar, parity)) return true;
+  const long long t0 = clock64();
+  while (!mbar_try_wait(bar, parity))
+    if (clock64() - t0 > kWaitCycles) return false;
+  return true;
+}
+
+// The walk of one call over its Ghat tiles.  Four lanes share a row of the panel (lane p takes the 16-byte pieces
+// p, p + 4, ..).  The 64 signs of a panel are the fixed point of "decide every token from the current signs" (sweep k
+// makes token k final); in sweep 0, with no in-panel sign known, a row whose distance to its threshold exceeds the sum of
+// its in-panel |Ghat| is decided already, and if that holds for all rows (and none can FAIL) one sweep suffices.
+__global__ void __launch_bounds__(kWalkThreads)
+walk_kernel(Geom G, const CallSet calls, int call0, int level, const float* __restrict__ ghat, int tiles_per_call, int stages,
+            int8_t* __restrict__ eta_out, int8_t* __restrict__ dbg_eta, float* __restrict__ dbg_S, float* __restrict__ dbg_p,
+            unsigned long long* __restrict__ fail_count, int* __restrict__ status) {
+  extern __shared__ __align__(128) unsigned char sm[];
+  const int t = G.t, P = t / kTile;
+  float* tiles = reinterpret_cast<float*>(sm);                           // [stages][64 x 64]
+  float* etas = tiles + (size_t)stages * kTileFloats;                    // [t] final signs
+  float* cur = etas + t;                                                 // [2][64] the panel's signs, sweep by sweep
+  uint64_t* full = reinterpret_cast<uint64_t*>(cur + 2 * kTile);         // [stages], then [stages] empty
+  uint64_t* empty = full + kWalkStages;
+  const int call = call0 + blockIdx.x;
+  const CallDesc C = call_of(calls, G, call);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid == 0) {
+    for (int s = 0; s < stages; ++s) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&full[s])));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&empty[s])), "r"(kWalkWarps));
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  const int head = C.stream % G.H, layer = (C.stream / G.H) % G.L, seq = C.stream / (G.H * G.L);
+  const float c = G.c;
+  __syncthreads();
+  grid_wait_and_release();
+  if (warp == kWalkWarps) {
+    if (lane == 0) {
+      const float* src = ghat + (size_t)blockIdx.x * tiles_per_call * kTileFloats;
+      bool ok = true;
+      for (int i = 0; i < tiles_per_call && ok; ++i) {
+        const int s = i % stages;
+        if (i >= stages) ok = mbar_wait(&empty[s], (uint32_t)((i / stages - 1) & 1));
+        if (!ok) break;
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&full[s])), "r"(kTileBytes) : "memory");
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                     ::"r"(smem_u32(tiles + (size_t)s * kTileFloats)), "l"(src + (size_t)i * kTileFloats), "r"(kTileBytes),
+                     "r"(smem_u32(&full[s])) : "memory");
+      }
+    }
+  } else {
+    const int row = tid / 4, p = tid % 4;
+    const float* gp = tiles + row * kTile;
+    const int sw = (row & 1) << 4;
+    int fails = 0;
+    bool ok = true;
+    int i = 0;
+    auto wait_tile = [&](int tile) {                     // a warp's one polling lane, then the warp
+      bool got = true;
+      if (lane == 0) got = mbar_wait(&full[tile % stages], (uint32_t)((tile / stages) & 1));
+      got = __shfl_sync(0xffffffffu, got, 0);
+      __syncwarp();
+      return got;
+    };
+    for (int r = 0; r < P; ++r) {
+      const int j = r * kTile + row;
+      const float thr = c * (1.0f - 2.0f * walk_uniform(G.seed + (uint64_t)seq, layer, head, C.ordinal, level, j));
+      float acc = 0.f;
+      for (int k = 0; k < r; ++k, ++i) {
+        ok = ok && wait_tile(i);
+        if (ok) {
+          const float* g = gp + (size_t)(i % stages) * kTileFloats;
+          const float* e = etas + k * kTile;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const int col = 16 * q + 4 * p;
+            const float4 x = *reinterpret_cast<const float4*>(g + (col ^ sw)), y = *reinterpret_cast<const float4*>(e + col);
+            acc = fmaf(x.x, y.x, acc); acc = fmaf(x.y, y.y, acc); acc = fmaf(x.z, y.z, acc); acc = fmaf(x.w, y.w, acc);
+          }
+        }
+        __syncwarp();
+        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&empty[i % stages])) : "memory");
+      }
+      // ---- diagonal tile
+      ok = ok && wait_tile(i);
+      float4 g[4];
+      float absum = 0.f;
+      if (ok) {
+        const float* gt = gp + (size_t)(i % stages) * kTileFloats;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          g[q] = *reinterpret_cast<const float4*>(gt + ((16 * q + 4 * p) ^ sw));
+          absum += (fabsf(g[q].x) + fabsf(g[q].y)) + (fabsf(g[q].z) + fabsf(g[q].w));
+        }
+      }
+      __syncwarp();
+      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&empty[i % stages])) : "memory");
+      ++i;
+      if (walkers_or(!ok)) { ok = false; break; }        // uniform: everybody walks or everybody leaves
+      absum += __shfl_xor_sync(0xffffffffu, absum, 1);
+      absum += __shfl_xor_sync(0xffffffffu, absum, 2);
+      acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+      acc += __shfl_xor_sync(0xffffffffu, acc, 2);       // the earlier panels' part, the same in the row's four lanes
+      float S = acc;
+      bool plus = S < thr;
+      {
+        const float slack = 1e-5f * (fabsf(S) + absum) + 1e-30f;
+        const bool open = C.dbg_off >= 0 || !(fabsf(S - thr) > absum + slack) || !(fabsf(S) + absum + slack < c);
+        if (p == 0) cur[row] = plus ? 1.f : -1.f;
+        if (walkers_or(open)) {
+          for (int sweep = 1; sweep < kMaxSweeps; ++sweep) {
+            const float* e = cur + ((sweep - 1) & 1) * kTile;
+            float part = 0.f;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const float4 y = *reinterpret_cast<const float4*>(e + 16 * q + 4 * p);
+              part = fmaf(g[q].x, y.x, part); part = fmaf(g[q].y, y.y, part); part = fmaf(g[q].z, y.z, part); part = fmaf(g[q].w, y.w, part);
+            }
+            part += __shfl_xor_sync(0xffffffffu, part, 1);
+            part += __shfl_xor_sync(0xffffffffu, part, 2);
+            S = acc + part;
+            const bool now = S < thr, changed = now != plus;
+            plus = now;
+            if (p == 0) cur[(sweep & 1) * kTile + row] = plus ? 1.f : -1.f;
+            if (!walkers_or(changed)) break;
+          }
+        }
+      }
+      if (p == 0) {
+        etas[j] = plus ? 1.f : -1.f;
+        eta_out[(size_t)call * t + j] = plus ? 1 : -1;
+        if (fabsf(S) > c) ++fails;                       // FAIL of Algorithm 2: counted; the decision is the clamped one
+        if (C.dbg_off >= 0) {
+          dbg_eta[C.dbg_off + j] = plus ? 1 : -1;
+          dbg_S[C.dbg_off + j] = S;
+          dbg_p[C.dbg_off + j] = 0.5f - fminf(fmaxf(S, -c), c) / (2.0f * c);
+        }
+      }
+      walkers_or(false);                                 // the panel's signs are written
+    }
+    if (!ok && lane == 0) atomicCAS(status, kStatusOk, kStatusWaitTimeout);
     fails = (int)__reduce_add_sync(0xffffffffu, (unsigned)fails);
     if (lane == 0 && fails) atomicAdd(fail_count, (unsigned long long)fails);
   }
 }
 
-template <bool kBf16, int D>
-cudaError_t launch_one(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, int level,
-                       const CallStat* stats, const float* tok_shift, int8_t* eta, int8_t* dbg_eta, float* dbg_S,
-                       float* dbg_p, unsigned long long* fail_count, cudaStream_t st) {
-  const size_t smem = SimtSmem<D>::bytes(G.t);
-  auto kern = walk_simt_kernel<kBf16, D>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  const PdlConfig pc(dim3(n_calls), kThreads, smem, st);
-  return cudaLaunchKernelEx(&pc.cfg, kern, G, A, calls, level, stats, tok_shift, eta, dbg_eta, dbg_S, dbg_p, fail_count);
+size_t walk_smem(int t, int stages) { return (size_t)stages * kTileBytes + sizeof(float) * (t + 2 * kTile) + 2 * kWalkStages * sizeof(uint64_t); }
+int walk_stages(int tiles) { return std::min(kWalkStages, tiles); }
+
+template <typename E, int D, int RM, int CM>
+cudaError_t launch_ghat(const Geom& G, const Arena& A, const CallSet& calls, int call0, int n, const CallStat* stats,
+                        const float* tok_shift, float* ghat, int tiles, cudaStream_t st) {
+  auto kern = ghat_kernel<E, D, RM, CM>;
+  constexpr size_t smem = ghat_smem<E, CM>();
+  if (smem > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  int blocks = 0;
+  for (int r = 0; r < G.t / kTile; ++r) blocks += r * kTile / (16 * CM) + 1;
+  const PdlConfig pc(dim3(blocks, n), kGhatThreads<RM>, smem, st);
+  return cudaLaunchKernelEx(&pc.cfg, kern, G, A, calls, call0, stats, tok_shift, ghat, tiles);
+}
+
+template <typename E, int D>
+cudaError_t launch_ghat_d(const Geom& G, const Arena& A, const CallSet& calls, int call0, int n, const CallStat* stats,
+                          const float* tok_shift, float* ghat, int tiles, cudaStream_t st) {
+  // blocks of 64 x 128 where they fill the chip (two CTAs per SM), else 64 x 64 with twice the threads per entry
+  if ((int64_t)tiles / 2 * n >= 2 * 148) return launch_ghat<E, D, 8, 8>(G, A, calls, call0, n, stats, tok_shift, ghat, tiles, st);
+  return launch_ghat<E, D, 4, 4>(G, A, calls, call0, n, stats, tok_shift, ghat, tiles, st);
 }
 
 }  // namespace
 
 int walk_simt_supported(int d) { return d == 64 || d == 128; }
 
-size_t walk_simt_smem_bytes(int d, int t) { return d == 64 ? SimtSmem<64>::bytes(t) : SimtSmem<128>::bytes(t); }
+// Bytes of workspace per call of a launch.
+size_t walk_simt_bytes(int t) { return (size_t)(t / kTile) * (t / kTile + 1) / 2 * kTileBytes; }
 
+// ws: workspace of ws_calls calls; the calls run in groups of that many.
 cudaError_t launch_walk_simt(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, int level,
                              const CallStat* stats, const float* tok_shift, int8_t* eta, int8_t* dbg_eta,
-                             float* dbg_S, float* dbg_p, unsigned long long* fail_count, cudaStream_t st) {
-  if (n_calls <= 0) return cudaSuccess;
-  if (G.d == 128) {
-    return G.is_bf16 ? launch_one<true, 128>(G, A, calls, n_calls, level, stats, tok_shift, eta, dbg_eta, dbg_S, dbg_p, fail_count, st)
-                     : launch_one<false, 128>(G, A, calls, n_calls, level, stats, tok_shift, eta, dbg_eta, dbg_S, dbg_p, fail_count, st);
+                             float* dbg_S, float* dbg_p, unsigned long long* fail_count, int* status, float* ws, int ws_calls,
+                             cudaStream_t st) {
+  const int tiles = (int)(walk_simt_bytes(G.t) / kTileBytes), stages = walk_stages(tiles);
+  const size_t smem = walk_smem(G.t, stages);
+  cudaError_t e = cudaFuncSetAttribute(walk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (!G.center_keys) tok_shift = nullptr;
+  for (int call0 = 0; call0 < n_calls && e == cudaSuccess; call0 += ws_calls) {
+    const int n = std::min(ws_calls, n_calls - call0);
+    if (G.d == 128)
+      e = G.is_bf16 ? launch_ghat_d<__nv_bfloat16, 128>(G, A, calls, call0, n, stats, tok_shift, ws, tiles, st)
+                    : launch_ghat_d<float, 128>(G, A, calls, call0, n, stats, tok_shift, ws, tiles, st);
+    else
+      e = G.is_bf16 ? launch_ghat_d<__nv_bfloat16, 64>(G, A, calls, call0, n, stats, tok_shift, ws, tiles, st)
+                    : launch_ghat_d<float, 64>(G, A, calls, call0, n, stats, tok_shift, ws, tiles, st);
+    if (e != cudaSuccess) break;
+    const PdlConfig pc(dim3(n), kWalkThreads, smem, st);
+    e = cudaLaunchKernelEx(&pc.cfg, walk_kernel, G, calls, call0, level, static_cast<const float*>(ws), tiles, stages, eta, dbg_eta,
+                           dbg_S, dbg_p, fail_count, status);
   }
-  if (G.d == 64) {
-    return G.is_bf16 ? launch_one<true, 64>(G, A, calls, n_calls, level, stats, tok_shift, eta, dbg_eta, dbg_S, dbg_p, fail_count, st)
-                     : launch_one<false, 64>(G, A, calls, n_calls, level, stats, tok_shift, eta, dbg_eta, dbg_S, dbg_p, fail_count, st);
-  }
-  return cudaErrorInvalidValue;
+  return e;
 }
 
 }  // namespace bkv

@@ -32,3 +32,34 @@ def _run(cuda_lib, d, dtype, t, T, center, tol, walk_kernel, **kw):
 def test_tensor_core_walk_with_ragged_panels(cuda_lib, d, t, T, center):
     """Whole panels and a last panel of 64 tokens; d = 64 operands are a single 64-dim box."""
     _run(cuda_lib, d, "bf16", t, T, center, 5e-4 if center else 2e-4, 2)
+
+
+@pytest.mark.parametrize("d,dtype,t,T,center", [(64, "fp32", 64, 2, 0), (64, "fp32", 128, 1, 1), (128, "fp32", 192, 2, 0), (128, "fp32", 640, 1, 0),
+                                                (64, "fp32", 1024, 1, 0), (128, "bf16", 64, 2, 1), (64, "bf16", 320, 1, 0)])
+def test_cuda_core_walk(cuda_lib, d, dtype, t, T, center):
+    """One workspace tile, fewer tiles than stages and more, an odd number of row tiles (column blocks that reach past the
+    call), small and large launches of the kernel-matrix kernel."""
+    _run(cuda_lib, d, dtype, t, T, center, 5e-4 if center else 2e-5, 1, gram_path=1)
+
+
+def test_cuda_core_walk_in_groups_of_calls(cuda_lib):
+    """More calls than the workspace holds (512 MB: 60 calls of 2048 tokens), against the walk of each stream alone."""
+    import torch
+
+    S, t, n = 62, 2048, 2048
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    K = 0.1 * torch.randn(1, S, n, 64, device="cuda", generator=gen)
+    V = torch.randn(1, S, n, 64, device="cuda", generator=gen)
+    ctx = cuda_lib.Context(n_seqs=1, n_layers=1, n_kv_heads=S, n_q_heads=S, head_dim=64, dtype="fp32", block=t, levels=1, max_tokens=n,
+                           seed=3, c_override=0.75)
+    ctx.stream_append_layer(0, K, V)
+    ctx.compress()
+    one = cuda_lib.Context(n_seqs=1, n_layers=1, n_kv_heads=S, n_q_heads=S, head_dim=64, dtype="fp32", block=t, levels=1, max_tokens=n,
+                           seed=3, c_override=0.75)
+    for h in (0, 59, 60, 61):
+        one.stream_append(0, 0, h, K[0, h], V[0, h])
+        one.compress()
+        assert all(torch.equal(a, b) for a, b in zip(ctx.cache_view(0, 0, h), one.cache_view(0, 0, h))), h
+    assert ctx.stats()["device_status"] == 0 and one.stats()["device_status"] == 0
+    ctx.close()
+    one.close()

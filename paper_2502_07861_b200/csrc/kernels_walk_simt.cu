@@ -11,7 +11,8 @@
 // (grid: tiles of all calls) into a workspace of 64 x 64 tiles; walk_kernel (a CTA per call) streams the tiles back by
 // bulk copies, folds the tiles left of the diagonal with the signs that are final, and walks the diagonal tile.
 // What bounds it: the FFMA pipe in the first kernel, the chain of panels and the L2 reads (2 t^2 bytes per call) in the
-// second.  One CTA per call doing both left most of the chip idle and ran at a third of an SM's FFMA rate: @FIGURES@
+// second.  128 calls of 512 fp32 tokens x 128 dims: 253 + 18 us (62 % of the FMA pipe; one CTA per call doing both took
+// 408 us and as much for 64 calls, which take 128 + 18 now); one call of 256 x 64: 8 + 7 us (67).
 // All accumulation is fp32 in a fixed order, so two runs give identical bits.
 #include <algorithm>
 
@@ -36,32 +37,39 @@ __device__ inline void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
 
-// Four neighbouring elements in shared memory.
+// Four neighbouring elements in shared memory, as two pairs.
+struct Quad {
+  float2 a, b;
+};
 template <typename E>
-__device__ inline float4 lds4(const unsigned char* p) {
+__device__ inline Quad lds4(const unsigned char* p) {
   if constexpr (sizeof(E) == 4) {
-    return *reinterpret_cast<const float4*>(p);
+    const float4 w = *reinterpret_cast<const float4*>(p);
+    return Quad{make_float2(w.x, w.y), make_float2(w.z, w.w)};
   } else {
     const uint2 w = *reinterpret_cast<const uint2*>(p);
-    return make_float4(bf16_lo(w.x), bf16_hi(w.x), bf16_lo(w.y), bf16_hi(w.y));
+    return Quad{make_float2(bf16_lo(w.x), bf16_hi(w.x)), make_float2(bf16_lo(w.y), bf16_hi(w.y))};
   }
 }
 
-// A block of 64 rows x 16 CM columns of one call's Ghat: 16 columns of threads, thread (ty, tx) owns the rows
-// ty + (64 / RM) a and the columns tx + 16 b.  Operands pass through two stages of 32 dims (cp.async, rows padded by 16
-// bytes: the column operand's 16 rows of a warp's load fall on all banks), first those of K, then of V.
+// One 64 x 64 tile of one call's Ghat: 16 columns of threads, thread (ty, tx) owns the rows ty + (64 / RM) a and the
+// columns tx + 16 b.  Operands pass through two stages of 32 dims (cp.async, rows padded by 16 bytes: the column operand's
+// 16 rows of a warp's load fall on all banks), first those of K, then of V.  Products are packed pairs of neighbouring
+// dims (even and odd dims are summed apart).  Measured and not better: scalar FFMA with 8 x 8 entries per thread (290 us for
+// the 253 above: issue and operand fetch), 8 x 8 packed entries with the exponentials parked in shared memory (271).
+constexpr int CM = 4;                                   // 16 CM = 64 columns
 template <int RM>
 constexpr int kGhatThreads = kTile / RM * 16;
-template <typename E, int CM>
-constexpr size_t ghat_smem() { return 2 * (size_t)(kTile + 16 * CM) * (kChunk * sizeof(E) + 16); }
+template <typename E>
+constexpr size_t ghat_smem() { return 2 * (size_t)(2 * kTile) * (kChunk * sizeof(E) + 16); }
 
-template <typename E, int D, int RM, int CM>
-__global__ void __launch_bounds__(kGhatThreads<RM>, 2)
+template <typename E, int D, int RM>
+__global__ void __launch_bounds__(kGhatThreads<RM>, RM == 8 ? 3 : 2)
 ghat_kernel(Geom G, Arena A, const CallSet calls, int call0, const CallStat* __restrict__ stats,
             const float* __restrict__ tok_shift, float* __restrict__ ghat, int tiles_per_call) {
-  constexpr int kThreads = kGhatThreads<RM>, kCols = 16 * CM, kRowStep = kTile / RM;
+  constexpr int kThreads = kGhatThreads<RM>, kRowStep = kTile / RM;
   constexpr int kStride = kChunk * (int)sizeof(E) + 16, kPieces = kChunk * (int)sizeof(E) / 16;
-  constexpr int kStageBytes = (kTile + kCols) * kStride;
+  constexpr int kStageBytes = 2 * kTile * kStride;
   constexpr int kHalf = D / kChunk, kSteps = 2 * kHalf;
   extern __shared__ __align__(128) unsigned char sm[];
   __shared__ float red[2][kThreads / 32];
@@ -70,19 +78,19 @@ ghat_kernel(Geom G, Arena A, const CallSet calls, int call0, const CallStat* __r
   const CallDesc C = call_of(calls, G, call);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int t = G.t;
-  // block index -> (row tile r, column block cb): row tile r has r / (kCols / 64) + 1 column blocks
+  // block index -> tile (r, cb) of the lower triangle
   int r = 0, cb = blockIdx.x;
-  for (int n; cb >= (n = r * kTile / kCols + 1); ++r) cb -= n;
-  const int row0 = r * kTile, col0 = cb * kCols;
+  for (; cb > r; ++r) cb -= r + 1;
+  const int row0 = r * kTile, col0 = cb * kTile;
 
   const unsigned char* src[2] = {static_cast<const unsigned char*>(A.K) + (size_t)C.src_row * D * sizeof(E),
                                  static_cast<const unsigned char*>(A.V) + (size_t)C.src_row * D * sizeof(E)};
   auto issue = [&](int step) {
     unsigned char* st = sm + (step & 1) * kStageBytes;
     const unsigned char* base = src[step / kHalf] + (size_t)(step % kHalf) * kChunk * sizeof(E);
-    for (int i = tid; i < (kTile + kCols) * kPieces; i += kThreads) {
+    for (int i = tid; i < 2 * kTile * kPieces; i += kThreads) {
       const int row = i / kPieces, p = i % kPieces;
-      const int token = row < kTile ? row0 + row : min(col0 + row - kTile, t - 1);   // columns past the call are not stored
+      const int token = row < kTile ? row0 + row : col0 + row - kTile;
       cp_async16(st + row * kStride + p * 16, base + (size_t)token * D * sizeof(E) + p * 16);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
@@ -115,11 +123,12 @@ ghat_kernel(Geom G, Arena A, const CallSet calls, int call0, const CallStat* __r
   const float scale = 1.4426950408889634f * G.inv_sqrt_d;
 
   const int ty = tid / 16, tx = tid % 16;
-  float acc[RM][CM], ex[RM][CM];
+  float2 acc[RM][CM];
+  float ex[RM][CM];
 #pragma unroll
   for (int a = 0; a < RM; ++a)
 #pragma unroll
-    for (int b = 0; b < CM; ++b) acc[a][b] = 0.f;
+    for (int b = 0; b < CM; ++b) acc[a][b] = make_float2(0.f, 0.f);
 #pragma unroll 1
   for (int half = 0; half < 2; ++half) {
 #pragma unroll 1
@@ -132,19 +141,16 @@ ghat_kernel(Geom G, Arena A, const CallSet calls, int call0, const CallStat* __r
       const unsigned char* cols = rows + kTile * kStride;
 #pragma unroll 2
       for (int e = 0; e < kChunk; e += 4) {
-        float4 x[RM];
+        Quad x[RM];
 #pragma unroll
         for (int a = 0; a < RM; ++a) x[a] = lds4<E>(rows + (ty + kRowStep * a) * kStride + e * sizeof(E));
 #pragma unroll
         for (int b = 0; b < CM; ++b) {
-          const float4 y = lds4<E>(cols + (tx + 16 * b) * kStride + e * sizeof(E));
+          const Quad y = lds4<E>(cols + (tx + 16 * b) * kStride + e * sizeof(E));
 #pragma unroll
-          for (int a = 0; a < RM; ++a) {
-            acc[a][b] = fmaf(x[a].x, y.x, acc[a][b]);
-            acc[a][b] = fmaf(x[a].y, y.y, acc[a][b]);
-            acc[a][b] = fmaf(x[a].z, y.z, acc[a][b]);
-            acc[a][b] = fmaf(x[a].w, y.w, acc[a][b]);
-          }
+          for (int a = 0; a < RM; ++a) acc[a][b] = __ffma2_rn(x[a].a, y.a, acc[a][b]);
+#pragma unroll
+          for (int a = 0; a < RM; ++a) acc[a][b] = __ffma2_rn(x[a].b, y.b, acc[a][b]);
         }
       }
       __syncthreads();
@@ -159,24 +165,18 @@ ghat_kernel(Geom G, Arena A, const CallSet calls, int call0, const CallStat* __r
 #pragma unroll
         for (int b = 0; b < CM; ++b) {
           const int i = col0 + tx + 16 * b;
-          ex[a][b] = i < j ? exp2f((acc[a][b] - (shift ? shift[i] : 0.f) - off) * scale) : 0.f;   // only earlier tokens count
-          acc[a][b] = 0.f;
+          ex[a][b] = i < j ? exp2f((acc[a][b].x + acc[a][b].y - (shift ? shift[i] : 0.f) - off) * scale) : 0.f;   // only earlier tokens count
+          acc[a][b] = make_float2(0.f, 0.f);
         }
       }
     }
   }
-  float* out = ghat + ((size_t)blockIdx.y * tiles_per_call + (size_t)r * (r + 1) / 2 + col0 / kTile) * kTileFloats;
+  float* out = ghat + ((size_t)blockIdx.y * tiles_per_call + blockIdx.x) * kTileFloats;
 #pragma unroll
-  for (int b = 0; b < CM; ++b) {
-    const int ct = 16 * b / kTile, col = tx + 16 * b - ct * kTile;       // column tile of the block, column inside it
-    if (col0 / kTile + ct <= r) {
+  for (int a = 0; a < RM; ++a)
 #pragma unroll
-      for (int a = 0; a < RM; ++a) {
-        const int row = ty + kRowStep * a;
-        out[(size_t)ct * kTileFloats + tile_at(row, col)] = ex[a][b] != 0.f ? ex[a][b] * (acc[a][b] * inv_rv2) : 0.f;
-      }
-    }
-  }
+    for (int b = 0; b < CM; ++b)
+      out[tile_at(ty + kRowStep * a, tx + 16 * b)] = ex[a][b] != 0.f ? ex[a][b] * ((acc[a][b].x + acc[a][b].y) * inv_rv2) : 0.f;
 }
 
 constexpr int kWalkWarps = 8, kWalkThreads = 32 * kWalkWarps + 32;       // eight warps walk, one lane of the ninth fetches
@@ -221,7 +221,8 @@ walk_kernel(Geom G, const CallSet calls, int call0, int level, const float* __re
   const int t = G.t, P = t / kTile;
   float* tiles = reinterpret_cast<float*>(sm);                           // [stages][64 x 64]
   float* etas = tiles + (size_t)stages * kTileFloats;                    // [t] final signs
-  float* cur = etas + t;                                                 // [2][64] the panel's signs, sweep by sweep
+  float* thr_s = etas + t;                                               // [t] decision thresholds c (1 - 2 u_j)
+  float* cur = thr_s + t;                                                // [2][64] the panel's signs, sweep by sweep
   uint64_t* full = reinterpret_cast<uint64_t*>(cur + 2 * kTile);         // [stages], then [stages] empty
   uint64_t* empty = full + kWalkStages;
   const int call = call0 + blockIdx.x;
@@ -235,17 +236,23 @@ walk_kernel(Geom G, const CallSet calls, int call0, int level, const float* __re
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
-  const int head = C.stream % G.H, layer = (C.stream / G.H) % G.L, seq = C.stream / (G.H * G.L);
   const float c = G.c;
+  {
+    // the coins of the whole call, ahead of the grid dependency
+    const int head = C.stream % G.H, layer = (C.stream / G.H) % G.L, seq = C.stream / (G.H * G.L);
+    for (int j = tid; j < t; j += kWalkThreads)
+      thr_s[j] = c * (1.0f - 2.0f * walk_uniform(G.seed + (uint64_t)seq, layer, head, C.ordinal, level, j));
+  }
   __syncthreads();
   grid_wait_and_release();
   if (warp == kWalkWarps) {
     if (lane == 0) {
       const float* src = ghat + (size_t)blockIdx.x * tiles_per_call * kTileFloats;
       bool ok = true;
-      for (int i = 0; i < tiles_per_call && ok; ++i) {
-        const int s = i % stages;
-        if (i >= stages) ok = mbar_wait(&empty[s], (uint32_t)((i / stages - 1) & 1));
+      int s = 0;
+      uint32_t par = 1;                                    // of the next wait on stage s: none in the first round
+      for (int i = 0; i < tiles_per_call && ok; ++i, s = s + 1 == stages ? (par ^= 1u, 0) : s + 1) {
+        if (i >= stages) ok = mbar_wait(&empty[s], par);
         if (!ok) break;
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&full[s])), "r"(kTileBytes) : "memory");
         asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
@@ -259,48 +266,53 @@ walk_kernel(Geom G, const CallSet calls, int call0, int level, const float* __re
     const int sw = (row & 1) << 4;
     int fails = 0;
     bool ok = true;
-    int i = 0;
-    auto wait_tile = [&](int tile) {                     // a warp's one polling lane, then the warp
+    int s = 0;                                           // stage of the next tile, parity of its barrier
+    uint32_t par = 0;
+    auto wait_tile = [&]() {                             // a warp's one polling lane, then the warp
       bool got = true;
-      if (lane == 0) got = mbar_wait(&full[tile % stages], (uint32_t)((tile / stages) & 1));
+      if (lane == 0) got = mbar_wait(&full[s], par);
       got = __shfl_sync(0xffffffffu, got, 0);
       __syncwarp();
       return got;
     };
+    auto leave_tile = [&]() {
+      __syncwarp();
+      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&empty[s])) : "memory");
+      if (++s == stages) { s = 0; par ^= 1u; }
+    };
     for (int r = 0; r < P; ++r) {
       const int j = r * kTile + row;
-      const float thr = c * (1.0f - 2.0f * walk_uniform(G.seed + (uint64_t)seq, layer, head, C.ordinal, level, j));
-      float acc = 0.f;
-      for (int k = 0; k < r; ++k, ++i) {
-        ok = ok && wait_tile(i);
+      const float thr = thr_s[j];
+      float2 a2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+      for (int k = 0; k < r; ++k) {
+        ok = ok && wait_tile();
         if (ok) {
-          const float* g = gp + (size_t)(i % stages) * kTileFloats;
+          const float* g = gp + (size_t)s * kTileFloats;
           const float* e = etas + k * kTile;
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             const int col = 16 * q + 4 * p;
             const float4 x = *reinterpret_cast<const float4*>(g + (col ^ sw)), y = *reinterpret_cast<const float4*>(e + col);
-            acc = fmaf(x.x, y.x, acc); acc = fmaf(x.y, y.y, acc); acc = fmaf(x.z, y.z, acc); acc = fmaf(x.w, y.w, acc);
+            a2[0] = __ffma2_rn(make_float2(x.x, x.y), make_float2(y.x, y.y), a2[0]);
+            a2[1] = __ffma2_rn(make_float2(x.z, x.w), make_float2(y.z, y.w), a2[1]);
           }
         }
-        __syncwarp();
-        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&empty[i % stages])) : "memory");
+        leave_tile();
       }
       // ---- diagonal tile
-      ok = ok && wait_tile(i);
+      float acc = (a2[0].x + a2[0].y) + (a2[1].x + a2[1].y);
+      ok = ok && wait_tile();
       float4 g[4];
       float absum = 0.f;
       if (ok) {
-        const float* gt = gp + (size_t)(i % stages) * kTileFloats;
+        const float* gt = gp + (size_t)s * kTileFloats;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           g[q] = *reinterpret_cast<const float4*>(gt + ((16 * q + 4 * p) ^ sw));
           absum += (fabsf(g[q].x) + fabsf(g[q].y)) + (fabsf(g[q].z) + fabsf(g[q].w));
         }
       }
-      __syncwarp();
-      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&empty[i % stages])) : "memory");
-      ++i;
+      leave_tile();
       if (walkers_or(!ok)) { ok = false; break; }        // uniform: everybody walks or everybody leaves
       absum += __shfl_xor_sync(0xffffffffu, absum, 1);
       absum += __shfl_xor_sync(0xffffffffu, absum, 2);
@@ -349,30 +361,28 @@ walk_kernel(Geom G, const CallSet calls, int call0, int level, const float* __re
   }
 }
 
-size_t walk_smem(int t, int stages) { return (size_t)stages * kTileBytes + sizeof(float) * (t + 2 * kTile) + 2 * kWalkStages * sizeof(uint64_t); }
+size_t walk_smem(int t, int stages) { return (size_t)stages * kTileBytes + sizeof(float) * (2 * t + 2 * kTile) + 2 * kWalkStages * sizeof(uint64_t); }
 int walk_stages(int tiles) { return std::min(kWalkStages, tiles); }
 
-template <typename E, int D, int RM, int CM>
+template <typename E, int D, int RM>
 cudaError_t launch_ghat(const Geom& G, const Arena& A, const CallSet& calls, int call0, int n, const CallStat* stats,
                         const float* tok_shift, float* ghat, int tiles, cudaStream_t st) {
-  auto kern = ghat_kernel<E, D, RM, CM>;
-  constexpr size_t smem = ghat_smem<E, CM>();
+  auto kern = ghat_kernel<E, D, RM>;
+  constexpr size_t smem = ghat_smem<E>();
   if (smem > 48 * 1024) {
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  int blocks = 0;
-  for (int r = 0; r < G.t / kTile; ++r) blocks += r * kTile / (16 * CM) + 1;
-  const PdlConfig pc(dim3(blocks, n), kGhatThreads<RM>, smem, st);
+  const PdlConfig pc(dim3(tiles, n), kGhatThreads<RM>, smem, st);
   return cudaLaunchKernelEx(&pc.cfg, kern, G, A, calls, call0, stats, tok_shift, ghat, tiles);
 }
 
 template <typename E, int D>
 cudaError_t launch_ghat_d(const Geom& G, const Arena& A, const CallSet& calls, int call0, int n, const CallStat* stats,
                           const float* tok_shift, float* ghat, int tiles, cudaStream_t st) {
-  // blocks of 64 x 128 where they fill the chip (two CTAs per SM), else 64 x 64 with twice the threads per entry
-  if ((int64_t)tiles / 2 * n >= 2 * 148) return launch_ghat<E, D, 8, 8>(G, A, calls, call0, n, stats, tok_shift, ghat, tiles, st);
-  return launch_ghat<E, D, 4, 4>(G, A, calls, call0, n, stats, tok_shift, ghat, tiles, st);
+  // 8 x 4 entries per thread where the tiles fill the chip (three CTAs per SM), else 4 x 4: twice the threads per tile
+  if ((int64_t)tiles * n >= 2 * 148) return launch_ghat<E, D, 8>(G, A, calls, call0, n, stats, tok_shift, ghat, tiles, st);
+  return launch_ghat<E, D, 4>(G, A, calls, call0, n, stats, tok_shift, ghat, tiles, st);
 }
 
 }  // namespace

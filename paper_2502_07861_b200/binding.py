@@ -113,12 +113,15 @@ def _check(code: int, what: str):
 
 
 def _stream_ptr(stream):
+    """The cudaStream_t as an integer: of a torch stream, a raw one, or (None) the current stream of the current device."""
+    if isinstance(stream, int):          # a raw cudaStream_t
+        return stream
+    if stream is not None:
+        return stream.cuda_stream
     import torch
 
-    if isinstance(stream, int):          # a raw cudaStream_t
-        return C.c_void_p(stream)
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return C.c_void_p(s.cuda_stream)
+    # torch.cuda.current_stream() builds a stream object: 3.3 us of every call against 0.2 us for the handle alone
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _torch_dtype(dtype_code: int):
@@ -173,7 +176,7 @@ class Context:
     def _dev(self, t, name):
         if not t.is_cuda or t.dtype != self.dtype or not t.is_contiguous():
             raise ValueError(f"{name}: expected a contiguous CUDA tensor of dtype {self.dtype}")
-        return C.c_void_p(t.data_ptr())
+        return t.data_ptr()
 
     def stream_append(self, seq, layer, kv_head, K_blk, V_blk, stream=None):
         assert K_blk.shape == V_blk.shape and K_blk.shape[-1] == self.cfg.head_dim
@@ -301,16 +304,16 @@ class Context:
         return out
 
     def stream_step_host(self, layer, q_host, k_host, v_host, out_host, stream=None):
-        _check(self.lib.balancekv_stream_step_host(self._h, layer, C.c_void_p(q_host.data_ptr()),
-                                                   C.c_void_p(k_host.data_ptr()), C.c_void_p(v_host.data_ptr()),
-                                                   C.c_void_p(out_host.data_ptr()), _stream_ptr(stream)),
+        _check(self.lib.balancekv_stream_step_host(self._h, layer, q_host.data_ptr(),
+                                                   k_host.data_ptr(), v_host.data_ptr(),
+                                                   out_host.data_ptr(), _stream_ptr(stream)),
                "balancekv_stream_step_host")
         return out_host
 
     def decode_attn_host(self, layer, q_host, out_host, stream=None):
         assert not q_host.is_cuda and not out_host.is_cuda and q_host.dtype == self.dtype
-        _check(self.lib.balancekv_decode_attn_host(self._h, layer, C.c_void_p(q_host.data_ptr()),
-                                                   C.c_void_p(out_host.data_ptr()), _stream_ptr(stream)),
+        _check(self.lib.balancekv_decode_attn_host(self._h, layer, q_host.data_ptr(),
+                                                   out_host.data_ptr(), _stream_ptr(stream)),
                "balancekv_decode_attn_host")
         return out_host
 
@@ -414,10 +417,10 @@ def decode_attn_static(K, V, n_heavy, level, q, out=None, stream=None):
     assert K.shape == V.shape and K.dtype == V.dtype == q.dtype and q.shape[0] == K.shape[0] and q.shape[2] == K.shape[2]
     if out is None:
         out = torch.empty_like(q)
-    dtype_code = {torch.float32: 0, torch.bfloat16: 1}[K.dtype]
-    _check(load().balancekv_decode_attn_static(C.c_void_p(K.data_ptr()), C.c_void_p(V.data_ptr()), K.shape[0],
-                                               K.shape[1], n_heavy, level, C.c_void_p(q.data_ptr()),
-                                               C.c_void_p(out.data_ptr()), q.shape[1], K.shape[2], dtype_code,
+    dtype_code = 1 if K.dtype == torch.bfloat16 else {torch.float32: 0}[K.dtype]
+    _check(load().balancekv_decode_attn_static(K.data_ptr(), V.data_ptr(), K.shape[0],
+                                               K.shape[1], n_heavy, level, q.data_ptr(),
+                                               out.data_ptr(), q.shape[1], K.shape[2], dtype_code,
                                                _stream_ptr(stream)), "balancekv_decode_attn_static")
     return out
 

@@ -31,6 +31,8 @@
 // roles leave their loops, TMEM is freed and the kernel returns.
 #include <cuda.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace bkv {
@@ -149,6 +151,15 @@ __device__ inline void umma_tile_hi(uint32_t d_tmem, uint32_t a_lo, uint32_t b_l
   umma_bf16<1>(d_tmem, a_lo + kHalf + 2, b_lo + kHalf + 2);
   umma_bf16<1>(d_tmem, a_lo + kHalf + 4, b_lo + kHalf + 4);
   umma_bf16<1>(d_tmem, a_lo + kHalf + 6, b_lo + kHalf + 6);
+}
+// One lane of a converged warp, always the same: code under it stays warp-uniform for the compiler.
+__device__ inline bool elect_one() {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+  return r != 0;
 }
 __device__ inline void umma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
@@ -324,7 +335,7 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
                int* __restrict__ status, const float2* __restrict__ row_norms, const Arena A,
                const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV) {
   extern __shared__ unsigned char smem_raw[];
-  unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  unsigned char* sm = smem_raw + (-smem_u32(smem_raw) & 1023u);   // an offset, so that the compiler keeps seeing shared memory
   constexpr uint32_t kTileBytes = kTileBytesOf<D>, kSlotBytes = Smem<D>::kSlotBytes;
   constexpr int kBoxes = D / 64;                                          // boxes of 64 dims per tile
   // t is a multiple of 64: the last panel may hold 64 tokens only.  Its tile then covers 64 rows that are not the
@@ -347,7 +358,12 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
   int* abort_flag = reinterpret_cast<int*>(tmem_ptr_s + 1);
 
   const int call = blockIdx.x;
-  const CallDesc C = call_of(calls, G, call);
+  // The call's descriptor is derived where it is wanted: kept, it would take eight registers of every epilogue thread.
+  auto desc = [&]() {
+    int i = blockIdx.x;
+    asm volatile("" : "+r"(i));
+    return call_of(calls, G, i);
+  };
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
   if (tid == 0) {
@@ -366,6 +382,7 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
   // Everything above touches only this CTA's own state, and so do the coins: all of it overlaps the end of the previous
   // launch (programmatic serialization; the wait comes before the first row or norm is read).
   {
+    const CallDesc C = desc();
     const int head = C.stream % G.H, layer = (C.stream / G.H) % G.L, seq = C.stream / (G.H * G.L);
     for (int i = tid; i < t; i += kThreads)
       thr_s[i] = G.c * (1.0f - 2.0f * walk_uniform(G.seed + (uint64_t)seq, layer, head, C.ordinal, level, i));
@@ -386,6 +403,7 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
   if (warp == kTmaWarp) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
+      const int64_t src_row = desc().src_row;
       uint32_t used = 0, par = 0;        // per slot: loaded before; parity of the next wait on its empty barriers
       bool ok = true;
       auto load = [&](int slot, int tile_row) -> bool {
@@ -394,7 +412,7 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
         used |= 1u << slot;
         if (again) par ^= 1u << slot;
         unsigned char* st = sm + (uint32_t)slot * kSlotBytes;
-        const int y = (int)(C.src_row + (int64_t)tile_row * kTile);
+        const int y = (int)(src_row + (int64_t)tile_row * kTile);
 #pragma unroll
         for (int h = 0; h < kBoxes; ++h) {
           uint64_t* fk = full + 2 * slot + h;
@@ -417,42 +435,56 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
     __syncwarp();
   } else if (warp == kMmaWarp || warp == kMmaWarpV) {
     // ------------------------------------------------------------------ MMA issuers (K K^T and V V^T)
-    if (lane == 0) {
-      const int x = warp == kMmaWarpV ? 1 : 0;
+    // The whole warp walks the schedule and one elected lane issues: descriptors and addresses are then warp-uniform and
+    // sit in uniform registers.  (Issued from a branch on the lane index, with per-thread operands, an MMA took about 100
+    // cycles of the issuing thread instead of the 64 that the tensor core needs for it.)
+    auto issue = [&](auto product) {
+      constexpr int x = decltype(product)::value;
       int i = 0;
       uint32_t par = 0;                  // per slot: parity of the next wait on its full barrier
       bool ok = true;
       const uint32_t slot0 = umma_desc_lo(smem_u32(sm + (x ? kTileBytes : 0u)));
       constexpr uint32_t kSlotDesc = kSlotBytes >> 4;
+      const uint32_t d_base = __shfl_sync(0xffffffffu, tmem_base, 0) + (x ? 128u : 0u);
+      auto wait = [&](uint64_t* bar, uint32_t parity) { return __all_sync(0xffffffffu, wait_bar(bar, parity, abort_flag)) != 0; };
       for (int r = 0; r < P && ok; ++r) {
         const int rs = r % 3;
-        if (!(ok = wait_bar(full + 6 * x + 2 * rs, (par >> rs) & 1u, abort_flag))) break;
-        if (kBoxes == 2 && !(ok = wait_bar(full + 6 * x + 2 * rs + 1, (par >> rs) & 1u, abort_flag))) break;
+        if (!(ok = wait(full + 6 * x + 2 * rs, (par >> rs) & 1u))) break;
+        if (kBoxes == 2 && !(ok = wait(full + 6 * x + 2 * rs + 1, (par >> rs) & 1u))) break;
         par ^= 1u << rs;
         const uint32_t arow = slot0 + (uint32_t)rs * kSlotDesc;
         for (int c = 0; c <= r; ++c, ++i) {
           const int buf = i & 1;
-          if (!(ok = wait_bar(tmem_empty + buf, (uint32_t)(((i >> 1) & 1) ^ 1), abort_flag))) break;
+          if (!(ok = wait(tmem_empty + buf, (uint32_t)(((i >> 1) & 1) ^ 1)))) break;
           const int slot = c < r ? (r + 1 + (c & 1)) % 3 : rs;
           const uint32_t b = slot0 + (uint32_t)slot * kSlotDesc;
-          const uint32_t d_tmem = tmem_base + (uint32_t)buf * 256u + (x ? 128u : 0u);
+          const uint32_t d_tmem = d_base + (uint32_t)buf * 256u;
           const uint32_t ph = (par >> slot) & 1u;
           if (c < r) {
-            if (!(ok = wait_bar(full + 6 * x + 2 * slot, ph, abort_flag))) break;
+            if (!(ok = wait(full + 6 * x + 2 * slot, ph))) break;
             par ^= 1u << slot;
           }
           tc_fence_after();
-          umma_tile_lo(d_tmem, arow, b);
-          umma_commit(empty + 6 * x + 2 * slot);       // a column slot's box after its tile, the row slot's after the diagonal tile
-          if constexpr (kBoxes == 2) {
-            if (c < r && !(ok = wait_bar(full + 6 * x + 2 * slot + 1, ph, abort_flag))) break;
-            umma_tile_hi(d_tmem, arow, b);
-            umma_commit(empty + 6 * x + 2 * slot + 1);
+          if (elect_one()) {
+            umma_tile_lo(d_tmem, arow, b);
+            umma_commit(empty + 6 * x + 2 * slot);       // a column slot's box after its tile, the row slot's after the diagonal tile
           }
-          umma_commit(xdone + buf);
+          __syncwarp();
+          if constexpr (kBoxes == 2) {
+            if (c < r && !(ok = wait(full + 6 * x + 2 * slot + 1, ph))) break;
+            if (elect_one()) {
+              umma_tile_hi(d_tmem, arow, b);
+              umma_commit(empty + 6 * x + 2 * slot + 1);
+            }
+            __syncwarp();
+          }
+          if (elect_one()) umma_commit(xdone + buf);
+          __syncwarp();
         }
       }
-    }
+    };
+    if (warp == kMmaWarp) issue(std::integral_constant<int, 0>{});
+    else issue(std::integral_constant<int, 1>{});
     __syncwarp();
   } else {
     // ------------------------------------------------------------------ four epilogue warpgroups
@@ -513,9 +545,10 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
       // r_key^2, r_value^2 of the call (inputs of Algorithm 2) = maxima of the stored row norms,
       // unless a separate kernel has put them (key centering changes them) or they are fixed
       if (row_norms) {
+        const float2* norms = row_norms + desc().src_row;
         float mk = 0.f, mv = 0.f;
         for (int i = tid; i < t; i += kEpiThreads) {
-          const float2 n2 = row_norms[C.src_row + i];
+          const float2 n2 = norms[i];
           mk = fmaxf(mk, n2.x);
           mv = fmaxf(mv, n2.y);
         }
@@ -537,6 +570,7 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
       if (rv2 <= 0.f) rv2 = stats[call].rv2;
     }
     const float inv_rv2 = rv2 > 0.f ? 1.0f / rv2 : 0.f;
+    const bool record = calls.list && desc().dbg_off >= 0;
     // All waits of a panel come before its vote barrier (id 3); a thread whose wait timed out
     // skips to the vote, where everybody learns of it and leaves.  The sweep barriers (ids 1, 2)
     // come after the vote and contain no waits, so no thread can be left waiting at them.
@@ -607,16 +641,20 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
       // that holds for every row (and no row can FAIL, and S is not recorded) one sweep suffices.
       float absum = 0.f;
       if (below) {
+        float b4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int i = 0; i < 32; ++i) absum += fabsf(g[i]);
+        for (int i = 0; i < 32; i += 4) {
+          b4[0] += fabsf(g[i]); b4[1] += fabsf(g[i + 1]); b4[2] += fabsf(g[i + 2]); b4[3] += fabsf(g[i + 3]);
+        }
+        absum = (b4[0] + b4[1]) + (b4[2] + b4[3]);
       }
       if (wg > 0) xb[(wg - 1) * kTile + row] = absum;
       bool plus = false;
       float S = 0.f;
 #pragma unroll 1
       for (int sweep = 0; sweep < kMaxSweeps; ++sweep) {
-        float part = acc;
-        if (below) {
+        float part = acc;                                    // sweep 0: no in-panel sign is known yet
+        if (below && sweep > 0) {
           float2 a2 = make_float2(acc, 0.f), b2 = make_float2(0.f, 0.f);
 #pragma unroll
           for (int x = 0; x < 8; ++x) {
@@ -639,7 +677,7 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
           } else if (sweep == 0) {
             const float bound = ((absum + xb[row]) + (xb[kTile + row] + xb[2 * kTile + row])) * inv_rv2;
             const float slack = 1e-5f * (fabsf(S) + bound) + 1e-30f;
-            changed = C.dbg_off >= 0 || !(fabsf(S - thr) > bound + slack) || !(fabsf(S) + bound + slack < cw);
+            changed = record || !(fabsf(S - thr) > bound + slack) || !(fabsf(S) + bound + slack < cw);
           } else {
             changed = now != plus;
           }
@@ -651,9 +689,10 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
       if (wg == 0 && mine) {
         eta8[j] = plus ? 1 : -1;
         if (fabsf(S) > cw) ++fails;                          // FAIL of Algorithm 2: counted; the decision is the clamped one
-        if (C.dbg_off >= 0) {
-          dbg_S[C.dbg_off + j] = S;
-          dbg_p[C.dbg_off + j] = 0.5f - fminf(fmaxf(S, -cw), cw) / (2.0f * cw);
+        if (record) {
+          const int64_t off = desc().dbg_off + j;
+          dbg_S[off] = S;
+          dbg_p[off] = 0.5f - fminf(fmaxf(S, -cw), cw) / (2.0f * cw);
         }
       }
     }
@@ -667,6 +706,7 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
   if (*abort_flag) {
     if (tid == 0) atomicCAS(status, kStatusOk, kStatusWaitTimeout);
   } else {
+    const CallDesc C = desc();
     for (int i = tid; i < t; i += kThreads) {
       const int8_t e = eta8[i];
       eta_out[(size_t)call * t + i] = e;

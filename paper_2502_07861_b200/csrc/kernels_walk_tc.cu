@@ -19,18 +19,28 @@
 // TMEM is double buffered (2 x 256 columns); an epilogue hands its buffer back as soon as the
 // accumulator values are in registers.  Each of the two products of a tile has its own issuing
 // thread and its own barriers, so that one product's waits and commits overlap the other's
-// MMAs.  Operands live in three slots (K tile + V tile; 64 KB at d = 128) that rotate roles: panel r keeps
-// its rows in slot r % 3 and streams its column tiles through the other two, and the rows of
-// panel r + 1 are fetched into the slot that panel r's column tiles leave first, so the next
-// panel's first products are already in TMEM when the walk of the diagonal tile ends.
+// MMAs.  Operands live in three slots (K tile + V tile; 64 KB at d = 128) that rotate roles: one holds the panel's rows,
+// the column tiles stream through the other two, and the next panel's rows are fetched behind the last columns, so that its
+// first products are already in TMEM when the walk of the diagonal tile ends.  Where the rows of the resident calls exceed
+// L2, a panel begins with the two tiles that the one before left in shared memory: 107 loads instead of 136 for 2048 tokens,
+// 183 -> 169 us for 148 such calls.
 // Inside a slot every operand is two boxes of 64 dims with their own full/empty barriers: a box is
 // refilled as soon as the four MMAs that read it have retired.
 // Ghat never touches global memory.
+// What bounds it (cycles per off-diagonal tile at 148 calls, d = 128): the MMAs 1090, of which 1024 are the tensor core's; the
+// epilogue 1300, 900 of them for its 28 exponentials per thread on the special-function unit; the loads 1100 from L2, 1540
+// from HBM (calls of 2048 tokens).  A diagonal tile takes 2400, the selection 2100, the copy of 512 kept tokens 13000 at the
+// rate at which the chip takes the writes.  Measured and not taken: A from TMEM, which halves the operand reads from shared
+// memory (1740 per tile); accumulators read in two pipelined halves (1390); a CTA per SM that takes several calls, with the
+// next call's radii and thresholds prepared by a warp of its own (2 % faster from three calls per SM on, 1 to 6 % slower below,
+// from registers that the epilogue lacks); the copies spread over the next call's walk (20 us instead of 9 for 512 tokens, as
+// their loads queue behind the tiles) or left to that warp (75 us, by bulk copies 115).
 //
 // Every wait is bounded: a wait that runs out sets the abort flag and the status word, all
 // roles leave their loops, TMEM is freed and the kernel returns.
 #include <cuda.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "common.cuh"
@@ -225,6 +235,26 @@ struct Smem {
   static constexpr uint32_t kSlotBytes = 2 * kTileBytesOf<D>;
   static constexpr uint32_t kTilesEnd = 3 * kSlotBytes;
 };
+// The columns of panel r where tiles are reused: r - 1, then 0 .. r - 2 in a cycle that begins with the last column of panel
+// r - 1.  What a panel ends on is what the next one begins with, so that only the columns from the third on are loaded.
+struct Columns {
+  int c, next = 0, r = 0;
+  __device__ __forceinline__ void begin(int panel) { r = panel; c = panel - 1; }       // next: the last column of the panel before
+  __device__ __forceinline__ void step() { c = next; next = next + 1 < r - 1 ? next + 1 : 0; }
+  __device__ __forceinline__ void end() { next = r > 0 ? c : 0; }                      // c: the panel's last column
+};
+// The three slots' roles then, and how they change from panel r to r + 1.
+struct Slots {
+  uint32_t a = 0, b = 1, c = 2;
+  __device__ __forceinline__ uint32_t column(int k) const { return k & 1 ? c : b; }
+  __device__ __forceinline__ uint32_t next_rows(int r) const { return r & 1 ? c : b; }
+  __device__ __forceinline__ void advance(int r) {
+    const uint32_t rows = next_rows(r), last = r & 1 ? b : c;
+    b = a;
+    a = rows;
+    c = last;
+  }
+};
 constexpr int kMaxSweeps = kTile + 2;
 
 // Output of Algorithm 2 completed to exactly t/2 tokens (the implementation note of Appendix B:
@@ -293,6 +323,17 @@ __device__ inline void select_and_compact(const Geom& G, const Arena& A, const C
     for (int i = 0; i < ipt; ++i)
       if (mask & (1u << i)) kept_pos[pos++] = j0 + i;
   __syncthreads();
+  // positions and norms: the first two tokens' loads ahead of the rows, their stores after them (2 of 21 us for 256 tokens)
+  int32_t tok[2];
+  float2 nrm[2];
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int o = tid + u * kThreads;
+    if (o < half) {
+      tok[u] = A.idx[C.src_row + kept_pos[o]];
+      if (A.nrm) nrm[u] = A.nrm[C.src_row + kept_pos[o]];
+    }
+  }
   constexpr int kCh = D / 8;
   // copy: a survivor row of K and of V is 2 x d / 8 chunks of 16 bytes; eight loads in flight per thread.
   // (All CTAs of a wave reach this point together, so the copy runs at the chip's memory bandwidth
@@ -321,13 +362,21 @@ __device__ inline void select_and_compact(const Geom& G, const Arena& A, const C
       }
     }
   }
-  for (int o = tid; o < half; o += kThreads) {
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int o = tid + u * kThreads;
+    if (o < half) {
+      A.idx[C.dst_row + o] = tok[u];
+      if (A.nrm) A.nrm[C.dst_row + o] = nrm[u];
+    }
+  }
+  for (int o = tid + 2 * kThreads; o < half; o += kThreads) {
     A.idx[C.dst_row + o] = A.idx[C.src_row + kept_pos[o]];
     if (A.nrm) A.nrm[C.dst_row + o] = A.nrm[C.src_row + kept_pos[o]];
   }
 }
 
-template <int D, bool kCenter>
+template <int D, bool kCenter, bool kReuse>
 __global__ void __launch_bounds__(kThreads, 1)
 walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restrict__ stats,
                const float* __restrict__ tok_shift, int8_t* __restrict__ eta_out, int8_t* __restrict__ dbg_eta,
@@ -393,13 +442,13 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
   tc_fence_after();
   const uint32_t tmem_base = *tmem_ptr_s;
 
-  // Tiles are numbered in issue order i = 0, 1, ...: panel r contributes (r,0) .. (r,r).  Tile i
-  // uses TMEM buffer i & 1.  Panel r reads its rows from slot r % 3 and column tile c from slot
-  // (r + 1 + (c & 1)) % 3.  Loads happen in the order R0, R1, C(1,0), R2, C(2,0), C(2,1), R3, ...
-  // (R = row panel), which is also the order in which the MMA threads first touch them, so both
-  // sides count the uses of a slot alike.  Every barrier is waited on phase by phase by its one
-  // kind of waiter, and each next phase depends on that waiter having passed, so a parity wait
-  // can never be a phase behind.
+  // Tiles are numbered in issue order i = 0, 1, ...; tile i uses TMEM buffer i & 1.  Panel r visits its columns, then the
+  // diagonal.  Without kReuse: rows in slot r % 3, columns in ascending order, column c in slot (r + 1 + (c & 1)) % 3, the
+  // next panel's rows behind the last columns.  With kReuse: slot A holds the rows, the columns alternate between B and C in
+  // the order of Columns, whose first two are still there from panel r - 1 as its rows and its last column; the rows of panel
+  // r + 1 follow the last column but one into its slot, and the slots change roles.  All sides walk the same schedule and
+  // count a slot's loads alike.  Every barrier is waited on phase by phase by its one kind of waiter, and each next phase
+  // depends on that waiter having passed, so a parity wait can never be a phase behind.
   if (warp == kTmaWarp) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
@@ -427,9 +476,24 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
         return true;
       };
       ok = load(0, 0);
-      for (int r = 0; r < P && ok; ++r) {
-        for (int c = 0; c < r && ok; ++c) ok = load((r + 1 + (c & 1)) % 3, c);
-        if (ok && r + 1 < P) ok = load((r + 1) % 3, r + 1);
+      if constexpr (kReuse) {
+        Slots slots;
+        Columns col;
+        for (int r = 0; r < P && ok; ++r) {
+          col.begin(r);
+          for (int k = 1; k < r && ok; ++k) {
+            col.step();
+            if (k > 1) ok = load(slots.column(k), col.c);
+          }
+          col.end();
+          if (ok && r + 1 < P) ok = load(slots.next_rows(r), r + 1);
+          slots.advance(r);
+        }
+      } else {
+        for (int r = 0; r < P && ok; ++r) {
+          for (int c = 0; c < r && ok; ++c) ok = load((r + 1 + (c & 1)) % 3, c);
+          if (ok && r + 1 < P) ok = load((r + 1) % 3, r + 1);
+        }
       }
     }
     __syncwarp();
@@ -447,8 +511,9 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
       constexpr uint32_t kSlotDesc = kSlotBytes >> 4;
       const uint32_t d_base = __shfl_sync(0xffffffffu, tmem_base, 0) + (x ? 128u : 0u);
       auto wait = [&](uint64_t* bar, uint32_t parity) { return __all_sync(0xffffffffu, wait_bar(bar, parity, abort_flag)) != 0; };
-      for (int r = 0; r < P && ok; ++r) {
-        const int rs = r % 3;
+      Slots slots;
+      for (int r = 0; r < P && ok; slots.advance(r), ++r) {
+        const int rs = kReuse ? (int)slots.a : r % 3;
         if (!(ok = wait(full + 6 * x + 2 * rs, (par >> rs) & 1u))) break;
         if (kBoxes == 2 && !(ok = wait(full + 6 * x + 2 * rs + 1, (par >> rs) & 1u))) break;
         par ^= 1u << rs;
@@ -456,25 +521,27 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
         for (int c = 0; c <= r; ++c, ++i) {
           const int buf = i & 1;
           if (!(ok = wait(tmem_empty + buf, (uint32_t)(((i >> 1) & 1) ^ 1)))) break;
-          const int slot = c < r ? (r + 1 + (c & 1)) % 3 : rs;
+          const int slot = c == r ? rs : kReuse ? (int)slots.column(c) : (r + 1 + (c & 1)) % 3;   // c-th column visited
+          const bool loaded = c < r && (!kReuse || c >= 2);  // else the slot's content has been used before
+          const bool leaves = !kReuse || c < r - 1;          // else the next panel uses it once more
           const uint32_t b = slot0 + (uint32_t)slot * kSlotDesc;
           const uint32_t d_tmem = d_base + (uint32_t)buf * 256u;
           const uint32_t ph = (par >> slot) & 1u;
-          if (c < r) {
+          if (loaded) {
             if (!(ok = wait(full + 6 * x + 2 * slot, ph))) break;
             par ^= 1u << slot;
           }
           tc_fence_after();
           if (elect_one()) {
             umma_tile_lo(d_tmem, arow, b);
-            umma_commit(empty + 6 * x + 2 * slot);       // a column slot's box after its tile, the row slot's after the diagonal tile
+            if (leaves) umma_commit(empty + 6 * x + 2 * slot);   // a column slot's box after its tile, the row slot's after the diagonal tile
           }
           __syncwarp();
           if constexpr (kBoxes == 2) {
-            if (c < r && !(ok = wait(full + 6 * x + 2 * slot + 1, ph))) break;
+            if (loaded && !(ok = wait(full + 6 * x + 2 * slot + 1, ph))) break;
             if (elect_one()) {
               umma_tile_hi(d_tmem, arow, b);
-              umma_commit(empty + 6 * x + 2 * slot + 1);
+              if (leaves) umma_commit(empty + 6 * x + 2 * slot + 1);
             }
             __syncwarp();
           }
@@ -574,6 +641,7 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
     // All waits of a panel come before its vote barrier (id 3); a thread whose wait timed out
     // skips to the vote, where everybody learns of it and leaves.  The sweep barriers (ids 1, 2)
     // come after the vote and contain no waits, so no thread can be left waiting at them.
+    int next_col = 0;                                     // with kReuse: the column to follow, at a panel's start its second
     for (int r = 0; r < P; ++r) {
       const int j = r * kTile + row;                      // this thread's token in the panel
       const bool mine = j < t;
@@ -582,7 +650,14 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
       float acc = 0.f;
       const int col0 = 32 * wg;
       const bool below = wg <= q;                         // warp-uniform: the warp has columns below the diagonal
-      for (int c = 0; c < r && ok; ++c, ++tile_it) {
+      int c = kReuse ? r - 1 : 0;
+      for (int k = 0; k < r && ok; ++k, ++tile_it) {
+        if (!kReuse) {
+          c = k;
+        } else if (k > 0) {                                 // the order of Columns
+          c = next_col;
+          next_col = next_col + 1 < r - 1 ? next_col + 1 : 0;
+        }
         const int buf = tile_it & 1;
         if (!(ok = wait_bar(xdone + buf, (uint32_t)((tile_it >> 1) & 1), abort_flag))) break;
         tc_fence_after();
@@ -599,6 +674,7 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
         // signs of panel c are final since its walk
         acc = fold_regs(dk, dv, etas + c * kTile + 32 * wg, c * kTile + 32 * wg, nb, acc);
       }
+      if (kReuse) next_col = r > 0 ? c : 0;
       // ---- diagonal tile
       const int buf = tile_it & 1;
       if (ok) ok = wait_bar(xdone + buf, (uint32_t)((tile_it >> 1) & 1), abort_flag);
@@ -723,9 +799,14 @@ size_t tc_smem_bytes(int d, int t) {
   const size_t tp = (t + kTile - 1) / kTile * kTile;
   return 1024 + (d == 128 ? Smem<128>::kTilesEnd : Smem<64>::kTilesEnd) + tp * 9 + 2 * (kEpiGroups - 1) * kTile * 4 + 512;
 }
-auto kernel_for(int d, bool center) {
-  return d == 128 ? (center ? walk_tc_kernel<128, true> : walk_tc_kernel<128, false>)
-                  : (center ? walk_tc_kernel<64, true> : walk_tc_kernel<64, false>);
+// Tiles are reused where the rows that the resident CTAs visit exceed L2: only then are the loads what a tile waits for.  148
+// calls at d = 128, cycles per off-diagonal tile without and with reuse: 1340 and 1430 for 1024 tokens (78 MB; the epilogue
+// bounds both, and the order costs it some instructions), 1540 and 1460 for 2048 (155 MB).
+bool reuse_tiles(const Geom& G, int ctas) { return G.d == 128 && (int64_t)ctas * G.t * G.d * 4 > (int64_t)126 << 20; }
+auto kernel_for(int d, bool center, bool reuse) {
+  if (d == 64) return center ? walk_tc_kernel<64, true, false> : walk_tc_kernel<64, false, false>;
+  if (reuse) return center ? walk_tc_kernel<128, true, true> : walk_tc_kernel<128, false, true>;
+  return center ? walk_tc_kernel<128, true, false> : walk_tc_kernel<128, false, false>;
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -764,8 +845,8 @@ cudaError_t walk_tc_prepare(const Geom& G, const Arena& A, int64_t total_rows, v
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) { delete tm; return cudaErrorInvalidValue; }
   }
-  for (int i = 0; i < 2 && e == cudaSuccess; ++i)
-    e = cudaFuncSetAttribute(kernel_for(G.d, i != 0), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem_bytes(G.d, G.t));
+  for (int i = 0; i < 4 && e == cudaSuccess; ++i)
+    e = cudaFuncSetAttribute(kernel_for(G.d, (i & 1) != 0, i > 1), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem_bytes(G.d, G.t));
   if (e != cudaSuccess) { delete tm; return e; }
   *tmaps_out = tm;
   return cudaSuccess;
@@ -776,7 +857,7 @@ void walk_tc_release(void* tmaps) { delete static_cast<TensorMaps*>(tmaps); }
 cudaError_t launch_walk_tc(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, int level,
                            const CallStat* stats, const float* tok_shift, int8_t* eta, int8_t* dbg_eta,
                            float* dbg_S, float* dbg_p, unsigned long long* fail_count, int* status,
-                           const void* tmaps, const void* fuse_compaction, cudaStream_t st) {
+                           const void* tmaps, const void* fuse_compaction, int sm_count, cudaStream_t st) {
   if (n_calls <= 0) return cudaSuccess;
   if (!tmaps) return cudaErrorInvalidValue;
   const TensorMaps* tm = static_cast<const TensorMaps*>(tmaps);
@@ -784,7 +865,7 @@ cudaError_t launch_walk_tc(const Geom& G, const Arena& A, const CallSet& calls, 
   Arena Af = A;                       // K == nullptr: leave selection and compaction to the separate kernel
   if (!fuse_compaction) Af.K = nullptr;
   const PdlConfig pc(dim3(n_calls), kThreads, smem, st);
-  return cudaLaunchKernelEx(&pc.cfg, kernel_for(G.d, G.center_keys != 0), G, calls, level, stats, tok_shift,
+  return cudaLaunchKernelEx(&pc.cfg, kernel_for(G.d, G.center_keys != 0, reuse_tiles(G, std::min(n_calls, sm_count))), G, calls, level, stats, tok_shift,
                             eta, dbg_eta, dbg_S, dbg_p, fail_count, status, G.center_keys ? nullptr : A.nrm, Af, tm->k, tm->v);
 }
 

@@ -28,7 +28,7 @@ def _run(cuda_lib, d, dtype, t, T, center, tol, walk_kernel, **kw):
 
 
 @pytest.mark.parametrize("d", [64, 128])
-@pytest.mark.parametrize("t,T,center", [(128, 1, 0), (192, 2, 0), (192, 1, 1), (320, 1, 0), (1088, 1, 0), (2048, 1, 0)])
+@pytest.mark.parametrize("t,T,center", [(128, 1, 0), (192, 2, 0), (192, 1, 1), (320, 1, 0), (1088, 1, 0), (2048, 1, 0), (2560, 1, 0)])
 def test_tensor_core_walk_with_ragged_panels(cuda_lib, d, t, T, center):
     """Whole panels and a last panel of 64 tokens; d = 64 operands are a single 64-dim box."""
     _run(cuda_lib, d, "bf16", t, T, center, 5e-4 if center else 2e-4, 2)
@@ -61,5 +61,29 @@ def test_cuda_core_walk_in_groups_of_calls(cuda_lib):
         one.compress()
         assert all(torch.equal(a, b) for a, b in zip(ctx.cache_view(0, 0, h), one.cache_view(0, 0, h))), h
     assert ctx.stats()["device_status"] == 0 and one.stats()["device_status"] == 0
+    ctx.close()
+    one.close()
+
+
+def test_tensor_core_walk_beyond_l2(cuda_lib):
+    """Resident calls whose rows exceed L2 (148 of 2048 tokens) take the column order that reuses tiles; against the walk of each
+    stream alone, which does not.  Sums of 2048 terms in another order differ by about 1e-6 of a threshold range of 2 c: for the
+    8192 decisions compared, a chance of 1 in 100 that one flips, the same in every run of these inputs."""
+    import torch
+
+    S, t, d = 150, 2048, 128
+    gen = torch.Generator(device="cuda").manual_seed(11)
+    K = (0.3 * torch.randn(1, S, t, d, device="cuda", generator=gen)).bfloat16()
+    V = torch.randn(1, S, t, d, device="cuda", generator=gen).bfloat16()
+    make = lambda: cuda_lib.Context(n_seqs=1, n_layers=1, n_kv_heads=S, n_q_heads=S, head_dim=d, dtype="bf16", block=t, levels=1,
+                                    max_tokens=t, seed=3, c_override=0.75)
+    ctx, one = make(), make()
+    ctx.stream_append_layer(0, K, V)
+    ctx.compress()
+    for h in (0, 1, S // 2, S - 1):
+        one.stream_append(0, 0, h, K[0, h], V[0, h])
+        one.compress()
+        assert all(torch.equal(a, b) for a, b in zip(ctx.cache_view(0, 0, h), one.cache_view(0, 0, h))), h
+    assert ctx.stats()["device_status"] == 0 and ctx.stats()["walk_kernel"] == 2 and one.stats()["device_status"] == 0
     ctx.close()
     one.close()

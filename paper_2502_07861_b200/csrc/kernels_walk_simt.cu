@@ -362,6 +362,7 @@ walk_kernel(Geom G, const CallSet calls, int call0, int level, const float* __re
 }
 
 size_t walk_smem(int t, int stages) { return (size_t)stages * kTileBytes + sizeof(float) * (2 * t + 2 * kTile) + 2 * kWalkStages * sizeof(uint64_t); }
+constexpr int kMaxTokens = 4096;                         // largest block of a context
 int walk_stages(int tiles) { return std::min(kWalkStages, tiles); }
 
 template <typename E, int D, int RM>
@@ -399,7 +400,8 @@ cudaError_t launch_walk_simt(const Geom& G, const Arena& A, const CallSet& calls
                              cudaStream_t st) {
   const int tiles = (int)(walk_simt_bytes(G.t) / kTileBytes), stages = walk_stages(tiles);
   const size_t smem = walk_smem(G.t, stages);
-  cudaError_t e = cudaFuncSetAttribute(walk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // one limit for every block: it belongs to the function, and another thread's context may be launching it
+  cudaError_t e = cudaFuncSetAttribute(walk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)walk_smem(kMaxTokens, kWalkStages));
   if (!G.center_keys) tok_shift = nullptr;
   for (int call0 = 0; call0 < n_calls && e == cudaSuccess; call0 += ws_calls) {
     const int n = std::min(ws_calls, n_calls - call0);

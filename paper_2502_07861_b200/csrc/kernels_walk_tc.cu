@@ -799,6 +799,15 @@ size_t tc_smem_bytes(int d, int t) {
   const size_t tp = (t + kTile - 1) / kTile * kTile;
   return 1024 + (d == 128 ? Smem<128>::kTilesEnd : Smem<64>::kTilesEnd) + tp * 9 + 2 * (kEpiGroups - 1) * kTile * 4 + 512;
 }
+constexpr size_t kMaxSmem = (size_t)227 * 1024;
+// What the largest block that a kernel of this head size takes needs: every such kernel's limit, so that contexts with other
+// blocks never lower it.  (A function's limit belongs to the device, not to the context that sets it.)
+int tc_smem_limit(int d) {
+  size_t most = 0;
+  for (int t = kTile; t <= 4096; t += 64)
+    if (tc_smem_bytes(d, t) <= kMaxSmem) most = tc_smem_bytes(d, t);
+  return (int)most;
+}
 // Tiles are reused where the rows that the resident CTAs visit exceed L2: only then are the loads what a tile waits for.  148
 // calls at d = 128, cycles per off-diagonal tile without and with reuse: 1340 and 1430 for 1024 tokens (78 MB; the epilogue
 // bounds both, and the order costs it some instructions), 1540 and 1460 for 2048 (155 MB).
@@ -818,7 +827,7 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
 // Calls of a single half panel (t = 64) stay on CUDA cores: the tensor cores would work on 64 rows of 128.
 bool walk_tc_supported(const Geom& G) {
   return G.is_bf16 && (G.d == 128 || G.d == 64) && G.t % 64 == 0 && G.t >= kTile &&
-         tc_smem_bytes(G.d, G.t) <= (size_t)227 * 1024;
+         tc_smem_bytes(G.d, G.t) <= kMaxSmem;
 }
 
 // Encodes the two tensor maps (K and V arenas viewed as [total_rows, d] bf16, boxes of
@@ -846,7 +855,7 @@ cudaError_t walk_tc_prepare(const Geom& G, const Arena& A, int64_t total_rows, v
     if (r != CUDA_SUCCESS) { delete tm; return cudaErrorInvalidValue; }
   }
   for (int i = 0; i < 4 && e == cudaSuccess; ++i)
-    e = cudaFuncSetAttribute(kernel_for(G.d, (i & 1) != 0, i > 1), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem_bytes(G.d, G.t));
+    e = cudaFuncSetAttribute(kernel_for(G.d, (i & 1) != 0, i > 1), cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem_limit(G.d));
   if (e != cudaSuccess) { delete tm; return e; }
   *tmaps_out = tm;
   return cudaSuccess;

@@ -87,3 +87,30 @@ def test_tensor_core_walk_beyond_l2(cuda_lib):
     assert ctx.stats()["device_status"] == 0 and ctx.stats()["walk_kernel"] == 2 and one.stats()["device_status"] == 0
     ctx.close()
     one.close()
+
+
+@pytest.mark.parametrize("d,dtype,large,small", [(128, "bf16", 3072, 128), (64, "bf16", 4096, 192), (64, "fp32", 4096, 64)])
+def test_contexts_with_other_blocks_live_side_by_side(cuda_lib, d, dtype, large, small):
+    """A kernel's shared-memory limit belongs to the device: the context with the large blocks compresses after one with
+    small blocks was created and used, and keeps what it keeps alone."""
+    import torch
+
+    def make(t):
+        return cuda_lib.Context(n_seqs=1, n_layers=1, n_kv_heads=1, n_q_heads=1, head_dim=d, dtype=dtype, block=t, levels=1,
+                                max_tokens=t, seed=2, c_override=0.75)
+
+    def compress(ctx):
+        gen = torch.Generator(device="cuda").manual_seed(3)
+        K, V = (0.3 * torch.randn(1, 1, ctx.cfg.block, d, device="cuda", generator=gen).to(ctx.dtype) for _ in range(2))
+        ctx.reset()
+        ctx.stream_append_layer(0, K, V)
+        ctx.compress()
+        return ctx.cache_view(0, 0, 0)
+
+    a = make(large)
+    alone = compress(a)
+    b = make(small)
+    compress(b)
+    assert all(torch.equal(x, y) for x, y in zip(alone, compress(a)))
+    a.close()
+    b.close()

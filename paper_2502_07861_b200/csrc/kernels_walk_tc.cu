@@ -21,9 +21,9 @@
 // thread and its own barriers, so that one product's waits and commits overlap the other's
 // MMAs.  Operands live in three slots (K tile + V tile; 64 KB at d = 128) that rotate roles: one holds the panel's rows,
 // the column tiles stream through the other two, and the next panel's rows are fetched behind the last columns, so that its
-// first products are already in TMEM when the walk of the diagonal tile ends.  Where the rows of the resident calls exceed
-// L2, a panel begins with the two tiles that the one before left in shared memory: 107 loads instead of 136 for 2048 tokens,
-// 183 -> 169 us for 148 such calls.
+// first products are already in TMEM when the walk of the diagonal tile ends.  From 1792 tokens on (reuse_tiles) a panel
+// begins with the two tiles that the one before left in shared memory: 107 loads instead of 136 for 2048 tokens, 181 -> 169 us
+// for 148 such calls.
 // Inside a slot every operand is two boxes of 64 dims with their own full/empty barriers: a box is
 // refilled as soon as the four MMAs that read it have retired.
 // Ghat never touches global memory.
@@ -808,10 +808,12 @@ int tc_smem_limit(int d) {
     if (tc_smem_bytes(d, t) <= kMaxSmem) most = tc_smem_bytes(d, t);
   return (int)most;
 }
-// Tiles are reused where the rows that the resident CTAs visit exceed L2: only then are the loads what a tile waits for.  148
-// calls at d = 128, cycles per off-diagonal tile without and with reuse: 1340 and 1430 for 1024 tokens (78 MB; the epilogue
-// bounds both, and the order costs it some instructions), 1540 and 1460 for 2048 (155 MB).
-bool reuse_tiles(const Geom& G, int ctas) { return G.d == 128 && (int64_t)ctas * G.t * G.d * 4 > (int64_t)126 << 20; }
+// The order of a panel's columns is the order of summation of S_j, so it follows from the block alone: a call keeps the same
+// tokens whatever else shares its launch.  Tiles are reused from 1792 tokens on, where the rows of one call per SM exceed L2
+// (148 x 1792 x 512 bytes against 126 MB).  Ascending order / reuse, us per launch: 2048 tokens, 1 call 132.4 / 128.4, 148
+// calls 181 / 169, 1024 calls 1265 / 1185; 3072 tokens, 148 calls 428 / 388.
+constexpr int kReuseTokens = 1792;
+bool reuse_tiles(const Geom& G) { return G.d == 128 && G.t >= kReuseTokens; }
 auto kernel_for(int d, bool center, bool reuse) {
   if (d == 64) return center ? walk_tc_kernel<64, true, false> : walk_tc_kernel<64, false, false>;
   if (reuse) return center ? walk_tc_kernel<128, true, true> : walk_tc_kernel<128, false, true>;
@@ -866,7 +868,7 @@ void walk_tc_release(void* tmaps) { delete static_cast<TensorMaps*>(tmaps); }
 cudaError_t launch_walk_tc(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, int level,
                            const CallStat* stats, const float* tok_shift, int8_t* eta, int8_t* dbg_eta,
                            float* dbg_S, float* dbg_p, unsigned long long* fail_count, int* status,
-                           const void* tmaps, const void* fuse_compaction, int sm_count, cudaStream_t st) {
+                           const void* tmaps, const void* fuse_compaction, cudaStream_t st) {
   if (n_calls <= 0) return cudaSuccess;
   if (!tmaps) return cudaErrorInvalidValue;
   const TensorMaps* tm = static_cast<const TensorMaps*>(tmaps);
@@ -874,7 +876,7 @@ cudaError_t launch_walk_tc(const Geom& G, const Arena& A, const CallSet& calls, 
   Arena Af = A;                       // K == nullptr: leave selection and compaction to the separate kernel
   if (!fuse_compaction) Af.K = nullptr;
   const PdlConfig pc(dim3(n_calls), kThreads, smem, st);
-  return cudaLaunchKernelEx(&pc.cfg, kernel_for(G.d, G.center_keys != 0, reuse_tiles(G, std::min(n_calls, sm_count))), G, calls, level, stats, tok_shift,
+  return cudaLaunchKernelEx(&pc.cfg, kernel_for(G.d, G.center_keys != 0, reuse_tiles(G)), G, calls, level, stats, tok_shift,
                             eta, dbg_eta, dbg_S, dbg_p, fail_count, status, G.center_keys ? nullptr : A.nrm, Af, tm->k, tm->v);
 }
 

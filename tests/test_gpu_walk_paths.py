@@ -66,9 +66,7 @@ def test_cuda_core_walk_in_groups_of_calls(cuda_lib):
 
 
 def test_tensor_core_walk_beyond_l2(cuda_lib):
-    """Resident calls whose rows exceed L2 (148 of 2048 tokens) take the column order that reuses tiles; against the walk of each
-    stream alone, which does not.  Sums of 2048 terms in another order differ by about 1e-6 of a threshold range of 2 c: for the
-    8192 decisions compared, a chance of 1 in 100 that one flips, the same in every run of these inputs."""
+    """Resident calls whose rows exceed L2 (148 of 2048 tokens) keep what the walk of each stream alone keeps."""
     import torch
 
     S, t, d = 150, 2048, 128
@@ -114,3 +112,33 @@ def test_contexts_with_other_blocks_live_side_by_side(cuda_lib, d, dtype, large,
     assert all(torch.equal(x, y) for x, y in zip(alone, compress(a)))
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("t", [1728, 1792, 2048])
+def test_sums_do_not_depend_on_the_launch(cuda_lib, t):
+    """The running correlations S_j of a call, bit for bit: alone and among 150 calls, on both sides of the block size where
+    the order of the columns changes.  (Sums in another order differ in their last bits, and a token near its threshold then
+    falls differently.)"""
+    import torch
+
+    S, d = 150, 128
+    gen = torch.Generator(device="cuda").manual_seed(t)
+    K = (0.3 * torch.randn(1, S, t, d, device="cuda", generator=gen)).bfloat16()
+    V = torch.randn(1, S, t, d, device="cuda", generator=gen).bfloat16()
+    pair = []
+    for _ in range(2):
+        ctx = cuda_lib.Context(n_seqs=1, n_layers=1, n_kv_heads=S, n_q_heads=S, head_dim=d, dtype="bf16", block=t, levels=1,
+                               max_tokens=t, seed=3, c_override=0.75)
+        ctx.debug_enable()
+        pair.append(ctx)
+    pair[0].stream_append_layer(0, K, V)
+    pair[0].compress()
+    for h in (0, 77, S - 1):
+        pair[1].stream_append(0, 0, h, K[0, h], V[0, h])
+        pair[1].compress()
+        (eta, sums, p), alone = (ctx.debug_call(0, 0, h, 0, 0) for ctx in pair)
+        assert torch.equal(sums, alone[1]) and torch.equal(eta, alone[0]) and torch.equal(p, alone[2]), h
+        assert float(sums.abs().max()) > 1e-3           # sums of something
+    for ctx in pair:
+        assert ctx.stats()["device_status"] == 0 and ctx.stats()["walk_kernel"] == 2
+        ctx.close()

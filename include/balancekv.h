@@ -173,16 +173,19 @@ int balancekv_decode_attn_host(balancekv_ctx* ctx, int layer, const void* q_host
  * first call on a device -- of this function or of balancekv_decode_attn_static_status,
  * whichever host thread gets there first -- looks up the arrays' device addresses
  * (cudaGetSymbolAddress) and initialises them synchronously; make that first
- * call outside any stream capture.  Calls take the blocks in turn: of calls that overlap on the GPU (different
- * CUDA streams) more than four race on them -- issue the calls on one stream. */
+ * call outside any stream capture.  The first three CUDA streams of a device that call have a block of their own until
+ * the process exits: their calls may overlap.  Calls on any other stream, and captured calls, share the fourth block:
+ * order them (with events, or on one stream), graph replays included.  A call that meets another in a block gives
+ * wrong results, and so do later ones until balancekv_decode_attn_static_status has emptied it. */
 int balancekv_decode_attn_static(const void* K, const void* V, int n_streams, int cache_len, int n_heavy,
                                  int level, const void* q, void* out, int group, int head_dim, int dtype,
                                  void* stream);
 /* The entry point above returns before its kernel has run, so a bounded device-side wait that
  * gives up cannot show in its return value; it sets a status word in the built-in array
  * instead, which this call copies to *status_host (0 = fine, 1 = a wait gave up since the last
- * read; the outputs of that launch and of later ones are then not valid) and clears, the scratch with it.  Allocates nothing;
- * synchronises `stream`.  The paper has no counterpart. */
+ * read; the outputs of that launch and of later ones are then not valid) and clears.  It empties the scratch: the block of
+ * `stream` and the shared one -- it counts as one of the calls that the shared block's users order --, and with
+ * status 1 all of it.  Allocates nothing; synchronises `stream`, with status 1 the device.  The paper has no counterpart. */
 int balancekv_decode_attn_static_status(int* status_host, void* stream);
 
 /* Load an already-compressed set into level `level` of every stream of one layer

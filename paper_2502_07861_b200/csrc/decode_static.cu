@@ -33,18 +33,20 @@ namespace {
 // and ticket words of its streams would fill (balancekv.h states the formula).
 constexpr size_t kStaticBytes = (size_t)8 << 20;
 // Split-K rows, whose words are their own arrival flags: all of them hold the empty pattern between launches, and
-// every launch puts it back.  Four blocks, used in turn, so that calls on different
-// CUDA streams do not meet in one unless more than four of them overlap.  A block holds the rows of 2 x 148 CTAs with
+// every launch puts it back.  Launches that overlap must not meet in a block, so the block follows from the CUDA stream,
+// whose launches never overlap: the first streams that call get one of their own, all others and captured calls (a
+// graph may be replayed on any stream) share the last one and are ordered by the caller.  (Blocks taken in turn would let a
+// call on one stream meet the fourth call issued after it on another.)  A block holds the rows of 2 x 148 CTAs with
 // tiles (1.3 MB at 8 heads) and of most launches that split more streams than that; the split factor follows the room.
 constexpr size_t kRowBlockBytes = (size_t)22 << 17;
-constexpr int kRowBlocks = 4;
+constexpr int kOwnBlocks = 3, kRowBlocks = kOwnBlocks + 1;
 static __device__ __align__(256) unsigned char g_static_rows[kRowBlocks * kRowBlockBytes];
 static __device__ int g_static_status;
 
 constexpr int kMaxDevices = 64;
 unsigned char* g_rows_addr[kMaxDevices] = {};       // device addresses of the arrays, per device
 int* g_status_addr[kMaxDevices] = {};
-std::atomic<unsigned> g_next_rows[kMaxDevices];
+std::atomic<unsigned long long> g_block_owner[kMaxDevices][kOwnBlocks];   // stream number + 1; 0: not taken yet
 int g_sm_count[kMaxDevices] = {};
 std::once_flag g_setup_once[kMaxDevices];           // the per-device set-up runs once, whichever host thread comes first
 cudaError_t g_setup_err[kMaxDevices] = {};
@@ -83,6 +85,29 @@ int static_device(int* dev_out) {
   }
   *dev_out = dev;
   return BALANCEKV_OK;
+}
+
+// The block of the calls on st (take: a first call takes one that is free).  The stream's number is unique in the process,
+// unlike its handle.
+cudaError_t row_block(int dev, cudaStream_t st, bool take, float** rows) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  cudaError_t e = cudaStreamIsCapturing(st, &cap);
+  if (e == cudaErrorStreamCaptureImplicit) {          // the legacy stream while another one is captured: the launch will say so
+    (void)cudaGetLastError();
+    e = cudaSuccess;
+  }
+  int block = kOwnBlocks;
+  if (e == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
+    unsigned long long id = 0;
+    e = cudaStreamGetId(st, &id);
+    for (int b = 0; b < kOwnBlocks && e == cudaSuccess; ++b) {
+      unsigned long long owner = g_block_owner[dev][b].load(std::memory_order_relaxed);
+      if (owner == 0 && take && g_block_owner[dev][b].compare_exchange_strong(owner, id + 1)) owner = id + 1;
+      if (owner == id + 1) { block = b; break; }
+    }
+  }
+  *rows = reinterpret_cast<float*>(g_rows_addr[dev] + block * kRowBlockBytes);
+  return e;
 }
 
 }  // namespace
@@ -144,12 +169,13 @@ extern "C" int balancekv_decode_attn_static(const void* K, const void* V, int n_
   ap.splits = plan.splits;
   ap.inline_combine = plan.inline_combine;
   while (ap.splits > 1 && decode_scratch_bytes(G, ap.splits) > kRowBlockBytes) --ap.splits;
-  const unsigned block = g_next_rows[dev].fetch_add(1, std::memory_order_relaxed) % kRowBlocks;
-  float* rows = reinterpret_cast<float*>(g_rows_addr[dev] + block * kRowBlockBytes);
   const Arena A{const_cast<void*>(K), const_cast<void*>(V), nullptr, nullptr, nullptr};
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const cudaError_t e = dtype == 1 ? launch_decode_static_mma(G, A, ap, q, out, rows, g_status_addr[dev], st)
-                                   : launch_decode(G, A, 0, q, out, rows, ap, g_status_addr[dev], st);
+  float* rows = nullptr;
+  cudaError_t e = row_block(dev, st, true, &rows);
+  if (e == cudaSuccess)
+    e = dtype == 1 ? launch_decode_static_mma(G, A, ap, q, out, rows, g_status_addr[dev], st)
+                   : launch_decode(G, A, 0, q, out, rows, ap, g_status_addr[dev], st);
   if (e != cudaSuccess) {
     std::fprintf(stderr, "balancekv_decode_attn_static: launch failed: %s\n", cudaGetErrorString(e));
     return BALANCEKV_E_CUDA;
@@ -167,10 +193,17 @@ extern "C" int balancekv_decode_attn_static_status(int* status_host, void* strea
   if (cudaMemcpyAsync(&v, g_status_addr[dev], sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess) return BALANCEKV_E_CUDA;
   if (cudaMemsetAsync(g_status_addr[dev], 0, sizeof(int), st) != cudaSuccess) return BALANCEKV_E_CUDA;
   if (cudaStreamSynchronize(st) != cudaSuccess) return BALANCEKV_E_CUDA;
-  // a launch that gave up may have left partial rows behind
-  if (v != 0 && (cudaMemsetAsync(g_rows_addr[dev], 0xff, kRowBlocks * kRowBlockBytes, st) != cudaSuccess ||
-                 cudaStreamSynchronize(st) != cudaSuccess))
+  // Words left behind are emptied: after a wait that gave up all of them, with no launch in flight; else those of the block
+  // that this stream's calls use, which are idle now, and the shared block's.
+  float* own = nullptr;
+  if (v != 0) {
+    if (cudaDeviceSynchronize() != cudaSuccess || cudaMemsetAsync(g_rows_addr[dev], 0xff, kRowBlocks * kRowBlockBytes, st) != cudaSuccess)
+      return BALANCEKV_E_CUDA;
+  } else if (row_block(dev, st, false, &own) != cudaSuccess || cudaMemsetAsync(own, 0xff, kRowBlockBytes, st) != cudaSuccess ||
+             cudaMemsetAsync(g_rows_addr[dev] + kOwnBlocks * kRowBlockBytes, 0xff, kRowBlockBytes, st) != cudaSuccess) {
     return BALANCEKV_E_CUDA;
+  }
+  if (cudaStreamSynchronize(st) != cudaSuccess) return BALANCEKV_E_CUDA;
   *status_host = v;
   return BALANCEKV_OK;
 }

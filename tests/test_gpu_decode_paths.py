@@ -108,3 +108,43 @@ def test_cuda_core_decode(cuda_lib, dtype, d, g, splits, n_heavy, n_tail):
         _check_heads(out.reshape(1, H * g, d), K[:, :, :n], V[:, :, :n], w[:n], q, g, dtype, "static")
         assert cuda_lib.decode_attn_static_status() == 0
     ctx.close()
+
+
+def test_static_decode_on_overlapping_streams(cuda_lib):
+    """Calls that overlap never share split rows: a long call on one stream beside many short ones on two others (no other
+    test of this process takes a block but for the default stream's), and a captured call replayed in order with calls of
+    four more streams.  Bit for bit the results of the calls alone."""
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    more = [torch.cuda.Stream() for _ in range(4)]
+    for dtype in (torch.bfloat16, torch.float32):
+        gen = torch.Generator(device="cuda").manual_seed(8)
+        make = lambda S, n, g: tuple(torch.randn(*s, 128, device="cuda", generator=gen).to(dtype) for s in ((S, n), (S, n), (S, g)))
+        big, small = make(100, 16384, 4), [make(2, 2048 + 64 * i, 4) for i in range(8)]
+        run = lambda x, out=None: cuda_lib.decode_attn_static(x[0], x[1], 1024, 1, x[2], out)
+        want_big, want = run(big), [run(x) for x in small]
+        torch.cuda.synchronize()
+        for rep in range(5):
+            with torch.cuda.stream(streams[0]):
+                got_big = run(big)
+            got = []
+            for i in range(24):
+                with torch.cuda.stream(streams[1] if i % 3 else torch.cuda.default_stream()):
+                    got.append(run(small[i % 8]))
+            torch.cuda.synchronize()
+            assert torch.equal(got_big, want_big), (dtype, rep)
+            assert all(torch.equal(got[i], want[i % 8]) for i in range(24)), (dtype, rep)
+        out = torch.empty_like(small[0][2])
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            run(small[0], out)
+        for rep in range(2):
+            for i, st in enumerate(more):
+                with torch.cuda.stream(st):
+                    got = run(small[i])
+                st.synchronize()
+                assert torch.equal(got, want[i]), (dtype, rep, i)
+                out.zero_()
+                graph.replay()
+                torch.cuda.synchronize()
+                assert torch.equal(out, want[0]), (dtype, rep, i)
+    assert all(cuda_lib.decode_attn_static_status(st) == 0 for st in [None, *streams, *more])

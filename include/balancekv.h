@@ -326,6 +326,11 @@ int balancekv_debug_set_status(balancekv_ctx* ctx, int value);
  * every launch).  Synchronises the device.  words: host pointer. */
 int balancekv_debug_scratch_used(balancekv_ctx* ctx, int64_t* words);
 
+/* Testing aid: what a decode launch does when the partial results of split `missing` (of the context's largest split
+ * factor; -1: none) arrive only after the combining warps' bounded wait has run out: the status word is set, and the late
+ * words stay behind in the scratch.  Contexts whose decode kernel is 2 (balancekv_stats).  Synchronises the device. */
+int balancekv_debug_late_split(balancekv_ctx* ctx, int missing);
+
 /* Synchronises the device.  Returns BALANCEKV_E_TIMEOUT (record filled) if a device-side wait gave up. */
 int balancekv_stats(balancekv_ctx* ctx, balancekv_stats_t* out);
 const char* balancekv_strerror(int code);

@@ -25,6 +25,7 @@ EXPORTS = [
     "balancekv_stream_step", "balancekv_stream_step_host", "balancekv_stream_append_layer_keys",
     "balancekv_decode_attn_two", "balancekv_decode_attn_merged", "balancekv_stream_append_bucketed",
     "balancekv_stream_append_layer_bucketed", "balancekv_stream_append_layer_preserving", "balancekv_debug_set_status", "balancekv_decode_attn_static_status", "balancekv_debug_scratch_used",
+    "balancekv_debug_late_split",
 ]
 PROFILE_CLASSES = ("append", "radii", "gram_walk", "compact", "decode", "bookkeeping")
 
@@ -99,6 +100,7 @@ def load():
     lib.balancekv_decode_attn_static.argtypes = [vp, vp, ci, ci, ci, ci, vp, vp, ci, ci, ci, vp]
     lib.balancekv_decode_attn_static_status.argtypes = [vp, vp]
     lib.balancekv_debug_set_status.argtypes = [vp, ci]
+    lib.balancekv_debug_late_split.argtypes = [vp, ci]
     lib.balancekv_debug_scratch_used.argtypes = [vp, C.POINTER(C.c_int64)]
     for name in EXPORTS:
         if name != "balancekv_strerror":
@@ -371,6 +373,10 @@ class Context:
         n = C.c_int64(0)
         _check(self.lib.balancekv_debug_scratch_used(self._h, C.byref(n)), "balancekv_debug_scratch_used")
         return int(n.value)
+
+    def debug_late_split(self, missing):
+        """Testing aid: combine a head whose split ``missing`` (-1: none) arrives after the bounded wait has run out."""
+        _check(self.lib.balancekv_debug_late_split(self._h, int(missing)), "balancekv_debug_late_split")
 
     def debug_set_status(self, value):
         """Testing aid: overwrite the device status word (1 = a bounded wait gave up)."""

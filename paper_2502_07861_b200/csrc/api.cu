@@ -35,6 +35,8 @@ cudaError_t launch_merged_ratio(const float* acc, const float* ml, int n_parts, 
                                 void* out, int n_heads, int d, cudaStream_t st);
 cudaError_t launch_decode_step_mma(const Geom& G, const Arena& A, int layer, const void* q, void* out, float* scratch,
                                    const StepAppend& ap, int* status, const void* maps, cudaStream_t st);
+cudaError_t launch_combine_without(const Geom& G, const Arena& A, int splits, int missing, void* out, float* scratch, int* status,
+                                   cudaStream_t st);
 }  // namespace bkv
 
 #define BKV_CUDA(expr)                                                                    \
@@ -1395,6 +1397,19 @@ int balancekv_debug_set_status(balancekv_ctx* c, int value) {
   BKV_CUDA(cudaDeviceSynchronize());
   BKV_CUDA(cudaMemcpy(c->d_status, &value, sizeof(int), cudaMemcpyHostToDevice));
   *c->h_status = value;
+  return BALANCEKV_OK;
+}
+
+int balancekv_debug_late_split(balancekv_ctx* c, int missing) {
+  if (!c || !c->decode_maps || missing < -1 || missing >= c->max_splits) return BALANCEKV_E_INVAL;
+  BKV_CUDA(cudaDeviceSynchronize());
+  c->decode_chain = false;
+  void* out = nullptr;
+  BKV_CUDA(cudaMalloc(&out, (size_t)c->cfg.head_dim * c->esz));
+  const cudaError_t e = launch_combine_without(c->G, c->A, c->max_splits, missing, out, c->d_decode_scratch, c->d_status, nullptr);
+  cudaDeviceSynchronize();
+  cudaFree(out);
+  BKV_CUDA(e);
   return BALANCEKV_OK;
 }
 

@@ -461,7 +461,7 @@ struct HeadEnd {
       if (!pending) break;
       if (clock64() - t0 > kDecodeWaitCycles) { ok = false; break; }
     }
-    __syncwarp();
+    ok = __all_sync(0xffffffffu, ok);            // every lane polls words of its own, and any of them may have given up
     const float M = warp_max(fmaxf(ml[0].x, ml[1].x));
     const float f0 = ml[0].x == -INFINITY ? 0.f : fast_exp2(ml[0].x - M);
     const float f1 = ml[1].x == -INFINITY ? 0.f : fast_exp2(ml[1].x - M);

@@ -506,6 +506,16 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
   }
 }
 
+// Testing aid: the combine of one head of one stream, alone.
+template <int D>
+__global__ void __launch_bounds__(kThreads)
+combine_kernel(Geom G, Arena A, __nv_bfloat16* __restrict__ out, float* __restrict__ part, int* __restrict__ status, const StepAppend ap) {
+  __shared__ float fac[kWarps][kDecodeMaxSplits];
+  const int warp = threadIdx.x >> 5;
+  const HeadEnd<__nv_bfloat16, D> end{G, A, ap, nullptr, out, nullptr, nullptr, 0, 0, 1, warp, (int)threadIdx.x & 31, 1.f};
+  end.combine_head(0, part, 1, fac[warp], status);
+}
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -561,6 +571,29 @@ cudaError_t launch(const Geom& G, const Arena& A, int layer, const void* q, void
 }
 
 }  // namespace
+
+// Testing aid: combines one head over `splits` splits of which all have arrived but `missing`.  The rows are those of a launch
+// with one stream and one head; `out`: a result row.  Afterwards the split's words arrive late.
+cudaError_t launch_combine_without(const Geom& G, const Arena& A, int splits, int missing, void* out, float* scratch, int* status,
+                                   cudaStream_t st) {
+  StepAppend ap{};
+  ap.splits = splits;
+  const int copies = G.d / 32;
+  auto arrive = [&](int sp) {
+    cudaError_t e = cudaMemsetAsync(scratch + (size_t)sp * G.d, 0, sizeof(float) * G.d, st);
+    for (int c = 0; c < copies && e == cudaSuccess; ++c)
+      e = cudaMemsetAsync(scratch + (size_t)splits * G.d + ((size_t)c * splits + sp) * 2, 0, 2 * sizeof(float), st);
+    return e;
+  };
+  cudaError_t e = cudaSuccess;
+  for (int sp = 0; sp < splits && e == cudaSuccess; ++sp)
+    if (sp != missing) e = arrive(sp);
+  if (e != cudaSuccess) return e;
+  if (G.d == 128) combine_kernel<128><<<1, kThreads, 0, st>>>(G, A, static_cast<__nv_bfloat16*>(out), scratch, status, ap);
+  else combine_kernel<64><<<1, kThreads, 0, st>>>(G, A, static_cast<__nv_bfloat16*>(out), scratch, status, ap);
+  e = cudaGetLastError();
+  return e != cudaSuccess || missing < 0 || missing >= splits ? e : arrive(missing);
+}
 
 bool decode_mma_supported(const Geom& G) { return G.is_bf16 && (G.d == 128 || G.d == 64) && G.g <= 8; }
 int decode_mma_tile_tokens() { return kTN; }

@@ -148,3 +148,24 @@ def test_static_decode_on_overlapping_streams(cuda_lib):
                 torch.cuda.synchronize()
                 assert torch.equal(out, want[0]), (dtype, rep, i)
     assert all(cuda_lib.decode_attn_static_status(st) == 0 for st in [None, *streams, *more])
+
+
+@pytest.mark.parametrize("d", [128, 64])
+def test_combine_reports_any_split_that_does_not_arrive(cuda_lib, d):
+    """Each lane of a combining warp waits for words of its own; whichever split is missing, the status word says so, and
+    reset makes the context usable again."""
+    ctx = cuda_lib.Context(n_seqs=1, n_layers=1, n_kv_heads=1, n_q_heads=1, head_dim=d, dtype="bf16", block=64, levels=1, max_tokens=4096)
+    ctx.debug_late_split(-1)
+    assert ctx.stats()["device_status"] == 0 and ctx.debug_scratch_used() == 0
+    K = torch.randn(1, 1, 4096, d, device="cuda").bfloat16()
+    for missing in (0, 1, 2, 5, 31, 32, 33, 63):
+        ctx.debug_late_split(missing)
+        assert ctx.stats()["device_status"] == 1, missing
+        ctx.reset()
+        assert ctx.stats()["device_status"] == 0 and ctx.debug_scratch_used() == 0, missing
+    ctx.stream_append_layer(0, K, K)
+    q = torch.randn(1, 1, d, device="cuda").bfloat16()
+    out = ctx.decode_attn(0, q).float().cpu().numpy()
+    k = K[0, 0].float().cpu().numpy()
+    _check(out[0], oracle.weighted_attention(k, k, np.ones(4096), q[0].float().cpu().numpy()), "bf16", d)
+    ctx.close()

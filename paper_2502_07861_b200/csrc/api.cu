@@ -362,7 +362,7 @@ int balancekv_create(const balancekv_config* cfg, balancekv_ctx** out) {
     if (G.center_keys && (rc = dev_alloc(c, &c->d_tokshift, (size_t)c->max_calls * t + 64))) return fail(rc);
   }
   if ((rc = dev_alloc(c, &c->d_fail, 1))) return fail(rc);
-  if ((rc = dev_alloc(c, &c->d_status, 2))) return fail(rc);       // the word, and the counter of launch_reset
+  if ((rc = dev_alloc(c, &c->d_status, 1))) return fail(rc);
   if (cudaMemset(c->d_fail, 0, 256) != cudaSuccess || cudaMemset(c->d_status, 0, 256) != cudaSuccess) return fail(BALANCEKV_E_CUDA);
   if (cudaMallocHost(reinterpret_cast<void**>(&c->h_status), 64) != cudaSuccess) return fail(BALANCEKV_E_NOMEM);
   if (cudaHostGetDevicePointer(reinterpret_cast<void**>(&c->h_status_dev), c->h_status, 0) != cudaSuccess) return fail(BALANCEKV_E_CUDA);
@@ -1325,12 +1325,13 @@ int balancekv_reset(balancekv_ctx* c, void* stream) {
   for (StreamState& S : c->st) S = StreamState();
   c->bucket_vmax2.clear();
   c->bucket_erase_max.clear();
-  // one kernel: the segment table, and -- where a device-side wait has given up -- the split-K scratch and the status word,
-  // so that the context becomes usable again
+  // one kernel: the segment table, the split-K scratch and the status word, so that a context whose device-side wait has
+  // given up becomes usable again
   *c->h_status = 0;
   BKV_CUDA(launch_reset(c->A.seg, (size_t)c->n_streams * (c->cfg.levels + 1), c->d_decode_scratch,
-                        decode_scratch_bytes(c->G, c->max_splits) / 4, c->two_scratch,
-                        c->two_scratch ? c->two_scratch_words * BALANCEKV_MAX_MERGE : 0, c->d_status, c->h_status_dev, st));
+                        decode_scratch_bytes(c->G, c->max_splits), c->two_scratch,
+                        c->two_scratch ? c->two_scratch_words * 4 * BALANCEKV_MAX_MERGE : 0, c->d_status, c->h_status_dev,
+                        c->sm_count, st));
   c->kernels_launched++;
   return BALANCEKV_OK;
 }

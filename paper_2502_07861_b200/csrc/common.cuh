@@ -242,10 +242,10 @@ cudaError_t launch_move(const Geom& G, const Arena& A, const MoveDesc* descs, in
                         cudaStream_t st);
 cudaError_t launch_batch_end(const Geom& G, const Arena& A, const BatchEnd& E, int n_streams, const Seg* seg,
                              const int* status, int* status_host, cudaStream_t st);
-// Forget every stream (segment table) and, if a device-side wait has given up, restore the split-K scratch: n words of
-// `scratch` and n2 of `scratch2` (may be null).  status: the status word, behind it a zero word of scratch.
-cudaError_t launch_reset(Seg* seg, size_t n_seg, float* scratch, size_t n, float* scratch2, size_t n2, int* status,
-                         int* status_host, cudaStream_t st);
+// Forget every stream (segment table), empty the split-K scratch (`bytes` and `bytes2`, multiples of 16; scratch2 may be null)
+// and clear the status word.
+cudaError_t launch_reset(Seg* seg, size_t n_seg, void* scratch, size_t bytes, void* scratch2, size_t bytes2, int* status,
+                         int* status_host, int sm_count, cudaStream_t st);
 cudaError_t launch_center(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, CallStat* stats,
                           float* tok_shift, cudaStream_t st);
 cudaError_t launch_walk_simt(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, int level,

@@ -169,25 +169,20 @@ batch_end_kernel(Geom G, Arena A, BatchEnd E, SegRow row, const int* __restrict_
   }
 }
 
+// The split-K scratch is emptied whatever the status word says: a launch that gave up, or launches that met in it, may have
+// left partial rows behind.
 __global__ void __launch_bounds__(256)
-reset_kernel(Seg* __restrict__ seg, size_t n_seg, float* __restrict__ scratch, size_t n, float* __restrict__ scratch2, size_t n2,
+reset_kernel(Seg* __restrict__ seg, size_t n_seg, uint4* __restrict__ scratch, size_t n, uint4* __restrict__ scratch2, size_t n2,
              int* __restrict__ status, int* __restrict__ status_host) {
   grid_wait_and_release();
   const size_t i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x, step = (size_t)gridDim.x * blockDim.x;
   for (size_t i = i0; i < n_seg; i += step) seg[i] = Seg{0, 0};
-  if (*static_cast<volatile int*>(status) != kStatusOk) {      // a launch that gave up may have left partial rows behind
-    const float empty = __uint_as_float(0xffffffffu);
-    for (size_t i = i0; i < n; i += step) scratch[i] = empty;
-    for (size_t i = i0; i < n2; i += step) scratch2[i] = empty;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    if (atomicAdd(status + 1, 1) == (int)gridDim.x - 1) {      // every CTA has read the status word
-      status[0] = kStatusOk;
-      status[1] = 0;
-      *static_cast<volatile int*>(status_host) = kStatusOk;
-    }
+  const uint4 empty = make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu);
+  for (size_t i = i0; i < n; i += step) scratch[i] = empty;
+  for (size_t i = i0; i < n2; i += step) scratch2[i] = empty;
+  if (i0 == 0) {
+    *status = kStatusOk;
+    *static_cast<volatile int*>(status_host) = kStatusOk;
   }
 }
 
@@ -319,10 +314,12 @@ cudaError_t launch_batch_end(const Geom& G, const Arena& A, const BatchEnd& E, i
   return cudaLaunchKernelEx(&pc.cfg, batch_end_kernel, G, A, E, row, status, status_host);
 }
 
-cudaError_t launch_reset(Seg* seg, size_t n_seg, float* scratch, size_t n, float* scratch2, size_t n2, int* status,
-                         int* status_host, cudaStream_t st) {
-  const PdlConfig pc(dim3((unsigned)std::min<size_t>(148, (n_seg + 255) / 256 + 1)), 256, 0, st);
-  return cudaLaunchKernelEx(&pc.cfg, reset_kernel, seg, n_seg, scratch, n, scratch2, n2, status, status_host);
+cudaError_t launch_reset(Seg* seg, size_t n_seg, void* scratch, size_t bytes, void* scratch2, size_t bytes2, int* status,
+                         int* status_host, int sm_count, cudaStream_t st) {
+  const size_t n = bytes / 16, n2 = bytes2 / 16, most = std::max(std::max(n_seg, n), n2);
+  const PdlConfig pc(dim3((unsigned)std::min<size_t>(4 * sm_count, (most + 255) / 256)), 256, 0, st);
+  return cudaLaunchKernelEx(&pc.cfg, reset_kernel, seg, n_seg, static_cast<uint4*>(scratch), n, static_cast<uint4*>(scratch2), n2,
+                            status, status_host);
 }
 
 // stats must hold n_calls entries, tok_shift n_calls * t floats.

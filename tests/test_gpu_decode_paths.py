@@ -169,3 +169,21 @@ def test_combine_reports_any_split_that_does_not_arrive(cuda_lib, d):
     k = K[0, 0].float().cpu().numpy()
     _check(out[0], oracle.weighted_attention(k, k, np.ones(4096), q[0].float().cpu().numpy()), "bf16", d)
     ctx.close()
+
+
+@pytest.mark.parametrize("merged", [False, True])
+def test_reset_empties_the_split_scratch(cuda_lib, merged):
+    """Whatever the status word says: words that were left behind without a report would pass for the next launch's."""
+    ctx = cuda_lib.Context(n_seqs=1, n_layers=2, n_kv_heads=3, n_q_heads=15, head_dim=128, dtype="bf16", block=64, levels=1,
+                           max_tokens=4096)
+    if merged:                                        # the scratch of the decode merged over slots exists as well
+        K = torch.randn(1, 3, 500, 128, device="cuda").bfloat16()
+        for layer in range(2):
+            ctx.stream_append_layer(layer, K, K)
+        ctx.decode_attn_merged([0, 1], [0, 1], torch.randn(1, 15, 128, device="cuda").bfloat16())
+    ctx.debug_late_split(3)
+    ctx.debug_set_status(0)
+    assert ctx.debug_scratch_used() > 0
+    ctx.reset()
+    assert ctx.debug_scratch_used() == 0 and ctx.stats()["device_status"] == 0
+    ctx.close()

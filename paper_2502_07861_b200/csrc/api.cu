@@ -352,8 +352,8 @@ int balancekv_create(const balancekv_config* cfg, balancekv_ctx** out) {
   if (cudaMemset(c->A.nrm, 0, sizeof(float2) * (size_t)c->total_rows) != cudaSuccess) return fail(BALANCEKV_E_CUDA);
   if ((rc = dev_alloc(c, &c->A.seg, (size_t)c->n_streams * (T + 1)))) return fail(rc);
   if (cudaMemset(c->A.seg, 0, sizeof(Seg) * (size_t)c->n_streams * (T + 1)) != cudaSuccess) return fail(BALANCEKV_E_CUDA);
-  // rows that were never written must hold finite numbers: tiles of the decode kernels may
-  // cover rows past a segment's end, which are masked to weight zero but still multiplied
+  // rows that were never written read as zeros: tiles of the decode kernels may cover rows past a
+  // segment's end, whose scores and values are masked
   if (cudaMemset(c->A.K, 0, (size_t)c->total_rows * row_bytes) != cudaSuccess) return fail(BALANCEKV_E_CUDA);
   if (cudaMemset(c->A.V, 0, (size_t)c->total_rows * row_bytes) != cudaSuccess) return fail(BALANCEKV_E_CUDA);
   if (T > 0) {

@@ -24,9 +24,10 @@
 // stream is past its tiles, i.e. has finished reading the old segment table.
 // d = 64 takes this kernel too: on CUDA cores a launch over 8 streams x 2900 rows, 8 query heads each, took 24.6 us
 // (issue bound, and the last CTA of a stream summed the splits one load after the other), here 9.0 us.
-// Rows of a tile beyond a segment's end are masked in the scores; their V rows are whatever the stream's own region
-// holds there (zero-initialised at creation or finite older rows; zeros beyond the stream's last row: the tensor maps
-// have the stream as a dimension of their own) times an exact zero.
+// Rows of a tile beyond a segment's end (older rows of the stream, Inf and NaN among them; zeros beyond its last row: the
+// tensor maps have the stream as a dimension of their own) are masked in the scores, and the V operand has the last valid
+// row in their place.  (Zeros there instead, by masks on the loaded registers or by clearing the tile's rows, made a launch
+// over 24 streams x 5000 rows 0.25 and 0.6 us slower; this takes less than 0.1 of 14.5.)
 #include <cuda.h>
 
 #include "decode_common.cuh"
@@ -314,9 +315,11 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
       uint32_t va[kTB][kMB][4];
       if (!keys_only) {
 #pragma unroll
-        for (int tb = 0; tb < kTB; ++tb)
+        for (int tb = 0; tb < kTB; ++tb) {
+          const int tok = min(v_tok + 16 * tb, tr.rows - 1);    // past the segment's end its last row again, times zero
 #pragma unroll
-          for (int mb = 0; mb < kMB; ++mb) ldsm_x4_trans(Vt + tile_off(v_tok + 16 * tb, mb * 2 + v_chunk), va[tb][mb]);
+          for (int mb = 0; mb < kMB; ++mb) ldsm_x4_trans(Vt + tile_off(tok, mb * 2 + v_chunk), va[tb][mb]);
+        }
       }
       // this thread: per block tb the tokens tok0 (x[tb][0], x[tb][1]) and tok0 + 8 (x[tb][2], x[tb][3]),
       // heads 2 tq (even index) and 2 tq + 1

@@ -187,3 +187,37 @@ def test_reset_empties_the_split_scratch(cuda_lib, merged):
     ctx.reset()
     assert ctx.debug_scratch_used() == 0 and ctx.stats()["device_status"] == 0
     ctx.close()
+
+
+@pytest.mark.parametrize("dtype,d,g,n_heavy,n_tail", [("bf16", 64, 8, 65, 33), ("bf16", 64, 3, 1000, 1), ("bf16", 128, 5, 97, 31), ("bf16", 128, 4, 4100, 95),
+                                                      ("fp32", 64, 2, 65, 33), ("fp32", 128, 5, 97, 31)])
+def test_rows_of_an_earlier_request_have_no_part(cuda_lib, dtype, d, g, n_heavy, n_tail):
+    """A request whose rows held Inf and NaN leaves them behind the segments of the next one, in the tiles that the decode
+    kernels read: before and after the fused append, and merged over slots."""
+    H, T = 2, 2
+    ctx = cuda_lib.Context(n_seqs=1, n_layers=2, n_kv_heads=H, n_q_heads=H * g, head_dim=d, dtype=dtype, block=64, levels=T, max_tokens=20000)
+    bad = torch.empty(1, H, 2 * n_heavy + n_tail + 200, d, device="cuda", dtype=ctx.dtype)
+    bad[:, :, 0::3], bad[:, :, 1::3], bad[:, :, 2::3] = float("nan"), float("inf"), float("-inf")
+    for layer in range(2):
+        ctx.cache_load_level(layer, T, bad[:, :, :n_heavy + 100].contiguous(), bad[:, :, :n_heavy + 100].contiguous())
+        ctx.stream_append_layer(layer, bad, bad)
+    ctx.reset()
+    n = n_heavy + n_tail
+    K, V = synth.layer_kv("llama", 39, 0, 1, H, n + 2, d, dtype)
+    for layer in range(2):
+        ctx.cache_load_level(layer, T, to_device(K[:, :, :n_heavy], dtype), to_device(V[:, :, :n_heavy], dtype))
+        ctx.stream_append_layer(layer, to_device(K[:, :, n_heavy:n], dtype), to_device(V[:, :, n_heavy:n], dtype))
+    w = np.concatenate([np.full(n_heavy, 4.0), np.ones(n_tail + 2)])
+    for step in range(3):
+        q = synth.queries(39, 0, step, 1, H * g, d, dtype)
+        qt = to_device(q, dtype)
+        if step == 0 and dtype == "bf16" and d == 128:       # two slots with the same rows
+            _check_heads(ctx.decode_attn_merged([0, 1], [0, 1], qt).float().cpu().numpy(), K[:, :, :n], V[:, :, :n], w[:n], q, g, dtype, "merged")
+        m = n + step
+        if step == 0:
+            out = ctx.decode_attn(0, qt)
+        else:
+            out = ctx.stream_step(0, qt, to_device(K[:, :, m - 1], dtype), to_device(V[:, :, m - 1], dtype), qt.clone())
+        _check_heads(out.float().cpu().numpy(), K[:, :, :m], V[:, :, :m], w[:m], q, g, dtype, (g, step))
+    assert ctx.stats()["device_status"] == 0
+    ctx.close()

@@ -13,7 +13,7 @@
 // rounded up to a power of two).  For the scores LPT = 8 or 16 lanes share a token (16-byte pieces, conflict free) and
 // every lane sums LPT (token, head) pairs over its dims; LPT - 1 shuffles of a transposed reduction leave one score in
 // each lane, so that a batch costs one exponential per lane.  The probabilities go through 128 bytes of shared memory to
-// the value phase, where a lane owns d / 32 output columns.
+// the value phase, where a lane owns d / 32 output columns (zeros for tokens past the end: an exact zero times Inf is NaN).
 // Warps merge through shared memory; splits, the fused append and the result are HeadEnd's (decode_common.cuh).
 //
 // What bounds it: at batch sizes that fill the chip, instruction issue and HBM; otherwise the chain of one launch.
@@ -108,6 +108,7 @@ decode_kernel(Geom G, Arena A, int layer, const E* __restrict__ q, E* __restrict
   __shared__ int lvl_tiles[kMaxLevels + 1];
   __shared__ Seg seg_s[kMaxLevels + 1];
   __shared__ __align__(16) float probs[kWarps][32];   // read as float4
+  __shared__ __align__(16) unsigned char zero_row[kRowBytes];
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = G.g;
@@ -124,6 +125,7 @@ decode_kernel(Geom G, Arena A, int layer, const E* __restrict__ q, E* __restrict
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  if (tid < (int)kRowBytes / 4) reinterpret_cast<uint32_t*>(zero_row)[tid] = 0u;
   prefetch_operands<kRowBytes>(ap, q, sl, g);
   const bool early = ap.early && ap.n_seg;
   if (!early) grid_wait_and_release();
@@ -267,7 +269,7 @@ decode_kernel(Geom G, Arena A, int layer, const E* __restrict__ q, E* __restrict
         for (int e = 0; e < 4; ++e) {
           const int tk = (4 * k + e) / HP, h = (4 * k + e) % HP;
           if (e == 0 || h == 0)
-            load_cols<E, CPL>(Vt + (size_t)min(base + tk, n_rows - 1) * kRowBytes, lane, vf);
+            load_cols<E, CPL>(base + tk < n_rows ? Vt + (size_t)(base + tk) * kRowBytes : zero_row, lane, vf);
 #pragma unroll
           for (int c = 0; c < CPL / 2; ++c) acc[h][c] = __ffma2_rn(make_float2(pv[e], pv[e]), vf[c], acc[h][c]);
         }

@@ -221,3 +221,21 @@ def test_rows_of_an_earlier_request_have_no_part(cuda_lib, dtype, d, g, n_heavy,
         _check_heads(out.float().cpu().numpy(), K[:, :, :m], V[:, :, :m], w[:m], q, g, dtype, (g, step))
     assert ctx.stats()["device_status"] == 0
     ctx.close()
+
+
+@pytest.mark.parametrize("dtype,d,g,n", [("fp32", 128, 1, 33), ("fp32", 128, 8, 1001), ("fp32", 64, 4, 130), ("bf16", 128, 4, 75)])
+def test_cuda_core_decode_of_an_infinite_value(cuda_lib, dtype, d, g, n):
+    """The last row of a cache, which the batches repeat past the end, holds an infinite value in two columns: there the
+    result is that infinity, elsewhere what it is without it."""
+    ctx = cuda_lib.Context(n_seqs=1, n_layers=1, n_kv_heads=1, n_q_heads=g, head_dim=d, dtype=dtype, block=64, levels=1, max_tokens=4096, gram_path=1)
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    K, V = (torch.randn(1, 1, n, d, device="cuda", generator=gen).to(ctx.dtype) for _ in range(2))
+    q = torch.randn(1, g, d, device="cuda", generator=gen).to(ctx.dtype)
+    ctx.stream_append_layer(0, K, V)
+    want = ctx.decode_attn(0, q).clone()
+    V[0, 0, n - 1, 1], V[0, 0, n - 1, d - 1] = float("inf"), float("-inf")
+    want[:, :, 1], want[:, :, d - 1] = float("inf"), float("-inf")
+    ctx.reset()
+    ctx.stream_append_layer(0, K, V)
+    assert torch.equal(ctx.decode_attn(0, q), want)
+    ctx.close()

@@ -123,7 +123,8 @@ int balancekv_compress_layer(balancekv_ctx* ctx, int layer, int T, void* stream)
 /* Algorithm 1's output ratio / Theorem 3.3's estimator for one layer:
  * out[s,h,:] = sum_i w_i e^{<k_i,q>/sqrt d} v_i / sum_i w_i e^{<k_i,q>/sqrt d} over every
  * stored token of the stream of (s, h / g), w_i = 2^level.  q, out: [n_seqs, n_q_heads,
- * head_dim] in the context's dtype.  With T = 0 this is Eq. (1) exactly. */
+ * head_dim] in the context's dtype.  With T = 0 this is Eq. (1) exactly.  May be captured into a
+ * CUDA graph (after a first call outside of one): a replay attends the rows stored at that moment. */
 int balancekv_decode_attn(balancekv_ctx* ctx, int layer, const void* q, void* out, void* stream);
 
 /* One step of the streaming problem of Section 2.1: the triple (q_j, k_j, v_j) of every

@@ -793,6 +793,14 @@ static SplitPlan pick_splits(const balancekv_ctx* c, int64_t tiles, int n) {
   return pick_decode_splits(tiles, c->max_splits, c->decode_slots, n, c->G.g, warps);
 }
 
+// True while st records a graph.
+static bool capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
+  (void)cudaGetLastError();                           // the legacy stream while another one is captured
+  return false;
+}
+
 // One decode launch over the layer's current caches; with k_new / v_new given it also appends one token per stream
 // (row rel of the level-0 region, original position idx0, new level-0 length new_len) and the host's bookkeeping of
 // that append has not happened yet.
@@ -801,8 +809,8 @@ static int launch_decode_step(balancekv_ctx* c, int layer, const void* q, void* 
   StepAppend ap{};
   ap.k_new = k_new; ap.v_new = v_new;
   ap.rel_row = rel; ap.idx0 = idx0; ap.new_len = new_len;
-  const bool alike = layer_seg_hint(c, layer, ap.seg);
-  if (alike) {
+  const bool alike = layer_seg_hint(c, layer, ap.seg), captured = capturing(st);
+  if (alike && !captured) {       // a captured launch reads the table: at each replay it attends the rows of that moment
     ap.n_seg = c->cfg.levels + 1;
     ap.early = c->decode_chain && c->chain_stream == st;
   }
@@ -817,7 +825,7 @@ static int launch_decode_step(balancekv_ctx* c, int layer, const void* q, void* 
     BKV_CUDA(launch_decode_step_mma(c->G, c->A, layer, q, out, c->d_decode_scratch, ap, c->d_status, c->decode_maps, st));
   else
     BKV_CUDA(launch_decode(c->G, c->A, layer, q, out, c->d_decode_scratch, ap, c->d_status, st));
-  c->decode_chain = true;
+  c->decode_chain = !captured;
   c->chain_stream = st;
   c->kernels_launched++;
   return BALANCEKV_OK;

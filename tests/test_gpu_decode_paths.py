@@ -239,3 +239,40 @@ def test_cuda_core_decode_of_an_infinite_value(cuda_lib, dtype, d, g, n):
     ctx.stream_append_layer(0, K, V)
     assert torch.equal(ctx.decode_attn(0, q), want)
     ctx.close()
+
+
+@pytest.mark.parametrize("dtype,d,g", [("fp32", 128, 4), ("bf16", 64, 4), ("bf16", 128, 8)])
+def test_replayed_decode_attends_the_rows_of_the_moment(cuda_lib, dtype, d, g):
+    """A decode call captured into a graph reads the segment table at each replay: rows appended or compressed since the
+    capture count, and rows of an earlier request do not."""
+    H, t, n = 2, 64, 700
+    ctx = cuda_lib.Context(n_seqs=1, n_layers=1, n_kv_heads=H, n_q_heads=H * g, head_dim=d, dtype=dtype, block=t, levels=2, max_tokens=2048)
+    K, V = synth.layer_kv("llama", 41, 0, 1, H, n, d, dtype)
+    Kd, Vd = to_device(K, dtype), to_device(V, dtype)
+    q = synth.queries(41, 0, 0, 1, H * g, d, dtype)
+    qt = to_device(q, dtype)
+    out = torch.empty_like(qt)
+    ctx.stream_append_layer(0, Kd[:, :, :100].contiguous(), Vd[:, :, :100].contiguous())
+    ctx.decode_attn(0, qt, out)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        ctx.decode_attn(0, qt, out)
+
+    def replay():
+        out.zero_()
+        graph.replay()
+        return out.float().cpu().numpy()
+
+    _check_heads(replay(), K[:, :, :100], V[:, :, :100], np.ones(100), q, g, dtype, "as captured")
+    ctx.stream_append_layer(0, Kd[:, :, 100:].contiguous(), Vd[:, :, 100:].contiguous())
+    _check_heads(replay(), K, V, np.ones(n), q, g, dtype, "appended")
+    ctx.compress()
+    for h in range(H):
+        kv = [x.float().cpu().numpy() for x in ctx.cache_view(0, 0, h)[:3]]
+        assert len(kv[2]) < n
+        _check(replay()[0, h * g:(h + 1) * g], oracle.weighted_attention(*kv, q[0, h * g:(h + 1) * g]), dtype, ("compressed", h))
+    ctx.reset()
+    ctx.stream_append_layer(0, Kd[:, :, 5:8].contiguous(), Vd[:, :, 5:8].contiguous())
+    _check_heads(replay(), K[:, :, 5:8], V[:, :, 5:8], np.ones(3), q, g, dtype, "next request")
+    assert ctx.stats()["device_status"] == 0 and ctx.debug_scratch_used() == 0
+    ctx.close()

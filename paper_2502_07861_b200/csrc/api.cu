@@ -1011,12 +1011,13 @@ int balancekv_stream_step_host(balancekv_ctx* c, int layer, const void* q_host, 
   }
   // The three small inputs travel as one copy: packed into a pinned slot on the host, then one
   // host-to-device transfer into the slot's device twin on the library's copy stream, so that the
-  // transfer of a step runs while the previous step's kernel does.  With the fused step kernel no event
-  // ties the launch to the transfer (an event wait between two steps would keep the next step's CTAs
-  // from becoming resident early): a second small copy writes an arrival word behind the operands and
-  // the kernel waits, bounded, for that word.  Otherwise the step's kernels wait for the transfer
-  // through an event.  A slot is reused only after the kernel that read it has finished (one event
-  // per 16 steps).
+  // transfer of a step runs while the previous step's kernel does.  The step's kernels wait for the
+  // transfer through an event -- except the fused step of 128-dim bf16 heads, whose launch no event ties
+  // to it (an event wait between two steps would keep the next step's CTAs from becoming resident early:
+  // 16.7 us per step instead of 14.1): there a second small copy writes an arrival word behind the operands
+  // and the kernel waits for that word, for longer than any other wait, because transfers of other
+  // streams may be ahead in the copy engines.  A slot is reused only after the kernel that read it has
+  // finished (one event per 16 steps).
   constexpr int kSlots = balancekv_ctx::kStepSlots, kGroup = kSlots / 4;
   const unsigned long long n = c->step_count++;
   const int slot = (int)(n % kSlots), group = slot / kGroup;
@@ -1026,9 +1027,9 @@ int balancekv_stream_step_host(balancekv_ctx* c, int layer, const void* q_host, 
   std::memcpy(h, q_host, qb);
   std::memcpy(h + qb, k_host, kb);
   std::memcpy(h + qb + kb, v_host, kb);
-  const bool fused = step_can_fuse(c, layer);
+  const bool flagged = c->decode_maps && c->cfg.head_dim == 128 && step_can_fuse(c, layer);
   BKV_CUDA(cudaMemcpyAsync(dev_in, h, qb + 2 * kb, cudaMemcpyHostToDevice, c->step_copy_stream));
-  if (fused) {
+  if (flagged) {
     const int expect = (int)((n + 1) & 0x7fffffffu);
     // the arrival word: a stream memory operation behind the transfer (a 16-byte copy where the driver has none)
     typedef CUresult (*WriteValueFn)(CUstream, CUdeviceptr, cuuint32_t, unsigned int);

@@ -13,6 +13,7 @@ constexpr int kDecodeMaxSplits = 64;
 constexpr int kInlineSplits = 16;            // most splits that the last split's CTA combines alone
 constexpr int kDecodeCtasPerSm = 2;          // both kernels: about 99 KB of shared memory per CTA
 constexpr long long kDecodeWaitCycles = 100000000LL;   // about 50 ms: a copy that has not landed by then never will
+constexpr long long kOperandWaitCycles = 4000000000LL; // about 2 s: 100 GB of transfers ahead of a step's operands
 
 // One appended token per stream of the layer (lockstep fill): source rows [B*H, d] and where they go.
 struct StepAppend {
@@ -229,7 +230,7 @@ __device__ inline void wait_operands(const StepAppend& ap, int* status) {
   if (threadIdx.x == 0) {
     const long long t0 = clock64();
     while (*reinterpret_cast<const volatile int*>(ap.in_flag) != ap.in_expect) {
-      if (clock64() - t0 > kDecodeWaitCycles) { atomicCAS(status, kStatusOk, kStatusWaitTimeout); break; }
+      if (clock64() - t0 > kOperandWaitCycles) { atomicCAS(status, kStatusOk, kStatusWaitTimeout); break; }
     }
     __threadfence();
   }

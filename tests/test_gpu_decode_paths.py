@@ -276,3 +276,38 @@ def test_replayed_decode_attends_the_rows_of_the_moment(cuda_lib, dtype, d, g):
     _check_heads(replay(), K[:, :, 5:8], V[:, :, 5:8], np.ones(3), q, g, dtype, "next request")
     assert ctx.stats()["device_status"] == 0 and ctx.debug_scratch_used() == 0
     ctx.close()
+
+
+@pytest.mark.parametrize("dtype,d", [("fp32", 64), ("bf16", 64), ("bf16", 128)])
+def test_host_steps_behind_other_transfers(cuda_lib, dtype, d):
+    """Host steps whose operands queue behind 8 GB of other transfers (0.15 s, three times the bound of the other waits)
+    attend what the same steps on device tensors attend."""
+    B, H, g, n = 1, 2, 4, 512
+    pair = [cuda_lib.Context(n_seqs=B, n_layers=1, n_kv_heads=H, n_q_heads=H * g, head_dim=d, dtype=dtype, block=64, levels=1, max_tokens=4096)
+            for _ in range(2)]
+    host, dev = pair
+    gen = torch.Generator(device="cuda").manual_seed(4)
+    draw = lambda *s: torch.randn(*s, d, device="cuda", generator=gen).to(host.dtype)
+    K, V = draw(B, H, n), draw(B, H, n)
+    for ctx in pair:
+        ctx.stream_append_layer(0, K, V)
+    steps = [(draw(B, H * g), draw(B, H), draw(B, H)) for _ in range(6)]
+    pinned = [tuple(x.cpu().pin_memory() for x in step) for step in steps]
+    out = torch.empty(6, B, H * g, d, dtype=host.dtype).pin_memory()
+    host.stream_step_host(0, *pinned[0], out[0])
+    src = torch.zeros(1 << 28, dtype=torch.uint8).pin_memory()
+    others = [(torch.cuda.Stream(), torch.empty_like(src, device="cuda")) for _ in range(4)]
+    torch.cuda.synchronize()
+    for _ in range(8):
+        for stream, dst in others:
+            with torch.cuda.stream(stream):
+                dst.copy_(src, non_blocking=True)
+    for i in range(1, 6):
+        host.stream_step_host(0, *pinned[i], out[i])
+    torch.cuda.synchronize()
+    assert host.stats()["device_status"] == 0
+    for i, (q, k, v) in enumerate(steps):
+        want = dev.stream_step(0, q, k, v, torch.empty_like(q))
+        assert torch.equal(out[i], want.cpu()), i
+    for ctx in pair:
+        ctx.close()

@@ -81,7 +81,9 @@ typedef struct balancekv_stats_t {
   int64_t decode_kernel;      /* decode attention: 1 CUDA cores, 2 tensor cores (mma + TMA)    */
 } balancekv_stats_t;
 
-/* Allocate a context: all cache memory for n_seqs*n_layers*n_kv_heads streams.
+/* Allocate a context: all cache memory for n_seqs*n_layers*n_kv_heads streams, and where the CUDA-core walk serves it
+ * (fp32, block 64, blocks too long for the tensor-core walk, gram_path 1) a workspace of 2 t (t + 64) bytes per call for up
+ * to 512 MB or 32 calls, but no more than half of the memory that is left.
  * E_INVAL on a bad field, E_NOMEM / E_CUDA if the device allocation fails.  The kernels that
  * serve the context follow from its shape (balancekv_stats reports them); if the tensor-core
  * kernels of a shape that has them cannot be prepared, the call fails with E_CUDA -- there is no

@@ -395,9 +395,23 @@ int balancekv_create(const balancekv_config* cfg, balancekv_ctx** out) {
   if (c->use_tc && walk_tc_prepare(G, c->A, c->total_rows, &c->tmaps) != cudaSuccess) return fail(BALANCEKV_E_CUDA);
   if (T > 0 && !c->use_tc) {
     if (!walk_simt_supported(G.d)) return fail(BALANCEKV_E_INVAL);
-    // workspace of the CUDA-core walk: the kernel matrices of up to 512 MB of calls at a time
-    c->ghat_calls = (int)std::max<int64_t>(1, std::min<int64_t>(c->max_calls, ((int64_t)512 << 20) / (int64_t)walk_simt_bytes(t)));
-    if ((rc = dev_alloc(c, reinterpret_cast<char**>(&c->d_ghat), walk_simt_bytes(t) * c->ghat_calls))) return fail(rc);
+    // Workspace of the CUDA-core walk: the kernel matrices of a group of calls.  Up to 512 MB, or 32 calls of long blocks,
+    // because walk_kernel runs on as many SMs as a group has calls (148 calls of 4096 x 64 fp32: 512 MB = 15 calls
+    // 15.4 ms, 32 calls 12.2; 148 of 1024 x 128: 64 MB 1.37 ms, 256 MB 1.18, 512 MB 1.12).  No more than half of the memory
+    // that is left, and less where even that fails: the groups get smaller, nothing else.
+    const int64_t per = (int64_t)walk_simt_bytes(t);
+    size_t left = 0, all = 0;
+    if (cudaMemGetInfo(&left, &all) != cudaSuccess) return fail(BALANCEKV_E_CUDA);
+    int64_t n = std::min<int64_t>(c->max_calls, std::max<int64_t>(32, ((int64_t)512 << 20) / per));
+    n = std::max<int64_t>(1, std::min<int64_t>(n, (int64_t)(left / 2) / per));
+    while (cudaMalloc(reinterpret_cast<void**>(&c->d_ghat), (size_t)(n * per)) != cudaSuccess) {
+      (void)cudaGetLastError();
+      c->d_ghat = nullptr;
+      if (n == 1) return fail(BALANCEKV_E_NOMEM);
+      n = (n + 1) / 2;
+    }
+    c->ghat_calls = (int)n;
+    c->bytes_resident += (size_t)(n * per);
   }
   *out = c;
   return BALANCEKV_OK;

@@ -142,3 +142,34 @@ def test_sums_do_not_depend_on_the_launch(cuda_lib, t):
     for ctx in pair:
         assert ctx.stats()["device_status"] == 0 and ctx.stats()["walk_kernel"] == 2
         ctx.close()
+
+
+def test_cuda_core_walk_with_little_memory(cuda_lib):
+    """A context whose workspace (62 calls: 536 MB) finds no room beside its 230 MB of rows takes a smaller one, and keeps
+    what it keeps with the whole workspace."""
+    import torch
+
+    S, t, d = 62, 2048, 64
+    gen = torch.Generator(device="cuda").manual_seed(6)
+    K = 0.1 * torch.randn(1, S, t, d, device="cuda", generator=gen)
+    V = torch.randn(1, S, t, d, device="cuda", generator=gen)
+
+    def kept():
+        ctx = cuda_lib.Context(n_seqs=1, n_layers=1, n_kv_heads=S, n_q_heads=S, head_dim=d, dtype="fp32", block=t, levels=1,
+                               max_tokens=t, seed=3, c_override=0.75)
+        ctx.stream_append_layer(0, K, V)
+        ctx.compress()
+        idx = [ctx.cache_view(0, 0, h)[3] for h in range(S)]
+        st = ctx.stats()
+        assert st["device_status"] == 0 and st["walk_kernel"] == 1
+        ctx.close()
+        return idx, st["bytes_resident"]
+
+    want, whole = kept()
+    torch.cuda.empty_cache()
+    hog = torch.empty(torch.cuda.mem_get_info()[0] - (500 << 20), dtype=torch.uint8, device="cuda")
+    got, small = kept()
+    del hog
+    torch.cuda.empty_cache()
+    assert small < whole - (200 << 20)
+    assert all(torch.equal(a, b) for a, b in zip(got, want))

@@ -122,8 +122,14 @@ def _stream_ptr(stream):
         return stream.cuda_stream
     import torch
 
-    # torch.cuda.current_stream() builds a stream object: 3.3 us of every call against 0.2 us for the handle alone
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    # torch.cuda.current_stream() builds a stream object: 3.3 us of every call against 0.3 us for the handle alone, which a
+    # torch without these two functions, not initialised yet, or forked since, does not give
+    if torch.cuda.is_initialized():
+        try:
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        except AttributeError:
+            pass
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _torch_dtype(dtype_code: int):

@@ -35,6 +35,25 @@ def test_strerror_and_argument_errors_without_a_device():
     assert lib.balancekv_plan_calls(3, 1, 0, None, 0, None, 0) == bk.binding.E_INVAL
 
 
+@pytest.mark.parametrize("initialized,private", [(False, True), (True, False)])
+def test_current_stream_through_the_public_call(monkeypatch, initialized, private):
+    """The handle of the current stream where torch's own shortcut cannot give it: before CUDA is initialised (in a forked
+    child the public call says what is wrong), and in a torch without that shortcut."""
+    import types
+
+    import torch
+
+    monkeypatch.setattr(torch.cuda, "is_initialized", lambda: initialized)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=1234))
+    if private:
+        monkeypatch.setattr(torch._C, "_cuda_getDevice", lambda: 0, raising=False)
+        monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda device: 99, raising=False)
+    else:
+        monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+    assert bk.binding._stream_ptr(None) == 1234
+    assert bk.binding._stream_ptr(7) == 7 and bk.binding._stream_ptr(types.SimpleNamespace(cuda_stream=8)) == 8
+
+
 @pytest.mark.parametrize("t,T,W,chunks", [
     (8, 1, 0, [64]), (8, 3, 0, [8 * 13]), (16, 2, 0, [50, 40, 91]), (16, 4, 0, [16] * 20),
     (16, 3, 24, [100, 3, 97]), (8, 2, 40, [20, 20, 20, 1, 1, 1, 100]), (4, 3, 0, [1] * 70), (64, 2, 5, [1000, 7, 640]),

@@ -311,3 +311,29 @@ def test_host_steps_behind_other_transfers(cuda_lib, dtype, d):
         assert torch.equal(out[i], want.cpu()), i
     for ctx in pair:
         ctx.close()
+
+
+@pytest.mark.parametrize("dtype,g", [("bf16", 1), ("bf16", 4), ("bf16", 8), ("fp32", 1), ("fp32", 4), ("fp32", 8)])
+def test_split_decode_over_several_waves(cuda_lib, dtype, g):
+    """More streams than half of the resident CTAs, long enough that each is split in three: 480 CTAs, whose combining ones
+    poll while the last of the others are not resident yet.  Plain decode, then a step with its append."""
+    S, d, T, n_heavy, n_tail = 160, 128, 1, 4001, 130
+    n = n_heavy + n_tail
+    ctx = cuda_lib.Context(n_seqs=S, n_layers=1, n_kv_heads=1, n_q_heads=g, head_dim=d, dtype=dtype, block=64, levels=T, max_tokens=2 * n)
+    gen = torch.Generator(device="cuda").manual_seed(g)
+    draw = lambda *s: torch.randn(*s, d, device="cuda", generator=gen).to(ctx.dtype)
+    K, V = draw(S, 1, n + 1), draw(S, 1, n + 1)
+    ctx.cache_load_level(0, T, K[:, :, :n_heavy].contiguous(), V[:, :, :n_heavy].contiguous())
+    ctx.stream_append_layer(0, K[:, :, n_heavy:n].contiguous(), V[:, :, n_heavy:n].contiguous())
+    w = np.concatenate([np.full(n_heavy, 2.0), np.ones(n_tail + 1)])
+    for m in (n, n + 1):
+        q = draw(S, g)
+        if m == n:
+            out = ctx.decode_attn(0, q)
+        else:
+            out = ctx.stream_step(0, q, K[:, :, n].contiguous(), V[:, :, n].contiguous(), torch.empty_like(q))
+        assert ctx.debug_scratch_used() == 0 and ctx.stats()["device_status"] == 0
+        for s in (0, 1, 77, 147, 148, S - 1):
+            k, v, x, o = (t.float().cpu().numpy() for t in (K[s, 0, :m], V[s, 0, :m], q[s], out[s]))
+            _check(o, oracle.weighted_attention(k, v, w[:m], x), dtype, (m, s))
+    ctx.close()

@@ -380,9 +380,9 @@ cudaError_t launch_ghat(const Geom& G, const Arena& A, const CallSet& calls, int
 
 template <typename E, int D>
 cudaError_t launch_ghat_d(const Geom& G, const Arena& A, const CallSet& calls, int call0, int n, const CallStat* stats,
-                          const float* tok_shift, float* ghat, int tiles, cudaStream_t st) {
+                          const float* tok_shift, float* ghat, int tiles, int sm_count, cudaStream_t st) {
   // 8 x 4 entries per thread where the tiles fill the chip (three CTAs per SM), else 4 x 4: twice the threads per tile
-  if ((int64_t)tiles * n >= 2 * 148) return launch_ghat<E, D, 8>(G, A, calls, call0, n, stats, tok_shift, ghat, tiles, st);
+  if ((int64_t)tiles * n >= 2 * sm_count) return launch_ghat<E, D, 8>(G, A, calls, call0, n, stats, tok_shift, ghat, tiles, st);
   return launch_ghat<E, D, 4>(G, A, calls, call0, n, stats, tok_shift, ghat, tiles, st);
 }
 
@@ -397,7 +397,7 @@ size_t walk_simt_bytes(int t) { return (size_t)(t / kTile) * (t / kTile + 1) / 2
 cudaError_t launch_walk_simt(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, int level,
                              const CallStat* stats, const float* tok_shift, int8_t* eta, int8_t* dbg_eta,
                              float* dbg_S, float* dbg_p, unsigned long long* fail_count, int* status, float* ws, int ws_calls,
-                             cudaStream_t st) {
+                             int sm_count, cudaStream_t st) {
   const int tiles = (int)(walk_simt_bytes(G.t) / kTileBytes), stages = walk_stages(tiles);
   const size_t smem = walk_smem(G.t, stages);
   // one limit for every block: it belongs to the function, and another thread's context may be launching it
@@ -406,11 +406,11 @@ cudaError_t launch_walk_simt(const Geom& G, const Arena& A, const CallSet& calls
   for (int call0 = 0; call0 < n_calls && e == cudaSuccess; call0 += ws_calls) {
     const int n = std::min(ws_calls, n_calls - call0);
     if (G.d == 128)
-      e = G.is_bf16 ? launch_ghat_d<__nv_bfloat16, 128>(G, A, calls, call0, n, stats, tok_shift, ws, tiles, st)
-                    : launch_ghat_d<float, 128>(G, A, calls, call0, n, stats, tok_shift, ws, tiles, st);
+      e = G.is_bf16 ? launch_ghat_d<__nv_bfloat16, 128>(G, A, calls, call0, n, stats, tok_shift, ws, tiles, sm_count, st)
+                    : launch_ghat_d<float, 128>(G, A, calls, call0, n, stats, tok_shift, ws, tiles, sm_count, st);
     else
-      e = G.is_bf16 ? launch_ghat_d<__nv_bfloat16, 64>(G, A, calls, call0, n, stats, tok_shift, ws, tiles, st)
-                    : launch_ghat_d<float, 64>(G, A, calls, call0, n, stats, tok_shift, ws, tiles, st);
+      e = G.is_bf16 ? launch_ghat_d<__nv_bfloat16, 64>(G, A, calls, call0, n, stats, tok_shift, ws, tiles, sm_count, st)
+                    : launch_ghat_d<float, 64>(G, A, calls, call0, n, stats, tok_shift, ws, tiles, sm_count, st);
     if (e != cudaSuccess) break;
     const PdlConfig pc(dim3(n), kWalkThreads, smem, st);
     e = cudaLaunchKernelEx(&pc.cfg, walk_kernel, G, calls, call0, level, static_cast<const float*>(ws), tiles, stages, eta, dbg_eta,

@@ -788,7 +788,7 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
       eta_out[(size_t)call * t + i] = e;
       if (C.dbg_off >= 0) dbg_eta[C.dbg_off + i] = e;
     }
-    if (A.K) select_and_compact<D>(G, A, C, eta8, reinterpret_cast<int*>(sm));
+    select_and_compact<D>(G, A, C, eta8, reinterpret_cast<int*>(sm));
   }
   if (warp == kMmaWarp) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
@@ -868,16 +868,14 @@ void walk_tc_release(void* tmaps) { delete static_cast<TensorMaps*>(tmaps); }
 cudaError_t launch_walk_tc(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, int level,
                            const CallStat* stats, const float* tok_shift, int8_t* eta, int8_t* dbg_eta,
                            float* dbg_S, float* dbg_p, unsigned long long* fail_count, int* status,
-                           const void* tmaps, const void* fuse_compaction, cudaStream_t st) {
+                           const void* tmaps, cudaStream_t st) {
   if (n_calls <= 0) return cudaSuccess;
   if (!tmaps) return cudaErrorInvalidValue;
   const TensorMaps* tm = static_cast<const TensorMaps*>(tmaps);
   const size_t smem = tc_smem_bytes(G.d, G.t);
-  Arena Af = A;                       // K == nullptr: leave selection and compaction to the separate kernel
-  if (!fuse_compaction) Af.K = nullptr;
   const PdlConfig pc(dim3(n_calls), kThreads, smem, st);
   return cudaLaunchKernelEx(&pc.cfg, kernel_for(G.d, G.center_keys != 0, reuse_tiles(G)), G, calls, level, stats, tok_shift,
-                            eta, dbg_eta, dbg_S, dbg_p, fail_count, status, G.center_keys ? nullptr : A.nrm, Af, tm->k, tm->v);
+                            eta, dbg_eta, dbg_S, dbg_p, fail_count, status, G.center_keys ? nullptr : A.nrm, A, tm->k, tm->v);
 }
 
 }  // namespace bkv

@@ -19,6 +19,7 @@ def _views(ctx):
     (128, "bf16", 192, 2, 5, 0, (400, 192, 777)),
     (64, "fp32", 64, 3, 0, 0, (64, 65, 700, 63, 320)),
     (64, "bf16", 64, 2, 100, 1, (333, 64, 500)),
+    (128, "bf16", 2048, 2, 0, 0, (4096, 2048, 6200)),
 ])
 @pytest.mark.parametrize("per_layer", [False, True])
 def test_lockstep_compress_equals_the_listed_calls(cuda_lib, d, dtype, t, T, W, center, chunks, per_layer):

@@ -89,7 +89,8 @@ typedef struct balancekv_stats_t {
  * kernels of a shape that has them cannot be prepared, the call fails with E_CUDA -- there is no
  * quiet change to other kernels.
  *
- * Device-side waits are bounded (about 50 ms).  One that gives up sets the context's status word:
+ * Device-side waits are bounded (about 50 ms; about 2 s for the operands of a host step, whose transfer may queue
+ * behind those of other streams).  One that gives up sets the context's status word:
  * balancekv_stats then returns BALANCEKV_E_TIMEOUT (after filling the record), and so does every
  * later call that would enqueue work once the host has seen the word (it is copied back behind
  * every compress batch); results computed after that point are not valid.  balancekv_reset clears

@@ -82,7 +82,9 @@ inline int inline_limit(int g, int warps, int64_t tiles) {
 // stream.  Measured (d = 128, splits with / without combiners of their own): 8 streams x 8192 rows, g = 4: 34 splits
 // 10.2 us / 16 splits 13.3; 8 x 2048, g = 8: 28 splits 7.4 / 8 splits 9.1; but 24 x 1024, g = 4: 8 splits 9.3 / 6.7, and
 // 64 x 4096, g = 5, where the combiners left room for one split: 49.8 / 4 splits 28.1 (they take slots, and their polls
-// delay the tiles).
+// delay the tiles).  With two heads per warp inline is slower and combiners of their own pay down to fewer splits; the line is
+// at 11 (8 heads x 4096 rows, 15 / 16 / 18 streams = room for 12 / 11 / 9 splits: 9.8 / 9.9 / 11.8 us with combiners of their
+// own, 11.9 / 12.0 / 11.8 inline).
 //
 // More streams: the share of the slots that the launch's waves fill, less 0.08 per further split for what a split costs
 // (16384 rows: 160 streams, 1 / 3 splits 217 / 199 us; 200 streams, 1 / 4: 244 / 244; 256 streams, 1 / 2:
@@ -462,7 +464,9 @@ struct HeadEnd {
       if (!pending) break;
       if (clock64() - t0 > kDecodeWaitCycles) { ok = false; break; }
     }
-    ok = __all_sync(0xffffffffu, ok);            // every lane polls words of its own, and any of them may have given up
+    // Every lane polls words of its own, and any of them may have given up.  The vote also brings the lanes together after
+    // their loops: 11.9 -> 11.6 us per launch (8 streams x 8272 rows, g = 4, four layers in turn).
+    ok = __all_sync(0xffffffffu, ok);
     const float M = warp_max(fmaxf(ml[0].x, ml[1].x));
     const float f0 = ml[0].x == -INFINITY ? 0.f : fast_exp2(ml[0].x - M);
     const float f1 = ml[1].x == -INFINITY ? 0.f : fast_exp2(ml[1].x - M);

@@ -15,11 +15,12 @@
 // groups take tiles in turn.  Warp w of a group owns tokens 32w..32w+31 of a tile -- the tokens are the M
 // dimension of both products -- and keeps a private online softmax (running max, sum, d x 8 accumulator)
 // in registers; warps merge through shared memory, splits through a global scratch whose words are their own
-// arrival flags: with more than one split, head 0 of a stream is combined by the CTA of its last split and
-// head h > 0 by a CTA of its own (grid y = splits + h - 1), which polls the partial rows of its head.
+// arrival flags.  Few splits (StepAppend::inline_combine, at most 16) are combined by the CTA of a stream's last split, a warp
+// per head; of more, head 0 is combined by that CTA and head h > 0 by a CTA of its own (grid y = splits + h - 1), which
+// polls the partial rows of its head.
 // Fused decode step: with k_new / v_new given, the launch also appends one token per stream
 // (Algorithm 3's C^0 <- C^0 + {(k_j, v_j)}).  The new token never goes through the tiles: the combining
-// CTAs score it in fp32 and add it as one more partial (weight 1), and the combiner of head 0 writes its
+// warps score it in fp32 and add it as one more partial (weight 1), and that of head 0 writes its
 // row, its position and the stream's new level-0 length once its polls have shown that every CTA of the
 // stream is past its tiles, i.e. has finished reading the old segment table.
 // d = 64 takes this kernel too: on CUDA cores a launch over 8 streams x 2900 rows, 8 query heads each, took 24.6 us

@@ -1,5 +1,5 @@
 // SoftmaxBalance (Algorithm 2) on CUDA cores, for the contexts that the tensor-core kernel does not serve: fp32 inputs,
-// blocks of 64 tokens, and bf16 contexts that ask for this family.
+// blocks of 64 tokens, 128-dim blocks of more than 3456 tokens, and bf16 contexts that ask for this family.
 //
 // For every token j of the call, in stream order,
 //   S_j   = sum_{i<j} eta_i * Ghat_ij,   Ghat_ij = exp((<k_i,k_j> - r_key^2)/sqrt d) <v_i,v_j> / r_value^2
@@ -11,7 +11,7 @@
 // (grid: tiles of all calls) into a workspace of 64 x 64 tiles; walk_kernel (a CTA per call) streams the tiles back by
 // bulk copies, folds the tiles left of the diagonal with the signs that are final, and walks the diagonal tile.
 // What bounds it: the FFMA pipe in the first kernel, the chain of panels and the L2 reads (2 t^2 bytes per call) in the
-// second.  128 calls of 512 fp32 tokens x 128 dims: 253 + 18 us (62 % of the FMA pipe; one CTA per call doing both took
+// second.  128 calls of 512 fp32 tokens x 128 dims: 253 + 18 us (38 TFLOP/s, half of the FMA pipe's rate; one CTA per call doing both took
 // 408 us and as much for 64 calls, which take 128 + 18 now); one call of 256 x 64: 8 + 7 us (67).
 // All accumulation is fp32 in a fixed order, so two runs give identical bits.
 #include <algorithm>

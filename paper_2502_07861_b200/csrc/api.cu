@@ -141,9 +141,11 @@ struct balancekv_ctx {
   // Chain of decode launches: true while the last work this context enqueued was a launch of the
   // tensor-core decode kernel on chain_stream.  The next decode launch on that stream may then fetch
   // cache tiles before its grid dependency resolves (only the previous launch can still be running,
-  // and it writes one row per stream).  Every other enqueuing call breaks the chain.
+  // and it writes one row per stream).  Every other enqueuing call breaks the chain, and launches recorded to a graph
+  // form chains of their own.
   bool decode_chain = false;
   cudaStream_t chain_stream = nullptr;
+  unsigned long long chain_capture = 0;
 
   // value-norm buckets (Algorithm 1): running v_max^2 and the largest erased bucket index, indexed
   // by the stream of the first bucket slot; routing buffers sized for the largest block so far
@@ -807,12 +809,13 @@ static SplitPlan pick_splits(const balancekv_ctx* c, int64_t tiles, int n) {
   return pick_decode_splits(tiles, c->max_splits, c->decode_slots, n, c->G.g, warps);
 }
 
-// True while st records a graph.
-static bool capturing(cudaStream_t st) {
+// Number of the capture that st records to, 0 if none.
+static unsigned long long capture_of(cudaStream_t st) {
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  if (cudaStreamGetCaptureInfo(st, &cap, &id) == cudaSuccess) return cap == cudaStreamCaptureStatusNone ? 0 : id;
   (void)cudaGetLastError();                           // the legacy stream while another one is captured
-  return false;
+  return 0;
 }
 
 // One decode launch over the layer's current caches; with k_new / v_new given it also appends one token per stream
@@ -823,10 +826,13 @@ static int launch_decode_step(balancekv_ctx* c, int layer, const void* q, void* 
   StepAppend ap{};
   ap.k_new = k_new; ap.v_new = v_new;
   ap.rel_row = rel; ap.idx0 = idx0; ap.new_len = new_len;
-  const bool alike = layer_seg_hint(c, layer, ap.seg), captured = capturing(st);
-  if (alike && !captured) {       // a captured launch reads the table: at each replay it attends the rows of that moment
+  const bool alike = layer_seg_hint(c, layer, ap.seg);
+  const unsigned long long capture = capture_of(st);
+  // A captured plain decode reads the table: at each replay it attends the rows of that moment.  A captured step keeps the
+  // segments that its row follows: a replay puts its token in the same place again.
+  if (alike && (k_new || !capture)) {
     ap.n_seg = c->cfg.levels + 1;
-    ap.early = c->decode_chain && c->chain_stream == st;
+    ap.early = c->decode_chain && c->chain_stream == st && c->chain_capture == capture;
   }
   const SplitPlan plan = pick_splits(c, decode_tiles(c, layer, alike ? ap.seg : nullptr), c->cfg.n_seqs * c->cfg.n_kv_heads);
   ap.splits = plan.splits;
@@ -839,8 +845,9 @@ static int launch_decode_step(balancekv_ctx* c, int layer, const void* q, void* 
     BKV_CUDA(launch_decode_step_mma(c->G, c->A, layer, q, out, c->d_decode_scratch, ap, c->d_status, c->decode_maps, st));
   else
     BKV_CUDA(launch_decode(c->G, c->A, layer, q, out, c->d_decode_scratch, ap, c->d_status, st));
-  c->decode_chain = !captured;
+  c->decode_chain = true;
   c->chain_stream = st;
+  c->chain_capture = capture;
   c->kernels_launched++;
   return BALANCEKV_OK;
 }

@@ -337,3 +337,38 @@ def test_split_decode_over_several_waves(cuda_lib, dtype, g):
             k, v, x, o = (t.float().cpu().numpy() for t in (K[s, 0, :m], V[s, 0, :m], q[s], out[s]))
             _check(o, oracle.weighted_attention(k, v, w[:m], x), dtype, (m, s))
     ctx.close()
+
+
+@pytest.mark.parametrize("dtype,d,g", [("fp32", 128, 4), ("bf16", 64, 4), ("bf16", 128, 8)])
+def test_replayed_step_puts_its_token_in_the_same_place(cuda_lib, dtype, d, g):
+    """A captured step: each replay attends the rows before it and the token that its operands then hold, and stores that
+    token in the step's row.  Behind the capture, launches of the stream wait for the append that preceded it."""
+    H, n = 2, 700
+    ctx = cuda_lib.Context(n_seqs=1, n_layers=1, n_kv_heads=H, n_q_heads=H * g, head_dim=d, dtype=dtype, block=64, levels=2, max_tokens=2048)
+    K, V = synth.layer_kv("llama", 43, 0, 1, H, n + 3, d, dtype)
+    Kd, Vd = to_device(K, dtype), to_device(V, dtype)
+    q = synth.queries(43, 0, 0, 1, H * g, d, dtype)
+    qt, k, v = to_device(q, dtype), Kd[:, :, n].clone(), Vd[:, :, n].clone()
+    out = torch.empty_like(qt)
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        ctx.stream_append_layer(0, Kd[:, :, :10].contiguous(), Vd[:, :, :10].contiguous())
+        ctx.decode_attn(0, qt, out)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        ctx.stream_append_layer(0, Kd[:, :, 10:n].contiguous(), Vd[:, :, 10:n].contiguous())
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        ctx.stream_step(0, qt, k, v, out)
+    for i in (n, n + 1, n + 2):
+        k.copy_(Kd[:, :, i])
+        v.copy_(Vd[:, :, i])
+        graph.replay()
+        rows = [*range(n), i]
+        _check_heads(out.float().cpu().numpy(), K[:, :, rows], V[:, :, rows], np.ones(n + 1), q, g, dtype, i)
+    with torch.cuda.stream(stream):
+        got = ctx.decode_attn(0, qt)
+    torch.cuda.synchronize()
+    _check_heads(got.float().cpu().numpy(), K[:, :, rows], V[:, :, rows], np.ones(n + 1), q, g, dtype, "behind")
+    assert ctx.stats()["device_status"] == 0 and ctx.debug_scratch_used() == 0
+    ctx.close()

@@ -29,12 +29,17 @@
 // Ghat never touches global memory.
 // What bounds it (cycles per off-diagonal tile at 148 calls, d = 128): the MMAs 1090, of which 1024 are the tensor core's; the
 // epilogue 1300, 900 of them for its 28 exponentials per thread on the special-function unit; the loads 1100 from L2, 1540
-// from HBM (calls of 2048 tokens).  A diagonal tile takes 2400, the selection 2100, the copy of 512 kept tokens 13000 at the
-// rate at which the chip takes the writes.  Measured and not taken: A from TMEM, which halves the operand reads from shared
-// memory (1740 per tile); accumulators read in two pipelined halves (1390); a CTA per SM that takes several calls, with the
-// next call's radii and thresholds prepared by a warp of its own (2 % faster from three calls per SM on, 1 to 6 % slower below,
-// from registers that the epilogue lacks); the copies spread over the next call's walk (20 us instead of 9 for 512 tokens, as
-// their loads queue behind the tiles) or left to that warp (75 us, by bulk copies 115).
+// from HBM (calls of 2048 tokens).  A diagonal tile takes 2400, the selection 2000, the copy of 512 kept tokens 12000 (copy_rows).
+// A call of 1024 tokens: 78000 cycles (86800 before its first loads were asked for together and the role warps left at the
+// walk's end): 4500 up to the first panel, 58000 for 28 tiles and 8 diagonals, 14000 for selection and copy.  592 such calls
+// 209 -> 189 us, 592 of 128 tokens 37.9 -> 33.8, 592 of 64-dim heads 187 -> 163.
+// Measured and not taken: A from TMEM, which halves the operand reads from shared memory (1740 per tile); accumulators read in two
+// pipelined halves (1390); two teams of warpgroups on alternate tiles (247 us for the 209); no vote before the diagonal tile,
+// failed waits running into the sweeps' limit (212); one polling lane per warp (218); the four warpgroups started 40 to 150
+// cycles apart, or other shares of the exponentials on the FMA pipe (no change); rows picked by TMA gather4 where a level reads
+// what the one before kept, in place of the copies (75 cycles per gather4: 734); a CTA per SM that takes several calls, with
+// each role going on by itself and the copy left to a warp of its own (128 tokens 29.7 us, 1024 tokens 201, 2048 tokens 3 %
+// slower: the rows to copy have left L2 by then, and their loads delay those of the tiles).
 //
 // Every wait is bounded: a wait that runs out sets the abort flag and the status word, all
 // roles leave their loops, TMEM is freed and the kernel returns.
@@ -53,7 +58,9 @@ constexpr int kTile = 128;
 constexpr int kEpiGroups = 4;              // epilogue + walk warpgroups: warps 0-15 (warp % 4 = TMEM lane quadrant)
 constexpr int kEpiWarps = 4 * kEpiGroups;
 constexpr int kTmaWarp = kEpiWarps, kMmaWarp = kEpiWarps + 1, kMmaWarpV = kEpiWarps + 2;   // TMA, MMA (K K^T), MMA (V V^T)
-constexpr int kThreads = 32 * (kEpiWarps + 3);
+constexpr int kEpiThreads = 32 * kEpiWarps;
+constexpr int kThreads = kEpiThreads + 32 * 4;   // a 20th warp idles: it takes no registers from the others (96 each), and the code
+                                                 // for 20 warps is the faster one (592 calls of 1024: 189 us, with 19 warps 193)
 constexpr uint32_t kHalfBytes = 16384;     // [128 rows][64 bf16] = one swizzle-atom column of a tile
 template <int D>
 constexpr uint32_t kTileBytesOf = (D / 64) * kHalfBytes;   // a K or V tile: [128 rows][d bf16]
@@ -122,6 +129,15 @@ __device__ inline void tma_load_2d(void* dst, const CUtensorMap* map, int x, int
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
       ::"r"(smem_u32(dst)), "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(y) : "memory");
+}
+
+// The same, and L2 may give its lines up first.
+__device__ inline void tma_load_2d_leaving(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
+  uint64_t policy;
+  asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4}], [%2], %5;"
+      ::"r"(smem_u32(dst)), "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(y), "l"(policy) : "memory");
 }
 
 // Shared-memory matrix descriptor of a K-major, 128B-swizzled bf16 operand: rows of 128 bytes,
@@ -256,130 +272,136 @@ struct Slots {
   }
 };
 constexpr int kMaxSweeps = kTile + 2;
+constexpr int kMiscBytes = 512;            // barriers, jobs
+
+// A call as its CTA's warps hand it on: rows of the arena (fewer than 2^31) and debug record.
+struct Job {
+  int32_t src_row, dst_row;
+  int32_t record;                          // debug records: number of the call's, or -1
+};
 
 // Output of Algorithm 2 completed to exactly t/2 tokens (the implementation note of Appendix B:
-// "strictly select n/2"), and Algorithm 3's C^{i+1} <- C^{i+1} + SoftmaxBalance(C^i): the smaller
-// sign class (ties: +1) plus the latest tokens of the other class, in stream order, copied to the
-// call's destination rows with their positions and norms.  Runs at the tail of the call's CTA, whose
-// operand slots are idle by then: `scratch` holds the kept positions.  The rows were read by this
-// CTA microseconds ago and come from L2.  All kThreads threads take part.
-template <int D>
-__device__ inline void select_and_compact(const Geom& G, const Arena& A, const CallDesc& C, const int8_t* eta8, int* scratch) {
-  const int t = G.t, half = t / 2;
+// "strictly select n/2"): the smaller sign class (ties: +1) plus the latest tokens of the other class, in stream order.  By the
+// epilogue warps; a token's sign is the sign bit of its entry in etas, `words` are 3 t / 32 words of scratch, kept[t / 2] the
+// positions.  Sign words of 32 tokens, scanned by one warp (block scans over sign bytes took 3100 cycles, this 2000).
+__device__ inline void select_half(const Geom& G, const float* etas, uint32_t* words, uint16_t* kept, int8_t* dbg_eta, int record) {
+  const int t = G.t, half = t / 2, nw = t / 32;    // at most 128 words
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  constexpr int kScan = 512;                       // scanning threads (warps 0-15)
-  int* warp_sums = scratch;                        // [16] + [16]
-  int* kept_pos = scratch + 64;                    // [t/2]
-  const int ipt = (t + kScan - 1) / kScan;         // consecutive tokens per scanning thread (<= 8)
-  const int j0 = tid * ipt;
-  int plus = 0;
-  if (tid < kScan)
-    for (int i = 0; i < ipt; ++i) plus += (j0 + i < t && eta8[j0 + i] > 0) ? 1 : 0;
-  // exclusive scan of `plus` over the scanning threads
-  int inc = plus;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int n = __shfl_up_sync(0xffffffffu, inc, o);
-    if (lane >= o) inc += n;
+  uint32_t* mask_s = words + nw;                   // [nw] tokens kept
+  uint32_t* base_s = mask_s + nw;                  // [nw] their number before the word
+  for (int j = tid; j < t; j += kEpiThreads) {     // t is a multiple of 64: whole warps
+    const bool plus = !(__float_as_uint(etas[j]) >> 31);
+    const uint32_t w = __ballot_sync(0xffffffffu, plus);
+    if (lane == 0) words[j >> 5] = w;
+    if (record >= 0) dbg_eta[(int64_t)record * t + j] = plus ? 1 : -1;
   }
-  if (tid < kScan && lane == 31) warp_sums[warp] = inc;
-  __syncthreads();
-  int base = 0, total_plus = 0;
+  bar_sync(3, kEpiThreads);
+  if (warp == 0) {
+    auto exclusive = [&](int x, int& total) {
+      int inc = x;
 #pragma unroll
-  for (int w = 0; w < kScan / 32; ++w) {
-    const int sv = warp_sums[w];
-    if (w < warp) base += sv;
-    total_plus += sv;
-  }
-  const int plus_before = base + inc - plus;
-  const int keep_sign = (total_plus <= t - total_plus) ? 1 : -1;
-  const int have = keep_sign > 0 ? total_plus : t - total_plus;
-  const int first_other_kept = (t - have) - (half - have);   // rank (in stream order) from which the other class is kept
-  int other_rank = keep_sign > 0 ? (min(j0, t) - plus_before) : plus_before;
-  int keep_cnt = 0;
-  unsigned mask = 0;
-  if (tid < kScan)
-    for (int i = 0; i < ipt; ++i) {
-      const int j = j0 + i;
-      if (j >= t) break;
-      const bool mine = (eta8[j] > 0) == (keep_sign > 0);
-      bool keep = mine;
-      if (!mine) { keep = other_rank >= first_other_kept; ++other_rank; }
-      if (keep) { mask |= 1u << i; ++keep_cnt; }
+      for (int o = 1; o < 32; o <<= 1) {
+        const int n = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += n;
+      }
+      total = __shfl_sync(0xffffffffu, inc, 31);
+      return inc - x;
+    };
+    uint32_t w[4];                                 // words 4 lane ..
+    int plus = 0, total_plus, kept_here = 0, total_kept;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      w[i] = 4 * lane + i < nw ? words[4 * lane + i] : 0u;
+      plus += __popc(w[i]);
     }
-  inc = keep_cnt;
+    const int plus_before = exclusive(plus, total_plus);
+    const bool keep_plus = total_plus <= t - total_plus;
+    const int have = keep_plus ? total_plus : t - total_plus;
+    const int first_other = (t - have) - (half - have);        // rank (in stream order) from which the other class is kept
+    int other_before = keep_plus ? 128 * lane - plus_before : plus_before;
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int n = __shfl_up_sync(0xffffffffu, inc, o);
-    if (lane >= o) inc += n;
-  }
-  if (tid < kScan && lane == 31) warp_sums[16 + warp] = inc;
-  __syncthreads();
-  int pos = inc - keep_cnt;
-#pragma unroll
-  for (int w = 0; w < kScan / 32; ++w)
-    if (w < warp) pos += warp_sums[16 + w];
-  if (tid < kScan)
-    for (int i = 0; i < ipt; ++i)
-      if (mask & (1u << i)) kept_pos[pos++] = j0 + i;
-  __syncthreads();
-  // positions and norms: the first two tokens' loads ahead of the rows, their stores after them (2 of 21 us for 256 tokens)
-  int32_t tok[2];
-  float2 nrm[2];
-#pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    const int o = tid + u * kThreads;
-    if (o < half) {
-      tok[u] = A.idx[C.src_row + kept_pos[o]];
-      if (A.nrm) nrm[u] = A.nrm[C.src_row + kept_pos[o]];
+    for (int i = 0; i < 4; ++i) {
+      const uint32_t mine = keep_plus ? w[i] : ~w[i];
+      uint32_t other = ~mine;
+      const int n = __popc(other), skip = min(max(first_other - other_before, 0), n);
+      other_before += n;
+      if (skip == n) other = 0u;
+      else
+        for (int k = 0; k < skip; ++k) other &= other - 1;     // in one word at most
+      w[i] = 4 * lane + i < nw ? mine | other : 0u;
+      kept_here += __popc(w[i]);
     }
+    int base = exclusive(kept_here, total_kept);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (4 * lane + i < nw) {
+        mask_s[4 * lane + i] = w[i];
+        base_s[4 * lane + i] = (uint32_t)base;
+        base += __popc(w[i]);
+      }
   }
-  constexpr int kCh = D / 8;
-  // copy: a survivor row of K and of V is 2 x d / 8 chunks of 16 bytes; eight loads in flight per thread.
-  // (All CTAs of a wave reach this point together, so the copy runs at the chip's memory bandwidth
-  // whichever engine moves the bytes; the bulk-copy engine was measured and is no faster.)
-  const uint4* Ks = reinterpret_cast<const uint4*>(A.K) + (size_t)C.src_row * kCh;
-  const uint4* Vs = reinterpret_cast<const uint4*>(A.V) + (size_t)C.src_row * kCh;
-  uint4* Kd = reinterpret_cast<uint4*>(A.K) + (size_t)C.dst_row * kCh;
-  uint4* Vd = reinterpret_cast<uint4*>(A.V) + (size_t)C.dst_row * kCh;
+  bar_sync(3, kEpiThreads);
+  for (int k = warp; k < nw; k += kEpiWarps) {
+    const uint32_t m = mask_s[k];
+    if ((m >> lane) & 1u) kept[base_s[k] + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(32 * k + lane);
+  }
+  bar_sync(3, kEpiThreads);
+}
+
+// Algorithm 3's C^{i+1} <- C^{i+1} + SoftmaxBalance(C^i): the kept rows, positions and norms to the call's destination, by all
+// epilogue threads.  The rows were read by this CTA microseconds ago and come from L2, for the last time: streaming loads and
+// stores, which leave L2 to the rows that the other calls read again (512 streams x 8192 tokens, t = 2048: 3590 -> 3520 us).
+// What bounds it: an SM stores 31 bytes per clock, whichever instruction does it (512 rows of K and V, 256 KB: 8400 cycles for the
+// stores alone, on one SM or on all; 12000 with the loads).
+template <int D>
+__device__ inline void copy_rows(const Geom& G, const Arena& A, int src_row, int dst_row, const uint16_t* kept) {
+  const int tid = threadIdx.x, half = G.t / 2;
+  // positions and norms: a thread's first token's loads ahead of the rows, their stores after them
+  int32_t tok = 0;
+  float2 nrm = make_float2(0.f, 0.f);
+  if (tid < half) {
+    tok = A.idx[src_row + kept[tid]];
+    if (A.nrm) nrm = A.nrm[src_row + kept[tid]];
+  }
+  constexpr int kCh = D / 8;                       // 16-byte pieces of a row
+  const uint4* Ks = reinterpret_cast<const uint4*>(A.K) + (size_t)src_row * kCh;
+  const uint4* Vs = reinterpret_cast<const uint4*>(A.V) + (size_t)src_row * kCh;
+  uint4* Kd = reinterpret_cast<uint4*>(A.K) + (size_t)dst_row * kCh;
+  uint4* Vd = reinterpret_cast<uint4*>(A.V) + (size_t)dst_row * kCh;
   const int items = half * 2 * kCh;
-  for (int i0 = tid; i0 < items; i0 += 8 * kThreads) {
+  for (int i0 = tid; i0 < items; i0 += 8 * kEpiThreads) {
     uint4 v[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      const int i = i0 + u * kThreads;
+      const int i = i0 + u * kEpiThreads;
       if (i < items) {
         const int o = i / (2 * kCh), c = i % (2 * kCh);
-        v[u] = (c < kCh ? Ks : Vs)[(size_t)kept_pos[o] * kCh + c % kCh];
+        v[u] = __ldcs((c < kCh ? Ks : Vs) + (size_t)kept[o] * kCh + c % kCh);
       }
     }
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      const int i = i0 + u * kThreads;
+      const int i = i0 + u * kEpiThreads;
       if (i < items) {
         const int o = i / (2 * kCh), c = i % (2 * kCh);
-        (c < kCh ? Kd : Vd)[(size_t)o * kCh + c % kCh] = v[u];
+        __stcs((c < kCh ? Kd : Vd) + (size_t)o * kCh + c % kCh, v[u]);
       }
     }
   }
-#pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    const int o = tid + u * kThreads;
-    if (o < half) {
-      A.idx[C.dst_row + o] = tok[u];
-      if (A.nrm) A.nrm[C.dst_row + o] = nrm[u];
-    }
+  if (tid < half) {
+    A.idx[dst_row + tid] = tok;
+    if (A.nrm) A.nrm[dst_row + tid] = nrm;
   }
-  for (int o = tid + 2 * kThreads; o < half; o += kThreads) {
-    A.idx[C.dst_row + o] = A.idx[C.src_row + kept_pos[o]];
-    if (A.nrm) A.nrm[C.dst_row + o] = A.nrm[C.src_row + kept_pos[o]];
+  for (int o = tid + kEpiThreads; o < half; o += kEpiThreads) {
+    A.idx[dst_row + o] = A.idx[src_row + kept[o]];
+    if (A.nrm) A.nrm[dst_row + o] = A.nrm[src_row + kept[o]];
   }
 }
 
 template <int D, bool kCenter, bool kReuse>
 __global__ void __launch_bounds__(kThreads, 1)
-walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restrict__ stats,
-               const float* __restrict__ tok_shift, int8_t* __restrict__ eta_out, int8_t* __restrict__ dbg_eta,
+walk_tc_kernel(Geom G, const CallSet calls, int resident, int level, const CallStat* __restrict__ stats,
+               const float* __restrict__ tok_shift, int8_t* __restrict__ dbg_eta,
                float* __restrict__ dbg_S, float* __restrict__ dbg_p, unsigned long long* __restrict__ fail_count,
                int* __restrict__ status, const float2* __restrict__ row_norms, const Arena A,
                const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV) {
@@ -390,12 +412,12 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
   // t is a multiple of 64: the last panel may hold 64 tokens only.  Its tile then covers 64 rows that are not the
   // call's; what is computed for them goes nowhere.
   const int t = G.t, P = (t + kTile - 1) / kTile, tp = P * kTile;
-  float* etas = reinterpret_cast<float*>(sm + Smem<D>::kTilesEnd);       // [tp] signs scaled by 1/r_value^2 (0 = undecided)
+  float* etas = reinterpret_cast<float*>(sm + Smem<D>::kTilesEnd);       // [tp] signs scaled by 1/r_value^2
   float* xs = etas + tp;                                                   // [3][128] partial correlations of column quarters 1..3
   float* xb = xs + (kEpiGroups - 1) * kTile;                              // [3][128] ... and of their sums of |Ghat|
   float* thr_s = xb + (kEpiGroups - 1) * kTile;                           // [tp] decision thresholds c (1 - 2 u_j)
-  int8_t* eta8 = reinterpret_cast<int8_t*>(thr_s + tp);                   // [tp] signs
-  uint64_t* bars = reinterpret_cast<uint64_t*>(eta8 + tp);
+  uint16_t* kept = reinterpret_cast<uint16_t*>(thr_s + tp);               // [tp / 2] positions of the tokens kept
+  uint64_t* bars = reinterpret_cast<uint64_t*>(kept + tp / 2);
   // x = 0: the K K^T product, x = 1: the V V^T product
   // An operand tile travels as two boxes of 64 dims (h = 0, 1); a box is refilled as soon as the
   // four MMAs that read it are done, which lengthens the prefetch distance of the column ring.
@@ -403,19 +425,27 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
   uint64_t* empty = bars + 12;       // [x][3][h] product x no longer reads that box -> producer
   uint64_t* xdone = bars + 24;       // [2] both products of the tile in TMEM buffer b finished (one arrival per product) -> epilogue
   uint64_t* tmem_empty = bars + 28;  // [2] all epilogue warps have drained buffer b
-  uint32_t* tmem_ptr_s = reinterpret_cast<uint32_t*>(bars + 30);
+  Job* job = reinterpret_cast<Job*>(bars + 30);
+  uint32_t* tmem_ptr_s = reinterpret_cast<uint32_t*>(job + 1);
   int* abort_flag = reinterpret_cast<int*>(tmem_ptr_s + 1);
+  static_assert(30 * 8 + sizeof(Job) + 8 <= kMiscBytes, "shared memory behind the positions");
+  float* radii_s = xb;                                                    // [2 kEpiWarps] maxima of the epilogue warps, before the walk
 
-  const int call = blockIdx.x;
-  // The call's descriptor is derived where it is wanted: kept, it would take eight registers of every epilogue thread.
-  auto desc = [&]() {
-    int i = blockIdx.x;
-    asm volatile("" : "+r"(i));
-    return call_of(calls, G, i);
-  };
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-
-  if (tid == 0) {
+  const int call = blockIdx.x;
+  // rows row0 .. of the arena into the box h of operand slot `slot`, whose readers are done
+  auto load_box = [&](uint32_t slot, int h, int row0, const CUtensorMap* map, int x) {
+    uint64_t* bar = full + 6 * x + 2 * slot + h;
+    mbar_expect_tx(bar, kHalfBytes);
+    unsigned char* dst = sm + slot * kSlotBytes + (x ? kTileBytes : 0u) + h * kHalfBytes;
+    // Where the resident calls' rows exceed L2 (kReuse), the panels that few later ones read again leave it first: 512 streams x
+    // 8192 tokens, t = 2048: 3515 us without, 3434 / 3459 / 3514 from panel 9 / 11 / 13 of 16 on.
+    if (kReuse && row0 - job->src_row >= 5 * P / 8 * kTile) tma_load_2d_leaving(dst, map, 64 * h, row0, bar);
+    else tma_load_2d(dst, map, 64 * h, row0, bar);
+  };
+  if (warp == kTmaWarp && lane == 0) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&tmK) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&tmV) : "memory");
     for (int i = 0; i < 12; ++i) { mbar_init(full + i, 1); mbar_init(empty + i, 1); }
     for (int i = 0; i < 2; ++i) mbar_init(xdone + i, 2);
     for (int i = 0; i < 2; ++i) mbar_init(tmem_empty + i, kEpiWarps);       // one arrival per warp (lane 0 after __syncwarp)
@@ -423,20 +453,54 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
-  for (int i = tid; i < tp; i += kThreads) etas[i] = 0.f;
   if (warp == kMmaWarp) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_ptr_s)), "r"(kTmemCols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  // Everything above touches only this CTA's own state, and so do the coins: all of it overlaps the end of the previous
-  // launch (programmatic serialization; the wait comes before the first row or norm is read).
-  {
-    const CallDesc C = desc();
+  CallDesc C;
+  if (warp < kEpiWarps || (warp == kTmaWarp && lane == 0)) C = call_of(calls, G, call);
+  auto draw_coins = [&]() {
     const int head = C.stream % G.H, layer = (C.stream / G.H) % G.L, seq = C.stream / (G.H * G.L);
-    for (int i = tid; i < t; i += kThreads)
+    for (int i = tid; i < t; i += kEpiThreads)
       thr_s[i] = G.c * (1.0f - 2.0f * walk_uniform(G.seed + (uint64_t)seq, layer, head, C.ordinal, level, i));
-  }
+  };
+  const bool waits = call < resident;          // a CTA of the first wave may find the previous launch still running
+  if (waits && warp < kEpiWarps) draw_coins();
+  // Everything above touches only this CTA's own state and overlaps the end of the previous launch (programmatic
+  // serialization; the wait comes before the first row or norm is read).
   grid_wait_and_release();
+  // A call begins with two latencies of about 4000 cycles each, its first tile's and its row norms': both are asked for as
+  // soon as the grid dependency allows; the coins are drawn under them, or, in the first wave, before.  (Radii by two dependent
+  // rounds of loads behind the coins and a barrier: 10800 cycles before the first panel; now 4500.)
+  if (warp == kTmaWarp && lane == 0) {
+    job->src_row = (int)C.src_row;
+#pragma unroll
+    for (int h = 0; h < kBoxes; ++h) {
+      load_box(0, h, (int)C.src_row, &tmK, 0);
+      load_box(0, h, (int)C.src_row, &tmV, 1);
+    }
+    job->dst_row = (int)C.dst_row;
+    job->record = C.dbg_off >= 0 ? (int)(C.dbg_off / t) : -1;
+  } else if (warp < kEpiWarps) {
+    // r_key^2, r_value^2 of the call (inputs of Algorithm 2) = maxima of the stored row norms, unless a separate kernel has
+    // put them (key centering changes them) or they are fixed.  kDeep loads in flight per thread.
+    constexpr int kDeep = 4;
+    float2 n2[kDeep];
+#pragma unroll
+    for (int u = 0; u < kDeep; ++u) n2[u] = row_norms && tid + u * kEpiThreads < t ? row_norms[C.src_row + tid + u * kEpiThreads] : make_float2(0.f, 0.f);
+    if (!waits) draw_coins();
+    float mk = 0.f, mv = 0.f;
+#pragma unroll
+    for (int u = 0; u < kDeep; ++u) { mk = fmaxf(mk, n2[u].x); mv = fmaxf(mv, n2[u].y); }
+    if (row_norms)
+      for (int i = tid + kDeep * kEpiThreads; i < t; i += kEpiThreads) {
+        const float2 n = row_norms[C.src_row + i];
+        mk = fmaxf(mk, n.x);
+        mv = fmaxf(mv, n.y);
+      }
+    mk = warp_max(mk); mv = warp_max(mv);
+    if (lane == 0) { radii_s[2 * warp] = mk; radii_s[2 * warp + 1] = mv; }
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -449,110 +513,113 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
   // r + 1 follow the last column but one into its slot, and the slots change roles.  All sides walk the same schedule and
   // count a slot's loads alike.  Every barrier is waited on phase by phase by its one kind of waiter, and each next phase
   // depends on that waiter having passed, so a parity wait can never be a phase behind.
-  if (warp == kTmaWarp) {
-    // ------------------------------------------------------------------ TMA producer
-    if (lane == 0) {
-      const int64_t src_row = desc().src_row;
-      uint32_t used = 0, par = 0;        // per slot: loaded before; parity of the next wait on its empty barriers
-      bool ok = true;
-      auto load = [&](int slot, int tile_row) -> bool {
-        const bool again = (used >> slot) & 1u;
-        const uint32_t ph = (par >> slot) & 1u;
-        used |= 1u << slot;
-        if (again) par ^= 1u << slot;
-        unsigned char* st = sm + (uint32_t)slot * kSlotBytes;
-        const int y = (int)(src_row + (int64_t)tile_row * kTile);
+  if (warp >= kTmaWarp) {
+    if (warp == kTmaWarp) {
+      // ------------------------------------------------------------------ TMA producer
+      if (lane == 0) {
+        uint32_t used = 1, par = 0;        // per slot: loaded before (slot 0 above); parity of the next wait on its empty barriers
+        bool ok = true;
+        const int src_row = (int)C.src_row;
+        auto load = [&](int slot, int tile_row) -> bool {
+          const bool again = (used >> slot) & 1u;
+          const uint32_t ph = (par >> slot) & 1u;
+          used |= 1u << slot;
+          if (again) par ^= 1u << slot;
+          const int y = src_row + tile_row * kTile;
 #pragma unroll
-        for (int h = 0; h < kBoxes; ++h) {
-          uint64_t* fk = full + 2 * slot + h;
-          uint64_t* fv = full + 6 + 2 * slot + h;
-          if (again && !wait_bar(empty + 2 * slot + h, ph, abort_flag)) return false;
-          mbar_expect_tx(fk, kHalfBytes);
-          tma_load_2d(st + h * kHalfBytes, &tmK, 64 * h, y, fk);
-          if (again && !wait_bar(empty + 6 + 2 * slot + h, ph, abort_flag)) return false;
-          mbar_expect_tx(fv, kHalfBytes);
-          tma_load_2d(st + kTileBytes + h * kHalfBytes, &tmV, 64 * h, y, fv);
-        }
-        return true;
-      };
-      ok = load(0, 0);
-      if constexpr (kReuse) {
-        Slots slots;
-        Columns col;
-        for (int r = 0; r < P && ok; ++r) {
-          col.begin(r);
-          for (int k = 1; k < r && ok; ++k) {
-            col.step();
-            if (k > 1) ok = load(slots.column(k), col.c);
+          for (int h = 0; h < kBoxes; ++h) {
+            if (again && !wait_bar(empty + 2 * slot + h, ph, abort_flag)) return false;
+            load_box(slot, h, y, &tmK, 0);
+            if (again && !wait_bar(empty + 6 + 2 * slot + h, ph, abort_flag)) return false;
+            load_box(slot, h, y, &tmV, 1);
           }
-          col.end();
-          if (ok && r + 1 < P) ok = load(slots.next_rows(r), r + 1);
-          slots.advance(r);
-        }
-      } else {
-        for (int r = 0; r < P && ok; ++r) {
-          for (int c = 0; c < r && ok; ++c) ok = load((r + 1 + (c & 1)) % 3, c);
-          if (ok && r + 1 < P) ok = load((r + 1) % 3, r + 1);
+          return true;
+        };
+        if constexpr (kReuse) {
+          Slots slots;
+          Columns col;
+          for (int r = 0; r < P && ok; ++r) {
+            col.begin(r);
+            for (int k = 1; k < r && ok; ++k) {
+              col.step();
+              if (k > 1) ok = load(slots.column(k), col.c);
+            }
+            col.end();
+            if (ok && r + 1 < P) ok = load(slots.next_rows(r), r + 1);
+            slots.advance(r);
+          }
+        } else {
+          for (int r = 0; r < P && ok; ++r) {
+            for (int c = 0; c < r && ok; ++c) ok = load((r + 1 + (c & 1)) % 3, c);
+            if (ok && r + 1 < P) ok = load((r + 1) % 3, r + 1);
+          }
         }
       }
-    }
-    __syncwarp();
-  } else if (warp == kMmaWarp || warp == kMmaWarpV) {
-    // ------------------------------------------------------------------ MMA issuers (K K^T and V V^T)
-    // The whole warp walks the schedule and one elected lane issues: descriptors and addresses are then warp-uniform and
-    // sit in uniform registers.  (Issued from a branch on the lane index, with per-thread operands, an MMA took about 100
-    // cycles of the issuing thread instead of the 64 that the tensor core needs for it.)
-    auto issue = [&](auto product) {
-      constexpr int x = decltype(product)::value;
-      int i = 0;
-      uint32_t par = 0;                  // per slot: parity of the next wait on its full barrier
-      bool ok = true;
-      const uint32_t slot0 = umma_desc_lo(smem_u32(sm + (x ? kTileBytes : 0u)));
-      constexpr uint32_t kSlotDesc = kSlotBytes >> 4;
-      const uint32_t d_base = __shfl_sync(0xffffffffu, tmem_base, 0) + (x ? 128u : 0u);
-      auto wait = [&](uint64_t* bar, uint32_t parity) { return __all_sync(0xffffffffu, wait_bar(bar, parity, abort_flag)) != 0; };
-      Slots slots;
-      for (int r = 0; r < P && ok; slots.advance(r), ++r) {
-        const int rs = kReuse ? (int)slots.a : r % 3;
-        if (!(ok = wait(full + 6 * x + 2 * rs, (par >> rs) & 1u))) break;
-        if (kBoxes == 2 && !(ok = wait(full + 6 * x + 2 * rs + 1, (par >> rs) & 1u))) break;
-        par ^= 1u << rs;
-        const uint32_t arow = slot0 + (uint32_t)rs * kSlotDesc;
-        for (int c = 0; c <= r; ++c, ++i) {
-          const int buf = i & 1;
-          if (!(ok = wait(tmem_empty + buf, (uint32_t)(((i >> 1) & 1) ^ 1)))) break;
-          const int slot = c == r ? rs : kReuse ? (int)slots.column(c) : (r + 1 + (c & 1)) % 3;   // c-th column visited
-          const bool loaded = c < r && (!kReuse || c >= 2);  // else the slot's content has been used before
-          const bool leaves = !kReuse || c < r - 1;          // else the next panel uses it once more
-          const uint32_t b = slot0 + (uint32_t)slot * kSlotDesc;
-          const uint32_t d_tmem = d_base + (uint32_t)buf * 256u;
-          const uint32_t ph = (par >> slot) & 1u;
-          if (loaded) {
-            if (!(ok = wait(full + 6 * x + 2 * slot, ph))) break;
-            par ^= 1u << slot;
-          }
-          tc_fence_after();
-          if (elect_one()) {
-            umma_tile_lo(d_tmem, arow, b);
-            if (leaves) umma_commit(empty + 6 * x + 2 * slot);   // a column slot's box after its tile, the row slot's after the diagonal tile
-          }
-          __syncwarp();
-          if constexpr (kBoxes == 2) {
-            if (loaded && !(ok = wait(full + 6 * x + 2 * slot + 1, ph))) break;
+      __syncwarp();
+    } else if (warp == kMmaWarp || warp == kMmaWarpV) {
+      // ------------------------------------------------------------------ MMA issuers (K K^T and V V^T)
+      // The whole warp walks the schedule and one elected lane issues: descriptors and addresses are then warp-uniform and
+      // sit in uniform registers.  (Issued from a branch on the lane index, with per-thread operands, an MMA took about 100
+      // cycles of the issuing thread instead of the 64 that the tensor core needs for it.)
+      auto issue = [&](auto product) {
+        constexpr int x = decltype(product)::value;
+        int i = 0;
+        uint32_t par = 0;                  // per slot: parity of the next wait on its full barrier
+        bool ok = true;
+        const uint32_t slot0 = umma_desc_lo(smem_u32(sm + (x ? kTileBytes : 0u)));
+        constexpr uint32_t kSlotDesc = kSlotBytes >> 4;
+        const uint32_t d_base = __shfl_sync(0xffffffffu, tmem_base, 0) + (x ? 128u : 0u);
+        auto wait = [&](uint64_t* bar, uint32_t parity) { return __all_sync(0xffffffffu, wait_bar(bar, parity, abort_flag)) != 0; };
+        Slots slots;
+        for (int r = 0; r < P && ok; slots.advance(r), ++r) {
+          const int rs = kReuse ? (int)slots.a : r % 3;
+          if (!(ok = wait(full + 6 * x + 2 * rs, (par >> rs) & 1u))) break;
+          if (kBoxes == 2 && !(ok = wait(full + 6 * x + 2 * rs + 1, (par >> rs) & 1u))) break;
+          par ^= 1u << rs;
+          const uint32_t arow = slot0 + (uint32_t)rs * kSlotDesc;
+          for (int c = 0; c <= r; ++c, ++i) {
+            const int buf = i & 1;
+            if (!(ok = wait(tmem_empty + buf, (uint32_t)(((i >> 1) & 1) ^ 1)))) break;
+            const int slot = c == r ? rs : kReuse ? (int)slots.column(c) : (r + 1 + (c & 1)) % 3;   // c-th column visited
+            const bool loaded = c < r && (!kReuse || c >= 2);  // else the slot's content has been used before
+            const bool leaves = !kReuse || c < r - 1;          // else the next panel uses it once more
+            const uint32_t b = slot0 + (uint32_t)slot * kSlotDesc;
+            const uint32_t d_tmem = d_base + (uint32_t)buf * 256u;
+            const uint32_t ph = (par >> slot) & 1u;
+            if (loaded) {
+              if (!(ok = wait(full + 6 * x + 2 * slot, ph))) break;
+              par ^= 1u << slot;
+            }
+            tc_fence_after();
             if (elect_one()) {
-              umma_tile_hi(d_tmem, arow, b);
-              if (leaves) umma_commit(empty + 6 * x + 2 * slot + 1);
+              umma_tile_lo(d_tmem, arow, b);
+              if (leaves) umma_commit(empty + 6 * x + 2 * slot);   // a column slot's box after its tile, the row slot's after the diagonal tile
             }
             __syncwarp();
+            if constexpr (kBoxes == 2) {
+              if (loaded && !(ok = wait(full + 6 * x + 2 * slot + 1, ph))) break;
+              if (elect_one()) {
+                umma_tile_hi(d_tmem, arow, b);
+                if (leaves) umma_commit(empty + 6 * x + 2 * slot + 1);
+              }
+              __syncwarp();
+            }
+            if (elect_one()) umma_commit(xdone + buf);
+            __syncwarp();
           }
-          if (elect_one()) umma_commit(xdone + buf);
-          __syncwarp();
         }
-      }
-    };
-    if (warp == kMmaWarp) issue(std::integral_constant<int, 0>{});
-    else issue(std::integral_constant<int, 1>{});
-    __syncwarp();
+      };
+      if (warp == kMmaWarp) issue(std::integral_constant<int, 0>{});
+      else issue(std::integral_constant<int, 1>{});
+      __syncwarp();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == kMmaWarp) {
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
+      if (lane == 0 && *abort_flag) atomicCAS(status, kStatusOk, kStatusWaitTimeout);
+    }
   } else {
     // ------------------------------------------------------------------ four epilogue warpgroups
     // Every tile is drained by all groups: group wg takes columns 32 wg .. 32 wg + 31 of the tile
@@ -607,37 +674,19 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
       }
     };
 
-    constexpr int kEpiThreads = 32 * kEpiWarps;
-    {
-      // r_key^2, r_value^2 of the call (inputs of Algorithm 2) = maxima of the stored row norms,
-      // unless a separate kernel has put them (key centering changes them) or they are fixed
-      if (row_norms) {
-        const float2* norms = row_norms + desc().src_row;
-        float mk = 0.f, mv = 0.f;
-        for (int i = tid; i < t; i += kEpiThreads) {
-          const float2 n2 = norms[i];
-          mk = fmaxf(mk, n2.x);
-          mv = fmaxf(mv, n2.y);
-        }
-        mk = warp_max(mk); mv = warp_max(mv);
-        if (lane == 0) { xs[2 * warp] = mk; xs[2 * warp + 1] = mv; }
-      }
-      bar_sync(3, kEpiThreads);
-    }
     float rk2 = G.fixed_rk2, rv2 = G.fixed_rv2;
     if (row_norms) {
       float mk = 0.f, mv = 0.f;
 #pragma unroll
-      for (int w = 0; w < kEpiWarps; ++w) { mk = fmaxf(mk, xs[2 * w]); mv = fmaxf(mv, xs[2 * w + 1]); }
+      for (int w = 0; w < kEpiWarps; ++w) { mk = fmaxf(mk, radii_s[2 * w]); mv = fmaxf(mv, radii_s[2 * w + 1]); }
       if (rk2 <= 0.f) rk2 = mk;
       if (rv2 <= 0.f) rv2 = mv;
-      bar_sync(3, kEpiThreads);                               // xs is reused by the first walk
     } else {
       if (rk2 <= 0.f) rk2 = stats[call].rk2;
       if (rv2 <= 0.f) rv2 = stats[call].rv2;
     }
     const float inv_rv2 = rv2 > 0.f ? 1.0f / rv2 : 0.f;
-    const bool record = calls.list && desc().dbg_off >= 0;
+    const bool record = job->record >= 0;
     // All waits of a panel come before its vote barrier (id 3); a thread whose wait timed out
     // skips to the vote, where everybody learns of it and leaves.  The sweep barriers (ids 1, 2)
     // come after the vote and contain no waits, so no thread can be left waiting at them.
@@ -763,10 +812,9 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
         if (!bar_red_or(2, kEpiThreads, changed)) break;  // all signs of this sweep are written; any change?
       }
       if (wg == 0 && mine) {
-        eta8[j] = plus ? 1 : -1;
         if (fabsf(S) > cw) ++fails;                          // FAIL of Algorithm 2: counted; the decision is the clamped one
         if (record) {
-          const int64_t off = desc().dbg_off + j;
+          const int64_t off = (int64_t)job->record * t + j;
           dbg_S[off] = S;
           dbg_p[off] = 0.5f - fminf(fmaxf(S, -cw), cw) / (2.0f * cw);
         }
@@ -774,40 +822,20 @@ walk_tc_kernel(Geom G, const CallSet calls, int level, const CallStat* __restric
     }
     fails = (int)__reduce_add_sync(0xffffffffu, (unsigned)fails);
     if (lane == 0 && fails) atomicAdd(fail_count, (unsigned long long)fails);
-  }
-
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  if (*abort_flag) {
-    if (tid == 0) atomicCAS(status, kStatusOk, kStatusWaitTimeout);
-  } else {
-    const CallDesc C = desc();
-    for (int i = tid; i < t; i += kThreads) {
-      const int8_t e = eta8[i];
-      eta_out[(size_t)call * t + i] = e;
-      if (C.dbg_off >= 0) dbg_eta[C.dbg_off + i] = e;
+    tc_fence_before();
+    __syncthreads();                                       // TMEM is drained
+    if (ok) {
+      select_half(G, etas, reinterpret_cast<uint32_t*>(thr_s), kept, dbg_eta, job->record);
+      copy_rows<D>(G, A, job->src_row, job->dst_row, kept);
     }
-    select_and_compact<D>(G, A, C, eta8, reinterpret_cast<int*>(sm));
-  }
-  if (warp == kMmaWarp) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
   }
 }
 
 size_t tc_smem_bytes(int d, int t) {
   const size_t tp = (t + kTile - 1) / kTile * kTile;
-  return 1024 + (d == 128 ? Smem<128>::kTilesEnd : Smem<64>::kTilesEnd) + tp * 9 + 2 * (kEpiGroups - 1) * kTile * 4 + 512;
+  return 1024 + (d == 128 ? Smem<128>::kTilesEnd : Smem<64>::kTilesEnd) + tp * 9 + 2 * (kEpiGroups - 1) * kTile * 4 + kMiscBytes;
 }
-constexpr size_t kMaxSmem = (size_t)227 * 1024;
-// What the largest block that a kernel of this head size takes needs: every such kernel's limit, so that contexts with other
-// blocks never lower it.  (A function's limit belongs to the device, not to the context that sets it.)
-int tc_smem_limit(int d) {
-  size_t most = 0;
-  for (int t = kTile; t <= 4096; t += 64)
-    if (tc_smem_bytes(d, t) <= kMaxSmem) most = tc_smem_bytes(d, t);
-  return (int)most;
-}
+constexpr size_t kMaxSmem = (size_t)227 * 1024;         // of every kernel: the limit belongs to the device, not to the context that sets it
 // The order of a panel's columns is the order of summation of S_j, so it follows from the block alone: a call keeps the same
 // tokens whatever else shares its launch.  Tiles are reused from 1792 tokens on, where the rows of one call per SM exceed L2
 // (148 x 1792 x 512 bytes against 126 MB).  Ascending order / reuse, us per launch: 2048 tokens, 1 call 132.4 / 128.4, 148
@@ -857,7 +885,7 @@ cudaError_t walk_tc_prepare(const Geom& G, const Arena& A, int64_t total_rows, v
     if (r != CUDA_SUCCESS) { delete tm; return cudaErrorInvalidValue; }
   }
   for (int i = 0; i < 4 && e == cudaSuccess; ++i)
-    e = cudaFuncSetAttribute(kernel_for(G.d, (i & 1) != 0, i > 1), cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem_limit(G.d));
+    e = cudaFuncSetAttribute(kernel_for(G.d, (i & 1) != 0, i > 1), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
   if (e != cudaSuccess) { delete tm; return e; }
   *tmaps_out = tm;
   return cudaSuccess;
@@ -866,16 +894,15 @@ cudaError_t walk_tc_prepare(const Geom& G, const Arena& A, int64_t total_rows, v
 void walk_tc_release(void* tmaps) { delete static_cast<TensorMaps*>(tmaps); }
 
 cudaError_t launch_walk_tc(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, int level,
-                           const CallStat* stats, const float* tok_shift, int8_t* eta, int8_t* dbg_eta,
+                           const CallStat* stats, const float* tok_shift, int8_t* dbg_eta,
                            float* dbg_S, float* dbg_p, unsigned long long* fail_count, int* status,
-                           const void* tmaps, cudaStream_t st) {
+                           const void* tmaps, int sm_count, cudaStream_t st) {
   if (n_calls <= 0) return cudaSuccess;
   if (!tmaps) return cudaErrorInvalidValue;
   const TensorMaps* tm = static_cast<const TensorMaps*>(tmaps);
-  const size_t smem = tc_smem_bytes(G.d, G.t);
-  const PdlConfig pc(dim3(n_calls), kThreads, smem, st);
-  return cudaLaunchKernelEx(&pc.cfg, kernel_for(G.d, G.center_keys != 0, reuse_tiles(G)), G, calls, level, stats, tok_shift,
-                            eta, dbg_eta, dbg_S, dbg_p, fail_count, status, G.center_keys ? nullptr : A.nrm, A, tm->k, tm->v);
+  const PdlConfig pc(dim3(n_calls), kThreads, tc_smem_bytes(G.d, G.t), st);
+  return cudaLaunchKernelEx(&pc.cfg, kernel_for(G.d, G.center_keys != 0, reuse_tiles(G)), G, calls, sm_count, level, stats, tok_shift,
+                            dbg_eta, dbg_S, dbg_p, fail_count, status, G.center_keys ? nullptr : A.nrm, A, tm->k, tm->v);
 }
 
 }  // namespace bkv

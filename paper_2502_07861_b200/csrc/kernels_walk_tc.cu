@@ -634,44 +634,34 @@ walk_tc_kernel(Geom G, const CallSet calls, int resident, int level, const CallS
     int tile_it = 0, fails = 0;
     bool ok = true;
 
-    // Ghat' (without 1/r_value^2) of two neighbouring columns, packed fp32
-    auto ghat2 = [&](float k0, float k1, float v0, float v1, float nb, bool poly) -> float2 {
-      const float2 ex = __ffma2_rn(make_float2(k0, k1), make_float2(scale, scale), make_float2(nb, nb));
+    // Ghat' (without 1/r_value^2) of two neighbouring columns, packed fp32.  sh: the columns' key shifts (key centering).
+    auto ghat2 = [&](float k0, float k1, float v0, float v1, float nb, float2 sh, bool poly) -> float2 {
+      float2 ex = __ffma2_rn(make_float2(k0, k1), make_float2(scale, scale), make_float2(nb, nb));
+      if constexpr (kCenter) ex = __ffma2_rn(sh, make_float2(-scale, -scale), ex);
       const float2 ee = poly ? poly_exp2x2(ex) : make_float2(fast_exp2(ex.x), fast_exp2(ex.y));
       return __fmul2_rn(ee, make_float2(v0, v1));
     };
+    // key shifts of the columns first + 4 x .., four at a time (16-byte aligned: a call's shifts begin at a multiple of 64)
+    auto shift4 = [&](int first, int x) -> float4 {
+      if constexpr (kCenter) return __ldg(reinterpret_cast<const float4*>(shift + first) + x);
+      else return make_float4(0.f, 0.f, 0.f, 0.f);
+    };
     // acc += sum over this group's 32 columns of Ghat' * sign, from accumulator values in registers
-    auto fold_regs = [&](const float (&dk)[32], const float (&dv)[32], const float* signs, int shift_base, float nb,
-                         float acc) -> float {
+    auto fold_regs = [&](const float (&dk)[32], const float (&dv)[32], const float* signs, int first, float nb, float acc) -> float {
       const float4* e4 = reinterpret_cast<const float4*>(signs);
-      if constexpr (kCenter) {
+      float2 a2[2] = {make_float2(acc, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll
-        for (int x = 0; x < 8; ++x) {
-          const float4 e = e4[x];
-          const float ev[4] = {e.x, e.y, e.z, e.w};
+      for (int x = 0; x < 8; ++x) {
+        const float4 e = e4[x], sh = shift4(first, x);
 #pragma unroll
-          for (int y = 0; y < 4; ++y) {
-            const int i = 4 * x + y;
-            const float ex = fmaf(dk[i], scale, nb) - shift[shift_base + i] * scale;
-            acc = fmaf(fast_exp2(ex) * dv[i], ev[y], acc);
-          }
+        for (int h = 0; h < 2; ++h) {
+          const int i = 4 * x + 2 * h, pair = 2 * x + h;
+          const float2 g = ghat2(dk[i], dk[i + 1], dv[i], dv[i + 1], nb, h ? make_float2(sh.z, sh.w) : make_float2(sh.x, sh.y), (pair & 7) < kPolyOf8);
+          a2[pair & 1] = __ffma2_rn(g, h ? make_float2(e.z, e.w) : make_float2(e.x, e.y), a2[pair & 1]);
         }
-        return acc;
-      } else {
-        float2 a2[2] = {make_float2(acc, 0.f), make_float2(0.f, 0.f)};
-#pragma unroll
-        for (int x = 0; x < 8; ++x) {
-          const float4 e = e4[x];
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const int i = 4 * x + 2 * h, pair = 2 * x + h;
-            const float2 g = ghat2(dk[i], dk[i + 1], dv[i], dv[i + 1], nb, (pair & 7) < kPolyOf8);
-            a2[pair & 1] = __ffma2_rn(g, h ? make_float2(e.z, e.w) : make_float2(e.x, e.y), a2[pair & 1]);
-          }
-        }
-        const float2 s2 = __fadd2_rn(a2[0], a2[1]);
-        return s2.x + s2.y;
       }
+      const float2 s2 = __fadd2_rn(a2[0], a2[1]);
+      return s2.x + s2.y;
     };
 
     float rk2 = G.fixed_rk2, rv2 = G.fixed_rv2;
@@ -746,12 +736,8 @@ walk_tc_kernel(Geom G, const CallSet calls, int resident, int level, const CallS
         for (int i = 0; i < 32; i += 2) {
           float2 v = make_float2(0.f, 0.f);
           if (below) {
-            if constexpr (kCenter) {
-              v.x = fast_exp2(fmaf(dk[i], scale, nb) - shift[r * kTile + col0 + i] * scale) * dv[i];
-              v.y = fast_exp2(fmaf(dk[i + 1], scale, nb) - shift[r * kTile + col0 + i + 1] * scale) * dv[i + 1];
-            } else {
-              v = ghat2(dk[i], dk[i + 1], dv[i], dv[i + 1], nb, false);
-            }
+            const float4 sh = shift4(r * kTile + col0, i / 4);
+            v = ghat2(dk[i], dk[i + 1], dv[i], dv[i + 1], nb, i & 2 ? make_float2(sh.z, sh.w) : make_float2(sh.x, sh.y), false);
           }
           g[i] = col0 + i < row ? v.x : 0.f;
           g[i + 1] = col0 + i + 1 < row ? v.y : 0.f;

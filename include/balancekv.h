@@ -76,8 +76,11 @@ typedef struct balancekv_stats_t {
   int64_t device_status;      /* 0, or the first device-side error code                       */
   int64_t bytes_resident;     /* device memory owned by the context                           */
   int64_t kernels_launched;   /* kernels of this library launched so far                      */
-  int64_t walk_kernel;        /* Algorithm 2's kernel: 0 none (T = 0), 1 CUDA cores (fp32 FMA),
-                                 2 tensor cores (tcgen05); fixed at create time by the shape    */
+  int64_t walk_kernel;        /* Algorithm 2's kernel: 0 none (T = 0), 1 from a workspace
+                                 (its kernel matrix by fp32 FMA, or, fp32 rows and blocks from
+                                 128 tokens on, by tcgen05 products of split rows),
+                                 2 fused on tensor cores (tcgen05); fixed at create time by the
+                                 shape                                                          */
   int64_t decode_kernel;      /* decode attention: 1 CUDA cores, 2 tensor cores (mma + TMA)    */
 } balancekv_stats_t;
 

@@ -345,6 +345,7 @@ int balancekv_create(const balancekv_config* cfg, balancekv_ctx** out) {
   G.fixed_rv2 = f.r_value > 0 ? (float)((double)f.r_value * f.r_value) : 0.f;
   G.seed = f.seed;
   G.center_keys = f.center_keys ? 1 : 0;
+  G.split_gram = !f.dtype && f.gram_path != 1 && t >= 128;
 
   auto fail = [&](int code) { balancekv_destroy(c); return code; };
   if ((rc = dev_alloc(c, reinterpret_cast<char**>(&c->A.K), (size_t)c->total_rows * row_bytes))) return fail(rc);

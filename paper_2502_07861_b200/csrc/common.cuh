@@ -111,6 +111,7 @@ struct Geom {
   float fixed_rk2, fixed_rv2;         // > 0: fixed radii
   uint64_t seed;
   int32_t center_keys;
+  int32_t split_gram;                 // the CUDA-core walk's kernel matrices of fp32 rows come from the tensor cores
 };
 
 __host__ __device__ inline int lockstep_stream(const Geom& G, int layer, int pos) {
@@ -279,5 +280,10 @@ cudaError_t launch_bucket_scatter(const Geom& G, const Arena& A, const void* K, 
                                   const float* ns, const BucketDst* dst, cudaStream_t st);
 int walk_simt_supported(int d);
 size_t walk_simt_bytes(int t);
+cudaError_t launch_ghat_tc(const Geom& G, const Arena& A, const CallSet& calls, int call0, int n, const CallStat* stats,
+                           const float* tok_shift, float* ghat, int tiles_per_call, int* status, cudaStream_t st);
+// 16-byte piece p of a row of a 64 x 64 workspace tile sits at p ^ ghat_swizzle(row): four lanes per row read two rows without
+// bank conflicts, and so does a lane per row write eight.
+__host__ __device__ inline int ghat_swizzle(int row) { return ((row & 1) << 2) | ((row >> 1) & 3); }
 
 }  // namespace bkv

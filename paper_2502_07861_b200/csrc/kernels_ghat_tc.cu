@@ -1,0 +1,299 @@
+// The kernel matrices of fp32 calls (the first half of the CUDA-core walk, see kernels_walk_simt.cu) on the tensor cores.
+//
+// An fp32 value is the sum of three bf16 values, a = a1 + a2 + a3, each the rounding of what the ones before leave, so a
+// product of fp32 rows is a sum of products of bf16 rows, which the tensor core multiplies exactly:
+//   <a, b> = <a1, b1> + (<a1, b2> + <a2, b1> + <a2, b2> + <a1, b3> + <a3, b1>) + what is left, below 2^-26 |a||b|.
+// Its accumulator drops the bits of a sum that do not fit its 24.  So that none are dropped where it counts, a1 is rounded to a
+// grid of 2^(floor(log2 |a|) - 10), |a| the row's norm: the products of a1 and b1 are multiples of the two grids' product, and
+// by Cauchy-Schwarz no partial sum of theirs exceeds 2^22 of them, i.e. <a1, b1> is exact.  The small products have an
+// accumulator of their own, 2^-8 of the size, and the two are added in fp32.
+// Error of S_j against 64 bits, relative (2-norm), 12 draws each, FFMA / here: N(0, 0.3^2) keys d = 128 2.3e-7 / 1.6e-7; two channels x 8
+// 9.8e-6 / 3.9e-6; four channels x 10 with a mean 2.0e-5 / 1.2e-5; Student-t 2.4e-6 / 2.6e-6 (the rounding of r_key^2, the same
+// for both, is most of it); d = 64 2.1e-7 / 1.6e-7, 9.7e-6 / 7.2e-6, 2.9e-5 / 1.0e-5, 3.3e-6 / 3.2e-6.
+//
+// One CTA of eight warps and a ninth per 128 x 64 tile of a call's lower triangle, two CTAs per SM.  The eight split a stage (32 dims
+// of K, then of V) into six operand planes in shared memory and the ninth issues its 12 MMAs; the planes hold 64 dims, so that
+// one half is written while the MMAs of the other run, and the rows of the stage after next are on their way.  The accumulators
+// then become Ghat (exponential, product) and leave by bulk stores in the layout of the workspace.
+// What bounds it: shared memory, which at 64 columns feeds an MMA in 48 cycles and takes the planes in between (a stage: 576 + 290
+// cycles of either CTA; measured 1250 for both), then a CTA's 4400 cycles ahead of its first stage and 3200 behind its last, which the other
+// CTA covers in part.  128 calls of 512 tokens x 128 dims: FFMA 255 us, here 119; with stages of 64 dims and no second half 140;
+// with the MMAs issued by one of the eight warps 133.
+//
+// Every wait is bounded: a wait that runs out sets the abort flag and the status word, and the kernel returns.
+#include <algorithm>
+
+#include "common.cuh"
+#include "tcgen05.cuh"
+
+namespace bkv {
+
+namespace {
+
+using namespace tc;
+
+constexpr int kRows = 128, kCols = 64;                   // a tile
+constexpr int kWorkers = 256, kThreads = kWorkers + 32;
+constexpr uint32_t kPlaneA = kRows * 128, kPlaneB = kCols * 128;      // [rows][64 bf16], 128-byte swizzle
+constexpr uint32_t kPlanes = 3 * (kPlaneA + kPlaneB);
+constexpr size_t kSmem = 1024 + kPlanes + 128;
+constexpr uint32_t kTmemCols = 256;                      // K main, K small, V main, V small: 64 columns each
+constexpr int kGhatTile = 64, kGhatTileBytes = kGhatTile * kGhatTile * 4;
+
+// 1.5 * 2^23 times the grid of a row with squared norm n2: (a + m) - m rounds a to that grid.
+__device__ inline float grid_magic(float n2) {
+  const int e = (int)(__float_as_uint(n2) >> 23) - 127;                // floor(log2 n2)
+  return __uint_as_float((uint32_t)((e >> 1) + 13 + 127) << 23 | 0x400000u);
+}
+
+template <int D>
+__global__ void __launch_bounds__(320, 2)       // ten warps: 96 registers, so that the 18 of two CTAs fit the SM's four register files
+
+ghat_tc_kernel(Geom G, Arena A, const CallSet calls, int call0, const CallStat* __restrict__ stats, const float* __restrict__ tok_shift,
+               float* __restrict__ ghat, int tiles_per_call, int* __restrict__ status) {
+  constexpr int kPer = D / 32, kStages = 2 * kPer;       // 32-dim stages: of K, then of V
+  constexpr int kUnits = 3;                              // of a thread and stage: (row, 8 dims), two of the rows' operand and one of the columns'
+  extern __shared__ unsigned char smem_raw[];
+  __shared__ float red[2][kWorkers / 32];
+  unsigned char* sm = smem_raw + (-smem_u32(smem_raw) & 1023u);
+  uint64_t* mma_done = reinterpret_cast<uint64_t*>(sm + kPlanes);       // [2] the MMAs of a half
+  uint64_t* full = mma_done + 2;                                        // [2] the planes of a half are written
+  uint32_t* tmem_s = reinterpret_cast<uint32_t*>(full + 2);
+  int* abort_flag = reinterpret_cast<int*>(tmem_s + 1);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int t = G.t;
+  int R = 0, c64 = blockIdx.x;                           // block index -> tile: 128-row panel R has 2 R + 2 column tiles
+  for (; c64 >= 2 * R + 2; ++R) c64 -= 2 * R + 2;
+  const int row0 = R * kRows, col0 = c64 * kCols;
+  const bool own = c64 >= 2 * R;                         // the columns are among the tile's rows
+  if (tid == 0) {
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(mma_done + i, 1);
+      mbar_init(full + i, kWorkers);
+    }
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 8) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_s)), "r"(kTmemCols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  grid_wait_and_release();
+  const int64_t src_row = call_of(calls, G, call0 + blockIdx.y).src_row;
+  const float* src[2] = {static_cast<const float*>(A.K) + (size_t)src_row * D, static_cast<const float*>(A.V) + (size_t)src_row * D};
+  const float2* nrm = A.nrm + src_row;
+  // eight lanes store rows r and r + 4: no bank conflicts under the swizzle
+  const int piece = tid & 3, urow = 8 * warp + 4 * ((lane >> 2) & 1) + (lane >> 3);
+  // The unit's token.  Rows behind the call's last (a panel of 64 rows) are its last row again; nobody reads what they give.
+  auto token = [&](int k) { return min(k < 2 ? row0 + urow + 64 * k : col0 + urow, t - 1); };
+  float4 v[2][2 * kUnits];
+  float magic[2][kUnits];
+  auto fetch = [&](int s, float4 (&to)[2 * kUnits]) {
+    const float* base = src[s / kPer] + 32 * (s % kPer) + 8 * piece;
+#pragma unroll
+    for (int k = 0; k < kUnits; ++k) {
+      if (k >= 2 && own) break;
+      const float4* p = reinterpret_cast<const float4*>(base + (size_t)token(k) * D);
+      to[2 * k] = p[0];
+      to[2 * k + 1] = p[1];
+    }
+  };
+  float mk = 0.f, mv = 0.f;                              // maxima of the stored norms
+  if (warp < 8) {
+    fetch(0, v[0]);
+    fetch(1, v[1]);
+#pragma unroll
+    for (int k = 0; k < kUnits; ++k) {
+      const float2 n = nrm[token(k)];
+      magic[0][k] = grid_magic(n.x);
+      magic[1][k] = grid_magic(n.y);
+    }
+    for (int j = tid; j < t; j += kWorkers) {
+      const float2 n = nrm[j];
+      mk = fmaxf(mk, n.x);
+      mv = fmaxf(mv, n.y);
+    }
+    mk = warp_max(mk); mv = warp_max(mv);
+    if (lane == 0) { red[0][warp] = mk; red[1][warp] = mv; }
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_s, 0);          // warp-uniform, so that the MMAs' operands sit in uniform registers
+  bool ok = true;
+  if (warp < 8) {
+#pragma unroll
+    for (int s = 0; s < kStages; ++s) {
+      if (s > 1) ok = ok && wait_bar(mma_done + (s & 1), (uint32_t)((s >> 1) - 1) & 1u, abort_flag);     // the half has been read
+      if (ok) {
+#pragma unroll
+        for (int k = 0; k < kUnits; ++k) {
+          if (k >= 2 && own) break;
+          const int row = urow + (k == 1 ? 64 : 0);
+          unsigned char* to = sm + (k < 2 ? 0u : 3 * kPlaneA) + row * 128 + (((4 * (s & 1) + piece) ^ (row & 7)) << 4);
+          const float4 x0 = v[s & 1][2 * k], x1 = v[s & 1][2 * k + 1];
+          const float x[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+          const float2 m = make_float2(magic[s / kPer][k], magic[s / kPer][k]), neg = make_float2(-m.x, -m.x);
+          uint32_t w[3][4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            float2 a = make_float2(x[2 * i], x[2 * i + 1]);
+            const float2 a1 = __fadd2_rn(__fadd2_rn(a, m), neg);
+#pragma unroll
+            for (int p = 0; p < 3; ++p) {
+              const __nv_bfloat162 h = p == 0 ? __floats2bfloat162_rn(a1.x, a1.y) : __floats2bfloat162_rn(a.x, a.y);
+              w[p][i] = *reinterpret_cast<const uint32_t*>(&h);
+              a = __ffma2_rn(make_float2(bf16_lo(w[p][i]), bf16_hi(w[p][i])), make_float2(-1.f, -1.f), a);
+            }
+          }
+#pragma unroll
+          for (int p = 0; p < 3; ++p)
+            *reinterpret_cast<uint4*>(to + p * (k < 2 ? kPlaneA : kPlaneB)) = make_uint4(w[p][0], w[p][1], w[p][2], w[p][3]);
+        }
+      }
+      if (s + 2 < kStages) fetch(s + 2, v[s & 1]);
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      mbar_arrive(full + (s & 1));
+    }
+#pragma unroll
+    for (int w = 0; w < kWorkers / 32; ++w) { mk = fmaxf(mk, red[0][w]); mv = fmaxf(mv, red[1][w]); }
+    // r_key^2, r_value^2 (inputs of Algorithm 2): maxima of the stored row norms, unless center_kernel has put them or they are fixed
+    float rk2 = G.fixed_rk2, rv2 = G.fixed_rv2;
+    if (rk2 <= 0.f) rk2 = tok_shift ? stats[call0 + blockIdx.y].rk2 : mk;
+    if (rv2 <= 0.f) rv2 = tok_shift ? stats[call0 + blockIdx.y].rv2 : mv;
+    const float inv_rv2 = rv2 > 0.f ? 1.0f / rv2 : 0.f;
+    const float scale = 1.4426950408889634f * G.inv_sqrt_d;
+    const float* shift = tok_shift ? tok_shift + (size_t)(call0 + blockIdx.y) * t : nullptr;
+    // thread = row of the tile; warps 0-3 its columns 0 .. 31, warps 4-7 the others
+    const int row = 32 * (warp & 3) + lane, ch = warp >> 2;
+    const int j = row0 + row, i0 = col0 + 32 * ch;
+    const float off = (shift && j < t ? shift[j] : 0.f) + rk2;
+    // the last stage of either half (a commit covers all MMAs before it, but each phase is waited for)
+    ok = ok && wait_bar(mma_done, (uint32_t)(kStages / 2 - 1) & 1u, abort_flag) && wait_bar(mma_done + 1, (uint32_t)(kStages / 2 - 1) & 1u, abort_flag);
+    ok = __all_sync(0xffffffffu, ok);
+    if (ok) {
+      tc_fence_after();
+      const uint32_t tl = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(32 * ch);
+      // the planes are free: two 64 x 64 tiles of the workspace, the panel's halves
+      unsigned char* tile = sm + (row >> 6) * kGhatTileBytes + (row & 63) * (kGhatTile * 4);
+      const int sw = ghat_swizzle(row);
+      const bool plain = !(mk < INFINITY && mv < INFINITY);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {                       // 16 columns at a time
+        const int c0 = i0 + 16 * h;
+        float ex[16], vv[16];
+        {
+          float lo[16], lv[16];
+          tmem_ld16(tl + 16 * h, ex);
+          tmem_ld16(tl + 64 + 16 * h, lo);
+          tmem_ld16(tl + 128 + 16 * h, vv);
+          tmem_ld16(tl + 192 + 16 * h, lv);
+          tmem_ld_wait();
+#pragma unroll
+          for (int i = 0; i < 16; ++i) { ex[i] += lo[i]; vv[i] += lv[i]; }
+        }
+        if (shift) {
+#pragma unroll
+          for (int i = 0; i < 16; i += 4) {
+            const float4 a = *reinterpret_cast<const float4*>(shift + c0 + i);
+            ex[i] -= a.x; ex[i + 1] -= a.y; ex[i + 2] -= a.z; ex[i + 3] -= a.w;
+          }
+        }
+        // only earlier tokens count (a select behind the exponential: a branch per entry cost 3000 cycles a tile)
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          const float e = exp2f((ex[i] - off) * scale);
+          ex[i] = c0 + i < j ? e : 0.f;
+        }
+        // Infinite entries have no remainders: such calls (a row's norm shows it) are formed by FFMA, as on the CUDA cores.
+        if (plain && j < t)
+          for (int i = 0; i < 16; ++i) {
+            const int c = c0 + i;
+            float dot[2] = {0.f, 0.f};
+            for (int x = 0; c < j && x < 2; ++x) {
+              float2 s = make_float2(0.f, 0.f);
+              for (int e = 0; e < D; e += 2)
+                s = __ffma2_rn(*reinterpret_cast<const float2*>(src[x] + (size_t)j * D + e), *reinterpret_cast<const float2*>(src[x] + (size_t)c * D + e), s);
+              dot[x] = s.x + s.y;
+            }
+            const float xk = c < j ? exp2f((dot[0] - (shift ? shift[c] : 0.f) - off) * scale) : 0.f;
+#pragma unroll
+            for (int u = 0; u < 16; ++u)                  // a dynamic index would put the arrays into local memory
+              if (u == i) { ex[u] = xk; vv[u] = dot[1]; }
+          }
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+          float o[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float x = ex[4 * p + i] * (vv[4 * p + i] * inv_rv2);
+            o[i] = ex[4 * p + i] != 0.f ? x : 0.f;
+          }
+          *reinterpret_cast<float4*>(tile + (((8 * ch + 4 * h + p) ^ sw) << 4)) = make_float4(o[0], o[1], o[2], o[3]);
+        }
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+  } else {
+#pragma unroll
+    for (int s = 0; s < kStages; ++s) {
+      ok = ok && __all_sync(0xffffffffu, wait_bar(full + (s & 1), (uint32_t)(s >> 1) & 1u, abort_flag));
+      if (!ok) break;
+      tc_fence_after();
+      if (elect_one()) {
+        const uint32_t main = tmem + (uint32_t)(s / kPer) * 128u, small = main + 64u;
+        const uint32_t a = umma_desc_lo(smem_u32(sm)) + 4 * (s & 1);
+        const uint32_t b = own ? a + (uint32_t)(c64 & 1) * (kPlaneB >> 4) : a + ((3 * kPlaneA) >> 4);
+        const uint32_t bp = own ? kPlaneA >> 4 : kPlaneB >> 4;      // from one of the columns' planes to the next
+        constexpr uint32_t ap = kPlaneA >> 4;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          if (s % kPer == 0 && k == 0) {
+            umma_bf16<0, kCols>(main, a, b);
+            umma_bf16<0, kCols>(small, a + 2 * ap, b);
+          } else {
+            umma_bf16<1, kCols>(main, a + 2 * k, b + 2 * k);
+            umma_bf16<1, kCols>(small, a + 2 * ap + 2 * k, b + 2 * k);
+          }
+          umma_bf16<1, kCols>(small, a + 2 * k, b + 2 * bp + 2 * k);
+          umma_bf16<1, kCols>(small, a + ap + 2 * k, b + bp + 2 * k);
+          umma_bf16<1, kCols>(small, a + ap + 2 * k, b + 2 * k);
+          umma_bf16<1, kCols>(small, a + 2 * k, b + bp + 2 * k);
+        }
+        umma_commit(mma_done + (s & 1));
+      }
+      __syncwarp();
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 8) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+  if (*abort_flag) {
+    if (tid == 0) atomicCAS(status, kStatusOk, kStatusWaitTimeout);
+  } else if (tid < 2) {
+    const int r = 2 * R + tid;
+    if (c64 <= r && r < t / kGhatTile) {
+      float* to = ghat + ((size_t)blockIdx.y * tiles_per_call + r * (r + 1) / 2 + c64) * (kGhatTile * kGhatTile);
+      asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
+                   ::"l"(to), "r"(smem_u32(sm + tid * kGhatTileBytes)), "r"(kGhatTileBytes) : "memory");
+      asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+      asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the stores end with the grid, which the walk waits for
+    }
+  }
+}
+
+}  // namespace
+
+// Calls call0 .. call0 + n - 1 of the set; ghat: their workspace, tiles_per_call 64 x 64 tiles each.
+cudaError_t launch_ghat_tc(const Geom& G, const Arena& A, const CallSet& calls, int call0, int n, const CallStat* stats,
+                           const float* tok_shift, float* ghat, int tiles_per_call, int* status, cudaStream_t st) {
+  auto kern = G.d == 128 ? ghat_tc_kernel<128> : ghat_tc_kernel<64>;
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+  if (e != cudaSuccess) return e;
+  const int P = (G.t + kRows - 1) / kRows, last = G.t % kRows ? 1 : 0;   // a last panel of 64 rows has one column tile less
+  const PdlConfig pc(dim3(P * (P + 1) - last, n), kThreads, kSmem, st);
+  return cudaLaunchKernelEx(&pc.cfg, kern, G, A, calls, call0, stats, tok_shift, ghat, tiles_per_call, status);
+}
+
+}  // namespace bkv

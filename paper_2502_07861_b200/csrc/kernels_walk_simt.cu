@@ -8,7 +8,8 @@
 // with u_j the Philox uniform of (seed, layer, head, call ordinal, level, j).
 //
 // Two kernels.  Ghat does not depend on the signs, so ghat_kernel forms its lower triangle with FFMA over the whole chip
-// (grid: tiles of all calls) into a workspace of 64 x 64 tiles; walk_kernel (a CTA per call) streams the tiles back by
+// (grid: tiles of all calls) into a workspace of 64 x 64 tiles (Geom::split_gram: fp32 rows and blocks from 128 tokens on, the
+// kernel of kernels_ghat_tc.cu does, in 119 us where this one takes 255); walk_kernel (a CTA per call) streams the tiles back by
 // bulk copies, folds the tiles left of the diagonal with the signs that are final, and walks the diagonal tile.
 // What bounds it: the FFMA pipe in the first kernel, the chain of panels and the L2 reads (2 t^2 bytes per call) in the
 // second.  128 calls of 512 fp32 tokens x 128 dims: 253 + 18 us (38 TFLOP/s, half of the FMA pipe's rate; one CTA per call doing both took
@@ -28,9 +29,8 @@ constexpr uint32_t kTileBytes = kTileFloats * 4;
 constexpr int kChunk = 32;                              // dims per pipeline stage of ghat_kernel
 constexpr long long kWaitCycles = 100000000LL;          // about 50 ms: a bulk copy that has not landed by then never will
 
-// Float index of (row, column) inside a workspace tile: 16-byte pieces, odd rows with the halves of every 128 bytes
-// swapped, so that four lanes per row read two rows without bank conflicts.
-__device__ inline int tile_at(int row, int col) { return row * kTile + (col ^ ((row & 1) << 4)); }
+// Float index of (row, column) inside a workspace tile.
+__device__ inline int tile_at(int row, int col) { return row * kTile + (col ^ (ghat_swizzle(row) << 2)); }
 
 __device__ inline uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ inline void cp_async16(void* dst, const void* src) {
@@ -263,7 +263,7 @@ walk_kernel(Geom G, const CallSet calls, int call0, int level, const float* __re
   } else {
     const int row = tid / 4, p = tid % 4;
     const float* gp = tiles + row * kTile;
-    const int sw = (row & 1) << 4;
+    const int sw = ghat_swizzle(row) << 2;
     int fails = 0;
     bool ok = true;
     int s = 0;                                           // stage of the next tile, parity of its barrier
@@ -405,7 +405,9 @@ cudaError_t launch_walk_simt(const Geom& G, const Arena& A, const CallSet& calls
   if (!G.center_keys) tok_shift = nullptr;
   for (int call0 = 0; call0 < n_calls && e == cudaSuccess; call0 += ws_calls) {
     const int n = std::min(ws_calls, n_calls - call0);
-    if (G.d == 128)
+    if (G.split_gram)
+      e = launch_ghat_tc(G, A, calls, call0, n, stats, tok_shift, ws, tiles, status, st);
+    else if (G.d == 128)
       e = G.is_bf16 ? launch_ghat_d<__nv_bfloat16, 128>(G, A, calls, call0, n, stats, tok_shift, ws, tiles, sm_count, st)
                     : launch_ghat_d<float, 128>(G, A, calls, call0, n, stats, tok_shift, ws, tiles, sm_count, st);
     else

@@ -42,6 +42,35 @@ def test_cuda_core_walk(cuda_lib, d, dtype, t, T, center):
     _run(cuda_lib, d, dtype, t, T, center, 5e-4 if center else 2e-5, 1, gram_path=1)
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("t,T,center", [(128, 2, 0), (192, 1, 1), (320, 1, 0), (640, 1, 0), (1024, 1, 0)])
+def test_kernel_matrix_of_fp32_rows_on_tensor_cores(cuda_lib, d, t, T, center):
+    """Whole panels and a last panel of 64 tokens, columns that are among the tile's rows and others; the tolerances of FFMA."""
+    _run(cuda_lib, d, "fp32", t, T, center, 5e-4 if center else 2e-5, 1)
+
+
+@pytest.mark.parametrize("value", [float("inf"), float("-inf"), 3.4e38])
+def test_fp32_call_with_an_infinite_row(cuda_lib, value):
+    """A row whose norm is infinite: its call is formed as on the CUDA cores, bit by bit."""
+    import torch
+
+    S, t, d = 2, 192, 64
+    gen = torch.Generator(device="cuda").manual_seed(9)
+    K = 0.3 * torch.randn(1, S, t, d, device="cuda", generator=gen)
+    V = torch.randn(1, S, t, d, device="cuda", generator=gen)
+    K[0, 0, 70, 5] = value
+    views = []
+    for path in (0, 1):
+        ctx = cuda_lib.Context(n_seqs=1, n_layers=1, n_kv_heads=S, n_q_heads=S, head_dim=d, dtype="fp32", block=t, levels=1, max_tokens=t,
+                               seed=3, c_override=0.75, gram_path=path)
+        ctx.stream_append_layer(0, K, V)
+        ctx.compress()
+        views.append(ctx.cache_view(0, 0, 0))
+        assert ctx.stats()["device_status"] == 0
+        ctx.close()
+    assert all(torch.equal(a, b) for a, b in zip(*views))
+
+
 def test_cuda_core_walk_in_groups_of_calls(cuda_lib):
     """More calls than the workspace holds (512 MB: 60 calls of 2048 tokens), against the walk of each stream alone."""
     import torch

@@ -55,6 +55,8 @@ struct StepAppend {
   // last split combines all heads (HeadEnd::combine_inline).
   int splits;
   int inline_combine;
+  // Share of every CTA's tiles, its first ones, that is loaded so that L2 gives it up first (see l2_leaving in api.cu).
+  float leaving;
 };
 
 // CTAs per stream of a launch.

@@ -75,6 +75,14 @@ __device__ inline void tma_load_3d(void* dst, const CUtensorMap* map, int x, int
       "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
       ::"r"(smem_u32(dst)), "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(z) : "memory");
 }
+// The same, and L2 may give its lines up first.
+__device__ inline void tma_load_3d_leaving(void* dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar) {
+  uint64_t policy;
+  asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4, %5}], [%2], %6;"
+      ::"r"(smem_u32(dst)), "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(z), "l"(policy) : "memory");
+}
 __device__ inline void tma_prefetch_3d(const CUtensorMap* map, int x, int y, int z) {
   asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(map), "r"(x), "r"(y), "r"(z) : "memory");
 }
@@ -125,8 +133,9 @@ __device__ inline bool group_bar_or(int group, bool pred) {
 }
 
 // kInline: how the splits are combined (StepAppend::inline_combine).  Two kernels, because the code of the way not taken
-// costs a launch 0.8 us of instruction fetches (8 streams x 8272 rows: 12.2 against 13.0 us).
-template <int D, bool kInline>
+// costs a launch 0.8 us of instruction fetches (8 streams x 8272 rows: 12.2 against 13.0 us).  kLeaving: StepAppend::leaving > 0; apart
+// for the same reason (0.2 us).
+template <int D, bool kInline, bool kLeaving>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ out,
                   float* __restrict__ part_base, int* __restrict__ status,
@@ -194,12 +203,23 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
   const int t_begin = (int)((long long)n_tiles * split / splits);
   const int t_end = (int)((long long)n_tiles * (split + 1) / splits);
   const int my_tiles = split < splits ? t_end - t_begin : 0;
+  const int n_leaving = kLeaving ? (int)ceilf(ap.leaving * (float)my_tiles) : 0;      // the CTA's tiles that L2 may give up first
 
   auto issue = [&](int i) {   // one thread
     const TileRef tr = locate_tile<kTN>(t_begin + i, lvl_tiles, seg_s, G.T, G.region_off);
     unsigned char* st = tiles + (size_t)(i % kStages) * kStageBytes;
     uint64_t* bar = &full[i % kBars];
     mbar_expect_tx(bar, keys_only ? kTensorBytes : kStageBytes);
+#pragma unroll
+    if (kLeaving && i < n_leaving) {
+#pragma unroll
+      for (int b = 0; b < D / 64; ++b) tma_load_3d_leaving(st + b * kHalf, &tmK, 64 * b, tr.row, stream, bar);
+      if (!keys_only) {
+#pragma unroll
+        for (int b = 0; b < D / 64; ++b) tma_load_3d_leaving(st + kTensorBytes + b * kHalf, &tmV, 64 * b, tr.row, stream, bar);
+      }
+      return;
+    }
 #pragma unroll
     for (int b = 0; b < D / 64; ++b) tma_load_3d(st + b * kHalf, &tmK, 64 * b, tr.row, stream, bar);
     if (!keys_only) {
@@ -555,22 +575,26 @@ cudaError_t encode_maps(DecodeMaps* tm, void* K, void* V, int d, int64_t rows, i
   return cudaSuccess;
 }
 
-auto kernel_for(int d, bool inline_combine) {
-  return d == 128 ? (inline_combine ? decode_mma_kernel<128, true> : decode_mma_kernel<128, false>)
-                  : (inline_combine ? decode_mma_kernel<64, true> : decode_mma_kernel<64, false>);
+template <int D>
+auto kernel_for_d(bool inline_combine, bool leaving) {
+  if (leaving) return inline_combine ? decode_mma_kernel<D, true, true> : decode_mma_kernel<D, false, true>;
+  return inline_combine ? decode_mma_kernel<D, true, false> : decode_mma_kernel<D, false, false>;
+}
+auto kernel_for(int d, bool inline_combine, bool leaving) {
+  return d == 128 ? kernel_for_d<128>(inline_combine, leaving) : kernel_for_d<64>(inline_combine, leaving);
 }
 size_t smem_bytes(int d) { return d == 128 ? Dim<128>::kSmemBytes : Dim<64>::kSmemBytes; }
 cudaError_t set_smem(int d) {
   cudaError_t e = cudaSuccess;
-  for (int i = 0; i < 2 && e == cudaSuccess; ++i)
-    e = cudaFuncSetAttribute(kernel_for(d, i != 0), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes(d));
+  for (int i = 0; i < 4 && e == cudaSuccess; ++i)
+    e = cudaFuncSetAttribute(kernel_for(d, (i & 1) != 0, i > 1), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes(d));
   return e;
 }
 
 cudaError_t launch(const Geom& G, const Arena& A, int layer, const void* q, void* out, float* part, int* status,
                    const StepAppend& ap, const DecodeMaps& tm, int n_slots, cudaStream_t st) {
   const PdlConfig pc(dim3(G.B * G.H, decode_grid_y(G, ap), n_slots), kThreads, smem_bytes(G.d), st);
-  return cudaLaunchKernelEx(&pc.cfg, kernel_for(G.d, ap.inline_combine), G, A, layer,
+  return cudaLaunchKernelEx(&pc.cfg, kernel_for(G.d, ap.inline_combine, ap.leaving > 0.f), G, A, layer,
                             static_cast<const __nv_bfloat16*>(q), static_cast<__nv_bfloat16*>(out), part, status, ap, tm.k, tm.v);
 }
 

@@ -590,7 +590,7 @@ static int run_calls(balancekv_ctx* c, const CallSet& calls, int n, int l, cudaS
   if (c->use_tc) {
     ProfScope ps(c, 2, st);
     BKV_CUDA(launch_walk_tc(G, c->A, calls, n, l, c->d_stats, c->d_tokshift, c->dbg_eta, c->dbg_S,
-                            c->dbg_p, c->d_fail, c->d_status, c->tmaps, c->sm_count, st));   // selection + compaction fused at the tail
+                            c->dbg_p, c->d_fail, c->d_status, c->tmaps, c->sm_count, c->l2_bytes, st));   // selection + compaction fused at the tail
   } else {
     ProfScope ps(c, 2, st);
     BKV_CUDA(launch_walk_simt(G, c->A, calls, n, l, c->d_stats, c->d_tokshift, c->d_eta, c->dbg_eta, c->dbg_S,

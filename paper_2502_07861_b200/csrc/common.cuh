@@ -256,7 +256,7 @@ cudaError_t launch_walk_simt(const Geom& G, const Arena& A, const CallSet& calls
 cudaError_t launch_walk_tc(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, int level,
                            const CallStat* stats, const float* tok_shift, int8_t* dbg_eta,
                            float* dbg_S, float* dbg_p, unsigned long long* fail_count, int* status,
-                           const void* tmaps, int sm_count, cudaStream_t st);
+                           const void* tmaps, int sm_count, int l2_bytes, cudaStream_t st);
 cudaError_t launch_compact(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, int level,
                            const int8_t* eta, cudaStream_t st);
 struct StepAppend;      // decode_common.cuh

@@ -21,7 +21,7 @@
 // thread and its own barriers, so that one product's waits and commits overlap the other's
 // MMAs.  Operands live in three slots (K tile + V tile; 64 KB at d = 128) that rotate roles: one holds the panel's rows,
 // the column tiles stream through the other two, and the next panel's rows are fetched behind the last columns, so that its
-// first products are already in TMEM when the walk of the diagonal tile ends.  From 1792 tokens on (reuse_tiles) a panel
+// first products are already in TMEM when the walk of the diagonal tile ends.  From 1792 tokens on (order_of) a panel
 // begins with the two tiles that the one before left in shared memory: 107 loads instead of 136 for 2048 tokens, 181 -> 169 us
 // for 148 such calls.
 // Inside a slot every operand is two boxes of 64 dims with their own full/empty barriers: a box is
@@ -64,6 +64,7 @@ constexpr int kTmaWarp = kEpiWarps, kMmaWarp = kEpiWarps + 1, kMmaWarpV = kEpiWa
 constexpr int kEpiThreads = 32 * kEpiWarps;
 constexpr int kThreads = kEpiThreads + 32 * 4;   // a 20th warp idles: it takes no registers from the others (96 each), and the code
                                                  // for 20 warps is the faster one (592 calls of 1024: 189 us, with 19 warps 193)
+constexpr int kSplitRegs = 96;
 constexpr uint32_t kHalfBytes = 16384;     // [128 rows][64 bf16] = one swizzle-atom column of a tile
 template <int D>
 constexpr uint32_t kTileBytesOf = (D / 64) * kHalfBytes;   // a K or V tile: [128 rows][d bf16]
@@ -181,6 +182,7 @@ struct Slots {
   }
 };
 constexpr int kMaxSweeps = kTile + 2;
+enum Order : int { kAscending, kReuseStaying, kReuseLeaving };   // of a panel's columns, and whether late panels leave L2 first
 constexpr int kMiscBytes = 512;            // barriers, jobs
 
 // A call as its CTA's warps hand it on: rows of the arena (fewer than 2^31) and debug record.
@@ -257,6 +259,11 @@ __device__ inline void select_half(const Geom& G, const float* etas, uint32_t* w
   bar_sync(3, kEpiThreads);
 }
 
+// As a call of its own, which gives the loops of the kernel that reuses tiles better registers (one call of 2048: 132 -> 130 us).
+__device__ __noinline__ void select_half_apart(const Geom& G, const float* etas, uint32_t* words, uint16_t* kept, int8_t* dbg_eta, int record) {
+  select_half(G, etas, words, kept, dbg_eta, record);
+}
+
 // Algorithm 3's C^{i+1} <- C^{i+1} + SoftmaxBalance(C^i): the kept rows, positions and norms to the call's destination, by all
 // epilogue threads.  The rows were read by this CTA microseconds ago and come from L2, for the last time: streaming loads and
 // stores, which leave L2 to the rows that the other calls read again (512 streams x 8192 tokens, t = 2048: 3590 -> 3520 us).
@@ -307,7 +314,7 @@ __device__ inline void copy_rows(const Geom& G, const Arena& A, int src_row, int
   }
 }
 
-template <int D, bool kCenter, bool kReuse>
+template <int D, bool kCenter, int kOrder>
 __global__ void __launch_bounds__(kThreads, 1)
 walk_tc_kernel(Geom G, const CallSet calls, int resident, int level, const CallStat* __restrict__ stats,
                const float* __restrict__ tok_shift, int8_t* __restrict__ dbg_eta,
@@ -318,6 +325,7 @@ walk_tc_kernel(Geom G, const CallSet calls, int resident, int level, const CallS
   unsigned char* sm = smem_raw + (-smem_u32(smem_raw) & 1023u);   // an offset, so that the compiler keeps seeing shared memory
   constexpr uint32_t kTileBytes = kTileBytesOf<D>, kSlotBytes = Smem<D>::kSlotBytes;
   constexpr int kBoxes = D / 64;                                          // boxes of 64 dims per tile
+  constexpr bool kReuse = kOrder != kAscending, kLeaving = kOrder == kReuseLeaving;
   // t is a multiple of 64: the last panel may hold 64 tokens only.  Its tile then covers 64 rows that are not the
   // call's; what is computed for them goes nowhere.
   const int t = G.t, P = (t + kTile - 1) / kTile, tp = P * kTile;
@@ -347,9 +355,7 @@ walk_tc_kernel(Geom G, const CallSet calls, int resident, int level, const CallS
     uint64_t* bar = full + 6 * x + 2 * slot + h;
     mbar_expect_tx(bar, kHalfBytes);
     unsigned char* dst = sm + slot * kSlotBytes + (x ? kTileBytes : 0u) + h * kHalfBytes;
-    // Where the resident calls' rows exceed L2 (kReuse), the panels that few later ones read again leave it first: 512 streams x
-    // 8192 tokens, t = 2048: 3515 us without, 3434 / 3459 / 3514 from panel 9 / 11 / 13 of 16 on.
-    if (kReuse && row0 - job->src_row >= 5 * P / 8 * kTile) tma_load_2d_leaving(dst, map, 64 * h, row0, bar);
+    if (kLeaving && row0 - job->src_row >= 5 * P / 8 * kTile) tma_load_2d_leaving(dst, map, 64 * h, row0, bar);   // panels that few later ones read again
     else tma_load_2d(dst, map, 64 * h, row0, bar);
   };
   if (warp == kTmaWarp && lane == 0) {
@@ -422,13 +428,17 @@ walk_tc_kernel(Geom G, const CallSet calls, int resident, int level, const CallS
   // r + 1 follow the last column but one into its slot, and the slots change roles.  All sides walk the same schedule and
   // count a slot's loads alike.  Every barrier is waited on phase by phase by its one kind of waiter, and each next phase
   // depends on that waiter having passed, so a parity wait can never be a phase behind.
+  // kSplit: the two branches' register counts as they are (96), but the compiler allocates the branches apart (592 calls of 1024 x 128:
+  // 195 -> 191 us; 64-dim heads 165 -> 179, tiles in reuse order 130 either way: without).
+  constexpr bool kSplit = D == 128 && !kReuse;
   if (warp >= kTmaWarp) {
+    if constexpr (kSplit) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kSplitRegs));
     if (warp == kTmaWarp) {
       // ------------------------------------------------------------------ TMA producer
       if (lane == 0) {
         uint32_t used = 1, par = 0;        // per slot: loaded before (slot 0 above); parity of the next wait on its empty barriers
         bool ok = true;
-        const int src_row = (int)C.src_row;
+        const int src_row = job->src_row;
         auto load = [&](int slot, int tile_row) -> bool {
           const bool again = (used >> slot) & 1u;
           const uint32_t ph = (par >> slot) & 1u;
@@ -530,6 +540,7 @@ walk_tc_kernel(Geom G, const CallSet calls, int resident, int level, const CallS
       if (lane == 0 && *abort_flag) atomicCAS(status, kStatusOk, kStatusWaitTimeout);
     }
   } else {
+    if constexpr (kSplit) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kSplitRegs));
     // ------------------------------------------------------------------ four epilogue warpgroups
     // Every tile is drained by all groups: group wg takes columns 32 wg .. 32 wg + 31 of the tile
     // (thread = row) and keeps a partial running correlation of its row over those columns.
@@ -720,7 +731,8 @@ walk_tc_kernel(Geom G, const CallSet calls, int resident, int level, const CallS
     tc_fence_before();
     __syncthreads();                                       // TMEM is drained
     if (ok) {
-      select_half(G, etas, reinterpret_cast<uint32_t*>(thr_s), kept, dbg_eta, job->record);
+      if constexpr (kReuse) select_half_apart(G, etas, reinterpret_cast<uint32_t*>(thr_s), kept, dbg_eta, job->record);
+      else select_half(G, etas, reinterpret_cast<uint32_t*>(thr_s), kept, dbg_eta, job->record);
       copy_rows<D>(G, A, job->src_row, job->dst_row, kept);
     }
   }
@@ -736,11 +748,17 @@ constexpr size_t kMaxSmem = (size_t)227 * 1024;         // of every kernel: the 
 // (148 x 1792 x 512 bytes against 126 MB).  Ascending order / reuse, us per launch: 2048 tokens, 1 call 132.4 / 128.4, 148
 // calls 181 / 169, 1024 calls 1265 / 1185; 3072 tokens, 148 calls 428 / 388.
 constexpr int kReuseTokens = 1792;
-bool reuse_tiles(const Geom& G) { return G.d == 128 && G.t >= kReuseTokens; }
-auto kernel_for(int d, bool center, bool reuse) {
-  if (d == 64) return center ? walk_tc_kernel<64, true, false> : walk_tc_kernel<64, false, false>;
-  if (reuse) return center ? walk_tc_kernel<128, true, true> : walk_tc_kernel<128, false, true>;
-  return center ? walk_tc_kernel<128, true, false> : walk_tc_kernel<128, false, false>;
+// With more rows resident than L2 holds, the late panels of a call leave it first: 512 streams x 8192 tokens, t = 2048: 3515 us without,
+// 3434 / 3459 / 3514 from panel 9 / 11 / 13 of 16 on.  With fewer they must stay (one call of 3072: 267 without, 284 with).
+int order_of(const Geom& G, int n_calls, int sm_count, int l2_bytes) {
+  if (G.d != 128 || G.t < kReuseTokens) return kAscending;
+  return (int64_t)std::min(n_calls, sm_count) * G.t * G.d * 4 > l2_bytes ? kReuseLeaving : kReuseStaying;
+}
+auto kernel_for(int d, bool center, int order) {
+  if (d == 64) return center ? walk_tc_kernel<64, true, kAscending> : walk_tc_kernel<64, false, kAscending>;
+  if (order == kReuseLeaving) return center ? walk_tc_kernel<128, true, kReuseLeaving> : walk_tc_kernel<128, false, kReuseLeaving>;
+  if (order == kReuseStaying) return center ? walk_tc_kernel<128, true, kReuseStaying> : walk_tc_kernel<128, false, kReuseStaying>;
+  return center ? walk_tc_kernel<128, true, kAscending> : walk_tc_kernel<128, false, kAscending>;
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -779,8 +797,14 @@ cudaError_t walk_tc_prepare(const Geom& G, const Arena& A, int64_t total_rows, v
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) { delete tm; return cudaErrorInvalidValue; }
   }
-  for (int i = 0; i < 4 && e == cudaSuccess; ++i)
-    e = cudaFuncSetAttribute(kernel_for(G.d, (i & 1) != 0, i > 1), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
+  for (int i = 0; i < 6 && e == cudaSuccess; ++i) {
+    auto kern = kernel_for(G.d, (i & 1) != 0, i / 2);
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
+    // a kernel that names its branches' registers (kSplitRegs) has to be launched with that many
+    cudaFuncAttributes attr;
+    if (e == cudaSuccess && i / 2 == kAscending && G.d == 128 && (e = cudaFuncGetAttributes(&attr, kern)) == cudaSuccess && attr.numRegs != kSplitRegs)
+      e = cudaErrorInvalidConfiguration;
+  }
   if (e != cudaSuccess) { delete tm; return e; }
   *tmaps_out = tm;
   return cudaSuccess;
@@ -791,12 +815,12 @@ void walk_tc_release(void* tmaps) { delete static_cast<TensorMaps*>(tmaps); }
 cudaError_t launch_walk_tc(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, int level,
                            const CallStat* stats, const float* tok_shift, int8_t* dbg_eta,
                            float* dbg_S, float* dbg_p, unsigned long long* fail_count, int* status,
-                           const void* tmaps, int sm_count, cudaStream_t st) {
+                           const void* tmaps, int sm_count, int l2_bytes, cudaStream_t st) {
   if (n_calls <= 0) return cudaSuccess;
   if (!tmaps) return cudaErrorInvalidValue;
   const TensorMaps* tm = static_cast<const TensorMaps*>(tmaps);
   const PdlConfig pc(dim3(n_calls), kThreads, tc_smem_bytes(G.d, G.t), st);
-  return cudaLaunchKernelEx(&pc.cfg, kernel_for(G.d, G.center_keys != 0, reuse_tiles(G)), G, calls, sm_count, level, stats, tok_shift,
+  return cudaLaunchKernelEx(&pc.cfg, kernel_for(G.d, G.center_keys != 0, order_of(G, n_calls, sm_count, l2_bytes)), G, calls, sm_count, level, stats, tok_shift,
                             dbg_eta, dbg_S, dbg_p, fail_count, status, G.center_keys ? nullptr : A.nrm, A, tm->k, tm->v);
 }
 

@@ -157,7 +157,6 @@ struct balancekv_ctx {
   unsigned* bkt_vmax_bits = nullptr;
   int32_t* bkt_chunk_cnt = nullptr;     // per (stream, chunk of the block): counts, then their prefix
   size_t bkt_chunk_ints = 0;
-  BucketOut* bkt_out = nullptr;
   BucketOut* bkt_out_host = nullptr;    // pinned
   size_t bkt_rows = 0, bkt_streams = 0;
   int64_t bucket_dropped = 0;
@@ -215,8 +214,13 @@ int ring_push(balancekv_ctx* c, const void* data, size_t bytes, cudaStream_t st,
     if (c->ring_ev_valid[c->ring_cur]) BKV_CUDA(cudaEventSynchronize(c->ring_ev[c->ring_cur]));
   }
   const size_t off = (size_t)c->ring_cur * c->ring_half + c->ring_pos;
-  std::memcpy(c->h_ring + off, data, bytes);
-  BKV_CUDA(cudaMemcpyAsync(c->d_ring + off, c->h_ring + off, bytes, cudaMemcpyHostToDevice, st));
+  if (bytes <= kUploadBytes) {
+    BKV_CUDA(launch_upload(c->d_ring + off, data, bytes, st));
+    c->kernels_launched++;
+  } else {
+    std::memcpy(c->h_ring + off, data, bytes);
+    BKV_CUDA(cudaMemcpyAsync(c->d_ring + off, c->h_ring + off, bytes, cudaMemcpyHostToDevice, st));
+  }
   c->ring_pos += need;
   *dev = c->d_ring + off;
   return BALANCEKV_OK;
@@ -431,7 +435,7 @@ int balancekv_destroy(balancekv_ctx* c) {
                   c->view_idx, c->bounce_K, c->bounce_V, c->bounce_q, c->bounce_out, c->step_dev_in, c->step_dev_out, c->two_acc, c->two_ml, c->two_scratch, c->unit_V};
   for (void* p : ptrs)
     if (p) cudaFree(p);
-  void* bkt[] = {c->bkt_ns, c->bkt_slot, c->bkt_rank, c->bkt_vmax_bits, c->bkt_out, c->bkt_chunk_cnt, c->acr_scratch, c->acr_cls};
+  void* bkt[] = {c->bkt_ns, c->bkt_slot, c->bkt_rank, c->bkt_vmax_bits, c->bkt_chunk_cnt, c->acr_scratch, c->acr_cls};
   for (void* p : bkt)
     if (p) cudaFree(p);
   if (c->bkt_out_host) cudaFreeHost(c->bkt_out_host);
@@ -701,11 +705,9 @@ static int run_plan(balancekv_ctx* c, Plan& P, cudaStream_t st) {
       if (rc) return rc;
     }
     ProfScope ps(c, 5, st);
-    BKV_CUDA(launch_seg_update(c->A, static_cast<const SegUpdate*>(d_segs), (int)P.segs.size(), st));
+    BKV_CUDA(launch_seg_update(c->A, static_cast<const SegUpdate*>(d_segs), (int)P.segs.size(), c->d_status, c->h_status_dev, st));
     c->kernels_launched++;
   }
-  // refresh the host's view of the status word behind the batch (4 bytes, no synchronisation)
-  BKV_CUDA(cudaMemcpyAsync(c->h_status, c->d_status, sizeof(int), cudaMemcpyDeviceToHost, st));
   return BALANCEKV_OK;
 }
 
@@ -1219,11 +1221,11 @@ static int append_bucketed_impl(balancekv_ctx* c, const std::vector<std::pair<in
   // routing buffers (grown with the largest block; the call synchronises the stream anyway)
   if ((size_t)n_sl * n > c->bkt_rows || (size_t)n_sl > c->bkt_streams || bucket_chunk_count_ints(n_sl, n) > c->bkt_chunk_ints) {
     BKV_CUDA(cudaStreamSynchronize(st));
-    void* old[] = {c->bkt_ns, c->bkt_slot, c->bkt_rank, c->bkt_vmax_bits, c->bkt_out, c->bkt_chunk_cnt};
+    void* old[] = {c->bkt_ns, c->bkt_slot, c->bkt_rank, c->bkt_vmax_bits, c->bkt_chunk_cnt};
     for (void* p : old)
       if (p) cudaFree(p);
     if (c->bkt_out_host) cudaFreeHost(c->bkt_out_host);
-    c->bkt_ns = nullptr; c->bkt_slot = nullptr; c->bkt_rank = nullptr; c->bkt_vmax_bits = nullptr; c->bkt_out = nullptr;
+    c->bkt_ns = nullptr; c->bkt_slot = nullptr; c->bkt_rank = nullptr; c->bkt_vmax_bits = nullptr;
     c->bkt_out_host = nullptr; c->bkt_chunk_cnt = nullptr;
     c->bkt_chunk_ints = std::max(c->bkt_chunk_ints, bucket_chunk_count_ints(n_sl, n));
     BKV_CUDA(cudaMalloc(reinterpret_cast<void**>(&c->bkt_chunk_cnt), sizeof(int32_t) * c->bkt_chunk_ints));
@@ -1233,7 +1235,7 @@ static int append_bucketed_impl(balancekv_ctx* c, const std::vector<std::pair<in
     BKV_CUDA(cudaMalloc(reinterpret_cast<void**>(&c->bkt_slot), c->bkt_rows));
     BKV_CUDA(cudaMalloc(reinterpret_cast<void**>(&c->bkt_rank), sizeof(int32_t) * c->bkt_rows));
     BKV_CUDA(cudaMalloc(reinterpret_cast<void**>(&c->bkt_vmax_bits), sizeof(unsigned) * c->bkt_streams));
-    BKV_CUDA(cudaMalloc(reinterpret_cast<void**>(&c->bkt_out), sizeof(BucketOut) * c->bkt_streams));
+    BKV_CUDA(cudaMemsetAsync(c->bkt_vmax_bits, 0, sizeof(unsigned) * c->bkt_streams, st));   // later calls find it emptied by the one before
     BKV_CUDA(cudaMallocHost(reinterpret_cast<void**>(&c->bkt_out_host), sizeof(BucketOut) * c->bkt_streams));
   }
   std::vector<BucketIn> in(n_sl);
@@ -1267,11 +1269,10 @@ static int append_bucketed_impl(balancekv_ctx* c, const std::vector<std::pair<in
   {
     ProfScope ps(c, 0, st);
     BKV_CUDA(launch_bucket_route(c->G, V, n_sl, n, n_buckets, i_top, rho * rho, static_cast<const BucketIn*>(d_in),
-                                 c->bkt_vmax_bits, c->bkt_ns, c->bkt_slot, c->bkt_rank, c->bkt_chunk_cnt, c->bkt_out, forced, st));
+                                 c->bkt_vmax_bits, c->bkt_ns, c->bkt_slot, c->bkt_rank, c->bkt_chunk_cnt, c->bkt_out_host, forced, st));
   }
   c->kernels_launched += 3;
-  BKV_CUDA(cudaMemcpyAsync(c->bkt_out_host, c->bkt_out, sizeof(BucketOut) * n_sl, cudaMemcpyDeviceToHost, st));
-  BKV_CUDA(cudaStreamSynchronize(st));   // the counts decide the host bookkeeping of every instance
+  BKV_CUDA(cudaStreamSynchronize(st));   // the counts (written to the host's memory) decide its bookkeeping of every instance
   const BucketOut* out = c->bkt_out_host;
   const int T = Lo.T;
   const int max_pending = T == 0 ? f.max_tokens : (f.max_pending > 0 ? std::min(f.max_pending, f.max_tokens) : f.max_tokens);

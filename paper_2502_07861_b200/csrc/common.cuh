@@ -266,7 +266,11 @@ int decode_warps();
 cudaError_t launch_decode(const Geom& G, const Arena& A, int layer, const void* q, void* out, float* scratch,
                           const StepAppend& ap, int* status, cudaStream_t st);
 cudaError_t launch_fill_weights(float* w, int n, float value, cudaStream_t st);
-cudaError_t launch_seg_update(const Arena& A, const SegUpdate* ups, int n, cudaStream_t st);
+// Segment updates of a batch; a device-side failure is shown to the host behind them.
+cudaError_t launch_seg_update(const Arena& A, const SegUpdate* ups, int n, const int* status, int* status_host, cudaStream_t st);
+// A host array of at most kUploadBytes to the device, as a kernel's parameters.
+constexpr size_t kUploadBytes = 16384;
+cudaError_t launch_upload(void* dst, const void* data, size_t bytes, cudaStream_t st);
 int bucket_scan_chunks(int n);
 size_t bucket_chunk_count_ints(int n_sl, int n);   // ints of the per-chunk count table of the routing pass
 cudaError_t launch_bucket_route(const Geom& G, const void* V, int n_sl, int n, int n_buckets, int i_top, float rho2,

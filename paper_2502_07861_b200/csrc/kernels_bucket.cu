@@ -45,6 +45,7 @@ __device__ inline float sumsq_piece(const uint4& v) {
 template <bool kBf16>
 __global__ void __launch_bounds__(256)
 bucket_norms_kernel(const void* __restrict__ V, int n, int chunks, float* __restrict__ ns, unsigned* __restrict__ vmax2_bits) {
+  grid_wait_and_release();
   const int sl = blockIdx.y;
   const int rows_per_pass = blockDim.x / chunks;         // 32, 16 or 8
   const int row_in = threadIdx.x / chunks, piece = threadIdx.x % chunks;
@@ -114,6 +115,7 @@ bucket_scan_kernel(const float* __restrict__ ns, int n, int n_chunks, int n_buck
                    int32_t* __restrict__ rank, int32_t* __restrict__ chunk_cnt, const int8_t* __restrict__ forced) {
   constexpr int kWarps = kScanThreads / 32, kRounds = kScanChunk / kScanThreads;
   __shared__ int warp_tot[kCountCols][kWarps];
+  grid_wait_and_release();
   const int sl = blockIdx.y, chunk = blockIdx.x;
   const int erase_max = erase_index(rho2, in[sl], vmax2_bits[sl]);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -179,8 +181,9 @@ bucket_scan_kernel(const float* __restrict__ ns, int n, int n_chunks, int n_buck
 // Second part: per stream, the exclusive prefix of the chunks' counts (in place) and the totals.
 // grid (streams), kCountCols warps: warp b scans column b, 32 chunks at a time.
 __global__ void __launch_bounds__(kCountCols * 32)
-bucket_prefix_kernel(int n_chunks, float rho2, const BucketIn* __restrict__ in, const unsigned* __restrict__ vmax2_bits,
+bucket_prefix_kernel(int n_chunks, float rho2, const BucketIn* __restrict__ in, unsigned* __restrict__ vmax2_bits,
                      int32_t* __restrict__ chunk_cnt, BucketOut* __restrict__ out) {
+  grid_wait_and_release();
   const int sl = blockIdx.x, col = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int32_t* c = chunk_cnt + (size_t)sl * n_chunks * kCountCols + col;
   int carry = 0;
@@ -204,6 +207,7 @@ bucket_prefix_kernel(int n_chunks, float rho2, const BucketIn* __restrict__ in, 
   if (threadIdx.x == 0) {
     out[sl].erase_max = erase_index(rho2, in[sl], vmax2_bits[sl]);
     out[sl].vmax2 = fmaxf(in[sl].prev_vmax2, __uint_as_float(vmax2_bits[sl]));
+    vmax2_bits[sl] = 0u;                     // for the next call
   }
 }
 
@@ -216,6 +220,7 @@ bucket_scatter_kernel(Geom G, Arena A, const void* __restrict__ Ksrc, const void
                       int n_buckets, const int8_t* __restrict__ slot, const int32_t* __restrict__ rank,
                       const int32_t* __restrict__ chunk_base, int n_chunks, const float* __restrict__ ns,
                       const BucketDst* __restrict__ dst) {
+  grid_wait_and_release();
   const int sl = blockIdx.y;
   const int rows_per_pass = blockDim.x / chunks;
   const int row_in = threadIdx.x / chunks, piece = threadIdx.x % chunks;
@@ -259,16 +264,15 @@ cudaError_t launch_bucket_route(const Geom& G, const void* V, int n_sl, int n, i
                                 const BucketIn* in, unsigned* vmax2_bits, float* ns, int8_t* slot, int32_t* rank,
                                 int32_t* chunk_cnt, BucketOut* out, const int8_t* forced_slot, cudaStream_t st) {
   const int chunks = G.d * (G.is_bf16 ? 2 : 4) / 16;
-  cudaError_t e = cudaMemsetAsync(vmax2_bits, 0, sizeof(unsigned) * n_sl, st);
-  if (e != cudaSuccess) return e;
-  dim3 grid((n + kRowsPerBlock - 1) / kRowsPerBlock, n_sl);
-  if (G.is_bf16) bucket_norms_kernel<true><<<grid, 256, 0, st>>>(V, n, chunks, ns, vmax2_bits);
-  else bucket_norms_kernel<false><<<grid, 256, 0, st>>>(V, n, chunks, ns, vmax2_bits);
+  const PdlConfig norms(dim3((n + kRowsPerBlock - 1) / kRowsPerBlock, n_sl), 256, 0, st);
+  cudaError_t e = cudaLaunchKernelEx(&norms.cfg, G.is_bf16 ? bucket_norms_kernel<true> : bucket_norms_kernel<false>, V, n, chunks, ns, vmax2_bits);
   const int n_chunks = bucket_scan_chunks(n);
-  bucket_scan_kernel<<<dim3(n_chunks, n_sl), kScanThreads, 0, st>>>(ns, n, n_chunks, n_buckets, i_top, rho2, in, vmax2_bits,
-                                                                   slot, rank, chunk_cnt, forced_slot);
-  bucket_prefix_kernel<<<n_sl, kCountCols * 32, 0, st>>>(n_chunks, rho2, in, vmax2_bits, chunk_cnt, out);
-  return cudaGetLastError();
+  const PdlConfig scan(dim3(n_chunks, n_sl), kScanThreads, 0, st);
+  if (e == cudaSuccess)
+    e = cudaLaunchKernelEx(&scan.cfg, bucket_scan_kernel, static_cast<const float*>(ns), n, n_chunks, n_buckets, i_top, rho2, in,
+                           static_cast<const unsigned*>(vmax2_bits), slot, rank, chunk_cnt, forced_slot);
+  const PdlConfig prefix(dim3(n_sl), kCountCols * 32, 0, st);
+  return e != cudaSuccess ? e : cudaLaunchKernelEx(&prefix.cfg, bucket_prefix_kernel, n_chunks, rho2, in, vmax2_bits, chunk_cnt, out);
 }
 
 cudaError_t launch_bucket_scatter(const Geom& G, const Arena& A, const void* K, const void* V, int n_sl, int n,
@@ -276,12 +280,9 @@ cudaError_t launch_bucket_scatter(const Geom& G, const Arena& A, const void* K, 
                                   const float* ns, const BucketDst* dst, cudaStream_t st) {
   const int chunks = G.d * (G.is_bf16 ? 2 : 4) / 16;
   const int n_chunks = bucket_scan_chunks(n);
-  dim3 grid((n + kRowsPerBlock - 1) / kRowsPerBlock, n_sl);
-  if (G.is_bf16)
-    bucket_scatter_kernel<true><<<grid, 256, 0, st>>>(G, A, K, V, n, chunks, n_buckets, slot, rank, chunk_base, n_chunks, ns, dst);
-  else
-    bucket_scatter_kernel<false><<<grid, 256, 0, st>>>(G, A, K, V, n, chunks, n_buckets, slot, rank, chunk_base, n_chunks, ns, dst);
-  return cudaGetLastError();
+  const PdlConfig pc(dim3((n + kRowsPerBlock - 1) / kRowsPerBlock, n_sl), 256, 0, st);
+  return cudaLaunchKernelEx(&pc.cfg, G.is_bf16 ? bucket_scatter_kernel<true> : bucket_scatter_kernel<false>, G, A, K, V, n, chunks, n_buckets, slot,
+                            rank, chunk_base, n_chunks, ns, dst);
 }
 
 }  // namespace bkv

@@ -3,6 +3,7 @@
 //   level-0 remainder move
 //   the optional key shift of a call and its radii r_key^2, r_value^2 (inputs of Algorithm 2)
 #include <algorithm>
+#include <cstring>
 
 #include "common.cuh"
 
@@ -150,6 +151,7 @@ __device__ inline void move_rows(const Geom& G, const Arena& A, const MoveDesc& 
 
 __global__ void __launch_bounds__(256)
 move_kernel(Geom G, Arena A, const MoveDesc* __restrict__ descs) {
+  grid_wait_and_release();
   move_rows(G, A, descs[blockIdx.x], blockIdx.y * kCopyRows);
 }
 
@@ -186,9 +188,32 @@ reset_kernel(Seg* __restrict__ seg, size_t n_seg, uint4* __restrict__ scratch, s
   }
 }
 
-__global__ void seg_update_kernel(Arena A, const SegUpdate* __restrict__ ups, int n) {
+__global__ void seg_update_kernel(Arena A, const SegUpdate* __restrict__ ups, int n, const int* __restrict__ status,
+                                  int* __restrict__ status_host) {
+  grid_wait_and_release();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) A.seg[ups[i].index] = Seg{ups[i].start, ups[i].len};
+  if (i == 0 && *status != kStatusOk) *static_cast<volatile int*>(status_host) = *status;
+}
+
+// Descriptors travel as a kernel's parameters: a transfer between two kernels ends their overlap and took 8 us of a batch's
+// chain where this takes 2.
+template <size_t kBytes>
+struct Blob {
+  uint4 w[kBytes / 16];
+};
+template <size_t kBytes>
+__global__ void __launch_bounds__(256)
+upload_kernel(uint4* __restrict__ dst, int n, const __grid_constant__ Blob<kBytes> data) {
+  for (int i = threadIdx.x; i < n; i += 256) dst[i] = data.w[i];
+  grid_wait_and_release();                   // what follows waits for this kernel alone
+}
+template <size_t kBytes>
+cudaError_t upload(void* dst, const void* data, size_t bytes, cudaStream_t st) {
+  Blob<kBytes> b;
+  std::memcpy(&b, data, bytes);
+  const PdlConfig pc(dim3(1), 256, 0, st);
+  return cudaLaunchKernelEx(&pc.cfg, upload_kernel<kBytes>, static_cast<uint4*>(dst), (int)((bytes + 15) / 16), b);
 }
 
 // Key centering: one CTA per call.  The mean of the call's keys (fixed summation order, so the result is reproducible),
@@ -302,8 +327,8 @@ cudaError_t launch_move(const Geom& G, const Arena& A, const MoveDesc* descs, in
   if (n_desc <= 0) return cudaSuccess;
   dim3 grid(n_desc, (max_rows + kCopyRows - 1) / kCopyRows);
   if (grid.y == 0) grid.y = 1;
-  move_kernel<<<grid, 256, 0, st>>>(G, A, descs);
-  return cudaGetLastError();
+  const PdlConfig pc(grid, 256, 0, st);
+  return cudaLaunchKernelEx(&pc.cfg, move_kernel, G, A, descs);
 }
 
 cudaError_t launch_batch_end(const Geom& G, const Arena& A, const BatchEnd& E, int n_streams, const Seg* seg,
@@ -329,10 +354,16 @@ cudaError_t launch_center(const Geom& G, const Arena& A, const CallSet& calls, i
   return cudaLaunchKernelEx(&pc.cfg, G.is_bf16 ? center_kernel<true> : center_kernel<false>, G, A, calls, stats, tok_shift);
 }
 
-cudaError_t launch_seg_update(const Arena& A, const SegUpdate* ups, int n, cudaStream_t st) {
+cudaError_t launch_seg_update(const Arena& A, const SegUpdate* ups, int n, const int* status, int* status_host, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  seg_update_kernel<<<(n + 255) / 256, 256, 0, st>>>(A, ups, n);
-  return cudaGetLastError();
+  const PdlConfig pc(dim3((n + 255) / 256), 256, 0, st);
+  return cudaLaunchKernelEx(&pc.cfg, seg_update_kernel, A, ups, n, status, status_host);
+}
+
+cudaError_t launch_upload(void* dst, const void* data, size_t bytes, cudaStream_t st) {
+  if (bytes <= 1024) return upload<1024>(dst, data, bytes, st);
+  if (bytes <= 4096) return upload<4096>(dst, data, bytes, st);
+  return bytes <= kUploadBytes ? upload<kUploadBytes>(dst, data, bytes, st) : cudaErrorInvalidValue;
 }
 
 cudaError_t launch_fill_weights(float* w, int n, float value, cudaStream_t st) {

@@ -226,6 +226,7 @@ walk_kernel(Geom G, const CallSet calls, int call0, int level, const float* __re
   uint64_t* full = reinterpret_cast<uint64_t*>(cur + 2 * kTile);         // [stages], then [stages] empty
   uint64_t* empty = full + kWalkStages;
   const int call = call0 + blockIdx.x;
+  if (calls.list) asm volatile("griddepcontrol.wait;" ::: "memory");   // its descriptor comes from a kernel of this batch
   const CallDesc C = call_of(calls, G, call);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (tid == 0) {

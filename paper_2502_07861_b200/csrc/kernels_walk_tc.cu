@@ -372,6 +372,8 @@ walk_tc_kernel(Geom G, const CallSet calls, int resident, int level, const CallS
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_ptr_s)), "r"(kTmemCols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  // A listed call's descriptor may come from the kernel right before this one.
+  if (calls.list) asm volatile("griddepcontrol.wait;" ::: "memory");
   CallDesc C;
   if (warp < kEpiWarps || (warp == kTmaWarp && lane == 0)) C = call_of(calls, G, call);
   auto draw_coins = [&]() {

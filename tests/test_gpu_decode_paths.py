@@ -372,3 +372,31 @@ def test_replayed_step_puts_its_token_in_the_same_place(cuda_lib, dtype, d, g):
     _check_heads(got.float().cpu().numpy(), K[:, :, rows], V[:, :, rows], np.ones(n + 1), q, g, dtype, "behind")
     assert ctx.stats()["device_status"] == 0 and ctx.debug_scratch_used() == 0
     ctx.close()
+
+
+@pytest.mark.parametrize("B,d,g,rows", [(1, 128, 4, 8192), (8, 128, 5, 1024), (2, 64, 8, 8000), (1, 128, 1, 8211)])
+def test_caches_beyond_l2_decode_as_they_do_alone(cuda_lib, B, d, g, rows):
+    """Layers that together exceed L2 load part of their tiles to leave it first; each gives what it gives in a context of its own."""
+    import torch
+
+    L, H = 4, 8
+    gen = torch.Generator(device="cuda").manual_seed(21)
+    make = lambda layers: cuda_lib.Context(n_seqs=B, n_layers=layers, n_kv_heads=H, n_q_heads=H * g, head_dim=d, dtype="bf16", block=64,
+                                           levels=2, max_tokens=4 * rows + 64, max_pending=64)
+    q, kn, vn = (torch.randn(B, n, d, device="cuda", generator=gen).bfloat16() for n in (H * g, H, H))
+    ctx, alone = make(L), make(1)
+    for layer in range(L):
+        K, V = (torch.randn(B, H, rows, d, device="cuda", generator=gen).bfloat16() for _ in range(2))
+        outs = []
+        for c, at in ((ctx, layer), (alone, 0)):
+            if c is alone:
+                c.reset()
+            c.cache_load_level(at, 2, K, V)
+            step = torch.empty_like(q)
+            first = c.decode_attn(at, q)
+            c.stream_step(at, q, kn, vn, step)
+            outs.append([first, step, c.decode_attn(at, q)])
+        assert all(torch.equal(a, b) for a, b in zip(*outs)), layer
+    assert ctx.stats()["device_status"] == 0 and alone.stats()["device_status"] == 0
+    ctx.close()
+    alone.close()

@@ -584,7 +584,7 @@ int balancekv_cache_load_level(balancekv_ctx* c, int layer, int level, const voi
 }
 
 // One level of a batch: radii -> walk -> selection/compaction for n calls.
-static int run_calls(balancekv_ctx* c, const CallSet& calls, int n, int l, cudaStream_t st) {
+static int run_calls(balancekv_ctx* c, const CallSet& calls, int n, int l, const BatchTail& tail, cudaStream_t st) {
   const Geom& G = c->G;
   if (G.center_keys) {          // else the walk takes the radii from the stored row norms itself
     ProfScope ps(c, 1, st);
@@ -603,7 +603,7 @@ static int run_calls(balancekv_ctx* c, const CallSet& calls, int n, int l, cudaS
   }
   if (!c->use_tc) {
     ProfScope ps(c, 3, st);
-    BKV_CUDA(launch_compact(G, c->A, calls, n, l, c->d_eta, st));
+    BKV_CUDA(launch_compact(G, c->A, calls, n, c->d_eta, tail, st));
     c->kernels_launched++;
   }
   c->kernels_launched++;
@@ -622,11 +622,15 @@ static int run_lockstep(balancekv_ctx* c, int layer, int first, int n, int nb, c
   BatchEnd E;
   Seg seg[kMaxLevels + 1];
   plan_lockstep(c->Lo, S, nb, layer, first, sets, calls, E, seg);
+  // Without rows to move, the compaction of the last level ends the batch as well (a launch of its own: 2.5 us of a small one).
+  const bool ends = !c->use_tc && E.move_rows == 0;
   for (int l = 0; l < c->G.T; ++l) {
     if (calls[l] == 0) break;
-    if (const int rc = run_calls(c, sets[l], n * calls[l], l, st)) return rc;
+    BatchTail tail{};
+    if (ends && (l + 1 == c->G.T || calls[l + 1] == 0)) tail = BatchTail{layer, first, n, seg_row(c->G.T, seg), c->d_status, c->h_status_dev};
+    if (const int rc = run_calls(c, sets[l], n * calls[l], l, tail, st)) return rc;
   }
-  {
+  if (!ends) {
     ProfScope ps(c, 5, st);
     BKV_CUDA(launch_batch_end(c->G, c->A, E, n, seg, c->d_status, c->h_status_dev, st));
     c->kernels_launched++;
@@ -685,7 +689,7 @@ static int run_plan(balancekv_ctx* c, Plan& P, cudaStream_t st) {
       }
       CallSet set{};
       set.list = static_cast<const CallDesc*>(d_calls);
-      if (const int rc = run_calls(c, set, n, l, st)) return rc;
+      if (const int rc = run_calls(c, set, n, l, BatchTail{}, st)) return rc;
     }
   }
   if (!P.moves.empty()) {

@@ -95,6 +95,22 @@ struct Seg {  // one level of one stream: rows [start, start+len) of the level's
   int32_t start, len;
 };
 
+struct SegRow {  // the segments of a lockstep stream after a batch
+  Seg seg[kMaxLevels + 1];
+};
+inline SegRow seg_row(int T, const Seg* seg) {
+  SegRow row;
+  for (int l = 0; l <= kMaxLevels; ++l) row.seg[l] = l <= T ? seg[l] : Seg{0, 0};
+  return row;
+}
+// What compact_kernel does for a batch whose last launch it is: the segments of its lockstep streams (n_streams = 0: nothing).
+struct BatchTail {
+  int32_t layer, first, n_streams;
+  SegRow row;
+  const int* status;
+  int* status_host;
+};
+
 // Per-call radii of Algorithm 2 and the key shift.
 struct CallStat {
   float rk2, rv2;    // r_key^2, r_value^2
@@ -257,8 +273,8 @@ cudaError_t launch_walk_tc(const Geom& G, const Arena& A, const CallSet& calls, 
                            const CallStat* stats, const float* tok_shift, int8_t* dbg_eta,
                            float* dbg_S, float* dbg_p, unsigned long long* fail_count, int* status,
                            const void* tmaps, int sm_count, int l2_bytes, cudaStream_t st);
-cudaError_t launch_compact(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, int level,
-                           const int8_t* eta, cudaStream_t st);
+cudaError_t launch_compact(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, const int8_t* eta, const BatchTail& tail,
+                           cudaStream_t st);
 struct StepAppend;      // decode_common.cuh
 size_t decode_scratch_bytes(const Geom& G, int splits);
 int decode_tile_tokens(const Geom& G);

@@ -40,7 +40,7 @@ __device__ inline int block_exclusive_scan(int v, int* warp_sums, int& total) {
 }
 
 __global__ void __launch_bounds__(kThreads)
-compact_kernel(Geom G, Arena A, const CallSet calls, const int8_t* __restrict__ eta) {
+compact_kernel(Geom G, Arena A, const CallSet calls, const int8_t* __restrict__ eta, const BatchTail tail) {
   extern __shared__ int kept_pos[];  // [t/2]
   __shared__ int warp_sums[kThreads / 32];
   grid_wait_and_release();
@@ -80,31 +80,47 @@ compact_kernel(Geom G, Arena A, const CallSet calls, const int8_t* __restrict__ 
   const int chunks = G.d * esz / 16;
   const int o0 = blockIdx.y * kRowsPerCta;
   const int rows = min(kRowsPerCta, half - o0);
-  const int per_row = 2 * chunks;
-  for (int i = threadIdx.x; i < rows * per_row; i += kThreads) {
-    const int o = o0 + i / per_row;
-    const int rem = i % per_row;
-    const int which = rem / chunks, ch = rem % chunks;
-    const char* src = static_cast<const char*>(which ? A.V : A.K) + (size_t)(C.src_row + kept_pos[o]) * G.d * esz;
-    char* dst = static_cast<char*>(which ? A.V : A.K) + (size_t)(C.dst_row + o) * G.d * esz;
-    reinterpret_cast<uint4*>(dst)[ch] = reinterpret_cast<const uint4*>(src)[ch];
+  const int sh = 31 - __clz(chunks);                          // a row has 8, 16 or 32 pieces of 16 bytes
+  const int items = rows << (sh + 1);
+  const uint4* Ks = static_cast<const uint4*>(A.K) + ((size_t)C.src_row << sh);
+  const uint4* Vs = static_cast<const uint4*>(A.V) + ((size_t)C.src_row << sh);
+  uint4* Kd = static_cast<uint4*>(A.K) + ((size_t)C.dst_row << sh);
+  uint4* Vd = static_cast<uint4*>(A.V) + ((size_t)C.dst_row << sh);
+  // kDeep loads in flight per thread
+  constexpr int kDeep = 8;
+  for (int i0 = threadIdx.x; i0 < items; i0 += kDeep * kThreads) {
+    uint4 v[kDeep];
+#pragma unroll
+    for (int u = 0; u < kDeep; ++u) {
+      const int i = i0 + u * kThreads, o = i >> (sh + 1), ch = i & (chunks - 1);
+      if (i < items) v[u] = ((i >> sh) & 1 ? Vs : Ks)[((size_t)kept_pos[o0 + o] << sh) + ch];
+    }
+#pragma unroll
+    for (int u = 0; u < kDeep; ++u) {
+      const int i = i0 + u * kThreads, o = i >> (sh + 1), ch = i & (chunks - 1);
+      if (i < items) ((i >> sh) & 1 ? Vd : Kd)[((size_t)(o0 + o) << sh) + ch] = v[u];
+    }
   }
   for (int i = threadIdx.x; i < rows; i += kThreads) {
     A.idx[C.dst_row + o0 + i] = A.idx[C.src_row + kept_pos[o0 + i]];
     if (A.nrm) A.nrm[C.dst_row + o0 + i] = A.nrm[C.src_row + kept_pos[o0 + i]];
   }
+  if ((int)blockIdx.x < tail.n_streams && blockIdx.y == 0) {
+    const int stream = lockstep_stream(G, tail.layer, tail.first + blockIdx.x);
+    if (threadIdx.x <= G.T) A.seg[(size_t)stream * (G.T + 1) + threadIdx.x] = tail.row.seg[threadIdx.x];
+    if (blockIdx.x == 0 && threadIdx.x == 0 && *tail.status != kStatusOk) *static_cast<volatile int*>(tail.status_host) = *tail.status;
+  }
 }
 
 }  // namespace
 
-cudaError_t launch_compact(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, int level,
-                           const int8_t* eta, cudaStream_t st) {
+cudaError_t launch_compact(const Geom& G, const Arena& A, const CallSet& calls, int n_calls, const int8_t* eta, const BatchTail& tail,
+                           cudaStream_t st) {
   if (n_calls <= 0) return cudaSuccess;
   const int half = G.t / 2;
   dim3 grid(n_calls, (half + kRowsPerCta - 1) / kRowsPerCta);
-  (void)level;
   const PdlConfig pc(grid, kThreads, sizeof(int) * half, st);
-  return cudaLaunchKernelEx(&pc.cfg, compact_kernel, G, A, calls, eta);
+  return cudaLaunchKernelEx(&pc.cfg, compact_kernel, G, A, calls, eta, tail);
 }
 
 }  // namespace bkv

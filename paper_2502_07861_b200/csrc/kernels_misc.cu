@@ -155,9 +155,6 @@ move_kernel(Geom G, Arena A, const MoveDesc* __restrict__ descs) {
   move_rows(G, A, descs[blockIdx.x], blockIdx.y * kCopyRows);
 }
 
-struct SegRow {            // the segments of a lockstep stream after a batch
-  Seg seg[kMaxLevels + 1];
-};
 // grid (streams, row groups of the move)
 __global__ void __launch_bounds__(256)
 batch_end_kernel(Geom G, Arena A, BatchEnd E, SegRow row, const int* __restrict__ status, int* __restrict__ status_host) {
@@ -333,8 +330,7 @@ cudaError_t launch_move(const Geom& G, const Arena& A, const MoveDesc* descs, in
 
 cudaError_t launch_batch_end(const Geom& G, const Arena& A, const BatchEnd& E, int n_streams, const Seg* seg,
                              const int* status, int* status_host, cudaStream_t st) {
-  SegRow row;
-  for (int l = 0; l <= kMaxLevels; ++l) row.seg[l] = l <= G.T ? seg[l] : Seg{0, 0};
+  const SegRow row = seg_row(G.T, seg);
   const PdlConfig pc(dim3(n_streams, std::max(1, (E.move_rows + kCopyRows - 1) / kCopyRows)), 256, 0, st);
   return cudaLaunchKernelEx(&pc.cfg, batch_end_kernel, G, A, E, row, status, status_host);
 }

@@ -154,6 +154,10 @@ __device__ inline float2 poly_exp2x2(float2 x) {
 // Of the 16 column pairs of a 32-column chunk, pairs with (index % 8) < kPolyOf8 take the
 // polynomial path, the others the special-function unit.
 constexpr int kPolyOf8 = 1;
+// Not with key centering: a fixed radius that the shifted keys exceed gives exponents beyond the polynomial's range, whose overflow
+// the special-function unit turns into infinity (592 calls of 1024 x 128 339 us either way).
+template <bool kCenter>
+constexpr int kPolyPairs = kCenter ? 0 : kPolyOf8;
 
 template <int D>
 struct Smem {
@@ -578,7 +582,7 @@ walk_tc_kernel(Geom G, const CallSet calls, int resident, int level, const CallS
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const int i = 4 * x + 2 * h, pair = 2 * x + h;
-          const float2 g = ghat2(dk[i], dk[i + 1], dv[i], dv[i + 1], nb, h ? make_float2(sh.z, sh.w) : make_float2(sh.x, sh.y), (pair & 7) < kPolyOf8);
+          const float2 g = ghat2(dk[i], dk[i + 1], dv[i], dv[i + 1], nb, h ? make_float2(sh.z, sh.w) : make_float2(sh.x, sh.y), (pair & 7) < kPolyPairs<kCenter>);
           a2[pair & 1] = __ffma2_rn(g, h ? make_float2(e.z, e.w) : make_float2(e.x, e.y), a2[pair & 1]);
         }
       }

@@ -202,3 +202,27 @@ def test_cuda_core_walk_with_little_memory(cuda_lib):
     torch.cuda.empty_cache()
     assert small < whole - (200 << 20)
     assert all(torch.equal(a, b) for a, b in zip(got, want))
+
+
+def test_centered_call_beyond_a_fixed_radius(cuda_lib):
+    """Keys that a fixed radius is far too small for: the exponential overflows, and the sum with it, on both kernel families.
+    (Token 0 and token 200 share a key; token 0 is a column of token 200's panel.)"""
+    import torch
+
+    t, d = 256, 128
+    gen = torch.Generator(device="cuda").manual_seed(4)
+    K = torch.zeros(1, 1, t, d, device="cuda")
+    K[0, 0, 0] = K[0, 0, 200] = 3.5
+    V = torch.rand(1, 1, t, d, device="cuda", generator=gen)
+    sums = []
+    for path in (0, 1):
+        ctx = cuda_lib.Context(n_seqs=1, n_layers=1, n_kv_heads=1, n_q_heads=1, head_dim=d, dtype="bf16", block=t, levels=1, max_tokens=t,
+                               seed=3, c_override=0.75, center_keys=1, r_key=1.0, gram_path=path)
+        ctx.debug_enable()
+        ctx.stream_append_layer(0, K.bfloat16(), V.bfloat16())
+        ctx.compress()
+        sums.append(ctx.debug_call(0, 0, 0, 0, 0)[1])
+        assert ctx.stats()["device_status"] == 0 and ctx.stats()["walk_kernel"] == 2 - path
+        ctx.close()
+    assert torch.isinf(sums[1][200]) and sums[0][200].abs() == sums[1][200].abs()
+    assert torch.isfinite(sums[0][:200]).all()

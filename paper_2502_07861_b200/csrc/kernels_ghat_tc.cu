@@ -46,10 +46,118 @@ __device__ inline float grid_magic(float n2) {
   return __uint_as_float((uint32_t)((e >> 1) + 13 + 127) << 23 | 0x400000u);
 }
 
+__device__ inline void workers_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kWorkers) : "memory"); }
+
+// r_key^2, r_value^2 (inputs of Algorithm 2): maxima of the stored row norms, unless center_kernel has put them or they are fixed.
+__device__ inline float2 radii(const Geom& G, float mk, float mv, const CallStat* put) {
+  float2 r = make_float2(G.fixed_rk2, G.fixed_rv2);
+  if (r.x <= 0.f) r.x = put ? put->rk2 : mk;
+  if (r.y <= 0.f) r.y = put ? put->rv2 : mv;
+  return r;
+}
+
+// A block index' 128-row panel R and column tile: the panel has 2 R + 2 of them.
+__device__ inline int2 tile_of(int block) {
+  int R = 0;
+  for (; block >= 2 * R + 2; ++R) block -= 2 * R + 2;
+  return make_int2(R, block);
+}
+
+// The panel's halves as 64 x 64 tiles at sm, to the workspace.
+__device__ inline void store_tiles(float* ghat, int tiles_per_call, int t, int2 at, const unsigned char* sm) {
+  const int half = threadIdx.x, r = 2 * at.x + half;
+  if (half < 2 && at.y <= r && r < t / kGhatTile) {
+    float* to = ghat + ((size_t)blockIdx.y * tiles_per_call + r * (r + 1) / 2 + at.y) * (kGhatTile * kGhatTile);
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
+                 ::"l"(to), "r"(smem_u32(sm + half * kGhatTileBytes)), "r"(kGhatTileBytes) : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+    asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the stores end with the grid, which the walk waits for
+  }
+}
+
+// The CTA's tiles by FFMA, bit by bit what ghat_kernel gives (kernels_walk_simt.cu: 4 x 4 entries per thread, two stages of 32 dims),
+// by way of the planes' memory.  For the eight splitting warps.
+template <int D>
+__device__ __noinline__ void ffma_tiles(const Geom& G, const Arena& A, const CallSet& calls, int call0, const CallStat* stats, const float* tok_shift,
+                                        float* ghat, int tiles_per_call, const float (*red)[kWorkers / 32], unsigned char* sm) {
+  constexpr int kChunk = 32, kStride = kChunk * 4 + 16, kStageBytes = 2 * kGhatTile * kStride, kHalf = D / kChunk, kSteps = 2 * kHalf;
+  static_assert(2 * kGhatTileBytes + 2 * kStageBytes <= (int)kPlanes, "the planes' memory");
+  const int call = call0 + blockIdx.y, t = G.t, ty = threadIdx.x / 16, tx = threadIdx.x % 16;
+  const int2 at = tile_of(blockIdx.x);
+  float mk = 0.f, mv = 0.f;
+  for (int w = 0; w < kWorkers / 32; ++w) { mk = fmaxf(mk, red[0][w]); mv = fmaxf(mv, red[1][w]); }
+  const float2 r2 = radii(G, mk, mv, tok_shift ? stats + call : nullptr);
+  const float inv_rv2 = r2.y > 0.f ? 1.0f / r2.y : 0.f, scale = 1.4426950408889634f * G.inv_sqrt_d;
+  const float* shift = tok_shift ? tok_shift + (size_t)call * t : nullptr;
+  const size_t first = (size_t)call_of(calls, G, call).src_row * D;
+  unsigned char* stages = sm + 2 * kGhatTileBytes;
+#pragma unroll 1
+  for (int h = 0; h < 2; ++h) {
+    const int row0 = (2 * at.x + h) * kGhatTile, col0 = at.y * kGhatTile;
+    if (row0 >= t || col0 > row0) continue;
+    auto issue = [&](int step) {
+      unsigned char* st = stages + (step & 1) * kStageBytes;
+      const float* base = static_cast<const float*>(step < kHalf ? A.K : A.V) + first + (step % kHalf) * kChunk;
+      for (int i = threadIdx.x; i < 2 * kGhatTile * 8; i += kWorkers) {
+        const int row = i / 8, p = i % 8, token = row < kGhatTile ? row0 + row : col0 + row - kGhatTile;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(st + row * kStride + p * 16)), "l"(base + (size_t)token * D + p * 4) : "memory");
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    issue(0);
+    issue(1);
+    float2 acc[4][4];
+    float ex[4][4];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) acc[i / 4][i % 4] = make_float2(0.f, 0.f);
+#pragma unroll 1
+    for (int step = 0; step < kSteps; ++step) {
+      if (step + 1 < kSteps) asm volatile("cp.async.wait_group 1;" ::: "memory");
+      else asm volatile("cp.async.wait_group 0;" ::: "memory");
+      workers_sync();
+      const unsigned char* rows = stages + (step & 1) * kStageBytes + ty * kStride;
+      const unsigned char* cols = stages + (step & 1) * kStageBytes + (kGhatTile + tx) * kStride;
+#pragma unroll 1
+      for (int e = 0; e < kChunk; e += 4) {
+        float4 x[4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) x[a] = *reinterpret_cast<const float4*>(rows + 16 * a * kStride + 4 * e);
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          const float4 y = *reinterpret_cast<const float4*>(cols + 16 * b * kStride + 4 * e);
+#pragma unroll
+          for (int a = 0; a < 4; ++a) acc[a][b] = __ffma2_rn(make_float2(x[a].x, x[a].y), make_float2(y.x, y.y), acc[a][b]);
+#pragma unroll
+          for (int a = 0; a < 4; ++a) acc[a][b] = __ffma2_rn(make_float2(x[a].z, x[a].w), make_float2(y.z, y.w), acc[a][b]);
+        }
+      }
+      workers_sync();
+      if (step + 2 < kSteps) issue(step + 2);
+      if (step + 1 != kHalf) continue;
+#pragma unroll
+      for (int k = 0; k < 16; ++k) {
+        const int a = k / 4, b = k % 4, j = row0 + ty + 16 * a, i = col0 + tx + 16 * b;
+        const float off = (shift ? shift[j] : 0.f) + r2.x;
+        ex[a][b] = i < j ? exp2f((acc[a][b].x + acc[a][b].y - (shift ? shift[i] : 0.f) - off) * scale) : 0.f;   // only earlier tokens count
+        acc[a][b] = make_float2(0.f, 0.f);
+      }
+    }
+    float* out = reinterpret_cast<float*>(sm + h * kGhatTileBytes);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      const int a = k / 4, b = k % 4, row = ty + 16 * a, col = tx + 16 * b;
+      out[row * kGhatTile + (col ^ (ghat_swizzle(row) << 2))] = ex[a][b] != 0.f ? ex[a][b] * ((acc[a][b].x + acc[a][b].y) * inv_rv2) : 0.f;
+    }
+  }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  workers_sync();
+  store_tiles(ghat, tiles_per_call, t, at, sm);
+}
+
 template <int D>
 __global__ void __launch_bounds__(320, 2)       // ten warps: 96 registers, so that the 18 of two CTAs fit the SM's four register files
 
-ghat_tc_kernel(Geom G, Arena A, const CallSet calls, int call0, const CallStat* __restrict__ stats, const float* __restrict__ tok_shift,
+ghat_tc_kernel(const __grid_constant__ Geom G, const __grid_constant__ Arena A, const __grid_constant__ CallSet calls, int call0, const CallStat* __restrict__ stats, const float* __restrict__ tok_shift,
                float* __restrict__ ghat, int tiles_per_call, int* __restrict__ status) {
   constexpr int kPer = D / 32, kStages = 2 * kPer;       // 32-dim stages: of K, then of V
   constexpr int kUnits = 3;                              // of a thread and stage: (row, 8 dims), two of the rows' operand and one of the columns'
@@ -62,8 +170,8 @@ ghat_tc_kernel(Geom G, Arena A, const CallSet calls, int call0, const CallStat* 
   int* abort_flag = reinterpret_cast<int*>(tmem_s + 1);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int t = G.t;
-  int R = 0, c64 = blockIdx.x;                           // block index -> tile: 128-row panel R has 2 R + 2 column tiles
-  for (; c64 >= 2 * R + 2; ++R) c64 -= 2 * R + 2;
+  const int2 at = tile_of(blockIdx.x);
+  const int R = at.x, c64 = at.y;
   const int row0 = R * kRows, col0 = c64 * kCols;
   const bool own = c64 >= 2 * R;                         // the columns are among the tile's rows
   if (tid == 0) {
@@ -121,7 +229,12 @@ ghat_tc_kernel(Geom G, Arena A, const CallSet calls, int call0, const CallStat* 
   tc_fence_after();
   const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_s, 0);          // warp-uniform, so that the MMAs' operands sit in uniform registers
   bool ok = true;
-  if (warp < 8) {
+  // Infinite entries have no remainders: such calls (a row's norm shows it) are formed by FFMA (below).
+#pragma unroll
+  for (int w = 0; w < kWorkers / 32; ++w) { mk = fmaxf(mk, red[0][w]); mv = fmaxf(mv, red[1][w]); }
+  const bool split = mk < INFINITY && mv < INFINITY;
+  if (!split) {
+  } else if (warp < 8) {
 #pragma unroll
     for (int s = 0; s < kStages; ++s) {
       if (s > 1) ok = ok && wait_bar(mma_done + (s & 1), (uint32_t)((s >> 1) - 1) & 1u, abort_flag);     // the half has been read
@@ -155,19 +268,14 @@ ghat_tc_kernel(Geom G, Arena A, const CallSet calls, int call0, const CallStat* 
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       mbar_arrive(full + (s & 1));
     }
-#pragma unroll
-    for (int w = 0; w < kWorkers / 32; ++w) { mk = fmaxf(mk, red[0][w]); mv = fmaxf(mv, red[1][w]); }
-    // r_key^2, r_value^2 (inputs of Algorithm 2): maxima of the stored row norms, unless center_kernel has put them or they are fixed
-    float rk2 = G.fixed_rk2, rv2 = G.fixed_rv2;
-    if (rk2 <= 0.f) rk2 = tok_shift ? stats[call0 + blockIdx.y].rk2 : mk;
-    if (rv2 <= 0.f) rv2 = tok_shift ? stats[call0 + blockIdx.y].rv2 : mv;
-    const float inv_rv2 = rv2 > 0.f ? 1.0f / rv2 : 0.f;
+    const float2 r2 = radii(G, mk, mv, tok_shift ? stats + call0 + blockIdx.y : nullptr);
+    const float inv_rv2 = r2.y > 0.f ? 1.0f / r2.y : 0.f;
     const float scale = 1.4426950408889634f * G.inv_sqrt_d;
     const float* shift = tok_shift ? tok_shift + (size_t)(call0 + blockIdx.y) * t : nullptr;
     // thread = row of the tile; warps 0-3 its columns 0 .. 31, warps 4-7 the others
     const int row = 32 * (warp & 3) + lane, ch = warp >> 2;
     const int j = row0 + row, i0 = col0 + 32 * ch;
-    const float off = (shift && j < t ? shift[j] : 0.f) + rk2;
+    const float off = (shift && j < t ? shift[j] : 0.f) + r2.x;
     // the last stage of either half (a commit covers all MMAs before it, but each phase is waited for)
     ok = ok && wait_bar(mma_done, (uint32_t)(kStages / 2 - 1) & 1u, abort_flag) && wait_bar(mma_done + 1, (uint32_t)(kStages / 2 - 1) & 1u, abort_flag);
     ok = __all_sync(0xffffffffu, ok);
@@ -177,7 +285,6 @@ ghat_tc_kernel(Geom G, Arena A, const CallSet calls, int call0, const CallStat* 
       // the planes are free: two 64 x 64 tiles of the workspace, the panel's halves
       unsigned char* tile = sm + (row >> 6) * kGhatTileBytes + (row & 63) * (kGhatTile * 4);
       const int sw = ghat_swizzle(row);
-      const bool plain = !(mk < INFINITY && mv < INFINITY);
 #pragma unroll
       for (int h = 0; h < 2; ++h) {                       // 16 columns at a time
         const int c0 = i0 + 16 * h;
@@ -205,22 +312,6 @@ ghat_tc_kernel(Geom G, Arena A, const CallSet calls, int call0, const CallStat* 
           const float e = exp2f((ex[i] - off) * scale);
           ex[i] = c0 + i < j ? e : 0.f;
         }
-        // Infinite entries have no remainders: such calls (a row's norm shows it) are formed by FFMA, as on the CUDA cores.
-        if (plain && j < t)
-          for (int i = 0; i < 16; ++i) {
-            const int c = c0 + i;
-            float dot[2] = {0.f, 0.f};
-            for (int x = 0; c < j && x < 2; ++x) {
-              float2 s = make_float2(0.f, 0.f);
-              for (int e = 0; e < D; e += 2)
-                s = __ffma2_rn(*reinterpret_cast<const float2*>(src[x] + (size_t)j * D + e), *reinterpret_cast<const float2*>(src[x] + (size_t)c * D + e), s);
-              dot[x] = s.x + s.y;
-            }
-            const float xk = c < j ? exp2f((dot[0] - (shift ? shift[c] : 0.f) - off) * scale) : 0.f;
-#pragma unroll
-            for (int u = 0; u < 16; ++u)                  // a dynamic index would put the arrays into local memory
-              if (u == i) { ex[u] = xk; vv[u] = dot[1]; }
-          }
 #pragma unroll
         for (int p = 0; p < 4; ++p) {
           float o[4];
@@ -271,16 +362,13 @@ ghat_tc_kernel(Geom G, Arena A, const CallSet calls, int call0, const CallStat* 
   if (warp == 8) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
   if (*abort_flag) {
     if (tid == 0) atomicCAS(status, kStatusOk, kStatusWaitTimeout);
-  } else if (tid < 2) {
-    const int r = 2 * R + tid;
-    if (c64 <= r && r < t / kGhatTile) {
-      float* to = ghat + ((size_t)blockIdx.y * tiles_per_call + r * (r + 1) / 2 + c64) * (kGhatTile * kGhatTile);
-      asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
-                   ::"l"(to), "r"(smem_u32(sm + tid * kGhatTileBytes)), "r"(kGhatTileBytes) : "memory");
-      asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-      asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the stores end with the grid, which the walk waits for
-    }
+    return;
   }
+  if (!split) {
+    if (warp < 8) ffma_tiles<D>(G, A, calls, call0, stats, tok_shift, ghat, tiles_per_call, red, sm);
+    return;
+  }
+  store_tiles(ghat, tiles_per_call, t, at, sm);
 }
 
 }  // namespace

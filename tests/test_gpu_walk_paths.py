@@ -71,6 +71,32 @@ def test_fp32_call_with_an_infinite_row(cuda_lib, value):
     assert all(torch.equal(a, b) for a, b in zip(*views))
 
 
+@pytest.mark.parametrize("d,t,center,kind", [(64, 128, 0, "infinite"), (128, 320, 0, "infinite"), (128, 256, 1, "infinite")])
+def test_fp32_calls_formed_by_ffma(cuda_lib, d, t, center, kind):
+    """Calls whose rows are not split give the running sums of the CUDA cores bit by bit: whole panels and a last one of 64
+    tokens, columns that are among the tile's rows and others, key shifts."""
+    import torch
+
+    S = 2
+    gen = torch.Generator(device="cuda").manual_seed(t)
+    K = 0.1 * torch.randn(1, S, t, d, device="cuda", generator=gen)
+    V = torch.randn(1, S, t, d, device="cuda", generator=gen)
+    if kind == "infinite":
+        V[0, :, t - 1, 3] = float("inf")                # the last token's alone: every other sum stays finite
+    runs = []
+    for path in (0, 1):
+        ctx = cuda_lib.Context(n_seqs=1, n_layers=1, n_kv_heads=S, n_q_heads=S, head_dim=d, dtype="fp32", block=t, levels=1, max_tokens=t,
+                               seed=3, c_override=0.75, center_keys=center, r_value=float(d) ** 0.5, gram_path=path)
+        ctx.debug_enable()
+        ctx.stream_append_layer(0, K, V)
+        ctx.compress()
+        runs.append([x for h in range(S) for x in ctx.debug_call(0, 0, h, 0, 0)[:2]])
+        assert ctx.stats()["device_status"] == 0
+        ctx.close()
+    assert float(runs[0][1][: t - 1].abs().max()) > 1e-3      # sums of something
+    assert all(torch.equal(x.nan_to_num(7.0), y.nan_to_num(7.0)) for x, y in zip(*runs))
+
+
 def test_cuda_core_walk_in_groups_of_calls(cuda_lib):
     """More calls than the workspace holds (512 MB: 60 calls of 2048 tokens), against the walk of each stream alone."""
     import torch

@@ -1,15 +1,26 @@
 // The kernel matrices of fp32 calls (the first half of the CUDA-core walk, see kernels_walk_simt.cu) on the tensor cores.
 //
-// An fp32 value is the sum of three bf16 values, a = a1 + a2 + a3, each the rounding of what the ones before leave, so a
-// product of fp32 rows is a sum of products of bf16 rows, which the tensor core multiplies exactly:
-//   <a, b> = <a1, b1> + (<a1, b2> + <a2, b1> + <a2, b2> + <a1, b3> + <a3, b1>) + what is left, below 2^-26 |a||b|.
-// Its accumulator drops the bits of a sum that do not fit its 24.  So that none are dropped where it counts, a1 is rounded to a
-// grid of 2^(floor(log2 |a|) - 10), |a| the row's norm: the products of a1 and b1 are multiples of the two grids' product, and
-// by Cauchy-Schwarz no partial sum of theirs exceeds 2^22 of them, i.e. <a1, b1> is exact.  The small products have an
-// accumulator of their own, 2^-8 of the size, and the two are added in fp32.
-// Error of S_j against 64 bits, relative (2-norm), 12 draws each, FFMA / here: N(0, 0.3^2) keys d = 128 2.3e-7 / 1.6e-7; two channels x 8
-// 9.8e-6 / 3.9e-6; four channels x 10 with a mean 2.0e-5 / 1.2e-5; Student-t 2.4e-6 / 2.6e-6 (the rounding of r_key^2, the same
-// for both, is most of it); d = 64 2.1e-7 / 1.6e-7, 9.7e-6 / 7.2e-6, 2.9e-5 / 1.0e-5, 3.3e-6 / 3.2e-6.
+// A row is scaled by a power of two to a norm in [2^14, 2^15) and split into three f16 planes, a = a1 + a2 + a3, so that a product
+// of fp32 rows becomes products of f16 rows, which the tensor core multiplies exactly:
+//   <a, b> = <a1, b1> + (<a1, b2> + <a2, b1> + <a2, b2> + <a1, b3> + <a3, b1>) + what is left.
+// Its accumulator drops the bits of a sum that do not fit its 24.  So that none are dropped where it counts, a1 is a rounded to a
+// multiple of 16 (|a1| <= 2^15: 11 bits): the products of a1 and b1 are multiples of 256, and by Cauchy-Schwarz no partial sum of
+// theirs exceeds 2^30, i.e. <a1, b1> is exact.  The small products have an accumulator of their own, and the two are added in fp32.
+// a2 is the rounding of a - a1, |a - a1| <= 8, a3 that of what a2 leaves: an element keeps its 24 bits down to 2^-11 of its row's
+// norm, all but the last down to 2^-16 of it, and whatever exceeds 2^-39 of it.  What is left out, <a2, b3> + <a3, b2> + <a3, b3>
+// and the remainders, is at most d / 32 + 1/2 on that scale, where |a||b| >= 2^28: below 2^-25 |a||b|, typically 2^-33.
+//
+// That is more than FFMA keeps wherever the large elements of one row meet elements of the other that a1 holds.  Rows of a few large
+// elements and otherwise small ones (one channel a thousand times the others, another one from row to row) have products without a
+// main part, whose errors would be those of the small accumulator.  So a tile with a row of which a quarter of the channels and more
+// are not zero but within 24 on that scale (2^-10 of the norm) is formed by FFMA, as is a call with an infinite row, which has no
+// remainders.  Every other pair of channels is counted, which takes half the instructions (all: 3 % of the kernel).
+// Errors of products against 64 bits relative to sum |a_i b_i|, d = 128, 2-norm over 1536 pairs, FFMA / here: flat rows 2.0e-8 /
+// 3.5e-9, one channel x 30 in either row 5.3e-8 / 9.8e-9, four hot channels and a mean 9.8e-8 / 1.4e-8, one repeated value 4.6e-7 /
+// 2.5e-8, sparse rows 2.1e-8 / 6.4e-9, halves x 0.03 that meet the other row's large half 2.0e-8 / 1.8e-8; from one channel x 100
+// on the same.  Of S_j, relative, with the radii given, mean of 48 calls of 512 x 128: flat keys 2.1e-7 / 1.5e-7, two channels x 8
+// 5.4e-6 / 1.4e-6, four channels x 10 with a mean 1.5e-5 / 3.2e-6, Student-t 3.2e-6 / 1.6e-6; x 64: 1.7e-7 / 1.3e-7, 7.2e-6 / 2.2e-6,
+// 1.1e-5 / 4.1e-6, 2.4e-6 / 1.2e-6.  (The rounding of r_key^2, common to both, adds up to 5e-6 where r_key^2 is large.)
 //
 // One CTA of eight warps and a ninth per 128 x 64 tile of a call's lower triangle, two CTAs per SM.  The eight split a stage (32 dims
 // of K, then of V) into six operand planes in shared memory and the ninth issues its 12 MMAs; the planes hold 64 dims, so that
@@ -17,10 +28,13 @@
 // then become Ghat (exponential, product) and leave by bulk stores in the layout of the workspace.
 // What bounds it: shared memory, which at 64 columns feeds an MMA in 48 cycles and takes the planes in between (a stage: 576 + 290
 // cycles of either CTA; measured 1250 for both), then a CTA's 4400 cycles ahead of its first stage and 3200 behind its last, which the other
-// CTA covers in part.  128 calls of 512 tokens x 128 dims: FFMA 255 us, here 119; with stages of 64 dims and no second half 140;
-// with the MMAs issued by one of the eight warps 133.
+// CTA covers in part.  128 calls of 512 tokens x 128 dims: FFMA 255 us, here 125; with bf16 planes, which held fewer bits and needed
+// no scales, 117, with stages of 64 dims and no second half 140, with the MMAs issued by one of the eight warps 133 (both bf16).
+// The same calls with an infinite row or with uneven rows: 353 and 470 us.
 //
 // Every wait is bounded: a wait that runs out sets the abort flag and the status word, and the kernel returns.
+#include <cuda_fp16.h>
+
 #include <algorithm>
 
 #include "common.cuh"
@@ -37,14 +51,16 @@ constexpr int kWorkers = 256, kThreads = kWorkers + 32;
 constexpr uint32_t kPlaneA = kRows * 128, kPlaneB = kCols * 128;      // [rows][64 bf16], 128-byte swizzle
 constexpr uint32_t kPlanes = 3 * (kPlaneA + kPlaneB);
 constexpr size_t kSmem = 1024 + kPlanes + 128;
+constexpr float kTiny = 32.f;                            // an element that a1 holds as 0 or +-16 barely has a main part
 constexpr uint32_t kTmemCols = 256;                      // K main, K small, V main, V small: 64 columns each
 constexpr int kGhatTile = 64, kGhatTileBytes = kGhatTile * kGhatTile * 4;
 
-// 1.5 * 2^23 times the grid of a row with squared norm n2: (a + m) - m rounds a to that grid.
-__device__ inline float grid_magic(float n2) {
-  const int e = (int)(__float_as_uint(n2) >> 23) - 127;                // floor(log2 n2)
-  return __uint_as_float((uint32_t)((e >> 1) + 13 + 127) << 23 | 0x400000u);
-}
+// Rows are scaled by a power of two to a norm in [2^14, 2^15) (n2: the row's squared norm): where f16 keeps most of them.
+constexpr int kNormExponent = 14;
+__device__ inline int norm_exponent(float n2) { return ((int)(__float_as_uint(n2) >> 23 & 255u) - 127) >> 1; }     // floor(log2 |a|)
+__device__ inline float row_scale(float n2) { return __uint_as_float((uint32_t)(kNormExponent - norm_exponent(n2) + 127) << 23); }
+__device__ inline float row_unscale(float n2) { return __uint_as_float((uint32_t)(norm_exponent(n2) - kNormExponent + 127) << 23); }
+constexpr float kGridMagic = 1.5f * 0x1p27f;             // (y + it) - it rounds y to a multiple of 16, 2^-10 of the norm's power of two
 
 __device__ inline void workers_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kWorkers) : "memory"); }
 
@@ -163,11 +179,13 @@ ghat_tc_kernel(const __grid_constant__ Geom G, const __grid_constant__ Arena A, 
   constexpr int kUnits = 3;                              // of a thread and stage: (row, 8 dims), two of the rows' operand and one of the columns'
   extern __shared__ unsigned char smem_raw[];
   __shared__ float red[2][kWorkers / 32];
+  __shared__ __align__(16) float unscale[2][kCols];       // of the columns' rows
   unsigned char* sm = smem_raw + (-smem_u32(smem_raw) & 1023u);
   uint64_t* mma_done = reinterpret_cast<uint64_t*>(sm + kPlanes);       // [2] the MMAs of a half
   uint64_t* full = mma_done + 2;                                        // [2] the planes of a half are written
   uint32_t* tmem_s = reinterpret_cast<uint32_t*>(full + 2);
   int* abort_flag = reinterpret_cast<int*>(tmem_s + 1);
+  int* uneven = abort_flag + 1;                          // a row of the tile is not to be split
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int t = G.t;
   const int2 at = tile_of(blockIdx.x);
@@ -180,6 +198,7 @@ ghat_tc_kernel(const __grid_constant__ Geom G, const __grid_constant__ Arena A, 
       mbar_init(full + i, kWorkers);
     }
     *abort_flag = 0;
+    *uneven = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 8) {
@@ -195,7 +214,7 @@ ghat_tc_kernel(const __grid_constant__ Geom G, const __grid_constant__ Arena A, 
   // The unit's token.  Rows behind the call's last (a panel of 64 rows) are its last row again; nobody reads what they give.
   auto token = [&](int k) { return min(k < 2 ? row0 + urow + 64 * k : col0 + urow, t - 1); };
   float4 v[2][2 * kUnits];
-  float magic[2][kUnits];
+  float scales[2][kUnits];
   auto fetch = [&](int s, float4 (&to)[2 * kUnits]) {
     const float* base = src[s / kPer] + 32 * (s % kPer) + 8 * piece;
 #pragma unroll
@@ -213,8 +232,13 @@ ghat_tc_kernel(const __grid_constant__ Geom G, const __grid_constant__ Arena A, 
 #pragma unroll
     for (int k = 0; k < kUnits; ++k) {
       const float2 n = nrm[token(k)];
-      magic[0][k] = grid_magic(n.x);
-      magic[1][k] = grid_magic(n.y);
+      scales[0][k] = row_scale(n.x);
+      scales[1][k] = row_scale(n.y);
+    }
+    if (tid < kCols) {
+      const float2 n = nrm[col0 + tid];
+      unscale[0][tid] = row_unscale(n.x);
+      unscale[1][tid] = row_unscale(n.y);
     }
     for (int j = tid; j < t; j += kWorkers) {
       const float2 n = nrm[j];
@@ -235,10 +259,11 @@ ghat_tc_kernel(const __grid_constant__ Geom G, const __grid_constant__ Arena A, 
   const bool split = mk < INFINITY && mv < INFINITY;
   if (!split) {
   } else if (warp < 8) {
+    __half2 tiny[kUnits];                                // the units' elements, not zero, that a1 barely holds
 #pragma unroll
     for (int s = 0; s < kStages; ++s) {
       if (s > 1) ok = ok && wait_bar(mma_done + (s & 1), (uint32_t)((s >> 1) - 1) & 1u, abort_flag);     // the half has been read
-      if (ok) {
+      if (__all_sync(0xffffffffu, ok)) {
 #pragma unroll
         for (int k = 0; k < kUnits; ++k) {
           if (k >= 2 && own) break;
@@ -246,18 +271,28 @@ ghat_tc_kernel(const __grid_constant__ Geom G, const __grid_constant__ Arena A, 
           unsigned char* to = sm + (k < 2 ? 0u : 3 * kPlaneA) + row * 128 + (((4 * (s & 1) + piece) ^ (row & 7)) << 4);
           const float4 x0 = v[s & 1][2 * k], x1 = v[s & 1][2 * k + 1];
           const float x[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
-          const float2 m = make_float2(magic[s / kPer][k], magic[s / kPer][k]), neg = make_float2(-m.x, -m.x);
+          const float2 scale = make_float2(scales[s / kPer][k], scales[s / kPer][k]);
+          const float2 magic = make_float2(kGridMagic, kGridMagic), minus = make_float2(-1.f, -1.f);
           uint32_t w[3][4];
+          if (s % kPer == 0) tiny[k] = __half2half2(__ushort_as_half(0));
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
-            float2 a = make_float2(x[2 * i], x[2 * i + 1]);
-            const float2 a1 = __fadd2_rn(__fadd2_rn(a, m), neg);
-#pragma unroll
-            for (int p = 0; p < 3; ++p) {
-              const __nv_bfloat162 h = p == 0 ? __floats2bfloat162_rn(a1.x, a1.y) : __floats2bfloat162_rn(a.x, a.y);
-              w[p][i] = *reinterpret_cast<const uint32_t*>(&h);
-              a = __ffma2_rn(make_float2(bf16_lo(w[p][i]), bf16_hi(w[p][i])), make_float2(-1.f, -1.f), a);
-            }
+            const float2 e = make_float2(x[2 * i], x[2 * i + 1]);
+            const float2 y = __fmul2_rn(e, scale), a1 = __fadd2_rn(__fadd2_rn(y, magic), make_float2(-kGridMagic, -kGridMagic)), r1 = __ffma2_rn(a1, minus, y);
+            const __half2 h1 = __floats2half2_rn(a1.x, a1.y), h2 = __floats2half2_rn(r1.x, r1.y);
+            const float2 r2 = __ffma2_rn(__half22float2(h2), minus, r1);
+            const __half2 h3 = __floats2half2_rn(r2.x, r2.y);
+            if ((i + s) % 2 == 0)                           // half of the row's channels: enough to tell, and half the instructions
+              tiny[k] = __hfma2(__hlt2(__habs2(h1), __float2half2_rn(kTiny)), __hne2(h2, __half2half2(__ushort_as_half(0))), tiny[k]);
+            w[0][i] = *reinterpret_cast<const uint32_t*>(&h1);
+            w[1][i] = *reinterpret_cast<const uint32_t*>(&h2);
+            w[2][i] = *reinterpret_cast<const uint32_t*>(&h3);
+          }
+          if (s % kPer == kPer - 1) {
+            float n = __low2float(tiny[k]) + __high2float(tiny[k]);
+            n += __shfl_xor_sync(0xffffffffu, n, 1);
+            n += __shfl_xor_sync(0xffffffffu, n, 2);
+            if (n >= D / 8) *uneven = 1;
           }
 #pragma unroll
           for (int p = 0; p < 3; ++p)
@@ -276,6 +311,9 @@ ghat_tc_kernel(const __grid_constant__ Geom G, const __grid_constant__ Arena A, 
     const int row = 32 * (warp & 3) + lane, ch = warp >> 2;
     const int j = row0 + row, i0 = col0 + 32 * ch;
     const float off = (shift && j < t ? shift[j] : 0.f) + r2.x;
+    const float2 neg_off = make_float2(-off, -off), nj = nrm[min(j, t - 1)];
+    const float bk = row_unscale(nj.x), bv = row_unscale(nj.y) * inv_rv2;
+    const float2 back_k = make_float2(bk, bk), back_v = make_float2(bv, bv);
     // the last stage of either half (a commit covers all MMAs before it, but each phase is waited for)
     ok = ok && wait_bar(mma_done, (uint32_t)(kStages / 2 - 1) & 1u, abort_flag) && wait_bar(mma_done + 1, (uint32_t)(kStages / 2 - 1) & 1u, abort_flag);
     ok = __all_sync(0xffffffffu, ok);
@@ -297,19 +335,23 @@ ghat_tc_kernel(const __grid_constant__ Geom G, const __grid_constant__ Arena A, 
           tmem_ld16(tl + 192 + 16 * h, lv);
           tmem_ld_wait();
 #pragma unroll
-          for (int i = 0; i < 16; ++i) { ex[i] += lo[i]; vv[i] += lv[i]; }
-        }
-        if (shift) {
-#pragma unroll
-          for (int i = 0; i < 16; i += 4) {
-            const float4 a = *reinterpret_cast<const float4*>(shift + c0 + i);
-            ex[i] -= a.x; ex[i + 1] -= a.y; ex[i + 2] -= a.z; ex[i + 3] -= a.w;
+          for (int i = 0; i < 16; i += 2) {
+            const float2 ca = *reinterpret_cast<const float2*>(unscale[0] + 32 * ch + 16 * h + i), cb = *reinterpret_cast<const float2*>(unscale[1] + 32 * ch + 16 * h + i);
+            float2 o = neg_off;
+            if (shift) {
+              const float2 a = *reinterpret_cast<const float2*>(shift + c0 + i);
+              o.x -= a.x; o.y -= a.y;
+            }
+            const float2 k = __ffma2_rn(__fadd2_rn(make_float2(ex[i], ex[i + 1]), make_float2(lo[i], lo[i + 1])), __fmul2_rn(ca, back_k), o);
+            const float2 w = __fmul2_rn(__fadd2_rn(make_float2(vv[i], vv[i + 1]), make_float2(lv[i], lv[i + 1])), __fmul2_rn(cb, back_v));
+            ex[i] = k.x; ex[i + 1] = k.y;
+            vv[i] = w.x; vv[i + 1] = w.y;
           }
         }
         // only earlier tokens count (a select behind the exponential: a branch per entry cost 3000 cycles a tile)
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
-          const float e = exp2f((ex[i] - off) * scale);
+          const float e = exp2f(ex[i] * scale);
           ex[i] = c0 + i < j ? e : 0.f;
         }
 #pragma unroll
@@ -317,7 +359,7 @@ ghat_tc_kernel(const __grid_constant__ Geom G, const __grid_constant__ Arena A, 
           float o[4];
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
-            const float x = ex[4 * p + i] * (vv[4 * p + i] * inv_rv2);
+            const float x = ex[4 * p + i] * vv[4 * p + i];
             o[i] = ex[4 * p + i] != 0.f ? x : 0.f;
           }
           *reinterpret_cast<float4*>(tile + (((8 * ch + 4 * h + p) ^ sw) << 4)) = make_float4(o[0], o[1], o[2], o[3]);
@@ -340,16 +382,16 @@ ghat_tc_kernel(const __grid_constant__ Geom G, const __grid_constant__ Arena A, 
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
           if (s % kPer == 0 && k == 0) {
-            umma_bf16<0, kCols>(main, a, b);
-            umma_bf16<0, kCols>(small, a + 2 * ap, b);
+            umma<0, kInstrF16<kCols>>(main, a, b);
+            umma<0, kInstrF16<kCols>>(small, a + 2 * ap, b);
           } else {
-            umma_bf16<1, kCols>(main, a + 2 * k, b + 2 * k);
-            umma_bf16<1, kCols>(small, a + 2 * ap + 2 * k, b + 2 * k);
+            umma<1, kInstrF16<kCols>>(main, a + 2 * k, b + 2 * k);
+            umma<1, kInstrF16<kCols>>(small, a + 2 * ap + 2 * k, b + 2 * k);
           }
-          umma_bf16<1, kCols>(small, a + 2 * k, b + 2 * bp + 2 * k);
-          umma_bf16<1, kCols>(small, a + ap + 2 * k, b + bp + 2 * k);
-          umma_bf16<1, kCols>(small, a + ap + 2 * k, b + 2 * k);
-          umma_bf16<1, kCols>(small, a + 2 * k, b + bp + 2 * k);
+          umma<1, kInstrF16<kCols>>(small, a + 2 * k, b + 2 * bp + 2 * k);
+          umma<1, kInstrF16<kCols>>(small, a + ap + 2 * k, b + bp + 2 * k);
+          umma<1, kInstrF16<kCols>>(small, a + ap + 2 * k, b + 2 * k);
+          umma<1, kInstrF16<kCols>>(small, a + 2 * k, b + bp + 2 * k);
         }
         umma_commit(mma_done + (s & 1));
       }
@@ -364,7 +406,7 @@ ghat_tc_kernel(const __grid_constant__ Geom G, const __grid_constant__ Arena A, 
     if (tid == 0) atomicCAS(status, kStatusOk, kStatusWaitTimeout);
     return;
   }
-  if (!split) {
+  if (!split || *uneven) {
     if (warp < 8) ffma_tiles<D>(G, A, calls, call0, stats, tok_shift, ghat, tiles_per_call, red, sm);
     return;
   }

@@ -46,30 +46,34 @@ __device__ inline bool wait_bar(uint64_t* bar, uint32_t parity, int* abort_flag)
   return true;
 }
 
-// Shared-memory matrix descriptor of a K-major, 128B-swizzled bf16 operand: rows of 128 bytes,
+// Shared-memory matrix descriptor of a K-major, 128B-swizzled 16-bit operand: rows of 128 bytes,
 // 8-row groups 1024 bytes apart (stride byte offset), version 1, layout type SWIZZLE_128B.
 // Only the low word depends on the address: (addr >> 4) in bits [0,14), leading byte offset 1
 // (unused for swizzled K-major) in bits [16,30).  Stepping 16 elements along K adds 32 bytes,
 // i.e. 2 to the low word; the second 64-column half of a tile sits kHalfBytes further.
 constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
 __device__ inline uint32_t umma_desc_lo(uint32_t smem_addr) { return ((smem_addr & 0x3FFFFu) >> 4) | (1u << 16); }
-// kind::f16 instruction descriptor: D fp32, A and B bf16, both K-major, M = 128.
+// kind::f16 instruction descriptor: D fp32, A and B of one type (bf16: formats 1, f16: 0), both K-major, M = 128.
 template <int N>
-constexpr uint32_t kInstrDesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((128u >> 4) << 24);
+constexpr uint32_t kInstrF16 = (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((128u >> 4) << 24);
+template <int N>
+constexpr uint32_t kInstrBf16 = kInstrF16<N> | (1u << 7) | (1u << 10);
 
 // A tcgen05.mma is issued at the rate the tensor core retires them, so every other instruction
 // of the issuing thread is idle time of the pipe: descriptors come as ready-made words and the
 // accumulate flag is a compile-time constant.
-template <int kAccumulate, int N = 128>
-__device__ inline void umma_bf16(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo) {
+template <int kAccumulate, uint32_t kInstr>
+__device__ inline void umma(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
       "mov.b64 da, {%1, %3};\n\t"
       "mov.b64 db, {%2, %3};\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n\t}"
-      ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(kDescHi), "n"(kAccumulate), "r"(kInstrDesc<N>) : "memory");
+      ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(kDescHi), "n"(kAccumulate), "r"(kInstr) : "memory");
 }
+template <int kAccumulate>
+__device__ inline void umma_bf16(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo) { umma<kAccumulate, kInstrBf16<128>>(d_tmem, a_lo, b_lo); }
 // One lane of a converged warp, always the same: code under it stays warp-uniform for the compiler.
 __device__ inline bool elect_one() {
   uint32_t r;

@@ -71,7 +71,8 @@ def test_fp32_call_with_an_infinite_row(cuda_lib, value):
     assert all(torch.equal(a, b) for a, b in zip(*views))
 
 
-@pytest.mark.parametrize("d,t,center,kind", [(64, 128, 0, "infinite"), (128, 320, 0, "infinite"), (128, 256, 1, "infinite")])
+@pytest.mark.parametrize("d,t,center,kind", [(64, 128, 0, "infinite"), (128, 320, 0, "infinite"), (128, 256, 1, "infinite"),
+                                             (64, 192, 0, "uneven"), (128, 256, 1, "uneven")])
 def test_fp32_calls_formed_by_ffma(cuda_lib, d, t, center, kind):
     """Calls whose rows are not split give the running sums of the CUDA cores bit by bit: whole panels and a last one of 64
     tokens, columns that are among the tile's rows and others, key shifts."""
@@ -83,6 +84,8 @@ def test_fp32_calls_formed_by_ffma(cuda_lib, d, t, center, kind):
     V = torch.randn(1, S, t, d, device="cuda", generator=gen)
     if kind == "infinite":
         V[0, :, t - 1, 3] = float("inf")                # the last token's alone: every other sum stays finite
+    else:
+        V *= torch.where(torch.arange(t, device="cuda")[:, None] % d == torch.arange(d, device="cuda"), 1.0, 1e-4)
     runs = []
     for path in (0, 1):
         ctx = cuda_lib.Context(n_seqs=1, n_layers=1, n_kv_heads=S, n_q_heads=S, head_dim=d, dtype="fp32", block=t, levels=1, max_tokens=t,
@@ -93,7 +96,7 @@ def test_fp32_calls_formed_by_ffma(cuda_lib, d, t, center, kind):
         runs.append([x for h in range(S) for x in ctx.debug_call(0, 0, h, 0, 0)[:2]])
         assert ctx.stats()["device_status"] == 0
         ctx.close()
-    assert float(runs[0][1][: t - 1].abs().max()) > 1e-3      # sums of something
+    assert float(runs[0][1][: t - 1].abs().max()) > (1e-3 if kind == "infinite" else 1e-7)      # sums of something
     assert all(torch.equal(x.nan_to_num(7.0), y.nan_to_num(7.0)) for x, y in zip(*runs))
 
 
@@ -252,3 +255,70 @@ def test_centered_call_beyond_a_fixed_radius(cuda_lib):
         ctx.close()
     assert torch.isinf(sums[1][200]) and sums[0][200].abs() == sums[1][200].abs()
     assert torch.isfinite(sums[0][:200]).all()
+
+
+def _pair_rows(kind, n, d, gen):
+    """Two sets of n rows."""
+    import torch
+
+    a, b = (torch.randn(n, d, device="cuda", dtype=torch.float64, generator=gen) for _ in range(2))
+    if kind.startswith("one channel x"):                # another channel in either row
+        at = torch.arange(n, device="cuda")
+        size = float(kind.split("x")[1])
+        for x, c in ((a, at % (d // 2)), (b, d // 2 + at * 7 % (d // 2))):
+            x[at, c] = size * (1 + torch.rand(n, device="cuda", dtype=torch.float64, generator=gen))
+    elif kind == "one of two":
+        a[:, 3] *= 1000
+    elif kind == "one value":
+        a[:], b[:] = a[:, :1].clone(), b[:, :1].clone()
+    elif kind == "heavy tails":
+        a, b = (x / torch.randn(n, d, device="cuda", dtype=torch.float64, generator=gen).abs() for x in (a, b))
+    elif kind == "hot channels":
+        scale = torch.ones(d, device="cuda", dtype=torch.float64)
+        scale[:4] = 10
+        a, b = (a + 0.5) * scale, (b + 0.5) * scale
+    elif kind == "mean":
+        a, b = 7 + 1e-3 * a, 7 + 1e-3 * b
+    elif kind == "sparse":
+        keep = torch.rand(n, d, device="cuda", generator=gen)
+        a, b = a * (keep < 0.3), b * (keep < 0.3)
+    elif kind.startswith("halves x"):                   # the large elements of either row meet small ones
+        a[:, : d // 2] *= float(kind.split("x")[1])
+        b[:, d // 2:] *= float(kind.split("x")[1])
+    return a.float(), b.float()
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("t,first,second", [(128, 0, 1), (256, 0, 128)])
+@pytest.mark.parametrize("kind", ["flat", "one channel x100", "one channel x1000", "one channel x30000", "one channel x1e6", "one of two",
+                                  "one value", "heavy tails", "hot channels", "mean", "sparse", "halves x0.03", "halves x0.001"])
+def test_fp32_products_are_as_precise_as_ffma(cuda_lib, d, t, first, second, kind):
+    """Products of value rows against 64 bits; the limit is the error of the CUDA cores.  Tokens first + s m and second + s m have
+    the m-th axis as their key (of length r_key: the kernel is 1 between them and 0 elsewhere), so that a token's running sum is
+    the one product, up to the other token's sign.  Neighbours share a tile whose columns are among its rows, tokens 128 apart do not."""
+    import torch
+
+    S, n, r = 24, 64, 64.0
+    step = 2 if second == 1 else 1
+    gen = torch.Generator(device="cuda").manual_seed(d + t)
+    i, j = (x + step * torch.arange(n, device="cuda") for x in (first, second))
+    K, V = (torch.zeros(1, S, t, d, device="cuda") for _ in range(2))
+    for x in (i, j):
+        K[0, :, x, torch.arange(n, device="cuda")] = r
+    a, b = (x.reshape(S, n, d) for x in _pair_rows(kind, S * n, d, gen))
+    V[0, :, i], V[0, :, j] = a, b
+    exact, size = (a.double() * b.double()).sum(-1), (a.double() * b.double()).abs().sum(-1)
+    errors = []
+    for path in (0, 1):
+        ctx = cuda_lib.Context(n_seqs=1, n_layers=1, n_kv_heads=S, n_q_heads=S, head_dim=d, dtype="fp32", block=t, levels=1, max_tokens=t,
+                               seed=3, gram_path=path, r_key=r, r_value=1.0)
+        ctx.debug_enable()
+        ctx.stream_append_layer(0, K, V)
+        ctx.compress()
+        got = torch.stack([s[j] * e[i].float() for e, s, _ in (ctx.debug_call(0, 0, h, 0, 0) for h in range(S))])
+        assert ctx.stats()["device_status"] == 0
+        ctx.close()
+        errors.append((got.double() - exact).abs() / size)
+    assert float(errors[1].max()) < 3e-6                # sums of the right products
+    for of in (lambda e: e.square().mean().sqrt(), torch.median):
+        assert float(of(errors[0])) <= float(of(errors[1])), (float(of(errors[0])), float(of(errors[1])))

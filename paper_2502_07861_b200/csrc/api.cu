@@ -154,7 +154,6 @@ struct balancekv_ctx {
   float* bkt_ns = nullptr;
   int8_t* bkt_slot = nullptr;
   int32_t* bkt_rank = nullptr;
-  unsigned* bkt_vmax_bits = nullptr;
   int32_t* bkt_chunk_cnt = nullptr;     // per (stream, chunk of the block): counts, then their prefix
   size_t bkt_chunk_ints = 0;
   BucketOut* bkt_out_host = nullptr;    // pinned
@@ -435,7 +434,7 @@ int balancekv_destroy(balancekv_ctx* c) {
                   c->view_idx, c->bounce_K, c->bounce_V, c->bounce_q, c->bounce_out, c->step_dev_in, c->step_dev_out, c->two_acc, c->two_ml, c->two_scratch, c->unit_V};
   for (void* p : ptrs)
     if (p) cudaFree(p);
-  void* bkt[] = {c->bkt_ns, c->bkt_slot, c->bkt_rank, c->bkt_vmax_bits, c->bkt_chunk_cnt, c->acr_scratch, c->acr_cls};
+  void* bkt[] = {c->bkt_ns, c->bkt_slot, c->bkt_rank, c->bkt_chunk_cnt, c->acr_scratch, c->acr_cls};
   for (void* p : bkt)
     if (p) cudaFree(p);
   if (c->bkt_out_host) cudaFreeHost(c->bkt_out_host);
@@ -1225,11 +1224,11 @@ static int append_bucketed_impl(balancekv_ctx* c, const std::vector<std::pair<in
   // routing buffers (grown with the largest block; the call synchronises the stream anyway)
   if ((size_t)n_sl * n > c->bkt_rows || (size_t)n_sl > c->bkt_streams || bucket_chunk_count_ints(n_sl, n) > c->bkt_chunk_ints) {
     BKV_CUDA(cudaStreamSynchronize(st));
-    void* old[] = {c->bkt_ns, c->bkt_slot, c->bkt_rank, c->bkt_vmax_bits, c->bkt_chunk_cnt};
+    void* old[] = {c->bkt_ns, c->bkt_slot, c->bkt_rank, c->bkt_chunk_cnt};
     for (void* p : old)
       if (p) cudaFree(p);
     if (c->bkt_out_host) cudaFreeHost(c->bkt_out_host);
-    c->bkt_ns = nullptr; c->bkt_slot = nullptr; c->bkt_rank = nullptr; c->bkt_vmax_bits = nullptr;
+    c->bkt_ns = nullptr; c->bkt_slot = nullptr; c->bkt_rank = nullptr;
     c->bkt_out_host = nullptr; c->bkt_chunk_cnt = nullptr;
     c->bkt_chunk_ints = std::max(c->bkt_chunk_ints, bucket_chunk_count_ints(n_sl, n));
     BKV_CUDA(cudaMalloc(reinterpret_cast<void**>(&c->bkt_chunk_cnt), sizeof(int32_t) * c->bkt_chunk_ints));
@@ -1238,8 +1237,6 @@ static int append_bucketed_impl(balancekv_ctx* c, const std::vector<std::pair<in
     BKV_CUDA(cudaMalloc(reinterpret_cast<void**>(&c->bkt_ns), sizeof(float) * c->bkt_rows));
     BKV_CUDA(cudaMalloc(reinterpret_cast<void**>(&c->bkt_slot), c->bkt_rows));
     BKV_CUDA(cudaMalloc(reinterpret_cast<void**>(&c->bkt_rank), sizeof(int32_t) * c->bkt_rows));
-    BKV_CUDA(cudaMalloc(reinterpret_cast<void**>(&c->bkt_vmax_bits), sizeof(unsigned) * c->bkt_streams));
-    BKV_CUDA(cudaMemsetAsync(c->bkt_vmax_bits, 0, sizeof(unsigned) * c->bkt_streams, st));   // later calls find it emptied by the one before
     BKV_CUDA(cudaMallocHost(reinterpret_cast<void**>(&c->bkt_out_host), sizeof(BucketOut) * c->bkt_streams));
   }
   std::vector<BucketIn> in(n_sl);
@@ -1247,6 +1244,7 @@ static int append_bucketed_impl(balancekv_ctx* c, const std::vector<std::pair<in
     const int s0 = stream_id(c, heads[i].first, layer0, heads[i].second);
     in[i].prev_vmax2 = c->bucket_vmax2[s0];
     in[i].prev_erase_max = c->bucket_erase_max[s0];
+    in[i].block_vmax2 = 0u;
   }
   void* d_in = nullptr;
   int rc = ring_push(c, in.data(), in.size() * sizeof(BucketIn), st, &d_in);
@@ -1272,8 +1270,8 @@ static int append_bucketed_impl(balancekv_ctx* c, const std::vector<std::pair<in
   }
   {
     ProfScope ps(c, 0, st);
-    BKV_CUDA(launch_bucket_route(c->G, V, n_sl, n, n_buckets, i_top, rho * rho, static_cast<const BucketIn*>(d_in),
-                                 c->bkt_vmax_bits, c->bkt_ns, c->bkt_slot, c->bkt_rank, c->bkt_chunk_cnt, c->bkt_out_host, forced, st));
+    BKV_CUDA(launch_bucket_route(c->G, V, n_sl, n, n_buckets, i_top, rho * rho, static_cast<BucketIn*>(d_in),
+                                 c->bkt_ns, c->bkt_slot, c->bkt_rank, c->bkt_chunk_cnt, c->bkt_out_host, forced, st));
   }
   c->kernels_launched += 3;
   BKV_CUDA(cudaStreamSynchronize(st));   // the counts (written to the host's memory) decide its bookkeeping of every instance

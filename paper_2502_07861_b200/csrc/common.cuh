@@ -65,6 +65,7 @@ constexpr int kMaxBuckets = 8;
 struct BucketIn {
   float prev_vmax2;        // v_max^2 over the stream's earlier blocks
   int32_t prev_erase_max;  // largest bucket index erased so far (INT32_MIN: none)
+  uint32_t block_vmax2;    // bits of the block's largest squared norm: 0, then the norms kernel's maximum
 };
 struct BucketOut {
   int32_t count[kMaxBuckets];  // tokens of the block per slot
@@ -290,7 +291,7 @@ cudaError_t launch_upload(void* dst, const void* data, size_t bytes, cudaStream_
 int bucket_scan_chunks(int n);
 size_t bucket_chunk_count_ints(int n_sl, int n);   // ints of the per-chunk count table of the routing pass
 cudaError_t launch_bucket_route(const Geom& G, const void* V, int n_sl, int n, int n_buckets, int i_top, float rho2,
-                                const BucketIn* in, unsigned* vmax2_bits, float* ns, int8_t* slot, int32_t* rank,
+                                BucketIn* in, float* ns, int8_t* slot, int32_t* rank,
                                 int32_t* chunk_cnt, BucketOut* out, const int8_t* forced_slot, cudaStream_t st);
 size_t anticorr_scratch_floats(int n_sl, int n, int d);
 cudaError_t launch_anticorr_classes(const Geom& G, const void* K, int n_sl, int n, float tau, float* scratch, int8_t* cls,

@@ -44,7 +44,7 @@ __device__ inline float sumsq_piece(const uint4& v) {
 // all passes are issued before the first is reduced.
 template <bool kBf16>
 __global__ void __launch_bounds__(256)
-bucket_norms_kernel(const void* __restrict__ V, int n, int chunks, float* __restrict__ ns, unsigned* __restrict__ vmax2_bits) {
+bucket_norms_kernel(const void* __restrict__ V, int n, int chunks, float* __restrict__ ns, BucketIn* __restrict__ in) {
   grid_wait_and_release();
   const int sl = blockIdx.y;
   const int rows_per_pass = blockDim.x / chunks;         // 32, 16 or 8
@@ -80,7 +80,7 @@ bucket_norms_kernel(const void* __restrict__ V, int n, int chunks, float* __rest
     // squared norms are >= 0, so their bit patterns order like the values; one atomic per CTA,
     // and none once the stream's maximum is already at least this large
     const unsigned bits = __float_as_uint(mx);
-    if (bits > *reinterpret_cast<volatile unsigned*>(vmax2_bits + sl)) atomicMax(vmax2_bits + sl, bits);
+    if (bits > *const_cast<volatile uint32_t*>(&in[sl].block_vmax2)) atomicMax(&in[sl].block_vmax2, bits);
   }
 }
 
@@ -93,8 +93,8 @@ __device__ inline int bucket_of(float ns) {
 }
 
 // The largest erased bucket index after the block: 4^i <= rho^2 * v_max^2 (INT32_MIN: none).
-__device__ inline int erase_index(float rho2, const BucketIn& in, unsigned vmax2_bits) {
-  const float vmax2 = fmaxf(in.prev_vmax2, __uint_as_float(vmax2_bits));
+__device__ inline int erase_index(float rho2, const BucketIn& in) {
+  const float vmax2 = fmaxf(in.prev_vmax2, __uint_as_float(in.block_vmax2));
   int erase_max = INT32_MIN;
   const float thr = rho2 * vmax2;
   if (thr > 0.f) {
@@ -111,13 +111,13 @@ __device__ inline int erase_index(float rho2, const BucketIn& in, unsigned vmax2
 // (or -1) and its rank among the chunk's tokens of the same slot; per chunk, the counts.
 __global__ void __launch_bounds__(kScanThreads)
 bucket_scan_kernel(const float* __restrict__ ns, int n, int n_chunks, int n_buckets, int i_top, float rho2,
-                   const BucketIn* __restrict__ in, const unsigned* __restrict__ vmax2_bits, int8_t* __restrict__ slot,
+                   const BucketIn* __restrict__ in, int8_t* __restrict__ slot,
                    int32_t* __restrict__ rank, int32_t* __restrict__ chunk_cnt, const int8_t* __restrict__ forced) {
   constexpr int kWarps = kScanThreads / 32, kRounds = kScanChunk / kScanThreads;
   __shared__ int warp_tot[kCountCols][kWarps];
   grid_wait_and_release();
   const int sl = blockIdx.y, chunk = blockIdx.x;
-  const int erase_max = erase_index(rho2, in[sl], vmax2_bits[sl]);
+  const int erase_max = erase_index(rho2, in[sl]);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned lt = (1u << lane) - 1u;
   const size_t base = (size_t)sl * n;
@@ -181,8 +181,7 @@ bucket_scan_kernel(const float* __restrict__ ns, int n, int n_chunks, int n_buck
 // Second part: per stream, the exclusive prefix of the chunks' counts (in place) and the totals.
 // grid (streams), kCountCols warps: warp b scans column b, 32 chunks at a time.
 __global__ void __launch_bounds__(kCountCols * 32)
-bucket_prefix_kernel(int n_chunks, float rho2, const BucketIn* __restrict__ in, unsigned* __restrict__ vmax2_bits,
-                     int32_t* __restrict__ chunk_cnt, BucketOut* __restrict__ out) {
+bucket_prefix_kernel(int n_chunks, float rho2, const BucketIn* __restrict__ in, int32_t* __restrict__ chunk_cnt, BucketOut* __restrict__ out) {
   grid_wait_and_release();
   const int sl = blockIdx.x, col = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int32_t* c = chunk_cnt + (size_t)sl * n_chunks * kCountCols + col;
@@ -205,9 +204,8 @@ bucket_prefix_kernel(int n_chunks, float rho2, const BucketIn* __restrict__ in, 
     else out[sl].above = carry;
   }
   if (threadIdx.x == 0) {
-    out[sl].erase_max = erase_index(rho2, in[sl], vmax2_bits[sl]);
-    out[sl].vmax2 = fmaxf(in[sl].prev_vmax2, __uint_as_float(vmax2_bits[sl]));
-    vmax2_bits[sl] = 0u;                     // for the next call
+    out[sl].erase_max = erase_index(rho2, in[sl]);
+    out[sl].vmax2 = fmaxf(in[sl].prev_vmax2, __uint_as_float(in[sl].block_vmax2));
   }
 }
 
@@ -261,18 +259,18 @@ int bucket_scan_chunks(int n) { return (n + kScanChunk - 1) / kScanChunk; }
 size_t bucket_chunk_count_ints(int n_sl, int n) { return (size_t)n_sl * bucket_scan_chunks(n) * kCountCols; }
 
 cudaError_t launch_bucket_route(const Geom& G, const void* V, int n_sl, int n, int n_buckets, int i_top, float rho2,
-                                const BucketIn* in, unsigned* vmax2_bits, float* ns, int8_t* slot, int32_t* rank,
+                                BucketIn* in, float* ns, int8_t* slot, int32_t* rank,
                                 int32_t* chunk_cnt, BucketOut* out, const int8_t* forced_slot, cudaStream_t st) {
   const int chunks = G.d * (G.is_bf16 ? 2 : 4) / 16;
   const PdlConfig norms(dim3((n + kRowsPerBlock - 1) / kRowsPerBlock, n_sl), 256, 0, st);
-  cudaError_t e = cudaLaunchKernelEx(&norms.cfg, G.is_bf16 ? bucket_norms_kernel<true> : bucket_norms_kernel<false>, V, n, chunks, ns, vmax2_bits);
+  cudaError_t e = cudaLaunchKernelEx(&norms.cfg, G.is_bf16 ? bucket_norms_kernel<true> : bucket_norms_kernel<false>, V, n, chunks, ns, in);
   const int n_chunks = bucket_scan_chunks(n);
   const PdlConfig scan(dim3(n_chunks, n_sl), kScanThreads, 0, st);
   if (e == cudaSuccess)
-    e = cudaLaunchKernelEx(&scan.cfg, bucket_scan_kernel, static_cast<const float*>(ns), n, n_chunks, n_buckets, i_top, rho2, in,
-                           static_cast<const unsigned*>(vmax2_bits), slot, rank, chunk_cnt, forced_slot);
+    e = cudaLaunchKernelEx(&scan.cfg, bucket_scan_kernel, static_cast<const float*>(ns), n, n_chunks, n_buckets, i_top, rho2,
+                           static_cast<const BucketIn*>(in), slot, rank, chunk_cnt, forced_slot);
   const PdlConfig prefix(dim3(n_sl), kCountCols * 32, 0, st);
-  return e != cudaSuccess ? e : cudaLaunchKernelEx(&prefix.cfg, bucket_prefix_kernel, n_chunks, rho2, in, vmax2_bits, chunk_cnt, out);
+  return e != cudaSuccess ? e : cudaLaunchKernelEx(&prefix.cfg, bucket_prefix_kernel, n_chunks, rho2, static_cast<const BucketIn*>(in), chunk_cnt, out);
 }
 
 cudaError_t launch_bucket_scatter(const Geom& G, const Arena& A, const void* K, const void* V, int n_sl, int n,

@@ -165,6 +165,21 @@ def test_bucketed_per_stream_entry_and_refusals(cuda_lib, capacity):
         assert all(sum(ctx.level_sizes(0, s, 1)) <= capacity for s in range(4))
 
 
+def test_refused_block_leaves_no_maximum_behind(cuda_lib):
+    """The largest value norm of a block that was refused has no part in the next one's erasures."""
+    d, n = 64, 200
+    ctx = cuda_lib.Context(n_seqs=1, n_layers=4, n_kv_heads=1, n_q_heads=1, head_dim=d, dtype="fp32", block=64, levels=1, max_tokens=2 * n)
+    K = torch.randn(n, d, device="cuda")
+    V = torch.zeros(n, d, device="cuda")
+    V[:, 0] = 0.75                                            # bucket 0
+    with pytest.raises(Exception):
+        ctx.stream_append_bucketed(0, 0, 4, 3, 0, K, 1000 * V, 0.5)     # above 2^3
+    counts = ctx.stream_append_bucketed(0, 0, 4, 3, 0, K, V, 0.5)
+    assert [int(x) for x in counts] == [0, 0, 0, n, 0]        # erased: 2^i <= 0.375, not 2^i <= 375
+    assert ctx.stats()["device_status"] == 0
+    ctx.close()
+
+
 def test_bucketed_llama_layer_full_size_sampled_instances(cuda_lib):
     """The one-layer Llama-3.1-8B-shaped workload (8 KV heads x 32768 tokens, d = 128, bf16, block
     1024, T = 2) through the bucketed path: routing of every row of every stream against a direct

@@ -64,7 +64,7 @@ constexpr int kTmaWarp = kEpiWarps, kMmaWarp = kEpiWarps + 1, kMmaWarpV = kEpiWa
 constexpr int kEpiThreads = 32 * kEpiWarps;
 constexpr int kThreads = kEpiThreads + 32 * 4;   // a 20th warp idles: it takes no registers from the others (96 each), and the code
                                                  // for 20 warps is the faster one (592 calls of 1024: 189 us, with 19 warps 193)
-constexpr int kSplitRegs = 96;
+constexpr int kRegs = 96;                  // 20 warps: five on each of the SM's four register files
 constexpr uint32_t kHalfBytes = 16384;     // [128 rows][64 bf16] = one swizzle-atom column of a tile
 template <int D>
 constexpr uint32_t kTileBytesOf = (D / 64) * kHalfBytes;   // a K or V tile: [128 rows][d bf16]
@@ -319,7 +319,7 @@ __device__ inline void copy_rows(const Geom& G, const Arena& A, int src_row, int
 }
 
 template <int D, bool kCenter, int kOrder>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __maxnreg__(kRegs)
 walk_tc_kernel(Geom G, const CallSet calls, int resident, int level, const CallStat* __restrict__ stats,
                const float* __restrict__ tok_shift, int8_t* __restrict__ dbg_eta,
                float* __restrict__ dbg_S, float* __restrict__ dbg_p, unsigned long long* __restrict__ fail_count,
@@ -434,11 +434,12 @@ walk_tc_kernel(Geom G, const CallSet calls, int resident, int level, const CallS
   // r + 1 follow the last column but one into its slot, and the slots change roles.  All sides walk the same schedule and
   // count a slot's loads alike.  Every barrier is waited on phase by phase by its one kind of waiter, and each next phase
   // depends on that waiter having passed, so a parity wait can never be a phase behind.
-  // kSplit: the two branches' register counts as they are (96), but the compiler allocates the branches apart (592 calls of 1024 x 128:
-  // 195 -> 191 us; 64-dim heads 165 -> 179, tiles in reuse order 130 either way: without).
+  // kSplit: the two branches' register counts as they are, but the compiler allocates the branches apart (592 calls of 1024 x 128:
+  // 198 -> 194 us; 64-dim heads 165 -> 179, tiles in reuse order 130 either way: without).  A kernel that
+  // holds setmaxnreg is launched with exactly the registers that __maxnreg__ names.
   constexpr bool kSplit = D == 128 && !kReuse;
   if (warp >= kTmaWarp) {
-    if constexpr (kSplit) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kSplitRegs));
+    if constexpr (kSplit) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegs));
     if (warp == kTmaWarp) {
       // ------------------------------------------------------------------ TMA producer
       if (lane == 0) {
@@ -546,7 +547,7 @@ walk_tc_kernel(Geom G, const CallSet calls, int resident, int level, const CallS
       if (lane == 0 && *abort_flag) atomicCAS(status, kStatusOk, kStatusWaitTimeout);
     }
   } else {
-    if constexpr (kSplit) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kSplitRegs));
+    if constexpr (kSplit) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegs));
     // ------------------------------------------------------------------ four epilogue warpgroups
     // Every tile is drained by all groups: group wg takes columns 32 wg .. 32 wg + 31 of the tile
     // (thread = row) and keeps a partial running correlation of its row over those columns.
@@ -806,10 +807,6 @@ cudaError_t walk_tc_prepare(const Geom& G, const Arena& A, int64_t total_rows, v
   for (int i = 0; i < 6 && e == cudaSuccess; ++i) {
     auto kern = kernel_for(G.d, (i & 1) != 0, i / 2);
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
-    // a kernel that names its branches' registers (kSplitRegs) has to be launched with that many
-    cudaFuncAttributes attr;
-    if (e == cudaSuccess && i / 2 == kAscending && G.d == 128 && (e = cudaFuncGetAttributes(&attr, kern)) == cudaSuccess && attr.numRegs != kSplitRegs)
-      e = cudaErrorInvalidConfiguration;
   }
   if (e != cudaSuccess) { delete tm; return e; }
   *tmaps_out = tm;

@@ -359,7 +359,7 @@ walk_tc_kernel(Geom G, const CallSet calls, int resident, int level, const CallS
     uint64_t* bar = full + 6 * x + 2 * slot + h;
     mbar_expect_tx(bar, kHalfBytes);
     unsigned char* dst = sm + slot * kSlotBytes + (x ? kTileBytes : 0u) + h * kHalfBytes;
-    if (kLeaving && row0 - job->src_row >= 5 * P / 8 * kTile) tma_load_2d_leaving(dst, map, 64 * h, row0, bar);   // panels that few later ones read again
+    if (kLeaving && row0 - job->src_row >= 9 * P / 16 * kTile) tma_load_2d_leaving(dst, map, 64 * h, row0, bar);   // panels that few later ones read again
     else tma_load_2d(dst, map, 64 * h, row0, bar);
   };
   if (warp == kTmaWarp && lane == 0) {
@@ -752,11 +752,12 @@ size_t tc_smem_bytes(int d, int t) {
 constexpr size_t kMaxSmem = (size_t)227 * 1024;         // of every kernel: the limit belongs to the device, not to the context that sets it
 // The order of a panel's columns is the order of summation of S_j, so it follows from the block alone: a call keeps the same
 // tokens whatever else shares its launch.  Tiles are reused from 1792 tokens on, where the rows of one call per SM exceed L2
-// (148 x 1792 x 512 bytes against 126 MB).  Ascending order / reuse, us per launch: 2048 tokens, 1 call 132.4 / 128.4, 148
-// calls 181 / 169, 1024 calls 1265 / 1185; 3072 tokens, 148 calls 428 / 388.
+// (148 x 1792 x 512 bytes against 126 MB).  Ascending order / reuse, us per launch, as measured when the order was chosen: 2048
+// tokens, 1 call 132.4 / 128.4 (130 to 132 now), 148 calls 181 / 169 (167), 1024 calls 1265 / 1185; 3072 tokens, 148 calls 428 / 388.
 constexpr int kReuseTokens = 1792;
-// With more rows resident than L2 holds, the late panels of a call leave it first: 512 streams x 8192 tokens, t = 2048: 3515 us without,
-// 3434 / 3459 / 3514 from panel 9 / 11 / 13 of 16 on.  With fewer they must stay (one call of 3072: 267 without, 284 with).
+// With more rows resident than L2 holds, the late panels of a call leave it first, those from 9/16 on.  592 calls, us, from 9 / 10 /
+// 11 / 13 sixteenths on / without: 2048 tokens 665 / 668 / 671 / 677 / 672, 2560 tokens 1065 / 1078 / 1081 / 1097 / 1090; of 3072 and
+// 3456 tokens runs differ by 4 %, and no choice by more.  With fewer rows they must stay (one call of 3072: 267 without, 284 with).
 int order_of(const Geom& G, int n_calls, int sm_count, int l2_bytes) {
   if (G.d != 128 || G.t < kReuseTokens) return kAscending;
   return (int64_t)std::min(n_calls, sm_count) * G.t * G.d * 4 > l2_bytes ? kReuseLeaving : kReuseStaying;

@@ -70,7 +70,7 @@ struct balancekv_ctx {
   int max_calls = 0;
   CallStat* d_stats = nullptr;
   float* d_tokshift = nullptr;
-  int8_t* d_eta = nullptr;
+  int8_t* d_eta = nullptr;       // signs of the CUDA-core walk, for the compaction
   float* d_ghat = nullptr;       // workspace of the CUDA-core walk: ghat_calls calls
   int ghat_calls = 0;
   unsigned long long* d_fail = nullptr;
@@ -201,7 +201,9 @@ int dev_alloc(balancekv_ctx* c, T** p, size_t count) {
   return BALANCEKV_OK;
 }
 
-// Copies a host array into the descriptor ring and returns its device address.
+// Copies a host array into the descriptor ring and returns its device address.  upload_kernel writes ahead of its grid dependency:
+// what it overwrites is free, because a half is entered again only behind the event recorded when it was left, and every push's
+// consumer is launched before the next push.
 int ring_push(balancekv_ctx* c, const void* data, size_t bytes, cudaStream_t st, void** dev) {
   const size_t need = (bytes + 255) & ~(size_t)255;
   if (need > c->ring_half) return BALANCEKV_E_NOMEM;
@@ -365,7 +367,6 @@ int balancekv_create(const balancekv_config* cfg, balancekv_ctx** out) {
   if (cudaMemset(c->A.V, 0, (size_t)c->total_rows * row_bytes) != cudaSuccess) return fail(BALANCEKV_E_CUDA);
   if (T > 0) {
     if ((rc = dev_alloc(c, &c->d_stats, (size_t)c->max_calls))) return fail(rc);
-    if ((rc = dev_alloc(c, &c->d_eta, (size_t)c->max_calls * t))) return fail(rc);
     if (G.center_keys && (rc = dev_alloc(c, &c->d_tokshift, (size_t)c->max_calls * t + 64))) return fail(rc);
   }
   if ((rc = dev_alloc(c, &c->d_fail, 1))) return fail(rc);
@@ -402,6 +403,7 @@ int balancekv_create(const balancekv_config* cfg, balancekv_ctx** out) {
   if (c->use_tc && walk_tc_prepare(G, c->A, c->total_rows, &c->tmaps) != cudaSuccess) return fail(BALANCEKV_E_CUDA);
   if (T > 0 && !c->use_tc) {
     if (!walk_simt_supported(G.d)) return fail(BALANCEKV_E_INVAL);
+    if ((rc = dev_alloc(c, &c->d_eta, (size_t)c->max_calls * t))) return fail(rc);
     // Workspace of the CUDA-core walk: the kernel matrices of a group of calls.  Up to 512 MB, or 32 calls of long blocks,
     // because walk_kernel runs on as many SMs as a group has calls (148 calls of 4096 x 64 fp32: 512 MB = 15 calls
     // 15.4 ms, 32 calls 12.2; 148 of 1024 x 128: 64 MB 1.37 ms, 256 MB 1.18, 512 MB 1.12).  No more than half of the memory

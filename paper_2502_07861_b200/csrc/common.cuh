@@ -155,8 +155,9 @@ __host__ __device__ inline CallDesc call_of(const CallSet& S, const Geom& G, int
 }
 
 // Launches with programmatic stream serialization: the kernel may become resident while its predecessor on the stream is
-// finishing.  Every such kernel calls grid_wait() before it touches anything that an earlier kernel writes or reads; it
-// then releases its own dependents, which wait for its end in the same way.
+// finishing.  Every such kernel calls grid_wait_and_release() before it touches anything that an earlier kernel writes or reads
+// (upload_kernel alone writes before: ring_push hands it memory that no earlier kernel still reads); it then releases its own
+// dependents, which wait for its end in the same way.
 struct PdlConfig {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr;

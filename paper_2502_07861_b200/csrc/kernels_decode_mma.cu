@@ -142,8 +142,6 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
                   const StepAppend ap, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV) {
   constexpr int kStages = Dim<D>::kStages, kBars = Dim<D>::kBars, PS = Dim<D>::PS, kColWarps = Dim<D>::kColWarps;
   constexpr uint32_t kTensorBytes = Dim<D>::kTensorBytes, kStageBytes = Dim<D>::kStageBytes;
-  constexpr int kRowPieces = D / 8;                // 16-byte pieces of a row
-  constexpr int kLines = D / 64;                   // 128-byte lines of a row
   float* part = part_base;
   float* raw_acc = ap.raw_acc;
   float* raw_ml = ap.raw_ml;
@@ -210,7 +208,6 @@ decode_mma_kernel(Geom G, Arena A, int layer, const __nv_bfloat16* __restrict__ 
     unsigned char* st = tiles + (size_t)(i % kStages) * kStageBytes;
     uint64_t* bar = &full[i % kBars];
     mbar_expect_tx(bar, keys_only ? kTensorBytes : kStageBytes);
-#pragma unroll
     if (kLeaving && i < n_leaving) {
 #pragma unroll
       for (int b = 0; b < D / 64; ++b) tma_load_3d_leaving(st + b * kHalf, &tmK, 64 * b, tr.row, stream, bar);

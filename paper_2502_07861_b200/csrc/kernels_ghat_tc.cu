@@ -48,7 +48,7 @@ using namespace tc;
 
 constexpr int kRows = 128, kCols = 64;                   // a tile
 constexpr int kWorkers = 256, kThreads = kWorkers + 32;
-constexpr uint32_t kPlaneA = kRows * 128, kPlaneB = kCols * 128;      // [rows][64 bf16], 128-byte swizzle
+constexpr uint32_t kPlaneA = kRows * 128, kPlaneB = kCols * 128;      // [rows][64 f16], 128-byte swizzle
 constexpr uint32_t kPlanes = 3 * (kPlaneA + kPlaneB);
 constexpr size_t kSmem = 1024 + kPlanes + 128;
 constexpr float kTiny = 32.f;                            // an element that a1 holds as 0 or +-16 barely has a main part

@@ -194,7 +194,7 @@ __global__ void seg_update_kernel(Arena A, const SegUpdate* __restrict__ ups, in
 }
 
 // Descriptors travel as a kernel's parameters: a transfer between two kernels ends their overlap and took 8 us of a batch's
-// chain where this takes 2.
+// chain where this takes 2.  The destination is written ahead of the grid dependency (see ring_push).
 template <size_t kBytes>
 struct Blob {
   uint4 w[kBytes / 16];

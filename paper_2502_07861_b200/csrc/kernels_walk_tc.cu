@@ -672,9 +672,9 @@ walk_tc_kernel(Geom G, const CallSet calls, int resident, int level, const CallS
       }
       const float thr = thr_s[j];
       // The walk over the panel's 128 tokens by sweeps: group 0 owns the decisions, groups 1-3
-      // supply the partial sums of their columns.  Undecided signs are stored as 0.
+      // supply the partial sums of their columns.
       const float4* e4 = reinterpret_cast<const float4*>(etas + r * kTile + col0);
-      // In sweep 0 (all in-panel signs still 0, S = the earlier panels' part) a row whose distance
+      // In sweep 0 (no in-panel sign is read, S = the earlier panels' part) a row whose distance
       // to its threshold exceeds sum_j |Ghat_ij| of its in-panel columns is already decided; if
       // that holds for every row (and no row can FAIL, and S is not recorded) one sweep suffices.
       float absum = 0.f;

@@ -18,6 +18,7 @@ def _views(ctx):
     (128, "bf16", 256, 2, 0, 1, (256, 768, 1300)),
     (128, "bf16", 192, 2, 5, 0, (400, 192, 777)),
     (64, "fp32", 64, 3, 0, 0, (64, 65, 700, 63, 320)),
+    (128, "fp32", 192, 2, 0, 0, (384, 192, 1000)),
     (64, "bf16", 64, 2, 100, 1, (333, 64, 500)),
     (128, "bf16", 2048, 2, 0, 0, (4096, 2048, 6200)),
 ])

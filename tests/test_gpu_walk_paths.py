@@ -28,7 +28,8 @@ def _run(cuda_lib, d, dtype, t, T, center, tol, walk_kernel, **kw):
 
 
 @pytest.mark.parametrize("d", [64, 128])
-@pytest.mark.parametrize("t,T,center", [(128, 1, 0), (192, 2, 0), (192, 1, 1), (320, 1, 0), (1088, 1, 0), (2048, 1, 0), (2560, 1, 0)])
+@pytest.mark.parametrize("t,T,center", [(128, 1, 0), (192, 2, 0), (192, 1, 1), (320, 1, 0), (1088, 1, 0), (2048, 1, 0), (2560, 1, 0),
+                                        (1856, 1, 1), (2048, 1, 1)])
 def test_tensor_core_walk_with_ragged_panels(cuda_lib, d, t, T, center):
     """Whole panels and a last panel of 64 tokens; d = 64 operands are a single 64-dim box."""
     _run(cuda_lib, d, "bf16", t, T, center, 5e-4 if center else 2e-4, 2)
@@ -123,7 +124,8 @@ def test_cuda_core_walk_in_groups_of_calls(cuda_lib):
     one.close()
 
 
-def test_tensor_core_walk_beyond_l2(cuda_lib):
+@pytest.mark.parametrize("center", [0, 1])
+def test_tensor_core_walk_beyond_l2(cuda_lib, center):
     """Resident calls whose rows exceed L2 (148 of 2048 tokens) keep what the walk of each stream alone keeps."""
     import torch
 
@@ -132,7 +134,7 @@ def test_tensor_core_walk_beyond_l2(cuda_lib):
     K = (0.3 * torch.randn(1, S, t, d, device="cuda", generator=gen)).bfloat16()
     V = torch.randn(1, S, t, d, device="cuda", generator=gen).bfloat16()
     make = lambda: cuda_lib.Context(n_seqs=1, n_layers=1, n_kv_heads=S, n_q_heads=S, head_dim=d, dtype="bf16", block=t, levels=1,
-                                    max_tokens=t, seed=3, c_override=0.75)
+                                    max_tokens=t, seed=3, c_override=0.75, center_keys=center)
     ctx, one = make(), make()
     ctx.stream_append_layer(0, K, V)
     ctx.compress()

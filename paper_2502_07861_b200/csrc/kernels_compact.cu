@@ -40,7 +40,7 @@ __device__ inline int block_exclusive_scan(int v, int* warp_sums, int& total) {
 }
 
 __global__ void __launch_bounds__(kThreads)
-compact_kernel(Geom G, Arena A, const CallSet calls, const int8_t* __restrict__ eta, const BatchTail tail) {
+compact_kernel(Geom G, Arena A, const CallSet calls, const int8_t* __restrict__ eta, const __grid_constant__ BatchTail tail) {
   extern __shared__ int kept_pos[];  // [t/2]
   __shared__ int warp_sums[kThreads / 32];
   grid_wait_and_release();
@@ -87,7 +87,9 @@ compact_kernel(Geom G, Arena A, const CallSet calls, const int8_t* __restrict__ 
   uint4* Kd = static_cast<uint4*>(A.K) + ((size_t)C.dst_row << sh);
   uint4* Vd = static_cast<uint4*>(A.V) + ((size_t)C.dst_row << sh);
   // A piece per thread and pass: the CTAs' chains of scans hide one another, eight per SM.  With eight loads in flight per thread
-  // (61 registers, four CTAs) a pass of 2048 calls of 64 x 128 bf16 took 188.3 us for the 181.8, one of 592 fp32 calls and less the same.
+  // (61 registers, four CTAs) a pass of 2048 calls of 64 x 128 bf16 took 188.3 us for 181.8, one of few calls the same; and 176.8 now
+  // that the tail is a grid constant (its segments are picked by a dynamic index, for which every thread of a plain parameter
+  // keeps a copy in local memory).
   for (int i = threadIdx.x; i < items; i += kThreads) {
     const int o = i >> (sh + 1), ch = i & (chunks - 1);
     const bool value = (i >> sh) & 1;

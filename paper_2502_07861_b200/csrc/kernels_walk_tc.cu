@@ -333,12 +333,24 @@ walk_tc_kernel(Geom G, const CallSet calls, int resident, int level, const CallS
   // t is a multiple of 64: the last panel may hold 64 tokens only.  Its tile then covers 64 rows that are not the
   // call's; what is computed for them goes nowhere.
   const int t = G.t, P = (t + kTile - 1) / kTile, tp = P * kTile;
-  float* etas = reinterpret_cast<float*>(sm + Smem<D>::kTilesEnd);       // [tp] signs scaled by 1/r_value^2
-  float* xs = etas + tp;                                                   // [3][128] partial correlations of column quarters 1..3
-  float* xb = xs + (kEpiGroups - 1) * kTile;                              // [3][128] ... and of their sums of |Ghat|
-  float* thr_s = xb + (kEpiGroups - 1) * kTile;                           // [tp] decision thresholds c (1 - 2 u_j)
-  uint16_t* kept = reinterpret_cast<uint16_t*>(thr_s + tp);               // [tp / 2] positions of the tokens kept
-  uint64_t* bars = reinterpret_cast<uint64_t*>(kept + tp / 2);
+  float *etas, *xs, *xb, *thr_s;
+  uint16_t* kept;
+  uint64_t* bars;
+  if constexpr (kReuse) {            // what has a fixed size first: its addresses are constants
+    bars = reinterpret_cast<uint64_t*>(sm + Smem<D>::kTilesEnd);
+    xs = reinterpret_cast<float*>(sm + Smem<D>::kTilesEnd + kMiscBytes);
+    xb = xs + (kEpiGroups - 1) * kTile;
+    etas = xb + (kEpiGroups - 1) * kTile;
+    thr_s = etas + tp;
+    kept = reinterpret_cast<uint16_t*>(thr_s + tp);
+  } else {
+    etas = reinterpret_cast<float*>(sm + Smem<D>::kTilesEnd);       // [tp] signs scaled by 1/r_value^2
+    xs = etas + tp;                                                   // [3][128] partial correlations of column quarters 1..3
+    xb = xs + (kEpiGroups - 1) * kTile;                              // [3][128] ... and of their sums of |Ghat|
+    thr_s = xb + (kEpiGroups - 1) * kTile;                           // [tp] decision thresholds c (1 - 2 u_j)
+    kept = reinterpret_cast<uint16_t*>(thr_s + tp);               // [tp / 2] positions of the tokens kept
+    bars = reinterpret_cast<uint64_t*>(kept + tp / 2);
+  }
   // x = 0: the K K^T product, x = 1: the V V^T product
   // An operand tile travels as two boxes of 64 dims (h = 0, 1); a box is refilled as soon as the
   // four MMAs that read it are done, which lengthens the prefetch distance of the column ring.
@@ -437,7 +449,7 @@ walk_tc_kernel(Geom G, const CallSet calls, int resident, int level, const CallS
   // kSplit: the two branches' register counts as they are, but the compiler allocates the branches apart (592 calls of 1024 x 128:
   // 198 -> 194 us; 64-dim heads 165 -> 179, tiles in reuse order 130 either way: without).  A kernel that
   // holds setmaxnreg is launched with exactly the registers that __maxnreg__ names.
-  constexpr bool kSplit = D == 128 && !kReuse;
+  constexpr bool kSplit = D == 128;
   if (warp >= kTmaWarp) {
     if constexpr (kSplit) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegs));
     if (warp == kTmaWarp) {

@@ -821,10 +821,17 @@ static SplitPlan pick_splits(const balancekv_ctx* c, int64_t tiles, int n) {
 // The layers' caches are read in turn, token after token.  Together larger than L2, they push one another out of it, so the
 // share beyond 5/8 of L2 is loaded to leave first.  It is made of every CTA's first tiles, which a chain of launches fetches
 // ahead; the rest, whose latency shows, stays.  16 tokens, 8 streams x 8192 rows, 4 layers (135 MB): 753 us without, 692 / 693 / 696 / 733
-// with 60 / 80 / 100 / 115 MB kept; 3 layers 535 / 513, 8 layers 1502 / 1440, 16 layers 2994 / 2973 (80 MB); one token of 24 streams x
-// 5000 rows, 8 layers 125 / 121; 256 streams x 16384 rows 602 / 600.
-static float l2_leaving(const balancekv_ctx* c, int64_t tiles) {
+// with 60 / 80 / 100 / 115 MB kept.
+// Where it applies, with 70 to 200 MB of caches, with / without in us per token.  Plain decode: always (24 streams, 3 layers of 125 MB 30.6 /
+// 33.7, 8 layers of 105 MB 51.2 / 52.9; 8 streams, 16 layers of 88 MB 95.3 / 98.1; at worst the same).  Steps with combining
+// CTAs of their own: always (8 streams, 4 layers of 140 MB 40.4 / 43.4; 8 layers of 102 MB 54.0 / 55.9).  Steps combined by a
+// stream's last split: from 3.75 tiles per CTA on with more than 12 splits (16 streams, 4 layers of 120 MB 39.2 / 41.1; with two
+// tiles per CTA 8 streams, 16 layers of 105 MB 114.2 / 108.0), from 5.5 on with fewer (48 streams, 2 layers of 135 MB 28.1 / 30.7, 64
+// streams, one of 115 MB 21.0 / 24.6; with 5 and fewer 48 streams of 88 MB 21.5 / 20.3, 32 streams, 4 layers of 102 MB 36.7 / 34.0).
+// (A stream's share spread evenly over its splits in place of the whole tiles of every CTA: 1 to 3 % slower throughout.)
+static float l2_leaving(const balancekv_ctx* c, int64_t tiles, const SplitPlan& plan, bool step) {
   if (!c->decode_maps) return 0.f;
+  if (step && plan.inline_combine && 4 * tiles < (int64_t)plan.splits * (plan.splits > 12 ? 15 : 22)) return 0.f;
   const double all = (double)c->n_streams * (double)tiles * decode_mma_tile_tokens() * 2.0 * c->cfg.head_dim * c->esz;
   const double keep = 0.625 * c->l2_bytes;
   return all <= keep ? 0.f : (float)(1.0 - keep / all);
@@ -857,7 +864,7 @@ static int launch_decode_step(balancekv_ctx* c, int layer, const void* q, void* 
   }
   const int64_t tiles = decode_tiles(c, layer, alike ? ap.seg : nullptr);
   const SplitPlan plan = pick_splits(c, tiles, c->cfg.n_seqs * c->cfg.n_kv_heads);
-  ap.leaving = l2_leaving(c, tiles);
+  ap.leaving = l2_leaving(c, tiles, plan, k_new != nullptr);
   ap.splits = plan.splits;
   ap.inline_combine = plan.inline_combine;
   ap.in_flag = c->step_flag;

@@ -83,21 +83,21 @@ def decode_case(B, H, g, d, Lc, T, iters=50, max_layers=16, two_instance=False, 
 
 def run_compress(a):
     print(json.dumps(compress_case(a.streams, a.head_dim, a.context, a.block, a.levels, iters=a.iters, gram_path=a.gram_path,
-                                   c_override=a.c_override, outliers=a.outliers, window=a.window)))
+                                   c_override=a.c_override, outliers=a.outliers, window=a.window, dtype=a.dtype)))
 
 
-def compress_case(S, d, n, t, T, iters=10, gram_path=0, c_override=0.0, outliers=1, window=0):
+def compress_case(S, d, n, t, T, iters=10, gram_path=0, c_override=0.0, outliers=1, window=0, dtype="bf16"):
     """append + compress of `S` streams (one layer), timed per kernel class; returns a dict."""
     import types
 
     a = types.SimpleNamespace(iters=iters, gram_path=gram_path, c_override=c_override, outliers=outliers)
-    ctx = bk.Context(n_seqs=1, n_layers=1, n_kv_heads=S, n_q_heads=S, head_dim=d, dtype="bf16", block=t, levels=T,
+    ctx = bk.Context(n_seqs=1, n_layers=1, n_kv_heads=S, n_q_heads=S, head_dim=d, dtype=dtype, block=t, levels=T,
                      max_tokens=n, gram_path=a.gram_path, c_override=a.c_override, recent_window=window)
     K = torch.randn(1, S, n, d, device="cuda", dtype=torch.float32)
     if a.outliers:
         K[..., :4] *= 10.0
-    K = K.to(torch.bfloat16)
-    V = torch.randn(1, S, n, d, device="cuda", dtype=torch.float32).to(torch.bfloat16)
+    K = K.to(ctx.dtype)
+    V = torch.randn(1, S, n, d, device="cuda", dtype=torch.float32).to(ctx.dtype)
     flush = torch.empty(256 << 20, dtype=torch.uint8, device="cuda")
     for _ in range(2):
         ctx.reset(); ctx.stream_append_layer(0, K, V); ctx.compress()
@@ -121,7 +121,7 @@ def compress_case(S, d, n, t, T, iters=10, gram_path=0, c_override=0.0, outliers
     cp_n, cp_ms = prof["compact"]
     hbm, tf, src = _peaks()
     tfl = flop * a.iters / (gw_ms * 1e-3) / 1e12 if gw_ms else 0.0
-    cp_bytes = n_calls * ((t // 2) * (4 * d * 2 + 8 + 16) + t)   # rows, position, norms per survivor, sign bytes
+    cp_bytes = n_calls * ((t // 2) * (4 * d * (2 if dtype == "bf16" else 4) + 8 + 16) + t)   # rows, position, norms per survivor, sign bytes
     cp_gbs = cp_bytes * a.iters / (cp_ms * 1e-3) / 1e9 if cp_ms else 0.0
     st = ctx.stats()
     res = dict(kernel="compress", streams=S, context=n, block=t, levels=T, recent_window=window, calls=n_calls,
@@ -213,6 +213,7 @@ def main():
     c.add_argument("--levels", type=int, default=2)
     c.add_argument("--iters", type=int, default=10)
     c.add_argument("--gram-path", type=int, default=0)
+    c.add_argument("--dtype", choices=["bf16", "fp32"], default="bf16")
     c.add_argument("--c-override", type=float, default=0.0)
     c.add_argument("--outliers", type=int, default=1)
     c.add_argument("--window", type=int, default=0, help="recent window W (tokens kept out of the calls)")

@@ -9,7 +9,7 @@
 //
 // Two kernels.  Ghat does not depend on the signs, so ghat_kernel forms its lower triangle with FFMA over the whole chip
 // (grid: tiles of all calls) into a workspace of 64 x 64 tiles (Geom::split_gram: fp32 rows and blocks from 128 tokens on, the
-// kernel of kernels_ghat_tc.cu does, in 119 us where this one takes 255); walk_kernel (a CTA per call) streams the tiles back by
+// kernel of kernels_ghat_tc.cu does, in 125 us where this one takes 255); walk_kernel (a CTA per call) streams the tiles back by
 // bulk copies, folds the tiles left of the diagonal with the signs that are final, and walks the diagonal tile.
 // What bounds it: the FFMA pipe in the first kernel, the chain of panels and the L2 reads (2 t^2 bytes per call) in the
 // second.  128 calls of 512 fp32 tokens x 128 dims: 253 + 18 us (38 TFLOP/s, half of the FMA pipe's rate; one CTA per call doing both took
